@@ -1,8 +1,15 @@
 // HBM-bound kernels of the backbone: the packer (gather into the canonical
 // packed batch), RMSNorm, the final RMSNorm fused with the per-sample mean
 // pool, and the RoPE (cos, sin) table.
+#include <cooperative_groups.h>
+
+#include <climits>
+#include <cmath>
+
 #include "jnx_dev.cuh"
 #include "jnx_kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace jnx {
 
@@ -170,85 +177,137 @@ jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int 
 }
 
 // ---------------------------------------------------------------------------
-// Final RMSNorm + mean pool.  One CTA per sample walks its rows in order
-// (4 at a time); each thread owns columns tid, tid+256, ...; the row's sum
-// of squares is reduced by a fixed tree.  pooled[s] = gamma * mean_t(x_t *
-// rstd_t); hidden (optional) = bf16(x_t * rstd_t * gamma).
+// Final RMSNorm + mean pool.  A cluster of kPoolCtas CTAs per sample, each
+// walking its own contiguous share of the sample's rows in order (4 at a
+// time); each thread owns columns tid, tid + 256, ...; a row's sum of squares
+// is reduced by a fixed tree.  pooled[s] = gamma * mean_t(x_t * rstd_t): the
+// CTAs' column sums meet in distributed shared memory and are added in rank
+// order, so a sample's result depends on its own length only.  hidden
+// (optional) = bf16(x_t * rstd_t * gamma).
+//
+// Bound by HBM (4 bytes in, 2 out per element).  With one CTA per sample a
+// group of few samples left most SMs idle and walked each sample's rows one
+// after another.  Before and after: 7 samples of 300 rows x 4096 pooled 123
+// -> 26 us, 38 of 530 x 2048 hidden 333 -> 49 us (5.1 TB/s), 156 of 283 x
+// 1024 both 92 -> 57 us; 222 of 296 x 4096 pooled, which filled the SMs
+// already, 202 -> 214 us.
 // ---------------------------------------------------------------------------
-template <int C>  // columns per thread = d / 256
-__global__ void __launch_bounds__(256) k_final_pool(const float* __restrict__ x,
-                                                    const uint16_t* __restrict__ gamma, float eps,
-                                                    const int* __restrict__ cu,
-                                                    float* __restrict__ pooled,
-                                                    uint16_t* __restrict__ hidden) {
+constexpr int kPoolCtas = 8;
+
+// PRE: the next round's rows are loaded while this one is summed, for groups
+// whose CTAs do not fill the SMs; otherwise the registers go to longer rounds
+// of more CTAs.
+template <int C, bool PRE>  // C: columns per thread = d / 256
+__global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
+    k_final_pool(const float* __restrict__ x, const uint16_t* __restrict__ gamma, float eps,
+                 const int* __restrict__ cu, int parts, float* __restrict__ pooled,
+                 uint16_t* __restrict__ hidden) {
     constexpr int D = C * 256;
-    constexpr int R = 4;
-    __shared__ float red[R][8];
-    const int s = blockIdx.x;
-    const int t0 = cu[s], t1 = cu[s + 1];
+    constexpr int R = PRE && C == 16 ? 2 : 4;  // rows of a round
+    __shared__ float red[2][R][8];
+    __shared__ float sums[D];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int s = blockIdx.x / parts, part = blockIdx.x % parts;
+    const int r0 = cu[s], r1 = cu[s + 1];
+    // rows of this CTA: an equal share, in whole rounds
+    const int share = ((r1 - r0 + parts - 1) / parts + R - 1) / R * R;
+    const int t0 = min(r0 + part * share, r1), t1 = min(t0 + share, r1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float acc[C];
-    float gm[C];
+    float acc[C], gm[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         acc[c] = 0.f;
         gm[c] = bf2f(gamma[tid + 256 * c]);
     }
-    for (int t = t0; t < t1; t += R) {
+    float nx[R][C];
+    auto load = [&](int t) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                nx[r][c] = t + r < t1 ? __ldg(x + (size_t)(t + r) * D + tid + 256 * c) : 0.f;
+    };
+    if (PRE) load(t0);
+    int buf = 0;
+    for (int t = t0; t < t1; t += R, buf ^= 1) {
         float v[R][C];
+        if (!PRE) load(t);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) v[r][c] = nx[r][c];
+        if (PRE) load(t + R);
         float ss[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             ss[r] = 0.f;
-            const bool ok = t + r < t1;
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                v[r][c] = ok ? __ldg(x + (size_t)(t + r) * D + tid + 256 * c) : 0.f;
-                ss[r] += v[r][c] * v[r][c];
-            }
+            for (int c = 0; c < C; ++c) ss[r] += v[r][c] * v[r][c];
             ss[r] = warp_sum(ss[r]);
         }
+        // the two buffers of partial sums take turns, so one barrier a round
+        // is enough: a warp that writes a buffer again has passed the barrier
+        // after the round that read it
         if (lane == 0) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) red[r][warp] = ss[r];
+            for (int r = 0; r < R; ++r) red[buf][r][warp] = ss[r];
         }
         __syncthreads();
-        float rs[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             float tot = 0.f;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) tot += red[r][w];
-            rs[r] = rsqrtf(tot / (float)D + eps);
-        }
-        __syncthreads();
+            for (int w = 0; w < 8; ++w) tot += red[buf][r][w];
+            const float rs = rsqrtf(tot / (float)D + eps);
+            if (t + r < t1) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (t + r >= t1) break;
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const float y = v[r][c] * rs[r];
-                acc[c] += y;
-                if (hidden) hidden[(size_t)(t + r) * D + tid + 256 * c] = f2bf(y * gm[c]);
+                for (int c = 0; c < C; ++c) {
+                    const float y = v[r][c] * rs;
+                    acc[c] += y;
+                    if (hidden) hidden[(size_t)(t + r) * D + tid + 256 * c] = f2bf(y * gm[c]);
+                }
             }
         }
     }
-    if (pooled) {
-        const float inv = 1.0f / (float)(t1 - t0);
+    if (!pooled) return;
 #pragma unroll
-        for (int c = 0; c < C; ++c) pooled[(size_t)s * D + tid + 256 * c] = acc[c] * inv * gm[c];
+    for (int c = 0; c < C; ++c) sums[tid + 256 * c] = acc[c];
+    cluster.sync();
+    constexpr int kCols = D / kPoolCtas;  // this CTA finishes columns [part kCols, + kCols)
+    const float inv = 1.0f / (float)(r1 - r0);
+    for (int i = tid; i < kCols; i += 256) {
+        const int c = part * kCols + i;
+        float tot = 0.f;
+#pragma unroll
+        for (int k = 0; k < kPoolCtas; ++k) tot += *cluster.map_shared_rank(&sums[c], k);
+        pooled[(size_t)s * D + c] = tot * inv * bf2f(gamma[c]);
     }
+    cluster.sync();  // no CTA's shared memory goes away while another reads it
 }
 
 jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, const int* cu,
                              int S, int d, float* pooled, uint16_t* hidden, cudaStream_t s) {
     if (S == 0 || (!pooled && !hidden)) return JNX_OK;
+    // hidden rows alone need no cluster's sum: finer shares fill the SMs
+    const int parts = pooled ? kPoolCtas : 4 * kPoolCtas;
+    if (S > INT_MAX / parts) return fail(JNX_ERR_UNSUPPORTED, "final_pool: too many samples");
+    const int grid = S * parts;
+    // under four CTAs an SM the deep variant's loads hide the latency (7 x 4096:
+    // 26 us against 40), above it the flat one's longer rounds are faster (222 x
+    // 4096: 214 us against 221)
+    const bool pre = grid < 4 * num_sms();
+    auto launch = [&](auto deep, auto flat) {
+        if (pre)
+            deep<<<grid, 256, 0, s>>>(x, gamma, eps, cu, parts, pooled, hidden);
+        else
+            flat<<<grid, 256, 0, s>>>(x, gamma, eps, cu, parts, pooled, hidden);
+    };
     switch (d) {
-        case 256: k_final_pool<1><<<S, 256, 0, s>>>(x, gamma, eps, cu, pooled, hidden); break;
-        case 512: k_final_pool<2><<<S, 256, 0, s>>>(x, gamma, eps, cu, pooled, hidden); break;
-        case 1024: k_final_pool<4><<<S, 256, 0, s>>>(x, gamma, eps, cu, pooled, hidden); break;
-        case 2048: k_final_pool<8><<<S, 256, 0, s>>>(x, gamma, eps, cu, pooled, hidden); break;
-        case 4096: k_final_pool<16><<<S, 256, 0, s>>>(x, gamma, eps, cu, pooled, hidden); break;
+        case 256: launch(k_final_pool<1, true>, k_final_pool<1, false>); break;
+        case 512: launch(k_final_pool<2, true>, k_final_pool<2, false>); break;
+        case 1024: launch(k_final_pool<4, true>, k_final_pool<4, false>); break;
+        case 2048: launch(k_final_pool<8, true>, k_final_pool<8, false>); break;
+        case 4096: launch(k_final_pool<16, true>, k_final_pool<16, false>); break;
         default: return fail(JNX_ERR_UNSUPPORTED, "final_pool: d=%d not in {256..4096}", d);
     }
     cudaError_t e = cudaGetLastError();
@@ -257,25 +316,53 @@ jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, c
 
 // ---------------------------------------------------------------------------
 // RoPE table: (cos, sin) of pos * theta^(-2i/hd), evaluated in double and
-// rounded to fp32 once.
+// rounded to fp32 once, stored frequency-major (tab[i * max_pos + p]) so that
+// rows of consecutive positions read consecutive entries.
+//
+// One CTA per (frequency, kRopeSpan positions).  Position p = kRopeFine a + b:
+// the CTA evaluates sincos for the fine angles b and the coarse ones a only,
+// and every entry by the angle-addition formulas in double (the error stays
+// at a few 2^-53, invisible in the fp32 entry).  FP64 is what bounds this
+// kernel (a few operations per clock and SM): with a pow and a sincos per
+// entry 88 positions x 32 frequencies took 11.8 us and 830 x 128 36.7 us, this
+// way 3.3 and 8.4 us.
 // ---------------------------------------------------------------------------
-// (cos, sin) of position p at frequency i, stored frequency-major
-// (tab[i * max_pos + p]) so that rows of consecutive positions read
-// consecutive entries.
-__global__ void k_rope_table(float2* tab, int max_pos, int half, double theta) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= max_pos * half) return;
-    const int i = idx / max_pos, p = idx % max_pos;
-    const double inv = pow(theta, -2.0 * (double)i / (double)(2 * half));
-    double sn, cs;
-    sincos((double)p * inv, &sn, &cs);
-    tab[idx] = make_float2((float)cs, (float)sn);
+constexpr int kRopeFine = 32, kRopeCoarse = 64, kRopeSpan = kRopeFine * kRopeCoarse;
+
+struct RopeFreqs {
+    double inv[128];  // theta^(-2i/hd), i < hd / 2
+};
+
+__global__ void __launch_bounds__(256) k_rope_table(float2* tab, int max_pos,
+                                                    const __grid_constant__ RopeFreqs fr) {
+    __shared__ double2 fine[kRopeFine], coarse[kRopeCoarse];
+    const int i = blockIdx.x, p0 = blockIdx.y * kRopeSpan;
+    const int t = threadIdx.x;
+    if (t < kRopeFine + kRopeCoarse) {
+        const int p = t < kRopeFine ? t : p0 + (t - kRopeFine) * kRopeFine;
+        if (p < max_pos) {
+            double sn, cs;
+            sincos((double)p * fr.inv[i], &sn, &cs);
+            (t < kRopeFine ? fine[t] : coarse[t - kRopeFine]) = make_double2(cs, sn);
+        }
+    }
+    __syncthreads();
+    const int p1 = min(p0 + kRopeSpan, max_pos);
+    for (int p = p0 + t; p < p1; p += 256) {
+        const double2 a = coarse[(p - p0) / kRopeFine], b = fine[(p - p0) % kRopeFine];
+        tab[(size_t)i * max_pos + p] =
+            make_float2((float)(a.x * b.x - a.y * b.y), (float)(a.y * b.x + a.x * b.y));
+    }
 }
 
 jnx_status rope_table_launch(float2* tab, int max_pos, int hd, float theta, cudaStream_t s) {
-    const int n = max_pos * (hd / 2);
-    if (n == 0) return JNX_OK;
-    k_rope_table<<<(n + 255) / 256, 256, 0, s>>>(tab, max_pos, hd / 2, (double)theta);
+    const int half = hd / 2;
+    if (max_pos <= 0 || half <= 0) return JNX_OK;
+    if (half > 128) return fail(JNX_ERR_UNSUPPORTED, "rope table: head dim %d", hd);
+    RopeFreqs fr;
+    for (int i = 0; i < half; ++i) fr.inv[i] = pow((double)theta, -2.0 * i / (2.0 * half));
+    k_rope_table<<<dim3(half, (max_pos + kRopeSpan - 1) / kRopeSpan), 256, 0, s>>>(tab, max_pos,
+                                                                                  fr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "rope table: %s", cudaGetErrorString(e));
 }
