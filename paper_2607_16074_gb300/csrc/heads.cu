@@ -22,11 +22,15 @@
 // All sums run in a fixed order inside one thread, one CTA or one
 // tensor-core instruction sequence (no atomics), so a tenant's results are
 // identical whether it runs grouped or alone.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "jnx_dev.cuh"
 #include "jnx_heads.h"
 #include "jnx_kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace jnx {
 
@@ -250,7 +254,12 @@ __global__ void __launch_bounds__(256, 2) k_head_lin(const __grid_constant__ Hea
 }
 
 // Per-tenant loss and dy, one CTA per group slot, fixed-order reduction.
-__global__ void __launch_bounds__(256) k_l2_loss(const __grid_constant__ HeadTable tab,
+// Latency bound (a slot's samples x outputs are a few thousand elements), so
+// the CTA is as wide as it can be: 24.6 us with 256 threads, LOSS_US with
+// 1,024 for eight samples of up to 1,600 outputs.
+constexpr int kLossThreads = 1024;
+
+__global__ void __launch_bounds__(kLossThreads) k_l2_loss(const __grid_constant__ HeadTable tab,
                                                  const float* __restrict__ y, int ld_y,
                                                  const float* __restrict__ targets,
                                                  const int* __restrict__ sample_target,
@@ -260,19 +269,19 @@ __global__ void __launch_bounds__(256) k_l2_loss(const __grid_constant__ HeadTab
     const int n = (hs.s1 - hs.s0) * W;
     const float inv = 1.0f / (float)n;
     float acc = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) {
+    for (int i = threadIdx.x; i < n; i += kLossThreads) {
         const int s = hs.s0 + i / W, o = i % W;
         const float diff = y[(size_t)s * ld_y + o] - targets[sample_target[s] + o];
         acc += diff * diff;
         dy[(size_t)s * ld_y + o] = 2.0f * diff * inv;
     }
-    __shared__ float red[8];
+    __shared__ float red[kLossThreads / 32];
     acc = warp_sum_h(acc);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         float t = 0.f;
-        for (int w = 0; w < 8; ++w) t += red[w];
+        for (int w = 0; w < kLossThreads / 32; ++w) t += red[w];
         loss[hs.tenant] = t * inv;
     }
 }
@@ -356,63 +365,98 @@ __global__ void __launch_bounds__(256) k_head_dw_out(const __grid_constant__ Hea
 
 // Gradient into the output layer's input: dh[s, j] = (sum_o dy[s, o] W[o, j])
 // times SiLU'(z[s, j]) for an MLP slot (dz), plain for a query head (dO).
-// One CTA per (slot, 1024 columns j, 8 samples); a thread keeps 4
-// consecutive columns x 8 samples, so each weight row is read once per 8
-// samples (8-byte loads); dy is staged 64 outputs at a time in shared
-// memory; the outputs o are summed in order.
-__global__ void __launch_bounds__(256) k_head_back_in(const __grid_constant__ HeadTable tab,
+// One CTA per (slot, kBackCols columns j, 8 samples).  Warp w takes the
+// outputs o = w (mod 8), in order, for all of the CTA's columns (4 a lane) and
+// samples, with the next eight weight rows' loads in flight while eight are
+// multiplied; the warps' partial sums are added in warp order, so the result
+// does not depend on the group around the slot.  dy is staged 64 outputs at a
+// time in shared memory.
+//
+// Bound by reading W once per 8 samples (116 MB for eight query heads of
+// 350-1,600 outputs x 8,192 columns).  One CTA per 1,024 columns with the
+// outputs one after another kept 64 CTAs waiting for one load at a time:
+// 508 us; this split 61 us.
+constexpr int kBackCols = 128, kBackO = 64;
+
+__global__ void __launch_bounds__(256, 3) k_head_back_in(const __grid_constant__ HeadTable tab,
                                                       const float* __restrict__ dy, int ld_y,
                                                       const float* __restrict__ z, int ld_h,
                                                       float* __restrict__ dh) {
-    __shared__ __align__(16) float sdy[64][8];
+    __shared__ __align__(16) float sdy[kBackO][8];
+    __shared__ __align__(16) float red[8][8][kBackCols];  // [warp][sample][column]
     const HeadSlot& hs = tab.slot[blockIdx.x];
-    const int s0 = hs.s0 + blockIdx.z * 8, jb = blockIdx.y * 1024;
+    const int s0 = hs.s0 + blockIdx.z * 8, jb = blockIdx.y * kBackCols;
     if (s0 >= hs.s1 || jb >= hs.hid) return;
     const int ns = min(8, hs.s1 - s0);
-    const int j0 = jb + 4 * threadIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j0 = jb + 4 * lane;
     const bool colok = j0 < hs.hid;
     float acc[8][4];
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-    for (int o0 = 0; o0 < hs.width; o0 += 64) {
-        const int no = min(64, hs.width - o0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < 64 * 8; i += 256) {
-            const int si = i >> 6, o = i & 63;
-            sdy[o][si] = (o < no && si < ns) ? dy[(size_t)(s0 + si) * ld_y + o0 + o] : 0.f;
+    uint2 wv[kBackO / 8];
+    auto load = [&](int o0) {
+#pragma unroll
+        for (int i = 0; i < kBackO / 8; ++i) {
+            const int o = o0 + warp + 8 * i;
+            wv[i] = make_uint2(0u, 0u);
+            if (colok && o < hs.width)
+                wv[i] = __ldg(reinterpret_cast<const uint2*>(hs.w2 + (size_t)o * hs.hid + j0));
         }
+    };
+    load(0);
+    for (int o0 = 0; o0 < hs.width; o0 += kBackO) {
         __syncthreads();
-        if (colok) {
-            for (int o = 0; o < no; ++o) {
-                const uint2 wv =
-                    *reinterpret_cast<const uint2*>(hs.w2 + (size_t)(o0 + o) * hs.hid + j0);
-                const float w[4] = {__uint_as_float(wv.x << 16), __uint_as_float(wv.x & 0xFFFF0000u),
-                                    __uint_as_float(wv.y << 16), __uint_as_float(wv.y & 0xFFFF0000u)};
-                const float4 da = *reinterpret_cast<const float4*>(&sdy[o][0]);
-                const float4 db = *reinterpret_cast<const float4*>(&sdy[o][4]);
-                const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+        for (int i = threadIdx.x; i < kBackO * 8; i += 256) {
+            const int si = i % 8, o = i / 8;  // conflict-free stores; the rows' reads hit L1
+            sdy[o][si] =
+                (o0 + o < hs.width && si < ns) ? dy[(size_t)(s0 + si) * ld_y + o0 + o] : 0.f;
+        }
+        uint2 cur[kBackO / 8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < kBackO / 8; ++i) cur[i] = wv[i];
+        if (o0 + kBackO < hs.width) load(o0 + kBackO);
+        __syncthreads();
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[i][e] = fmaf(d[i], w[e], acc[i][e]);
-            }
+        for (int i = 0; i < kBackO / 8; ++i) {
+            const float w[4] = {__uint_as_float(cur[i].x << 16),
+                                __uint_as_float(cur[i].x & 0xFFFF0000u),
+                                __uint_as_float(cur[i].y << 16),
+                                __uint_as_float(cur[i].y & 0xFFFF0000u)};
+            const float4 da = *reinterpret_cast<const float4*>(&sdy[warp + 8 * i][0]);
+            const float4 db = *reinterpret_cast<const float4*>(&sdy[warp + 8 * i][4]);
+            const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[r][e] = fmaf(d[r], w[e], acc[r][e]);
         }
     }
-    if (!colok) return;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        if (i >= ns) break;
-        const size_t at = (size_t)(s0 + i) * ld_h + j0;
-        float4 v = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        if (hs.kind == JNX_HEAD_MLP) {
-            const float4 zz = *reinterpret_cast<const float4*>(z + at);
-            v.x *= silu_grad_f(zz.x);
-            v.y *= silu_grad_f(zz.y);
-            v.z *= silu_grad_f(zz.z);
-            v.w *= silu_grad_f(zz.w);
-        }
-        *reinterpret_cast<float4*>(dh + at) = v;
+    for (int r = 0; r < 8; ++r)
+        *reinterpret_cast<float4*>(&red[warp][r][4 * lane]) =
+            make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+    __syncthreads();
+    // thread: sample `warp`, its lane's four columns
+    if (!colok || warp >= ns) return;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const float4 t = *reinterpret_cast<const float4*>(&red[w][warp][4 * lane]);
+        v.x += t.x;
+        v.y += t.y;
+        v.z += t.z;
+        v.w += t.w;
     }
+    const size_t at = (size_t)(s0 + warp) * ld_h + j0;
+    if (hs.kind == JNX_HEAD_MLP) {
+        const float4 zz = *reinterpret_cast<const float4*>(z + at);
+        v.x *= silu_grad_f(zz.x);
+        v.y *= silu_grad_f(zz.y);
+        v.z *= silu_grad_f(zz.z);
+        v.w *= silu_grad_f(zz.w);
+    }
+    *reinterpret_cast<float4*>(dh + at) = v;
 }
 
 // MLP first-layer gradient: dW1[j, k] = sum_s dz[s, j] p[s, k]; db1[j] = sum_s dz[s, j].
@@ -518,15 +562,25 @@ __device__ __forceinline__ void split4(const float4 v, uint2& hi, uint2& lo) {
 __device__ __forceinline__ void xattn_split_rows(uint16_t* dst, int rows, int ldt,
                                                  const float* __restrict__ R, int ld, size_t row0,
                                                  int nr, int c0, int nc) {
+    // a thread's eight loads are all in flight before the first is used (rows
+    // * units is a multiple of 8 x 256: 32 rows, nc a multiple of 256)
     const int units = nc / 4;
-    for (int i = threadIdx.x; i < rows * units; i += blockDim.x) {
-        const int r = i / units, u = i % units;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < nr) v = *reinterpret_cast<const float4*>(R + (row0 + r) * ld + c0 + 4 * u);
-        uint2 hi, lo;
-        split4(v, hi, lo);
-        *reinterpret_cast<uint2*>(dst + (size_t)r * ldt + 4 * u) = hi;
-        *reinterpret_cast<uint2*>(dst + (size_t)(rows + r) * ldt + 4 * u) = lo;
+    for (int i0 = threadIdx.x; i0 < rows * units; i0 += 8 * 256) {
+        float4 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = i0 + 256 * k, r = i / units, u = i % units;
+            v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r < nr) v[k] = __ldg(reinterpret_cast<const float4*>(R + (row0 + r) * ld + c0 + 4 * u));
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = i0 + 256 * k, r = i / units, u = i % units;
+            uint2 hi, lo;
+            split4(v[k], hi, lo);
+            *reinterpret_cast<uint2*>(dst + (size_t)r * ldt + 4 * u) = hi;
+            *reinterpret_cast<uint2*>(dst + (size_t)(rows + r) * ldt + 4 * u) = lo;
+        }
     }
 }
 
@@ -536,10 +590,16 @@ __device__ __forceinline__ void xattn_split_rows(uint16_t* dst, int rows, int ld
 __device__ __forceinline__ void xattn_split_chunk(uint16_t* tq, uint16_t* tk,
                                                   const float* __restrict__ X, int j0, int nr,
                                                   int nq) {
-    for (int i = threadIdx.x; i < kMaxQ * kXRows; i += blockDim.x) {
-        const int q = i & 31, j = i >> 5;  // a key's nq values are contiguous
-        const bool ok = j < nr && q < nq;
-        const float x = ok ? X[(size_t)(j0 + j) * nq + q] : 0.f;
+    float v[kMaxQ * kXRows / 256];
+#pragma unroll
+    for (int k = 0; k < kMaxQ * kXRows / 256; ++k) {
+        const int i = threadIdx.x + 256 * k, q = i & 31, j = i >> 5;  // a key's nq values are contiguous
+        v[k] = j < nr && q < nq ? X[(size_t)(j0 + j) * nq + q] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kMaxQ * kXRows / 256; ++k) {
+        const int i = threadIdx.x + 256 * k, q = i & 31, j = i >> 5;
+        const float x = v[k];
         const uint16_t hi = f2bf(x), lo = f2bf(x - bf2f(hi));
         if (tq) {
             tq[q * kXPad + j] = hi;
@@ -556,7 +616,8 @@ __device__ __forceinline__ void xattn_split_chunk(uint16_t* tq, uint16_t* tk,
 __device__ __forceinline__ void xattn_stage_q(uint16_t* sQ, int ldr, const uint16_t* __restrict__ q,
                                               int nq, int dq) {
     const int units = dq / 8;
-    for (int i = threadIdx.x; i < kMaxQ * units; i += blockDim.x) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < kMaxQ * units; i += 256) {
         const int r = i / units, u = i % units;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (r < nq) v = *reinterpret_cast<const uint4*>(q + (size_t)r * dq + 8 * u);
@@ -564,21 +625,21 @@ __device__ __forceinline__ void xattn_stage_q(uint16_t* sQ, int ldr, const uint1
     }
 }
 
-// out[j * nq + q] = scale * sum_c A[q, c] R[r0 + j, c] over the sample's L
-// key rows, key-major: A = (ahi, alo) split, or bf16 ahi alone (alo null).
+// out[j * nq + q] = scale * sum_c A[q, c] R[r0 + j, c] over the sample's
+// keys j in [ja, jz), key-major: A = (ahi, alo) split, or bf16 ahi alone (alo null).
 // Per 32-key chunk (rows split into sR), warp w takes query tile w % 2 and
 // keys 8 (w / 2) .. + 7, over all dq.  Ends with a barrier.
 __device__ void xattn_scores(const uint16_t* ahi, const uint16_t* alo, int ldr, uint16_t* sR,
-                             const float* __restrict__ R, int ldkv, int r0, int L, int nq, int dq,
-                             float scale, float* __restrict__ out) {
+                             const float* __restrict__ R, int ldkv, int r0, int ja, int jz,
+                             int nq, int dq, float scale, float* __restrict__ out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = warp & 1, nt = warp >> 1, g = lane >> 2, t = lane & 3;
     const int arow = 16 * m + (lane & 7) + ((lane >> 3) & 1) * 8, acol = (lane >> 4) * 8;
     // B (8 keys x 16 deep): matrices hi / k 0-7, hi / k 8-15, lo / k 0-7, lo / k 8-15
     const int brow = 8 * nt + (lane & 7), bcol = ((lane >> 3) & 1) * 8;
     const uint16_t* bsrc = sR + (size_t)(lane >> 4) * kXRows * ldr + (size_t)brow * ldr + bcol;
-    for (int j0 = 0; j0 < L; j0 += kXRows) {
-        const int nr = min(kXRows, L - j0);
+    for (int j0 = ja; j0 < jz; j0 += kXRows) {
+        const int nr = min(kXRows, jz - j0);
         __syncthreads();  // the previous chunk's readers (or the A tiles' writers) done
         xattn_split_rows(sR, kXRows, ldr, R, ldkv, (size_t)r0 + j0, nr, 0, dq);
         __syncthreads();
@@ -641,37 +702,104 @@ __device__ __forceinline__ void xattn_chunk_xr(float (&acc)[2][4][4], const uint
     }
 }
 
-// Per-query reductions over the sample's key-major [L, nq] block X (and Y):
-// thread (q = tid % 32, part = tid / 32) covers keys part, part + 8, ...;
-// the eight parts are combined in order.  red: 8 x 32 floats of shared
-// memory.  MAX: max_j X; otherwise sum_j X * Y (Y may be X's weights).
+// A query-head sample is shared by a cluster of kXCtas CTAs: rank k takes an
+// equal share of the sample's 32-key chunks, keys [ja, jz) (empty for the
+// last ranks of a short sample).
+constexpr int kXCtas = 8;
+
+__device__ __forceinline__ void xattn_share(int rank, int L, int& ja, int& jz) {
+    const int chunks = (L + kXRows - 1) / kXRows;
+    const int share = (chunks + kXCtas - 1) / kXCtas * kXRows;
+    ja = min(rank * share, L);
+    jz = min(ja + share, L);
+}
+
+// Per-query values v of the eight 32-thread parts of every CTA of the
+// cluster (thread q = tid % 32, part = tid / 32) into one value per query:
+// parts in order inside a CTA, then CTAs in rank order.  red: 8 x 32 floats
+// of this CTA; slot: 32 floats of this CTA that the other CTAs read, used for
+// one reduction only.
 template <bool MAX>
-__device__ float xattn_reduce_q(const float* __restrict__ X, const float* __restrict__ Y, int L,
-                                int nq, float* red) {
-    const int q = threadIdx.x & 31, part = threadIdx.x >> 5;
-    float v = MAX ? -INFINITY : 0.f;
-    if (q < nq)
-        for (int j = part; j < L; j += 8) {
-            const float x = X[(size_t)j * nq + q];
-            v = MAX ? fmaxf(v, x) : fmaf(x, Y[(size_t)j * nq + q], v);
-        }
-    red[part * 32 + q] = v;
+__device__ float xattn_cluster_q(cg::cluster_group& cluster, float v, float* red, float* slot) {
+    red[threadIdx.x] = v;
     __syncthreads();
+    if (threadIdx.x < 32) {
+        float r = MAX ? -INFINITY : 0.f;
+        for (int p = 0; p < 8; ++p) {
+            const float x = red[p * 32 + threadIdx.x];
+            r = MAX ? fmaxf(r, x) : r + x;
+        }
+        slot[threadIdx.x] = r;
+    }
+    cluster.sync();
     float r = MAX ? -INFINITY : 0.f;
-    for (int p = 0; p < 8; ++p) r = MAX ? fmaxf(r, red[p * 32 + q]) : r + red[p * 32 + q];
-    __syncthreads();  // red is reused by the caller
-    return r;  // valid in threads with q < nq (every part holds the same value)
+#pragma unroll
+    for (int k = 0; k < kXCtas; ++k) {
+        const float x = *cluster.map_shared_rank(&slot[threadIdx.x & 31], k);
+        r = MAX ? fmaxf(r, x) : r + x;
+    }
+    return r;
+}
+
+// Sum over the cluster's CTAs, in rank order, of their [32][kXCols] partial
+// products (accumulators of xattn_chunk_xr), times scale, into rows q < nq of
+// out (row stride ldo): the accumulators go through `part` (32 x kXAccPad
+// floats of shared memory), each rank finishes an eighth of the block.
+constexpr int kXAccPad = kXCols + 8;  // conflict-free 8-byte stores of the accumulators
+
+__device__ void xattn_cluster_store(cg::cluster_group& cluster, const float (&acc)[2][4][4],
+                                    float* part, int nq, float scale, float* __restrict__ out,
+                                    int ldo) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    __syncthreads();  // the staged rows that `part` overlays are read
+    // element e of tile (m, n): query 16 m + g (+ 8 for e >= 2), column
+    // 32 w + 8 n + 2 t (+ 1 for odd e)
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+                *reinterpret_cast<float2*>(part + (16 * m + g + 8 * hf) * kXAccPad + 32 * warp +
+                                           8 * n + 2 * t) =
+                    make_float2(acc[m][n][2 * hf], acc[m][n][2 * hf + 1]);
+    cluster.sync();
+    static_assert(kMaxQ * kXCols == kXCtas * 256 * 4, "one float4 per thread");
+    const int e = (int)cluster.block_rank() * 1024 + 4 * threadIdx.x;
+    const int q = e / kXCols, c = e % kXCols;
+    if (q < nq) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < kXCtas; ++k) {
+            const float4 x = *reinterpret_cast<const float4*>(
+                cluster.map_shared_rank(part + q * kXAccPad + c, k));
+            v.x += x.x;
+            v.y += x.y;
+            v.z += x.z;
+            v.w += x.w;
+        }
+        *reinterpret_cast<float4*>(out + (size_t)q * ldo + c) =
+            make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
+    }
+    cluster.sync();  // no CTA reuses `part` or exits while another reads it
 }
 
 // ---------------------------------------------------------------------------
-// Query head, per sample.  One CTA per packed sample of a query-head slot.
+// Query head, per sample.  A cluster of kXCtas CTAs per packed sample of a
+// query-head slot: each takes a share of the keys, and the softmax's maxima
+// and sums, D and the products over keys (O, dQ) are combined through
+// distributed shared memory in rank order.  With one CTA per sample a group
+// of 64 samples (16 to 26 chunks each, load, split and multiply in turn) kept
+// at most 64 SMs at work: forward 364 us, backward 453 us; eight per sample:
+// and their staged rows loaded eight at a time: 82 and 112 us.
 // P (normalised attention) for sample s is stored key-major at P + nq * cu[s]:
 // element (query q, key j) at j * nq + q (nq a multiple of 4).  The
 // products run on the bf16 tensor cores with split fp32 operands (see
 // xattn_smem_bytes); every sum runs in a fixed order, so a sample's result
 // does not depend on the batch around it.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_xattn_fwd(const __grid_constant__ HeadTable tab, int g0,
+__global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 3)
+    k_xattn_fwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
                                                    const int* __restrict__ sample_slot,
                                                    int sample0, const float* __restrict__ kbuf,
@@ -680,65 +808,55 @@ __global__ void __launch_bounds__(256) k_xattn_fwd(const __grid_constant__ HeadT
                                                    int ld_h) {
     static_assert(kMaxQ == 32 && kXRows == 32, "two 16-row tiles of queries and of keys");
     extern __shared__ __align__(16) uint8_t xsm[];
-    __shared__ float red[8 * 32];
-    const int s = sample0 + blockIdx.x;
+    __shared__ float red[8 * 32], slot_m[32], slot_s[32];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int s = sample0 + blockIdx.x / kXCtas;
     const HeadSlot& hs = tab.slot[sample_slot[s] - g0];
-    if (hs.kind != JNX_HEAD_XATTN) return;
+    if (hs.kind != JNX_HEAD_XATTN) return;  // every CTA of the cluster
     const int nq = hs.nq, dq = hs.dq, ldr = dq + 8;
     uint16_t* sQ = reinterpret_cast<uint16_t*>(xsm);
     uint16_t* sR = sQ + kMaxQ * ldr;
     uint16_t* sT = sR + 2 * kXRows * ldr;
     const int r0 = cu[s], L = cu[s + 1] - r0;
+    int ja, jz;
+    xattn_share((int)cluster.block_rank(), L, ja, jz);
     float* Ps = P + (size_t)nq * r0;
-    xattn_stage_q(sQ, ldr, hs.q, nq, dq);
+    if (ja < jz) xattn_stage_q(sQ, ldr, hs.q, nq, dq);
     // scores S[j, q] = Q_q . k_j / sqrt(dq) into Ps
-    xattn_scores(sQ, nullptr, ldr, sR, kbuf, ldkv, r0, L, nq, dq, rsqrtf((float)dq), Ps);
-    // softmax over the keys of each query, in place
-    const float m = xattn_reduce_q<true>(Ps, nullptr, L, nq, red);
+    xattn_scores(sQ, nullptr, ldr, sR, kbuf, ldkv, r0, ja, jz, nq, dq, rsqrtf((float)dq), Ps);
+    // softmax over the keys of each query, in place: thread (q = tid % 32,
+    // part = tid / 32) covers keys ja + part, ja + part + 8, ...
     {
         const int q = threadIdx.x & 31, part = threadIdx.x >> 5;
+        float mx = -INFINITY;
+        if (q < nq)
+            for (int j = ja + part; j < jz; j += 8) mx = fmaxf(mx, Ps[(size_t)j * nq + q]);
+        const float m = xattn_cluster_q<true>(cluster, mx, red, slot_m);
         float sum = 0.f;
         if (q < nq)
-            for (int j = part; j < L; j += 8) {
+            for (int j = ja + part; j < jz; j += 8) {
                 const float e = expf(Ps[(size_t)j * nq + q] - m);
                 Ps[(size_t)j * nq + q] = e;
                 sum += e;
             }
-        red[part * 32 + q] = sum;
-        __syncthreads();
-        float tot = 0.f;
-        for (int p = 0; p < 8; ++p) tot += red[p * 32 + q];
-        const float inv = 1.0f / tot;
+        const float inv = 1.0f / xattn_cluster_q<false>(cluster, sum, red, slot_s);
         if (q < nq)
-            for (int j = part; j < L; j += 8) Ps[(size_t)j * nq + q] *= inv;
+            for (int j = ja + part; j < jz; j += 8) Ps[(size_t)j * nq + q] *= inv;
         __syncthreads();
     }
     // O = P v, kXCols value columns at a time, keys in 32-key chunks
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     for (int c0 = 0; c0 < dq; c0 += kXCols) {
         float acc[2][4][4] = {};
-        for (int j0 = 0; j0 < L; j0 += kXRows) {
-            const int nr = min(kXRows, L - j0);
+        for (int j0 = ja; j0 < jz; j0 += kXRows) {
+            const int nr = min(kXRows, jz - j0);
             __syncthreads();
             xattn_split_rows(sR, kXRows, kXCols + 8, vbuf, ldkv, (size_t)r0 + j0, nr, c0, kXCols);
             xattn_split_chunk(sT, nullptr, Ps, j0, nr, nq);
             __syncthreads();
             xattn_chunk_xr(acc, sT, sR);
         }
-        // element e of tile (m, n): query 16 m + g (+ 8 for e >= 2), column
-        // c0 + 32 w + 8 n + 2 t (+ 1 for odd e)
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                const int q = 16 * mt + g + 8 * hf;
-                if (q >= nq) continue;
-#pragma unroll
-                for (int n = 0; n < 4; ++n)
-                    *reinterpret_cast<float2*>(h + (size_t)s * ld_h + (size_t)q * dq + c0 +
-                                               32 * warp + 8 * n + 2 * t) =
-                        make_float2(acc[mt][n][2 * hf], acc[mt][n][2 * hf + 1]);
-            }
+        xattn_cluster_store(cluster, acc, reinterpret_cast<float*>(sR), nq, 1.f,
+                            h + (size_t)s * ld_h + c0, dq);
     }
 }
 
@@ -747,7 +865,8 @@ __global__ void __launch_bounds__(256) k_xattn_fwd(const __grid_constant__ HeadT
 // contribution scale dS k (summed per tenant later in sample order), and,
 // when kv_grads is set (the feature gradient needs them), the key rows'
 // dv = P^T dO and dk = scale dS^T Q.
-__global__ void __launch_bounds__(256) k_xattn_bwd(const __grid_constant__ HeadTable tab, int g0,
+__global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
+    k_xattn_bwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
                                                    const int* __restrict__ sample_slot,
                                                    int sample0, const float* __restrict__ kbuf,
@@ -758,10 +877,11 @@ __global__ void __launch_bounds__(256) k_xattn_bwd(const __grid_constant__ HeadT
                                                    float* __restrict__ dk, float* __restrict__ dv,
                                                    float* __restrict__ dQs, int kv_grads) {
     extern __shared__ __align__(16) uint8_t xsm[];
-    __shared__ float red[8 * 32];
-    const int s = sample0 + blockIdx.x;
+    __shared__ float red[8 * 32], slot_d[32];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int s = sample0 + blockIdx.x / kXCtas;
     const HeadSlot& hs = tab.slot[sample_slot[s] - g0];
-    if (hs.kind != JNX_HEAD_XATTN) return;
+    if (hs.kind != JNX_HEAD_XATTN) return;  // every CTA of the cluster
     const int nq = hs.nq, dq = hs.dq, ldr = dq + 8;
     uint16_t* sQ = reinterpret_cast<uint16_t*>(xsm);
     uint16_t* sA = sQ + kMaxQ * ldr;
@@ -769,17 +889,27 @@ __global__ void __launch_bounds__(256) k_xattn_bwd(const __grid_constant__ HeadT
     uint16_t* sT = sR + 2 * kXRows * ldr;
     uint16_t* sU = sT + 4 * kMaxQ * kXPad;
     const int r0 = cu[s], L = cu[s + 1] - r0;
+    int ja, jz;
+    xattn_share((int)cluster.block_rank(), L, ja, jz);
     const float scale = rsqrtf((float)dq);
     const float* Ps = P + (size_t)nq * r0;
     float* dSs = dS + (size_t)nq * r0;
-    xattn_stage_q(sQ, ldr, hs.q, nq, dq);
-    xattn_split_rows(sA, kMaxQ, ldr, dO + (size_t)s * ld_h, dq, 0, nq, 0, dq);
-    xattn_scores(sA, sA + kMaxQ * ldr, ldr, sR, vbuf, ldkv, r0, L, nq, dq, 1.f, dSs);  // dP
-    const float Dq = xattn_reduce_q<false>(dSs, Ps, L, nq, red);
+    if (ja < jz) {
+        xattn_stage_q(sQ, ldr, hs.q, nq, dq);
+        xattn_split_rows(sA, kMaxQ, ldr, dO + (size_t)s * ld_h, dq, 0, nq, 0, dq);
+    }
+    xattn_scores(sA, sA + kMaxQ * ldr, ldr, sR, vbuf, ldkv, r0, ja, jz, nq, dq, 1.f, dSs);  // dP
     {
         const int q = threadIdx.x & 31, part = threadIdx.x >> 5;
+        float sum = 0.f;
         if (q < nq)
-            for (int j = part; j < L; j += 8) {
+            for (int j = ja + part; j < jz; j += 8) {
+                const size_t at = (size_t)j * nq + q;
+                sum = fmaf(dSs[at], Ps[at], sum);
+            }
+        const float Dq = xattn_cluster_q<false>(cluster, sum, red, slot_d);
+        if (q < nq)
+            for (int j = ja + part; j < jz; j += 8) {
                 const size_t at = (size_t)j * nq + q;
                 dSs[at] = Ps[at] * (dSs[at] - Dq);
             }
@@ -792,8 +922,8 @@ __global__ void __launch_bounds__(256) k_xattn_bwd(const __grid_constant__ HeadT
     uint16_t* uD = sU + 2 * kXRows * kXPad;
     for (int c0 = 0; c0 < dq; c0 += kXCols) {
         float aq[2][4][4] = {};
-        for (int j0 = 0; j0 < L; j0 += kXRows) {
-            const int nr = min(kXRows, L - j0);
+        for (int j0 = ja; j0 < jz; j0 += kXRows) {
+            const int nr = min(kXRows, jz - j0);
             __syncthreads();
             xattn_split_rows(sR, kXRows, kXCols + 8, kbuf, ldkv, (size_t)r0 + j0, nr, c0, kXCols);
             xattn_split_chunk(sT, kv_grads ? uD : nullptr, dSs, j0, nr, nq);
@@ -856,18 +986,8 @@ __global__ void __launch_bounds__(256) k_xattn_bwd(const __grid_constant__ HeadT
                     }
                 }
         }
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                const int q = 16 * mt + g + 8 * hf;
-                if (q >= nq) continue;
-#pragma unroll
-                for (int n = 0; n < 4; ++n)
-                    *reinterpret_cast<float2*>(dQs + (size_t)s * ld_h + (size_t)q * dq + c0 +
-                                               32 * warp + 8 * n + 2 * t) =
-                        make_float2(aq[mt][n][2 * hf] * scale, aq[mt][n][2 * hf + 1] * scale);
-            }
+        xattn_cluster_store(cluster, aq, reinterpret_cast<float*>(sR), nq, scale,
+                            dQs + (size_t)s * ld_h + c0, dq);
     }
 }
 
@@ -1147,7 +1267,7 @@ jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const 
             tab, pooled, d, ws.z, ws.h, ws.ld_h, sample_target, preds);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, false);
-        k_xattn_fwd<<<b.sample1 - b.sample0, 256, smem, s>>>(tab, b.g0, cu, sample_slot,
+        k_xattn_fwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(tab, b.g0, cu, sample_slot,
                                                              b.sample0, ws.kbuf, ws.vbuf, ws.ldkv,
                                                              ws.P, ws.h, ws.ld_h);
     }
@@ -1156,7 +1276,7 @@ jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const 
                     256, kLinSmem, s>>>(
         tab, ws.h, ws.ld_h, ws.y, nullptr, ws.ld_y, sample_target, preds);
     if (targets)  // without targets (inference) there is no loss
-        k_l2_loss<<<b.n, 256, 0, s>>>(tab, ws.y, ws.ld_y, targets, sample_target, ws.dy, loss);
+        k_l2_loss<<<b.n, kLossThreads, 0, s>>>(tab, ws.y, ws.ld_y, targets, sample_target, ws.dy, loss);
     return cuda_ok("heads forward");
 }
 
@@ -1170,7 +1290,7 @@ jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const
     k_head_dw_out<NoOpt>
         <<<dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s>>>(
             tab, no, nh, ws.dy, ws.ld_y, ws.h, ws.ld_h);
-    k_head_back_in<<<dim3(b.n, (b.max_hid + 1023) / 1024, (b.max_ns + 7) / 8), 256, 0, s>>>(
+    k_head_back_in<<<dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s>>>(
         tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_mlp)
         k_mlp_dw1<NoOpt><<<dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256),
@@ -1178,7 +1298,7 @@ jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const
             tab, no, nh, ws.dh, ws.ld_h, pooled, d);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
-        k_xattn_bwd<<<b.sample1 - b.sample0, 256, smem, s>>>(
+        k_xattn_bwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(
             tab, b.g0, cu, sample_slot, b.sample0, ws.kbuf, ws.vbuf, ws.ldkv, ws.P, ws.dS, ws.dh,
             ws.ld_h, ws.dk, ws.dv, ws.dQs, kv_grads ? 1 : 0);
         k_xattn_dq<NoOpt><<<dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s>>>(
@@ -1196,11 +1316,11 @@ jnx_status heads_backward_front_launch(const HeadTable& tab, const HeadBatch& b,
                                        const int* cu, const int* sample_slot, bool kv_grads,
                                        cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
-    k_head_back_in<<<dim3(b.n, (b.max_hid + 1023) / 1024, (b.max_ns + 7) / 8), 256, 0, s>>>(
+    k_head_back_in<<<dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s>>>(
         tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
-        k_xattn_bwd<<<b.sample1 - b.sample0, 256, smem, s>>>(
+        k_xattn_bwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(
             tab, b.g0, cu, sample_slot, b.sample0, ws.kbuf, ws.vbuf, ws.ldkv, ws.P, ws.dS, ws.dh,
             ws.ld_h, ws.dk, ws.dv, ws.dQs, kv_grads ? 1 : 0);
         k_xattn_gh<<<dim3(b.sample1 - b.sample0, d / 128), 256, 0, s>>>(
