@@ -27,6 +27,7 @@
 // Every output element's K reduction runs in the same order whatever M is
 // or where the row sits, so packed (grouped) and per-tenant runs agree
 // bit for bit.
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -49,13 +50,29 @@ constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barrier
 constexpr int STG_SLOT_EW8 = 4096;
 constexpr int SMEM_BYTES_EW8 = SMEM_BYTES - STG_BYTES + 8 * STG_SLOT_EW8;
 static_assert(SMEM_BYTES_EW8 <= 227 * 1024, "shared memory per CTA");
-constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
+constexpr int RING_MAX = 24;  // stages of a narrow tile's ring, at most
 // LoRA operands of one tile (K = 16, 32-byte rows): t rows and B rows, a
 // 2-deep ring after the main stages.
 constexpr int LT_BYTES = BM * 16 * 2;
 constexpr int LB_BYTES = BN * 16 * 2;
 constexpr int LSTAGE = LT_BYTES + LB_BYTES;
 constexpr int SMEM_BYTES_LORA = SMEM_BYTES + 2 * LSTAGE;
+
+// Narrow tiles (128 x BN, BN = 128 or 64) for launches whose 256-wide tiles
+// leave SMs idle.  A tile's BN columns are two groups of BN / 2, so that one
+// tile still holds what an epilogue combines: a gate group and its up group,
+// or the two halves of a head that RoPE rotates.  Everything else is the wide
+// kernel: the same K order, the same MMA depth, the same epilogues, so a
+// result has the same bits whatever tile width the launch chose.
+// Shared memory: a ring of p.stages stages of a_rows (16 .. 128) A rows and BN
+// B rows, then the barriers and the staging slots.  The MMA always reads 128 A
+// rows; those past a_rows are whatever follows in shared memory and land in
+// accumulator rows that no epilogue stores.
+constexpr int NARROW_BAR = 512;  // barrier block of a narrow ring
+constexpr int narrow_smem(int bn, int stages, int a_rows, bool lora) {
+    return stages * (a_rows + bn) * BK * 2 + A_BYTES - a_rows * BK * 2 +
+           (lora ? 2 * (LT_BYTES + bn * 32) : 0) + 1024 + NARROW_BAR + STG_BYTES;
+}
 }  // namespace gemm
 
 // Descriptor of a K-major bf16 tile with 32-byte rows (K = 16) stored with
@@ -75,8 +92,11 @@ struct NoLora {};
 // Rows [row0, row_end) and column block nb of one output tile.  Without
 // LoRA, tiles are plain 128-row blocks of M; with LoRA they are laid out per
 // tenant segment so every tile belongs to one tenant (`seg`).
+// Its columns: the two groups start at weight rows c0 and c1 (a 256-wide
+// tile is one contiguous block, c1 = c0 + 128).
 struct TileGeo {
     int row0, row_end, nb, seg;
+    int c0, c1;
 };
 
 // Tile order: groups of `group_m` row-blocks, N fastest inside a group, so
@@ -174,22 +194,31 @@ __device__ __forceinline__ void stg_store_bf16(uint8_t* stg, int lane, const uin
 // fixed order; 1 without a folded norm.
 __device__ __forceinline__ float row_norm_scale(const GemmParams& p, int row, bool valid) {
     if (p.ss_in == nullptr || !valid) return 1.f;
-    const float* sp = p.ss_in + (size_t)row * p.ss_parts;
+    const float4* sp = reinterpret_cast<const float4*>(p.ss_in + (size_t)row * p.ss_parts);
     float t = 0.f;
-    for (int i = 0; i < p.ss_parts; ++i) t += sp[i];
+    for (int i = 0; i < p.ss_parts / 4; ++i) {
+        const float4 v = sp[i];
+        t += v.x;
+        t += v.y;
+        t += v.z;
+        t += v.w;
+    }
     return rsqrtf(t / (float)p.ss_cols + p.ss_eps);
 }
 
 // The accumulator tile at tbase (this warp's 32 TMEM lanes = rows
-// row_base..row_base+31, 256 fp32 columns) -> the epilogue's output.
+// row_base..row_base+31, BN fp32 columns) -> the epilogue's output.
 // NC, cb: the 32-column chunks [cb, cb + NC) of the tile this warp handles
-// (all 8, or one half of 4 with eight epilogue warps: EPI_BF16, EPI_F32,
-// EPI_RESID without a folded norm, EPI_GLU_BWD and EPI_GLU_DM only).  Ring slots are
-// indexed by the pass within this warp's range, so they stay compile-time.
-template <int EPI, int NC = 8>
+// (all of them, or one half of a 256-wide tile with eight epilogue warps:
+// EPI_GLU_BWD and EPI_GLU_DM).  Ring slots are indexed by the pass within
+// this warp's range, so they stay compile-time.
+template <int EPI, int NC, int BN>
 __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int lane,
-                                              int row_base, int row_end, int n0,
-                                              const GemmParams& p, int cb = 0) {
+                                              int row_base, int row_end, const TileGeo& geo,
+                                              const GemmParams& p, int cb) {
+    constexpr int HC = BN / 64;  // chunks of one column group
+    constexpr bool WIDE = BN == 256;
+    const int n0 = geo.c0;
     const int my_row = row_base + lane;
     const bool valid = my_row < row_end;
     const uint64_t pol = l2_evict_first_policy();  // outputs and residual are streamed
@@ -213,7 +242,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
         // loaded RD - 1 passes ahead of its use, so several passes' loads
         // are in flight while the accumulator is staged (a shallower ring for
         // half-tile warps, which run with fewer registers per thread)
-        constexpr int RD = NC == 4 ? 3 : 4;
+        constexpr int RD = WIDE && NC == 4 ? 3 : 4;
         float* dst = EPI == EPI_RESID ? p.resid : static_cast<float*>(p.out);
         const int ld = EPI == EPI_RESID ? p.ldr : p.ldo;
         float4 xr[RD][4];
@@ -239,8 +268,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
         }
         // folded RMSNorm (EPI_RESID with norm_gamma): y = bf16(x * gamma) and
         // the sums of x^2 of each of this lane's four rows over its columns,
-        // one per 128-column half of the tile (8 staging passes each)
-        float ssq[NC / 4][4] = {};
+        // one per 64-column block of the tile (4 staging passes each)
+        float ssq[NC / 2][4] = {};
 #pragma unroll
         for (int lc = 0; lc < NC; ++lc) {
             const int c = cb + lc;
@@ -289,7 +318,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
                                                      __float_as_uint(o.z), __float_as_uint(o.w)),
                                           pol);
                     if (EPI == EPI_RESID && norm) {
-                        ssq[lp / 8][i] += o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w;
+                        ssq[lp / 4][i] += o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w;
                         if (row < row_end)
                             *reinterpret_cast<uint2*>(p.norm_out + (size_t)row * p.N + col) =
                                 make_uint2(pack_bf2(o.x * gf[0], o.y * gf[1]),
@@ -300,10 +329,10 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
             }
         }
         if (norm) {
-            // the four lanes of a row hold each half's columns between them
-            const int parts = p.N / 128;
+            // the four lanes of a row hold each block's columns between them
+            const int parts = p.N / 64;
 #pragma unroll
-            for (int hb = 0; hb < NC / 4; ++hb)
+            for (int hb = 0; hb < NC / 2; ++hb)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float t = ssq[hb][i];
@@ -311,16 +340,16 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
                     t += __shfl_xor_sync(0xffffffffu, t, 2);
                     const int row = row_base + 8 * i + (lane >> 2);
                     if ((lane & 3) == 0 && row < row_end)
-                        p.ss_out[(size_t)row * parts + (n0 + 32 * cb) / 128 + hb] = t;
+                        p.ss_out[(size_t)row * parts + (n0 + 32 * cb) / 64 + hb] = t;
                 }
         }
     } else if constexpr (EPI == EPI_GLU) {
         const float rs = row_norm_scale(p, my_row, valid);
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < HC; ++c) {
             uint32_t g[32], u[32];
             tmem_ld32(tbase + c * 32, g);
-            tmem_ld32(tbase + (c + 4) * 32, u);
+            tmem_ld32(tbase + (c + HC) * 32, u);
             tmem_ld_wait();
             uint4 v[4];
 #pragma unroll
@@ -333,15 +362,15 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
                 v[q] = pack8_bf16(o);
             }
             stg_store_bf16(stg, lane, v, static_cast<bf16_t*>(p.out), p.ldo, row_base, row_end,
-                           n0 / 2 + c * 32, pol);
+                           geo.nb * (BN / 2) + c * 32, pol);
         }
     } else if constexpr (EPI == EPI_GLU_SAVE) {
         const float rs = row_norm_scale(p, my_row, valid);
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < HC; ++c) {
             uint32_t g[32], u[32];
             tmem_ld32(tbase + c * 32, g);
-            tmem_ld32(tbase + (c + 4) * 32, u);
+            tmem_ld32(tbase + (c + HC) * 32, u);
             tmem_ld_wait();
             uint4 vg[4], vu[4];
 #pragma unroll
@@ -360,7 +389,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
             stg_store_bf16(stg, lane, vg, static_cast<bf16_t*>(p.out), p.ldo, row_base, row_end,
                            n0 + c * 32, pol);
             stg_store_bf16(stg, lane, vu, static_cast<bf16_t*>(p.out), p.ldo, row_base, row_end,
-                           n0 + 128 + c * 32, pol);
+                           geo.c1 + c * 32, pol);
         }
     } else if constexpr (EPI == EPI_GLU_DM) {
         // as EPI_GLU_SAVE over the chunk pairs (gate c, up c + 4) of this
@@ -411,7 +440,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
             stg_store_bf16(stg, lane, vu, static_cast<bf16_t*>(p.out), p.ldo, row_base, row_end,
                            n0 + 128 + c * 32, pol);
         }
-    } else if constexpr (EPI == EPI_GLU_BWD && NC == 4) {
+    } else if constexpr (EPI == EPI_GLU_BWD && WIDE && NC == 4) {
         // half-tile warps (4 KB staging slot): one staging round per 32-column
         // chunk, so each lane takes 8 contiguous columns of rows 8 i + lane / 4
         // and its multiplier loads and result stores are 16 bytes; the next
@@ -565,9 +594,13 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
         if (valid && !pos_ok) report(p.status, JNX_ERR_DEVICE_BOUNDS);
         if (!pos_ok) pos = 0;
         const float rs = row_norm_scale(p, my_row, valid);
+        // a chunk pair's columns and its frequencies: a wide tile holds whole
+        // heads (partner chunk hc further), a narrow one the groups' chunks
+        const int pair = WIDE ? hc : HC;
+        const int fr0 = WIDE ? 0 : (n0 % p.hd) / 32;
 #pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
-            const int hchunk = c % (2 * hc);
+        for (int c = 0; c < (WIDE ? 8 : HC); ++c) {
+            const int hchunk = WIDE ? c % (2 * hc) : fr0 + c;
             if (hchunk >= hc) continue;  // handled with its lower partner
             const int col = n0 + c * 32;
             const bool rot = valid && pos_ok && col < p.rope_cols;
@@ -583,7 +616,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
             }
             uint32_t lo[32], hi[32];
             tmem_ld32(tbase + c * 32, lo);
-            tmem_ld32(tbase + (c + hc) * 32, hi);
+            tmem_ld32(tbase + (c + pair) * 32, hi);
             tmem_ld_wait();
             float a[32], b[32];
 #pragma unroll
@@ -613,13 +646,26 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
     }
 }
 
-template <bool LORA, class LG>
+template <int EPI, bool LORA, int BN, class LG>
 __device__ __forceinline__ TileGeo tile_geo(int tile, int num_m, int num_n, const GemmParams& p,
                                             const LG& lg) {
     int mb, nb;
     tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
     TileGeo g;
     g.nb = nb;
+    constexpr int HB = BN / 2;
+    if (BN < 256 && EPI == EPI_ROPE) {  // BN <= hd: a slice of one head and its rotation partner
+        const int per_head = p.hd / BN;
+        g.c0 = nb / per_head * p.hd + nb % per_head * HB;
+        g.c1 = g.c0 + p.hd / 2;
+    } else if (BN < 256 && (EPI == EPI_GLU || EPI == EPI_GLU_SAVE)) {
+        const int f = nb * HB;  // F columns f .. f + HB - 1: gate and up blocks of 128 in turn
+        g.c0 = 256 * (f / 128) + f % 128;
+        g.c1 = g.c0 + 128;
+    } else {
+        g.c0 = nb * BN;
+        g.c1 = g.c0 + HB;
+    }
     if constexpr (LORA) {
         int sg = 0;
         while (sg + 1 < lg.n_seg && lg.seg_tile0[sg + 1] <= mb) ++sg;
@@ -634,9 +680,8 @@ __device__ __forceinline__ TileGeo tile_geo(int tile, int num_m, int num_n, cons
     return g;
 }
 
-// The LoRA part holding column block nb, and the block's first column in it.
-__device__ __forceinline__ void lora_part(const LoraGemm& lg, int nb, int& part, int& c0) {
-    int c = nb * gemm::BN;
+// The LoRA part holding weight row c (of a tile's columns), and its place there.
+__device__ __forceinline__ void lora_part(const LoraGemm& lg, int c, int& part, int& c0) {
     part = 0;
     while (part + 1 < lg.n_parts && c >= lg.part_cols[part]) {
         c -= lg.part_cols[part];
@@ -645,19 +690,29 @@ __device__ __forceinline__ void lora_part(const LoraGemm& lg, int nb, int& part,
     c0 = c;
 }
 
-template <int EPI, bool LORA, int EW>
-__global__ void __launch_bounds__(64 + 32 * EW, 1)
+template <int EPI, bool LORA, int EW, int BN>
+__global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
     k_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
            const __grid_constant__ typename std::conditional<LORA, LoraGemm, NoLora>::type lg,
            GemmParams p) {
-    using namespace gemm;
+    using gemm::A_BYTES;
+    using gemm::BK;
+    using gemm::BM;
+    constexpr bool WIDE = BN == 256;
+    constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
+    constexpr int LT_BYTES = gemm::LT_BYTES, LSTAGE = LT_BYTES + BN * 32;
+    constexpr int RING = WIDE ? gemm::STAGES : gemm::RING_MAX;  // barriers per direction
+    constexpr uint32_t TMEM_COLS = 2 * BN;
+    const int stages = WIDE ? gemm::STAGES : p.stages;
+    const int a_bytes = WIDE ? A_BYTES : p.a_rows * BK * 2;
+    const int stage_bytes = a_bytes + BN * BK * 2;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* lsm = smem + STAGES * STAGE_BYTES;  // LoRA ring (LORA only)
+    uint8_t* lsm = smem + stages * stage_bytes + A_BYTES - a_bytes;  // LoRA ring (LORA only)
     uint64_t* full = reinterpret_cast<uint64_t*>(lsm + (LORA ? 2 * LSTAGE : 0));
-    uint64_t* empty = full + STAGES;
-    uint64_t* tfull = empty + STAGES;
+    uint64_t* empty = full + RING;
+    uint64_t* tfull = empty + RING;
     uint64_t* tempty = tfull + 2;
     uint64_t* drain = tempty + 2;
     uint64_t* lfull = drain + 1;   // [2]
@@ -667,11 +722,11 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1)
     volatile int* consumed = abort_flag + 1;
     volatile int* lconsumed = abort_flag + 2;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_uniform(threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < RING; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -699,7 +754,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
     int num_m;
     if constexpr (LORA)
@@ -712,137 +767,156 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1)
     int issued = 0, l_issued = 0;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int lj = 0;
-            uint32_t lphase = 0;
-            for (int tile = blockIdx.x; tile < num_tiles && !*abort_flag; tile += gridDim.x) {
-                const TileGeo g = tile_geo<LORA>(tile, num_m, num_n, p, lg);
-                for (int kb = 0; kb < num_k; ++kb) {
-                    if (!mbar_wait(&empty[stage], phase ^ 1)) {
-                        *abort_flag = 1;
-                        report(p.status, JNX_ERR_TIMEOUT);
-                        break;
-                    }
-                    mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
-                    uint8_t* sa = smem + stage * STAGE_BYTES;
-                    tma_load_2d(sa, &ta, kb * BK, g.row0, &full[stage]);
-                    int brow = g.nb * BN;
-                    if constexpr (LORA)
-                        if (lg.seg_b) brow += lg.seg_tenant[g.seg] * p.N;
-                    tma_load_2d(sa + A_BYTES, &tb, kb * BK, brow, &full[stage]);
-                    ++issued;
-                    if (++stage == STAGES) {
-                        stage = 0;
-                        phase ^= 1;
-                    }
+        int stage = 0;
+        uint32_t phase = 0;
+        int lj = 0;
+        uint32_t lphase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; ok && tile < num_tiles && !*abort_flag; tile += gridDim.x) {
+            const TileGeo g = tile_geo<EPI, LORA, BN>(tile, num_m, num_n, p, lg);
+            int brow = 0;
+            if constexpr (LORA)
+                if (lg.seg_b) brow = lg.seg_tenant[g.seg] * p.N;
+            for (int kb = 0; kb < num_k; ++kb) {
+                if (!mbar_wait(&empty[stage], phase ^ 1)) {
+                    ok = false;
+                    break;
                 }
-                if constexpr (LORA) {
-                    if (*abort_flag) break;
-                    if (lg.n_parts == 0) continue;  // segmented weights only
-                    // this tile's t rows (its part) and its tenant's B rows
-                    if (!mbar_wait(&lempty[lj], lphase ^ 1)) {
-                        *abort_flag = 1;
-                        report(p.status, JNX_ERR_TIMEOUT);
-                        break;
-                    }
-                    int part, c0;
-                    lora_part(lg, g.nb, part, c0);
+                if (elect_one()) {
+                    uint8_t* sa = smem + stage * stage_bytes;
+                    mbar_arrive_expect_tx(&full[stage], stage_bytes);
+                    tma_load_2d(sa, &ta, kb * BK, g.row0, &full[stage]);
+                    tma_load_2d(sa + a_bytes, &tb, kb * BK, brow + g.c0, &full[stage]);
+                    if constexpr (!WIDE)
+                        tma_load_2d(sa + a_bytes + BN / 2 * BK * 2, &tb, kb * BK, brow + g.c1,
+                                    &full[stage]);
+                }
+                __syncwarp();
+                ++issued;
+                if (++stage == stages) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+            }
+            if constexpr (LORA) {
+                if (!ok) break;
+                if (lg.n_parts == 0) continue;  // segmented weights only
+                // this tile's t rows (its part) and its tenant's B rows
+                if (!mbar_wait(&lempty[lj], lphase ^ 1)) {
+                    ok = false;
+                    break;
+                }
+                int part, c0;
+                lora_part(lg, g.c0, part, c0);
+                const int lrow = lg.seg_tenant[g.seg] * lg.part_cols[part] + c0;
+                if (elect_one()) {
                     uint8_t* lt = lsm + lj * LSTAGE;
                     mbar_arrive_expect_tx(&lfull[lj], LSTAGE);
                     tma_load_2d(lt, &lg.tt, part * 16, g.row0, &lfull[lj]);
-                    tma_load_2d(lt + LT_BYTES, &lg.tb[part], 0,
-                                lg.seg_tenant[g.seg] * lg.part_cols[part] + c0, &lfull[lj]);
-                    ++l_issued;
-                    if (++lj == 2) {
-                        lj = 0;
-                        lphase ^= 1;
-                    }
+                    tma_load_2d(lt + LT_BYTES, &lg.tb[part], 0, lrow, &lfull[lj]);
+                    if constexpr (!WIDE)  // both groups lie in one part
+                        tma_load_2d(lt + LT_BYTES + BN / 2 * 32, &lg.tb[part], 0,
+                                    lrow + g.c1 - g.c0, &lfull[lj]);
+                }
+                __syncwarp();
+                ++l_issued;
+                if (++lj == 2) {
+                    lj = 0;
+                    lphase ^= 1;
                 }
             }
         }
+        if (!ok) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int local = 0;
-            int lj = 0;
-            uint32_t lphase = 0;
-            for (int tile = blockIdx.x; tile < num_tiles && !*abort_flag;
-                 tile += gridDim.x, ++local) {
-                const int acc = local & 1;
-                const uint32_t acc_phase = (local >> 1) & 1;
-                if (!mbar_wait(&tempty[acc], acc_phase ^ 1)) {
-                    *abort_flag = 1;
-                    report(p.status, JNX_ERR_TIMEOUT);
+        int stage = 0, local = 0, lj = 0, n_used = 0, l_used = 0;
+        uint32_t phase = 0, lphase = 0;
+        bool ok = true;
+        const uint32_t a_lo = sw128_desc_lo(smem_u32(smem));
+        const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + a_bytes);
+        for (int tile = blockIdx.x; ok && tile < num_tiles && !*abort_flag;
+             tile += gridDim.x, ++local) {
+            const int acc = local & 1;
+            const uint32_t acc_phase = (local >> 1) & 1;
+            if (!mbar_wait(&tempty[acc], acc_phase ^ 1)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem_base + acc * BN;
+            for (int kb = 0; kb < num_k; ++kb) {
+                if (!mbar_wait(&full[stage], phase)) {
+                    ok = false;
                     break;
                 }
+                ++n_used;
                 tc_fence_after();
-                const uint32_t d = tmem_base + acc * BN;
-                bool ok = true;
-                for (int kb = 0; kb < num_k; ++kb) {
-                    if (!mbar_wait(&full[stage], phase)) {
-                        ok = false;
-                        break;
-                    }
-                    *consumed = *consumed + 1;
-                    tc_fence_after();
-                    const uint32_t a_addr = smem_u32(smem + stage * STAGE_BYTES);
-                    const uint32_t b_addr = a_addr + A_BYTES;
+                const uint32_t off = (uint32_t)(stage * stage_bytes) >> 4;
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk)
-                        tc_mma_f16(d, sw128_desc(a_addr + kk * 32), sw128_desc(b_addr + kk * 32),
-                                   IDESC, (kb | kk) != 0);
+                        tc_mma_f16(d, desc_of(a_lo + off + 2 * kk, kSw128DescHi),
+                                   desc_of(b_lo + off + 2 * kk, kSw128DescHi), IDESC,
+                                   (kb | kk) != 0);
                     tc_commit(&empty[stage]);
-                    if (++stage == STAGES) {
-                        stage = 0;
-                        phase ^= 1;
-                    }
                 }
-                if constexpr (LORA) {
-                    // D += t[rows, part] . B_part[tenant][cols]^T (one K = 16 step);
-                    // none with segmented weights only (n_parts == 0)
-                    if (ok && lg.n_parts > 0) {
-                        if (!mbar_wait(&lfull[lj], lphase)) {
-                            ok = false;
-                        } else {
-                            *lconsumed = *lconsumed + 1;
-                            tc_fence_after();
-                            const uint32_t la = smem_u32(lsm + lj * LSTAGE);
+                __syncwarp();
+                if (++stage == stages) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+            }
+            if constexpr (LORA) {
+                // D += t[rows, part] . B_part[tenant][cols]^T (one K = 16 step);
+                // none with segmented weights only (n_parts == 0)
+                if (ok && lg.n_parts > 0) {
+                    if (!mbar_wait(&lfull[lj], lphase)) {
+                        ok = false;
+                    } else {
+                        ++l_used;
+                        tc_fence_after();
+                        const uint32_t la = smem_u32(lsm + lj * LSTAGE);
+                        if (elect_one()) {
                             tc_mma_f16(d, sw32_desc(la), sw32_desc(la + LT_BYTES), IDESC, 1);
                             tc_commit(&lempty[lj]);
-                            if (++lj == 2) {
-                                lj = 0;
-                                lphase ^= 1;
-                            }
+                        }
+                        __syncwarp();
+                        if (++lj == 2) {
+                            lj = 0;
+                            lphase ^= 1;
                         }
                     }
                 }
-                if (!ok) {
-                    *abort_flag = 1;
-                    report(p.status, JNX_ERR_TIMEOUT);
-                    break;
-                }
-                tc_commit(&tfull[acc]);
             }
-            // make sure no MMA is still writing TMEM before teardown
-            tc_commit(drain);
-            mbar_wait(drain, 0);
+            if (!ok) break;
+            if (elect_one()) tc_commit(&tfull[acc]);
+            __syncwarp();
         }
+        if (!ok) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        }
+        *consumed = n_used;
+        *lconsumed = l_used;
+        // make sure no MMA is still writing TMEM before teardown
+        if (elect_one()) tc_commit(drain);
+        __syncwarp();
+        mbar_wait(drain, 0);
     } else {
         const int q = warp & 3;  // TMEM lane quarter this warp may access
         // with eight epilogue warps, warps 2-5 take chunks 0-3 of a tile and
         // warps 6-9 chunks 4-7 (the same lane quarters)
         const int cb = EW == 8 ? ((warp - 2) >> 2) * 4 : 0;
         // this warp's staging slot, after the barrier block
-        uint8_t* stg = reinterpret_cast<uint8_t*>(full) + 256 +
+        uint8_t* stg = reinterpret_cast<uint8_t*>(full) + (WIDE ? 256 : gemm::NARROW_BAR) +
                        (warp - 2) * (EW == 8 ? gemm::STG_SLOT_EW8 : 2048);
         int local = 0;
         for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x, ++local) {
             const int acc = local & 1;
             const uint32_t acc_phase = (local >> 1) & 1;
-            const TileGeo g = tile_geo<LORA>(tile, num_m, num_n, p, lg);
+            const TileGeo g = tile_geo<EPI, LORA, BN>(tile, num_m, num_n, p, lg);
             const int row_base = g.row0 + q * 32;
             if constexpr (EPI == EPI_GLU_DM) {
                 // this thread's dm for the tile (its row, its chunks of the
@@ -861,8 +935,9 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1)
                 break;
             }
             tc_fence_after();
-            epilogue_tile<EPI, EW == 8 ? 4 : 8>(tmem_base + acc * BN + ((uint32_t)(q * 32) << 16),
-                                                stg, lane, row_base, g.row_end, g.nb * BN, p, cb);
+            epilogue_tile<EPI, EW == 8 ? BN / 64 : BN / 32, BN>(
+                tmem_base + acc * BN + ((uint32_t)(q * 32) << 16), stg, lane, row_base, g.row_end,
+                g, p, cb);
             tc_fence_before();
             mbar_arrive(&tempty[acc]);
         }
@@ -874,7 +949,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1)
     if (*abort_flag && warp == 0 && lane == 0) {
         // wait (bounded) for TMA copies this CTA issued but nobody consumed
         for (int i = *consumed; i < issued; ++i)
-            mbar_wait(&full[i % STAGES], (i / STAGES) & 1, 100000000LL);
+            mbar_wait(&full[i % stages], (i / stages) & 1, 100000000LL);
         for (int i = *lconsumed; i < l_issued; ++i)
             mbar_wait(&lfull[i & 1], (i >> 1) & 1, 100000000LL);
     }
@@ -943,20 +1018,86 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
     return e;
 }
 
+// Width of a launch's output tiles: the one with the least estimated time,
+// (tiles an SM works through) x (its time per 64-deep K step).  The step times
+// are GB300's in microseconds, from launches of 8 to 10,000 tiles (K = 2,048 to
+// 16,384): a tile alone on its SM, and two narrow tiles sharing one, which is
+// how a narrow launch of more tiles than SMs runs.  A 256-wide tile is the
+// fastest per column, so narrower ones win only where it leaves SMs idle:
+// 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide tiles, 61 in 80 of 128
+// and 76 in 160 of 64; 300 rows 96, 60 and 55; 4,800 rows 196, 237 and 348.
+// RoPE needs a tile within one head; the GLU backward with dm has wide tiles
+// only.
+static int pick_bn(int m_tiles, const GemmParams& p) {
+    const int sms = num_sms();
+    auto rounds = [](long long tiles, int slots) { return (double)((tiles + slots - 1) / slots); };
+    const long long wide = (long long)m_tiles * (p.N / 256);
+    int best = 256;
+    double least = rounds(wide, sms) * 0.385;
+    if (p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn)) return best;
+    static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.235, 0.39},
+                                                                     {64, 0.215, 0.334}};
+    for (const auto& w : kNarrow) {
+        if (p.epi == EPI_ROPE && w.bn > p.hd) continue;
+        const long long tiles = (long long)m_tiles * (p.N / w.bn);
+        const double t = tiles <= sms ? w.alone : rounds(tiles, 2 * sms) * w.two;
+        if (t < least) {
+            best = w.bn;
+            least = t;
+        }
+    }
+    return best;
+}
+
+// The ring of a narrow launch: as many stages as fit one CTA's shared memory,
+// or half of it where the tiles are more than the SMs and two CTAs share one.
+static void narrow_ring(GemmParams& p, int bn, long long tiles, bool lora) {
+    const int budget = (tiles > num_sms() ? 112 : 224) * 1024;
+    p.stages = gemm::RING_MAX;
+    while (p.stages > 2 && gemm::narrow_smem(bn, p.stages, p.a_rows, lora) > budget) --p.stages;
+}
+
+template <int EPI, bool LORA, class LG, int EW, int BN>
+static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
+                             GemmParams p, long long tiles, cudaStream_t s) {
+    static_assert(EW == 4 || (EW == 8 && !LORA && BN == 256 &&
+                              (EPI == EPI_GLU_BWD || EPI == EPI_GLU_DM)),
+                  "eight epilogue warps: the epilogue-bound GLU backward only");
+    constexpr bool wide = BN == 256;
+    constexpr int limit = wide ? (LORA ? gemm::SMEM_BYTES_LORA
+                                       : (EW == 8 ? gemm::SMEM_BYTES_EW8 : gemm::SMEM_BYTES))
+                               : 224 * 1024;
+    if (!wide) narrow_ring(p, BN, tiles, LORA);
+    const int smem = wide ? limit : gemm::narrow_smem(BN, p.stages, p.a_rows, LORA);
+    const int per_sm = wide || smem > 112 * 1024 ? 1 : 2;
+    const int grid = (int)std::min<long long>(tiles, (long long)num_sms() * per_sm);
+    static std::atomic<uint64_t> attr{0};  // per instantiation, one bit per device
+    cudaError_t e =
+        set_smem_limit(reinterpret_cast<const void*>(k_gemm<EPI, LORA, EW, BN>), limit, attr);
+    if (e != cudaSuccess) return e;
+    k_gemm<EPI, LORA, EW, BN><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, lg, p);
+    return cudaGetLastError();
+}
+
+// The launch of one epilogue at the tile width bn.
 template <int EPI, bool LORA, class LG, int EW = 4>
 static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
-                              const GemmParams& p, int grid, cudaStream_t s) {
-    static_assert(EW == 4 || (EW == 8 && !LORA &&
-                              (EPI == EPI_BF16 || EPI == EPI_F32 || EPI == EPI_RESID ||
-                               EPI == EPI_GLU_BWD || EPI == EPI_GLU_DM)),
-                  "eight epilogue warps: column-splittable epilogues without LoRA only");
-    constexpr int smem = LORA ? gemm::SMEM_BYTES_LORA
-                              : (EW == 8 ? gemm::SMEM_BYTES_EW8 : gemm::SMEM_BYTES);
-    static std::atomic<uint64_t> attr{0};  // per instantiation, one bit per device
-    cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(k_gemm<EPI, LORA, EW>), smem, attr);
-    if (e != cudaSuccess) return e;
-    k_gemm<EPI, LORA, EW><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, lg, p);
-    return cudaGetLastError();
+                              const GemmParams& p, int bn, long long tiles, cudaStream_t s) {
+    if constexpr (EW == 4) {
+        if (bn == 64) return launch_bn<EPI, LORA, LG, EW, 64>(ta, tb, lg, p, tiles, s);
+        if (bn == 128) return launch_bn<EPI, LORA, LG, EW, 128>(ta, tb, lg, p, tiles, s);
+    }
+    return launch_bn<EPI, LORA, LG, EW, 256>(ta, tb, lg, p, tiles, s);
+}
+
+// Box rows of the two operands' tensor maps at tile width bn.
+static int b_box(int bn) { return bn == 256 ? 256 : bn / 2; }
+
+// Rows of A a narrow stage holds: the tallest tile's rows, in powers of two.
+static int a_box(int bn, int most_rows) {
+    int r = gemm::BM;
+    while (bn < 256 && r > 16 && r / 2 >= most_rows) r /= 2;
+    return r;
 }
 
 // Tile-order group height: enough 128-row blocks of A to hold ~40 MB in L2
@@ -978,36 +1119,36 @@ jnx_status gemm_check(int M, int N, int K) {
 }
 
 jnx_status gemm_launch(const uint16_t* A, int lda, const uint16_t* B, int ldb, GemmParams p,
-                       cudaStream_t s, int max_ctas) {
+                       cudaStream_t s) {
     jnx_status st = gemm_check(p.M, p.N, p.K);
     if (st != JNX_OK) return st;
     if (p.M == 0) return JNX_OK;
+    const int m_tiles = (p.M + gemm::BM - 1) / gemm::BM;
+    const int bn = pick_bn(m_tiles, p);
+    p.a_rows = a_box(bn, std::min(p.M, gemm::BM));
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, gemm::BM, gemm::BK) ||
-        !make_tmap_bf16(&tb, B, p.N, p.K, ldb, gemm::BN, gemm::BK))
+    if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) ||
+        !make_tmap_bf16(&tb, B, p.N, p.K, ldb, b_box(bn), gemm::BK))
         return fail(JNX_ERR_CUDA, "gemm: tensor map encode failed (alignment or driver)");
-    const int tiles = ((p.M + gemm::BM - 1) / gemm::BM) * (p.N / gemm::BN);
-    int grid = num_sms();
-    if (max_ctas > 0 && max_ctas < grid) grid = max_ctas;
-    if (tiles < grid) grid = tiles;
+    const long long tiles = (long long)m_tiles * (p.N / bn);
     if (p.group_m <= 0) p.group_m = default_group_m(p.K);
     cudaError_t e;
     const NoLora none{};
     switch (p.epi) {
-        case EPI_BF16: e = launch_epi<EPI_BF16, false>(ta, tb, none, p, grid, s); break;
+        case EPI_BF16: e = launch_epi<EPI_BF16, false>(ta, tb, none, p, bn, tiles, s); break;
         // eight epilogue warps only where the epilogue is the bottleneck: with
         // the fp32 and residual epilogues they slowed the GEMMs on GB300 (the
         // 7B-class O / down projections 1,314 / 1,460 -> 1,246 / 1,419 TFLOP/s)
-        case EPI_F32: e = launch_epi<EPI_F32, false>(ta, tb, none, p, grid, s); break;
-        case EPI_RESID: e = launch_epi<EPI_RESID, false>(ta, tb, none, p, grid, s); break;
-        case EPI_GLU: e = launch_epi<EPI_GLU, false>(ta, tb, none, p, grid, s); break;
-        case EPI_ROPE: e = launch_epi<EPI_ROPE, false>(ta, tb, none, p, grid, s); break;
+        case EPI_F32: e = launch_epi<EPI_F32, false>(ta, tb, none, p, bn, tiles, s); break;
+        case EPI_RESID: e = launch_epi<EPI_RESID, false>(ta, tb, none, p, bn, tiles, s); break;
+        case EPI_GLU: e = launch_epi<EPI_GLU, false>(ta, tb, none, p, bn, tiles, s); break;
+        case EPI_ROPE: e = launch_epi<EPI_ROPE, false>(ta, tb, none, p, bn, tiles, s); break;
         case EPI_GLU_BWD:
-            e = launch_epi<EPI_GLU_BWD, false, NoLora, 8>(ta, tb, none, p, grid, s);
+            e = launch_epi<EPI_GLU_BWD, false, NoLora, 8>(ta, tb, none, p, bn, tiles, s);
             break;
-        case EPI_GLU_SAVE: e = launch_epi<EPI_GLU_SAVE, false>(ta, tb, none, p, grid, s); break;
+        case EPI_GLU_SAVE: e = launch_epi<EPI_GLU_SAVE, false>(ta, tb, none, p, bn, tiles, s); break;
         case EPI_GLU_DM:
-            e = launch_epi<EPI_GLU_DM, false, NoLora, 8>(ta, tb, none, p, grid, s);
+            e = launch_epi<EPI_GLU_DM, false, NoLora, 8>(ta, tb, none, p, bn, tiles, s);
             break;
         default: return fail(JNX_ERR_INVALID_ARG, "gemm: unknown epilogue %d", p.epi);
     }
@@ -1028,7 +1169,7 @@ jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ld
     lg.n_parts = 0;
     lg.seg_b = 1;
     lg.n_seg = n_seg;
-    int tiles = 0;
+    int tiles = 0, most = 0;
     for (int i = 0; i < n_seg; ++i) {
         if (seg_r0[i] < 0 || seg_r1[i] < seg_r0[i] || seg_r1[i] > p.M || seg_tenant[i] < 0 ||
             seg_tenant[i] >= n_tenants)
@@ -1038,25 +1179,27 @@ jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ld
         lg.seg_tenant[i] = seg_tenant[i];
         lg.seg_tile0[i] = tiles;
         tiles += (seg_r1[i] - seg_r0[i] + gemm::BM - 1) / gemm::BM;
+        most = std::max(most, std::min(seg_r1[i] - seg_r0[i], gemm::BM));
     }
     lg.seg_tile0[n_seg] = tiles;
+    if (tiles == 0) return JNX_OK;
+    p.seg_bn = 1;
+    const int bn = pick_bn(tiles, p);
+    p.a_rows = a_box(bn, most);
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, gemm::BM, gemm::BK) ||
-        !make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.N, p.K, ldb, gemm::BN, gemm::BK))
+    if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) ||
+        !make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.N, p.K, ldb, b_box(bn), gemm::BK))
         return fail(JNX_ERR_CUDA, "gemm: tensor map encode failed (alignment or driver)");
-    const int total = tiles * (p.N / gemm::BN);
-    if (total == 0) return JNX_OK;
-    int grid = num_sms();
-    if (total < grid) grid = total;
+    const long long total = (long long)tiles * (p.N / bn);
     if (p.group_m <= 0) p.group_m = default_group_m(p.K);
     cudaError_t e;
     switch (p.epi) {
-        case EPI_BF16: e = launch_epi<EPI_BF16, true>(ta, tb, lg, p, grid, s); break;
-        case EPI_F32: e = launch_epi<EPI_F32, true>(ta, tb, lg, p, grid, s); break;
-        case EPI_RESID: e = launch_epi<EPI_RESID, true>(ta, tb, lg, p, grid, s); break;
-        case EPI_GLU: e = launch_epi<EPI_GLU, true>(ta, tb, lg, p, grid, s); break;
-        case EPI_GLU_SAVE: e = launch_epi<EPI_GLU_SAVE, true>(ta, tb, lg, p, grid, s); break;
-        case EPI_GLU_BWD: e = launch_epi<EPI_GLU_BWD, true>(ta, tb, lg, p, grid, s); break;
+        case EPI_BF16: e = launch_epi<EPI_BF16, true>(ta, tb, lg, p, bn, total, s); break;
+        case EPI_F32: e = launch_epi<EPI_F32, true>(ta, tb, lg, p, bn, total, s); break;
+        case EPI_RESID: e = launch_epi<EPI_RESID, true>(ta, tb, lg, p, bn, total, s); break;
+        case EPI_GLU: e = launch_epi<EPI_GLU, true>(ta, tb, lg, p, bn, total, s); break;
+        case EPI_GLU_SAVE: e = launch_epi<EPI_GLU_SAVE, true>(ta, tb, lg, p, bn, total, s); break;
+        case EPI_GLU_BWD: e = launch_epi<EPI_GLU_BWD, true>(ta, tb, lg, p, bn, total, s); break;
         default: return fail(JNX_ERR_INVALID_ARG, "gemm: epilogue %d unsupported here", p.epi);
     }
     if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
@@ -1096,23 +1239,23 @@ jnx_status gemm_launch_lora(const uint16_t* A, int lda, const uint16_t* B, int l
         tiles += (ls.seg_r1[i] - ls.seg_r0[i] + gemm::BM - 1) / gemm::BM;
     }
     lg.seg_tile0[ls.n_seg] = tiles;
+    if (tiles == 0) return JNX_OK;
+    const int bn = pick_bn(tiles, p);
+    p.a_rows = gemm::BM;  // the adapters' t rows come in whole tiles too
     CUtensorMap ta, tb;
-    bool ok = make_tmap_bf16(&ta, A, p.M, p.K, lda, gemm::BM, gemm::BK) &&
-              make_tmap_bf16(&tb, B, p.N, p.K, ldb, gemm::BN, gemm::BK) &&
+    bool ok = make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) &&
+              make_tmap_bf16(&tb, B, p.N, p.K, ldb, b_box(bn), gemm::BK) &&
               make_tmap_bf16(&lg.tt, ls.t, p.M, ls.ldt, ls.ldt, gemm::BM, 16, 32);
     for (int i = 0; i < ls.n_parts && ok; ++i) {
         lg.part_cols[i] = ls.cols[i];
         ok = make_tmap_bf16(&lg.tb[i], ls.b[i], (uint64_t)ls.n_tenants * ls.cols[i], kLoraRank,
-                            kLoraRank, gemm::BN, 16, 32);
+                            kLoraRank, b_box(bn), 16, 32);
     }
     if (!ok) return fail(JNX_ERR_CUDA, "gemm: LoRA tensor map encode failed");
-    const int total = tiles * (p.N / gemm::BN);
-    if (total == 0) return JNX_OK;
-    int grid = num_sms();
-    if (total < grid) grid = total;
+    const long long total = (long long)tiles * (p.N / bn);
     if (p.group_m <= 0) p.group_m = default_group_m(p.K);
-    cudaError_t e = p.epi == EPI_ROPE ? launch_epi<EPI_ROPE, true>(ta, tb, lg, p, grid, s)
-                                      : launch_epi<EPI_RESID, true>(ta, tb, lg, p, grid, s);
+    cudaError_t e = p.epi == EPI_ROPE ? launch_epi<EPI_ROPE, true>(ta, tb, lg, p, bn, total, s)
+                                      : launch_epi<EPI_RESID, true>(ta, tb, lg, p, bn, total, s);
     if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
     return JNX_OK;
 }

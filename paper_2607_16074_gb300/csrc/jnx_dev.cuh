@@ -290,6 +290,24 @@ __device__ __forceinline__ void tc_mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, 
         : "memory");
 }
 
+// One thread of a fully active warp (always the same one).  A warp that
+// issues tcgen05 or TMA instructions runs its loop with all lanes, so that
+// addresses and descriptors are warp-uniform values, and elects a thread for
+// the instructions themselves; in a branch of lane 0 every operand is moved
+// to the uniform registers those instructions read, one by one.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// A value that every lane of the warp holds, as one the compiler knows to be so.
+__device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 // Arrive on `bar` once all previously issued tcgen05 ops of this thread finish.
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
     asm volatile(
@@ -429,6 +447,16 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t smem_addr) {
     d |= (uint64_t)1 << 46;                         // descriptor version (sm_100 family)
     d |= (uint64_t)2 << 61;                         // layout: 128-byte swizzle
     return d;
+}
+
+// The two halves of sw128_desc: the low word moves with the address (16 bytes a
+// unit), the high word is a constant.
+constexpr uint32_t kSw128DescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t sw128_desc_lo(uint32_t smem_addr) {
+    return ((smem_addr & 0x3FFFF) >> 4) | (1u << 16);
+}
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo, uint32_t hi) {
+    return ((uint64_t)hi << 32) | lo;
 }
 
 // Descriptor for an MN-major bf16 operand stored with the 128-byte swizzle:

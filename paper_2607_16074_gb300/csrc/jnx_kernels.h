@@ -31,7 +31,7 @@ struct GemmParams {
     int* status;          // device status word
     // RMSNorm folded across two GEMMs.  EPI_RESID with norm_gamma set also
     // writes y = bf16(x_new * gamma[col]) to norm_out [M, N] and, per row and
-    // 128-column block, the partial sum of x_new^2 to ss_out [M, N / 128].
+    // 64-column block, the partial sum of x_new^2 to ss_out [M, N / 64].
     const uint16_t* norm_gamma;
     uint16_t* norm_out;
     float* ss_out;
@@ -60,6 +60,9 @@ struct GemmParams {
     // EPI_BF16 with pack_up set writes output column n to packed column
     // 256 (n / 128) + 128 + n % 128 (dm into the up columns for EPI_GLU_DM).
     int pack_up;
+    // set by the launchers: narrow tiles' ring (stages, A rows a stage holds),
+    // and that the launch is segmented
+    int stages, a_rows, seg_bn;
 };
 
 constexpr int kMaxRopePos = 1 << 16;  // longest sample a workspace reserves RoPE rows for
@@ -127,7 +130,7 @@ jnx_status lora_down_launch(const jnx_group* g, const uint16_t* x, int ldx, int 
 // GEMM C = A . B^T with A [M, K] (row stride lda), B [N, K] (row stride ldb).
 jnx_status gemm_check(int M, int N, int K);
 jnx_status gemm_launch(const uint16_t* A, int lda, const uint16_t* B, int ldb, GemmParams p,
-                       cudaStream_t s, int max_ctas = 0);
+                       cudaStream_t s);
 bool make_tmap_bf16(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols,
                     uint64_t row_stride_elems, uint32_t box_rows, uint32_t box_cols,
                     int swizzle_bytes = 128);
@@ -152,7 +155,7 @@ jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, c
                              int S, int d, float* pooled, uint16_t* hidden, cudaStream_t s);
 
 // Folded RMSNorm, first half: y = bf16(x * gamma) [M, d] and per row and
-// 128-column block the sum of x^2 (ss [M, d / 128]).
+// 64-column block the sum of x^2 (ss [M, d / 64]).
 jnx_status rms_prep_launch(const float* x, const uint16_t* gamma, int M, int d, uint16_t* y,
                            float* ss, cudaStream_t s);
 
