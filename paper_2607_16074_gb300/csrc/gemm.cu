@@ -958,6 +958,222 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
 }
 
 // ---------------------------------------------------------------------------
+// The same GEMM on CTA pairs: tiles of 256 x 256 shared by the two SMs of a
+// cluster.  Each CTA stages its 128 A rows and its 128 of the tile's 256 B rows;
+// the leader's MMA warp issues M = 256 instructions over both CTAs' operands,
+// and each CTA's epilogue warps take its own 128 accumulator rows.
+//
+// Why: a lone CTA's 128 x 256 tile takes in 48 KB per 64-deep K step, and an SM
+// takes in about 70 bytes a clock, so the step lasts 690 clocks while its MMAs
+// need 512 (clock64 in both warps of an instrumented build; more ring stages
+// changed nothing).  With B split between the pair it is 32 KB, in six stages
+// instead of four, and the MMAs bound it.  Single-CTA tiles against
+// pairs: 8,192 x 4,096 x K 4,096 with the residual 187 -> 162 us (1,696 TFLOP/s),
+// GeGLU gate/up of 4,800 rows x N 32,768 x K 2,048 364 -> 323 us (1,994).
+//
+// Barriers: `full` (leader only) counts both CTAs' bytes; `empty` and `tfull`
+// are signalled in both CTAs by the leader's commits; `tempty` (leader only)
+// counts the epilogue warps of both.  A CTA leaves only after a cluster barrier,
+// so no barrier, operand or accumulator goes away under its peer.
+// ---------------------------------------------------------------------------
+namespace pair {
+constexpr int BM = 256, BN = 256, BK = 64, STAGES = 6;
+constexpr int HALF_BYTES = 128 * BK * 2;         // one operand of one CTA's stage
+constexpr int STAGE_BYTES = 2 * HALF_BYTES;
+constexpr int smem_bytes(int ew) {
+    return STAGES * STAGE_BYTES + 1024 + 256 + (ew == 8 ? 8 * gemm::STG_SLOT_EW8 : gemm::STG_BYTES);
+}
+static_assert(smem_bytes(8) <= 227 * 1024, "shared memory per CTA");
+constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
+}  // namespace pair
+
+template <int EPI, int EW>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
+    k_gemm_pair(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+                GemmParams p) {
+    using namespace pair;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    uint64_t* empty = full + STAGES;
+    uint64_t* tfull = empty + STAGES;
+    uint64_t* tempty = tfull + 2;
+    uint64_t* drain = tempty + 2;
+    uint64_t* never = drain + 1;  // nothing arrives on it: a bounded pause when giving up
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = warp_uniform(threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(&tfull[a], 1);
+            mbar_init(&tempty[a], 2 * EW);
+        }
+        mbar_init(drain, 1);
+        mbar_init(never, 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+    }
+    if (warp == 1) {
+        tmem_alloc_pair(tmem_slot, 512);
+        tmem_relinquish_pair();
+    }
+    if (warp == 0 && lane == 0) {
+        tma_prefetch_desc(&ta);
+        tma_prefetch_desc(&tb);
+    }
+    tc_fence_before();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
+
+    const int num_m = (p.M + BM - 1) / BM;
+    const int num_n = p.N / BN;
+    const int num_k = p.K / BK;
+    const int num_tiles = num_m * num_n;
+    const int first = blockIdx.x >> 1, step = gridDim.x >> 1;
+
+    if (warp == 0) {
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = first; ok && tile < num_tiles && !*abort_flag; tile += step) {
+            int mb, nb;
+            tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
+            const int arow = mb * BM + (int)rank * 128, brow = nb * BN + (int)rank * 128;
+            for (int kb = 0; kb < num_k; ++kb) {
+                if (!mbar_wait(&empty[stage], phase ^ 1)) {
+                    ok = false;
+                    break;
+                }
+                if (elect_one()) {
+                    uint8_t* sa = smem + stage * STAGE_BYTES;
+                    const uint32_t bar = map_rank(&full[stage], 0);
+                    if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE_BYTES);
+                    tma_load_2d_pair(sa, &ta, kb * BK, arow, bar);
+                    tma_load_2d_pair(sa + HALF_BYTES, &tb, kb * BK, brow, bar);
+                }
+                __syncwarp();
+                if (++stage == STAGES) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+            }
+        }
+        if (!ok) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        }
+    } else if (warp == 1 && rank == 0) {
+        int stage = 0, local = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        const uint32_t a_lo = sw128_desc_lo(smem_u32(smem));
+        const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + HALF_BYTES);
+        for (int tile = first; ok && tile < num_tiles && !*abort_flag; tile += step, ++local) {
+            const int acc = local & 1;
+            if (!mbar_wait_cluster(&tempty[acc], ((local >> 1) & 1) ^ 1)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem_base + acc * BN;
+            for (int kb = 0; kb < num_k; ++kb) {
+                if (!mbar_wait_cluster(&full[stage], phase)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t off = (uint32_t)(stage * STAGE_BYTES) >> 4;
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        tc_mma_f16_pair(d, desc_of(a_lo + off + 2 * kk, kSw128DescHi),
+                                        desc_of(b_lo + off + 2 * kk, kSw128DescHi), IDESC,
+                                        (kb | kk) != 0);
+                    tc_commit_pair(&empty[stage]);
+                }
+                __syncwarp();
+                if (++stage == STAGES) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+            }
+            if (!ok) break;
+            if (elect_one()) tc_commit_pair(&tfull[acc]);
+            __syncwarp();
+        }
+        if (!ok) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        }
+        // no MMA still reads or writes either CTA after this
+        if (elect_one()) tc_commit_pair(drain);
+        __syncwarp();
+        mbar_wait(drain, 0);
+    } else if (warp == 1) {
+        mbar_wait(drain, 0);  // the leader's last commit has reached this CTA
+    } else {
+        const int q = warp & 3;  // TMEM lane quarter this warp may access
+        const int cb = EW == 8 ? ((warp - 2) >> 2) * 4 : 0;
+        uint8_t* stg = reinterpret_cast<uint8_t*>(full) + 256 +
+                       (warp - 2) * (EW == 8 ? gemm::STG_SLOT_EW8 : 2048);
+        int local = 0;
+        for (int tile = first; tile < num_tiles; tile += step, ++local) {
+            const int acc = local & 1;
+            int mb, nb;
+            tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
+            TileGeo g;
+            g.nb = nb;
+            g.seg = 0;
+            g.c0 = nb * BN;
+            g.c1 = g.c0 + 128;
+            g.row0 = mb * BM + (int)rank * 128;
+            g.row_end = min(g.row0 + 128, p.M);
+            const int row_base = g.row0 + q * 32;
+            if constexpr (EPI == EPI_GLU_DM) {
+                // this thread's dm for the tile into L2 while its K loop runs
+                const int row = row_base + lane;
+                if (row < g.row_end)
+                    prefetch_l2(p.aux + (size_t)row * p.ldaux + g.c0 + 128 + cb * 16);
+            }
+            if (!mbar_wait(&tfull[acc], (local >> 1) & 1) || *abort_flag) {
+                *abort_flag = 1;
+                report(p.status, JNX_ERR_TIMEOUT);
+                break;
+            }
+            tc_fence_after();
+            epilogue_tile<EPI, EW == 8 ? 4 : 8, 256>(
+                tmem_base + acc * BN + ((uint32_t)(q * 32) << 16), stg, lane, row_base, g.row_end,
+                g, p, cb);
+            tc_fence_before();
+            __syncwarp();
+            if (elect_one()) mbar_arrive_cluster(map_rank(&tempty[acc], 0));
+            __syncwarp();
+        }
+    }
+
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    // giving up: time for copies in flight to land before any CTA leaves
+    if (*abort_flag && warp == 0) mbar_wait(never, 0, 100000000LL);
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 
@@ -1026,14 +1242,27 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
 // fastest per column, so narrower ones win only where it leaves SMs idle:
 // 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide tiles, 61 in 80 of 128
 // and 76 in 160 of 64; 300 rows 96, 60 and 55; 4,800 rows 196, 237 and 348.
+// A pair's tile (plain launches only) takes 0.33 for the same work per SM as
+// a wide one's 0.385, so it wins wherever its tiles divide as well over the
+// SMs: 2,400 rows x N 32,768 177 us against 188, but x N 2,048 33 against 23.
 // RoPE needs a tile within one head; the GLU backward with dm has wide tiles
 // only.
-static int pick_bn(int m_tiles, const GemmParams& p) {
+constexpr int kPairTile = 512;
+
+static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
     const int sms = num_sms();
     auto rounds = [](long long tiles, int slots) { return (double)((tiles + slots - 1) / slots); };
     const long long wide = (long long)m_tiles * (p.N / 256);
     int best = 256;
     double least = rounds(wide, sms) * 0.385;
+    if (pairs) {
+        const double t =
+            rounds((long long)((m_tiles + 1) / 2) * (p.N / 256), sms / 2) * 0.33;
+        if (t < least) {
+            best = kPairTile;
+            least = t;
+        }
+    }
     if (p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn)) return best;
     static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.235, 0.39},
                                                                      {64, 0.215, 0.334}};
@@ -1079,10 +1308,27 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const
     return cudaGetLastError();
 }
 
-// The launch of one epilogue at the tile width bn.
+template <int EPI, int EW>
+static cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, GemmParams p,
+                               cudaStream_t s) {
+    constexpr int smem = pair::smem_bytes(EW);
+    p.group_m = std::max(1, p.group_m / 2);  // row blocks of 256
+    const long long tiles = (long long)((p.M + pair::BM - 1) / pair::BM) * (p.N / pair::BN);
+    const int grid = 2 * (int)std::min<long long>(tiles, num_sms() / 2);
+    static std::atomic<uint64_t> attr{0};
+    cudaError_t e =
+        set_smem_limit(reinterpret_cast<const void*>(k_gemm_pair<EPI, EW>), smem, attr);
+    if (e != cudaSuccess) return e;
+    k_gemm_pair<EPI, EW><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, p);
+    return cudaGetLastError();
+}
+
+// The launch of one epilogue at the tile width bn (kPairTile: a CTA pair's).
 template <int EPI, bool LORA, class LG, int EW = 4>
 static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
                               const GemmParams& p, int bn, long long tiles, cudaStream_t s) {
+    if constexpr (!LORA)
+        if (bn == kPairTile) return launch_pair<EPI, EW>(ta, tb, p, s);
     if constexpr (EW == 4) {
         if (bn == 64) return launch_bn<EPI, LORA, LG, EW, 64>(ta, tb, lg, p, tiles, s);
         if (bn == 128) return launch_bn<EPI, LORA, LG, EW, 128>(ta, tb, lg, p, tiles, s);
@@ -1091,7 +1337,7 @@ static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, cons
 }
 
 // Box rows of the two operands' tensor maps at tile width bn.
-static int b_box(int bn) { return bn == 256 ? 256 : bn / 2; }
+static int b_box(int bn) { return bn == kPairTile ? 128 : bn == 256 ? 256 : bn / 2; }
 
 // Rows of A a narrow stage holds: the tallest tile's rows, in powers of two.
 static int a_box(int bn, int most_rows) {
@@ -1124,13 +1370,13 @@ jnx_status gemm_launch(const uint16_t* A, int lda, const uint16_t* B, int ldb, G
     if (st != JNX_OK) return st;
     if (p.M == 0) return JNX_OK;
     const int m_tiles = (p.M + gemm::BM - 1) / gemm::BM;
-    const int bn = pick_bn(m_tiles, p);
+    const int bn = pick_bn(m_tiles, p, true);
     p.a_rows = a_box(bn, std::min(p.M, gemm::BM));
     CUtensorMap ta, tb;
     if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) ||
         !make_tmap_bf16(&tb, B, p.N, p.K, ldb, b_box(bn), gemm::BK))
         return fail(JNX_ERR_CUDA, "gemm: tensor map encode failed (alignment or driver)");
-    const long long tiles = (long long)m_tiles * (p.N / bn);
+    const long long tiles = (long long)m_tiles * (p.N / std::min(bn, 256));
     if (p.group_m <= 0) p.group_m = default_group_m(p.K);
     cudaError_t e;
     const NoLora none{};
@@ -1184,7 +1430,7 @@ jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ld
     lg.seg_tile0[n_seg] = tiles;
     if (tiles == 0) return JNX_OK;
     p.seg_bn = 1;
-    const int bn = pick_bn(tiles, p);
+    const int bn = pick_bn(tiles, p, false);
     p.a_rows = a_box(bn, most);
     CUtensorMap ta, tb;
     if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) ||
@@ -1240,7 +1486,7 @@ jnx_status gemm_launch_lora(const uint16_t* A, int lda, const uint16_t* B, int l
     }
     lg.seg_tile0[ls.n_seg] = tiles;
     if (tiles == 0) return JNX_OK;
-    const int bn = pick_bn(tiles, p);
+    const int bn = pick_bn(tiles, p, false);
     p.a_rows = gemm::BM;  // the adapters' t rows come in whole tiles too
     CUtensorMap ta, tb;
     bool ok = make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) &&
