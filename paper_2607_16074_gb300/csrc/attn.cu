@@ -120,6 +120,16 @@ __device__ __forceinline__ AttnWork attn_fetch(const AttnItems& it, const int* _
     return a;
 }
 
+// The item as warp-uniform values.
+__device__ __forceinline__ AttnWork attn_uniform(AttnWork a) {
+    a.h = warp_uniform(a.h);
+    a.qt = warp_uniform(a.qt);
+    a.start = warp_uniform(a.start);
+    a.L = warp_uniform(a.L);
+    a.valid = warp_uniform(a.valid);
+    return a;
+}
+
 // Epilogue staging of 16 output columns (32 bytes a row) through a 1 KB
 // slot per softmax warp: thread `lane` puts its row's two 16-byte units;
 // in round i thread `lane` gets row 16 i + lane / 2, unit lane % 2, so each
@@ -240,7 +250,7 @@ __global__ void __launch_bounds__(HD == 256 ? 384 : 640, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + C::OFF_BAR + C::NST * C::NBAR * 8);
     volatile int* fail_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     // stream of this warp: producers 0/1, MMA issuers 2/3, then per stream
     // 4 SPLIT softmax warps (stream t, half h, lane quarter q: warp
     // 4 + 4 SPLIT t + 4 h + q, so warp % 4 = q)
@@ -288,41 +298,52 @@ __global__ void __launch_bounds__(HD == 256 ? 384 : 640, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = *tmem_slot + (uint32_t)t * C::TSTRIDE;
+    const uint32_t tbase = warp_uniform(*tmem_slot) + (uint32_t)t * C::TSTRIDE;
 
     if (warp < 2) {
         // ---------------- producer of stream t ----------------
-        if (lane == 0 && t < C::NST) {
-            tma_prefetch_desc(&tq);
-            tma_prefetch_desc(&tkv);
+        // all lanes run the loop, an elected one issues (see elect_one)
+        if (t < C::NST) {
+            if (elect_one()) {
+                tma_prefetch_desc(&tq);
+                tma_prefetch_desc(&tkv);
+            }
             bool ok = true;
             int nq = 0;            // Q tiles loaded
             uint32_t gk = 0, gv = 0;  // K / V tiles loaded
             auto load_kv = [&](bool is_v, uint32_t& g, int y, int col) -> bool {
                 const int b = g & 1;
                 uint64_t* full = is_v ? &v_full[b] : &k_full[b];
-                if (!mbar_wait(is_v ? &v_empty[b] : &k_empty[b], ((g >> 1) & 1) ^ 1)) return false;
-                mbar_arrive_expect_tx(full, C::KB);
-                uint8_t* dst = is_v ? sV(b) : sK(b);
+                if (!mbar_wait_warp(is_v ? &v_empty[b] : &k_empty[b], ((g >> 1) & 1) ^ 1))
+                    return false;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, C::KB);
+                    uint8_t* dst = is_v ? sV(b) : sK(b);
 #pragma unroll
-                for (int c = 0; c < NCH; ++c)
-                    tma_load_2d(dst + c * BN * 128, &tkv, col + c * 64, y, full);
+                    for (int c = 0; c < NCH; ++c)
+                        tma_load_2d(dst + c * BN * 128, &tkv, col + c * 64, y, full);
+                }
+                __syncwarp();
                 ++g;
                 return true;
             };
             AttnWork nxt = attn_fetch(items, cu, H, w0, n_work);
-            for (int w = w0; w < n_work && ok && !*fail_flag; w += dw) {
-                const AttnWork a = nxt;
+            for (int w = w0; w < n_work && ok && !__any_sync(0xffffffffu, *fail_flag); w += dw) {
+                const AttnWork a = attn_uniform(nxt);
                 nxt = attn_fetch(items, cu, H, w + dw, n_work);
                 if (!a.valid) continue;
                 const int start = a.start, L = a.L, qt = a.qt, h = a.h;
                 const int n_kt = (L + BN - 1) / BN;
                 const int kvh = h / group;
-                if (nq > 0 && !(ok = mbar_wait(q_empty, (nq - 1) & 1))) break;
-                mbar_arrive_expect_tx(q_full, C::QB);
+                if (nq > 0 && !(ok = mbar_wait_warp(q_empty, (nq - 1) & 1))) break;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(q_full, C::QB);
 #pragma unroll
-                for (int c = 0; c < NCH; ++c)
-                    tma_load_2d(sQ + c * BM * 128, &tq, h * HD + c * 64, start + qt * BM, q_full);
+                    for (int c = 0; c < NCH; ++c)
+                        tma_load_2d(sQ + c * BM * 128, &tq, h * HD + c * 64, start + qt * BM,
+                                    q_full);
+                }
+                __syncwarp();
                 ++nq;
                 // K runs one tile ahead of V: S(kt + 1) is issued before PV(kt)
                 for (int j = 0; j <= n_kt && ok; ++j) {
@@ -332,18 +353,18 @@ __global__ void __launch_bounds__(HD == 256 ? 384 : 640, 1)
                 }
             }
             if (!ok) *fail_flag = 1;
-            // teardown: every copy this thread issued has landed before the
+            // teardown: every copy this warp issued has landed before the
             // CTA may exit (immediate in a normal run: the MMA warp has
             // consumed them all)
-            if (nq > 0) mbar_wait(q_full, (nq - 1) & 1);
+            if (nq > 0) mbar_wait_warp(q_full, (nq - 1) & 1);
             for (uint32_t k = 0; k < 2 && k < gk; ++k)
-                mbar_wait(&k_full[(gk - 1 - k) & 1], ((gk - 1 - k) >> 1) & 1);
+                mbar_wait_warp(&k_full[(gk - 1 - k) & 1], ((gk - 1 - k) >> 1) & 1);
             for (uint32_t k = 0; k < 2 && k < gv; ++k)
-                mbar_wait(&v_full[(gv - 1 - k) & 1], ((gv - 1 - k) >> 1) & 1);
+                mbar_wait_warp(&v_full[(gv - 1 - k) & 1], ((gv - 1 - k) >> 1) & 1);
         }
     } else if (warp < 4) {
         // ---------------- MMA issuer of stream t ----------------
-        if (lane == 0 && t < C::NST) {
+        if (t < C::NST) {
             constexpr uint32_t IDESC_S = idesc_bf16_f32(BM, BN);
             constexpr uint32_t IDESC_PV = idesc_bf16_f32(BM, HD) | (1u << 16);  // B MN-major
             bool ok = true, issued = false;
@@ -352,73 +373,86 @@ __global__ void __launch_bounds__(HD == 256 ? 384 : 640, 1)
             uint32_t gs = 0;             // S tiles issued (score buffer gs & 1)
             uint32_t gp = 0;             // p_full completions consumed = PVs issued
             int items_done = 0;
-            auto issue_s = [&](const uint32_t qa) -> bool {
+            const uint32_t q_lo = sw128_desc_lo(smem_u32(sQ));
+            auto issue_s = [&]() -> bool {
                 const int b = gk & 1;
-                if (!mbar_wait(&k_full[b], (gk >> 1) & 1)) return false;
+                if (!mbar_wait_warp(&k_full[b], (gk >> 1) & 1)) return false;
                 tc_fence_after();
-                const uint32_t ka = smem_u32(sK(b));
+                const uint32_t k_lo = sw128_desc_lo(smem_u32(sK(b)));
                 const uint32_t d = tbase + (gs & 1) * BN;
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < HD / 16; ++ks)
-                    tc_mma_f16(d, sw128_desc(qa + (ks >> 2) * BM * 128 + (ks & 3) * 32),
-                               sw128_desc(ka + (ks >> 2) * BN * 128 + (ks & 3) * 32), IDESC_S,
-                               ks > 0);
-                tc_commit(&s_full[gs & 1]);
-                tc_commit(&k_empty[b]);
+                    for (int ks = 0; ks < HD / 16; ++ks)
+                        tc_mma_f16(
+                            d, desc_of(q_lo + (ks >> 2) * BM * 8 + (ks & 3) * 2, kSw128DescHi),
+                            desc_of(k_lo + (ks >> 2) * BN * 8 + (ks & 3) * 2, kSw128DescHi),
+                            IDESC_S, ks > 0);
+                    tc_commit(&s_full[gs & 1]);
+                    tc_commit(&k_empty[b]);
+                }
+                __syncwarp();
                 ++gk;
                 ++gs;
                 issued = true;
                 return true;
             };
+            auto release_q = [&] {
+                if (elect_one()) tc_commit(q_empty);
+                __syncwarp();
+            };
             AttnWork nxt = attn_fetch(items, cu, H, w0, n_work);
-            for (int w = w0; w < n_work && ok && !*fail_flag; w += dw) {
-                const AttnWork a = nxt;
+            for (int w = w0; w < n_work && ok && !__any_sync(0xffffffffu, *fail_flag); w += dw) {
+                const AttnWork a = attn_uniform(nxt);
                 nxt = attn_fetch(items, cu, H, w + dw, n_work);
                 if (!a.valid) continue;
                 const int n_kt = (a.L + BN - 1) / BN;
-                if (!(ok = mbar_wait(q_full, nq & 1))) break;
+                if (!(ok = mbar_wait_warp(q_full, nq & 1))) break;
                 ++nq;
                 tc_fence_after();
-                const uint32_t qa = smem_u32(sQ);
                 // S(0), S(1): their score buffers were read before the
                 // previous item's last PVs were issued
-                ok = issue_s(qa) && (n_kt < 2 || issue_s(qa));
-                if (ok && n_kt <= 2) tc_commit(q_empty);
+                ok = issue_s() && (n_kt < 2 || issue_s());
+                if (ok && n_kt <= 2) release_q();
                 for (int kt = 0; kt < n_kt && ok; ++kt) {
                     // P(kt) is in TMEM, over S(kt) in score buffer gp & 1
                     const uint32_t pb = gp & 1;
-                    if (!(ok = mbar_wait(&p_full[pb], (gp >> 1) & 1))) break;
+                    if (!(ok = mbar_wait_warp(&p_full[pb], (gp >> 1) & 1))) break;
                     ++gp;
                     // the first PV of an item overwrites O: the previous
                     // item's epilogue must have read it
-                    if (kt == 0 && items_done > 0 && !(ok = mbar_wait(o_free, (items_done - 1) & 1)))
+                    if (kt == 0 && items_done > 0 &&
+                        !(ok = mbar_wait_warp(o_free, (items_done - 1) & 1)))
                         break;
                     const int b = gv & 1;
-                    if (!(ok = mbar_wait(&v_full[b], (gv >> 1) & 1))) break;
+                    if (!(ok = mbar_wait_warp(&v_full[b], (gv >> 1) & 1))) break;
                     tc_fence_after();
                     const uint32_t pa = tbase + pb * BN, va = smem_u32(sV(b));
+                    if (elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < BN / 16; ++ks)  // 16 keys = 8 TMEM columns of P
-                        tc_mma_f16_ts(tbase + C::O_COL, pa + ks * 8,
-                                      sw128_desc_mn(va + ks * 16 * 128, BN * 128, 1024), IDESC_PV,
-                                      kt > 0 || ks > 0);
-                    tc_commit(&o_done[pb]);
-                    tc_commit(&v_empty[b]);
+                        for (int ks = 0; ks < BN / 16; ++ks)  // 16 keys = 8 TMEM columns of P
+                            tc_mma_f16_ts(tbase + C::O_COL, pa + ks * 8,
+                                          sw128_desc_mn(va + ks * 16 * 128, BN * 128, 1024),
+                                          IDESC_PV, kt > 0 || ks > 0);
+                        tc_commit(&o_done[pb]);
+                        tc_commit(&v_empty[b]);
+                    }
+                    __syncwarp();
                     ++gv;
                     // S(kt + 2) reuses the score buffer of S(kt) / P(kt): the
-                    // tensor core runs this thread's MMAs in issue order, so
+                    // tensor core runs one thread's MMAs in issue order, so
                     // PV(kt) has read P(kt) before S(kt + 2) lands there
                     if (kt + 2 < n_kt) {
-                        ok = issue_s(qa);
-                        if (ok && kt + 3 == n_kt) tc_commit(q_empty);
+                        ok = issue_s();
+                        if (ok && kt + 3 == n_kt) release_q();
                     }
                 }
                 ++items_done;
             }
             if (!ok) *fail_flag = 1;
             if (issued) {
-                tc_commit(drain);
-                mbar_wait(drain, 0);
+                if (elect_one()) tc_commit(drain);
+                __syncwarp();
+                mbar_wait_warp(drain, 0);
             }
         }
     } else {

@@ -103,6 +103,16 @@ __device__ __forceinline__ BwdWork bwd_fetch(const BwdItems& it, const int* __re
     return a;
 }
 
+// The item as warp-uniform values.
+__device__ __forceinline__ BwdWork bwd_uniform(BwdWork a) {
+    a.tile = warp_uniform(a.tile);
+    a.hp = warp_uniform(a.hp);
+    a.start = warp_uniform(a.start);
+    a.L = warp_uniform(a.L);
+    a.valid = warp_uniform(a.valid);
+    return a;
+}
+
 template <int HD, int MODE>
 __global__ void __launch_bounds__(192, 1)
     k_attn_bwd(const __grid_constant__ CUtensorMap t_qkv_o, const __grid_constant__ CUtensorMap t_qkv_i,
@@ -137,7 +147,7 @@ __global__ void __launch_bounds__(192, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + abwd::kBars);
     volatile int* fail_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int group = H / Hkv;
     const int HP = IS_DQ ? H : Hkv;
     const int n_work = items.n * HP;
@@ -155,31 +165,39 @@ __global__ void __launch_bounds__(192, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = *tmem_slot;
+    const uint32_t tbase = warp_uniform(*tmem_slot);
     // inner tiles of an item
     auto n_inner = [&](int L) { return IS_DQ ? (L + BN - 1) / BN : group * ((L + BN - 1) / BN); };
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        if (lane == 0) {
-            tma_prefetch_desc(&t_qkv_o);
-            tma_prefetch_desc(&t_qkv_i);
-            tma_prefetch_desc(&t_do_o);
-            tma_prefetch_desc(&t_do_i);
+        // all lanes run the loop, an elected one issues (see elect_one)
+        {
+            if (elect_one()) {
+                tma_prefetch_desc(&t_qkv_o);
+                tma_prefetch_desc(&t_qkv_i);
+                tma_prefetch_desc(&t_do_o);
+                tma_prefetch_desc(&t_do_i);
+            }
             bool ok = true;
             int no = 0;              // outer tiles loaded
             uint32_t g1 = 0, g2 = 0;  // inner tiles loaded into each ring
             auto load_inner = [&](const CUtensorMap* map, uint8_t* dst, int col, int row,
                                   uint64_t* full) {
-                mbar_arrive_expect_tx(full, C::IB);
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, C::IB);
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) tma_load_2d(dst + c * BN * 128, map, col + c * 64, row, full);
+                    for (int c = 0; c < NCH; ++c)
+                        tma_load_2d(dst + c * BN * 128, map, col + c * 64, row, full);
+                }
+                __syncwarp();
             };
-            for (int w = blockIdx.x; w < n_work && ok && !*fail_flag; w += gridDim.x) {
-                const BwdWork a = bwd_fetch(items, cu, HP, w, n_work);
+            for (int w = blockIdx.x; w < n_work && ok && !__any_sync(0xffffffffu, *fail_flag); w += gridDim.x) {
+                const BwdWork a = bwd_uniform(bwd_fetch(items, cu, HP, w, n_work));
                 if (!a.valid) continue;
                 const int row0 = a.start + a.tile * BM;
-                if (no > 0 && !(ok = mbar_wait(o_empty, (no - 1) & 1))) break;
+                if (no > 0 && !(ok = mbar_wait_warp(o_empty, (no - 1) & 1))) break;
+                if (elect_one()) {
                 mbar_arrive_expect_tx(o_full, C::NEED_DP ? 2 * C::OB : C::OB);
                 if (IS_DQ) {
 #pragma unroll
@@ -197,6 +215,8 @@ __global__ void __launch_bounds__(192, 1)
                                         row0, o_full);
                     }
                 }
+                }
+                __syncwarp();
                 ++no;
                 const int n = n_inner(a.L);
                 const int nq = (a.L + BN - 1) / BN;
@@ -217,30 +237,30 @@ __global__ void __launch_bounds__(192, 1)
                         m2 = &t_do_i;
                     }
                     const int s1 = g1 % C::NB1;
-                    if (!(ok = mbar_wait(&b1_empty[s1], ((g1 / C::NB1) & 1) ^ 1))) break;
+                    if (!(ok = mbar_wait_warp(&b1_empty[s1], ((g1 / C::NB1) & 1) ^ 1))) break;
                     load_inner(&t_qkv_i, sB1(s1), c1, row, &b1_full[s1]);
                     ++g1;
                     const int s2 = g2 % C::NB2;
-                    if (!(ok = mbar_wait(&b2_empty[s2], ((g2 / C::NB2) & 1) ^ 1))) break;
+                    if (!(ok = mbar_wait_warp(&b2_empty[s2], ((g2 / C::NB2) & 1) ^ 1))) break;
                     load_inner(m2, sB2(s2), c2, row, &b2_full[s2]);
                     ++g2;
                 }
             }
             if (!ok) *fail_flag = 1;
             // teardown: every copy issued has landed before the CTA exits
-            if (no > 0) mbar_wait(o_full, (no - 1) & 1, 100000000LL);
+            if (no > 0) mbar_wait_warp(o_full, (no - 1) & 1, 100000000LL);
             for (uint32_t k = 0; k < (uint32_t)C::NB1 && k < g1; ++k) {
                 const uint32_t i = g1 - 1 - k;
-                mbar_wait(&b1_full[i % C::NB1], (i / C::NB1) & 1, 100000000LL);
+                mbar_wait_warp(&b1_full[i % C::NB1], (i / C::NB1) & 1, 100000000LL);
             }
             for (uint32_t k = 0; k < (uint32_t)C::NB2 && k < g2; ++k) {
                 const uint32_t i = g2 - 1 - k;
-                mbar_wait(&b2_full[i % C::NB2], (i / C::NB2) & 1, 100000000LL);
+                mbar_wait_warp(&b2_full[i % C::NB2], (i / C::NB2) & 1, 100000000LL);
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        {
             constexpr uint32_t IDESC_S = idesc_bf16_f32(BM, BN);
             constexpr uint32_t IDESC_ACC = idesc_bf16_f32(BM, HD) | (1u << 16);  // B MN-major
             bool ok = true, issued = false;
@@ -249,34 +269,44 @@ __global__ void __launch_bounds__(192, 1)
             uint32_t c1a = 0, c2a = 0;  // B1 / B2 tiles taken by the accumulating products
             uint32_t gs = 0, gp = 0;    // score tiles issued / P tiles consumed
             int items_done = 0;
-            const uint32_t a1 = smem_u32(sA1), a2 = smem_u32(sA2);
+            const uint32_t a1 = sw128_desc_lo(smem_u32(sA1)), a2 = sw128_desc_lo(smem_u32(sA2));
             auto issue_scores = [&]() -> bool {
                 const int s1 = c1s % C::NB1;
-                if (!mbar_wait(&b1_full[s1], (c1s / C::NB1) & 1)) return false;
+                if (!mbar_wait_warp(&b1_full[s1], (c1s / C::NB1) & 1)) return false;
                 tc_fence_after();
-                const uint32_t b1 = smem_u32(sB1(s1));
+                const uint32_t b1 = sw128_desc_lo(smem_u32(sB1(s1)));
                 const uint32_t d = tbase + C::S_COL + (gs & 1) * BN;
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < HD / 16; ++ks)
-                    tc_mma_f16(d, sw128_desc(a1 + (ks >> 2) * BM * 128 + (ks & 3) * 32),
-                               sw128_desc(b1 + (ks >> 2) * BN * 128 + (ks & 3) * 32), IDESC_S, ks > 0);
-                if (MODE == abwd::DV) tc_commit(&b1_empty[s1]);
+                    for (int ks = 0; ks < HD / 16; ++ks)
+                        tc_mma_f16(d,
+                                   desc_of(a1 + (ks >> 2) * BM * 8 + (ks & 3) * 2, kSw128DescHi),
+                                   desc_of(b1 + (ks >> 2) * BN * 8 + (ks & 3) * 2, kSw128DescHi),
+                                   IDESC_S, ks > 0);
+                    if (MODE == abwd::DV) tc_commit(&b1_empty[s1]);
+                }
+                __syncwarp();
                 ++c1s;
                 if (C::NEED_DP) {
                     const int s2 = c2s % C::NB2;
-                    if (!mbar_wait(&b2_full[s2], (c2s / C::NB2) & 1)) return false;
+                    if (!mbar_wait_warp(&b2_full[s2], (c2s / C::NB2) & 1)) return false;
                     tc_fence_after();
-                    const uint32_t b2 = smem_u32(sB2(s2));
+                    const uint32_t b2 = sw128_desc_lo(smem_u32(sB2(s2)));
                     const uint32_t d2 = tbase + C::DP_COL + (gs & 1) * BN;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < HD / 16; ++ks)
-                        tc_mma_f16(d2, sw128_desc(a2 + (ks >> 2) * BM * 128 + (ks & 3) * 32),
-                                   sw128_desc(b2 + (ks >> 2) * BN * 128 + (ks & 3) * 32), IDESC_S,
-                                   ks > 0);
-                    if (MODE == abwd::DQ || MODE == abwd::DK) tc_commit(&b2_empty[s2]);
+                        for (int ks = 0; ks < HD / 16; ++ks)
+                            tc_mma_f16(
+                                d2, desc_of(a2 + (ks >> 2) * BM * 8 + (ks & 3) * 2, kSw128DescHi),
+                                desc_of(b2 + (ks >> 2) * BN * 8 + (ks & 3) * 2, kSw128DescHi),
+                                IDESC_S, ks > 0);
+                        if (MODE == abwd::DQ || MODE == abwd::DK) tc_commit(&b2_empty[s2]);
+                    }
+                    __syncwarp();
                     ++c2s;
                 }
-                tc_commit(&s_full[gs & 1]);
+                if (elect_one()) tc_commit(&s_full[gs & 1]);
+                __syncwarp();
                 ++gs;
                 issued = true;
                 return true;
@@ -284,29 +314,36 @@ __global__ void __launch_bounds__(192, 1)
             // acc += X(tmem, 128 x 64 bf16) . B(smem inner tile, MN-major)
             auto acc_mma = [&](uint32_t acc_col, uint32_t xa, uint8_t* b, bool accumulate) {
                 const uint32_t ba = smem_u32(b);
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < BN / 16; ++ks)  // 16 inner rows = 8 TMEM columns of X
-                    tc_mma_f16_ts(tbase + acc_col, xa + ks * 8,
-                                  sw128_desc_mn(ba + ks * 16 * 128, BN * 128, 1024), IDESC_ACC,
-                                  accumulate || ks > 0);
+                    for (int ks = 0; ks < BN / 16; ++ks)  // 16 inner rows = 8 TMEM columns of X
+                        tc_mma_f16_ts(tbase + acc_col, xa + ks * 8,
+                                      sw128_desc_mn(ba + ks * 16 * 128, BN * 128, 1024), IDESC_ACC,
+                                      accumulate || ks > 0);
+                }
+                __syncwarp();
             };
-            for (int w = blockIdx.x; w < n_work && ok && !*fail_flag; w += gridDim.x) {
-                const BwdWork a = bwd_fetch(items, cu, HP, w, n_work);
+            auto commit = [&](uint64_t* bar) {
+                if (elect_one()) tc_commit(bar);
+                __syncwarp();
+            };
+            for (int w = blockIdx.x; w < n_work && ok && !__any_sync(0xffffffffu, *fail_flag); w += gridDim.x) {
+                const BwdWork a = bwd_uniform(bwd_fetch(items, cu, HP, w, n_work));
                 if (!a.valid) continue;
                 const int n = n_inner(a.L);
-                if (!(ok = mbar_wait(o_full, no & 1))) break;
+                if (!(ok = mbar_wait_warp(o_full, no & 1))) break;
                 ++no;
                 tc_fence_after();
                 ok = issue_scores() && (n < 2 || issue_scores());
-                if (ok && n <= 2) tc_commit(o_empty);
+                if (ok && n <= 2) commit(o_empty);
                 for (int kt = 0; kt < n && ok; ++kt) {
                     const uint32_t pb = gp & 1;
-                    if (!(ok = mbar_wait(&p_full[pb], (gp >> 1) & 1))) break;
+                    if (!(ok = mbar_wait_warp(&p_full[pb], (gp >> 1) & 1))) break;
                     ++gp;
                     // the first accumulating product of an item overwrites the
                     // accumulator: the previous item's epilogue must have read it
                     if (kt == 0 && items_done > 0 &&
-                        !(ok = mbar_wait(acc_free, (items_done - 1) & 1)))
+                        !(ok = mbar_wait_warp(acc_free, (items_done - 1) & 1)))
                         break;
                     tc_fence_after();
                     const uint32_t sb = tbase + C::S_COL + pb * BN;
@@ -314,21 +351,21 @@ __global__ void __launch_bounds__(192, 1)
                     if (MODE == abwd::DQ || MODE == abwd::DK) {
                         const int s1 = c1a % C::NB1;
                         acc_mma(C::ACC_COL, sb, sB1(s1), kt > 0);  // dS (over S) . B1
-                        tc_commit(&b1_empty[s1]);
+                        commit(&b1_empty[s1]);
                         ++c1a;
                     } else if (MODE == abwd::DV) {
                         const int s2 = c2a % C::NB2;
-                        if (!(ok = mbar_wait(&b2_full[s2], (c2a / C::NB2) & 1))) break;
+                        if (!(ok = mbar_wait_warp(&b2_full[s2], (c2a / C::NB2) & 1))) break;
                         tc_fence_after();
                         acc_mma(C::ACC_COL, sb, sB2(s2), kt > 0);  // P^T (over S) . dO
-                        tc_commit(&b2_empty[s2]);
+                        commit(&b2_empty[s2]);
                         ++c2a;
                     } else {  // DKV
                         const int s1 = c1a % C::NB1, s2 = c2a % C::NB2;
                         acc_mma(C::ACC_COL, db, sB1(s1), kt > 0);       // dS^T (over dP) . Q
                         acc_mma(C::ACC_COL + HD, sb, sB2(s2), kt > 0);  // P^T (over S) . dO
-                        tc_commit(&b1_empty[s1]);
-                        tc_commit(&b2_empty[s2]);
+                        commit(&b1_empty[s1]);
+                        commit(&b2_empty[s2]);
                         ++c1a;
                         ++c2a;
                     }
@@ -337,17 +374,17 @@ __global__ void __launch_bounds__(192, 1)
                     // the products above have read it before they land
                     if (kt + 2 < n) {
                         ok = issue_scores();
-                        if (ok && kt + 3 == n) tc_commit(o_empty);
+                        if (ok && kt + 3 == n) commit(o_empty);
                     }
                 }
                 if (!ok) break;
-                tc_commit(acc_full);
+                commit(acc_full);
                 ++items_done;
             }
             if (!ok) *fail_flag = 1;
             if (issued) {
-                tc_commit(drain);
-                mbar_wait(drain, 0, 100000000LL);
+                commit(drain);
+                mbar_wait_warp(drain, 0, 100000000LL);
             }
         }
     } else {

@@ -194,14 +194,13 @@ __device__ __forceinline__ void stg_store_bf16(uint8_t* stg, int lane, const uin
 // fixed order; 1 without a folded norm.
 __device__ __forceinline__ float row_norm_scale(const GemmParams& p, int row, bool valid) {
     if (p.ss_in == nullptr || !valid) return 1.f;
-    const float4* sp = reinterpret_cast<const float4*>(p.ss_in + (size_t)row * p.ss_parts);
+    // d / 128 of them, an even number
+    const float2* sp = reinterpret_cast<const float2*>(p.ss_in + (size_t)row * p.ss_parts);
     float t = 0.f;
-    for (int i = 0; i < p.ss_parts / 4; ++i) {
-        const float4 v = sp[i];
+    for (int i = 0; i < p.ss_parts / 2; ++i) {
+        const float2 v = sp[i];
         t += v.x;
         t += v.y;
-        t += v.z;
-        t += v.w;
     }
     return rsqrtf(t / (float)p.ss_cols + p.ss_eps);
 }
@@ -268,8 +267,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
         }
         // folded RMSNorm (EPI_RESID with norm_gamma): y = bf16(x * gamma) and
         // the sums of x^2 of each of this lane's four rows over its columns,
-        // one per 64-column block of the tile (4 staging passes each)
-        float ssq[NC / 2][4] = {};
+        // one per 128-column half of the tile (8 staging passes each)
+        float ssq[NC < 4 ? 1 : NC / 4][4] = {};
 #pragma unroll
         for (int lc = 0; lc < NC; ++lc) {
             const int c = cb + lc;
@@ -318,7 +317,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
                                                      __float_as_uint(o.z), __float_as_uint(o.w)),
                                           pol);
                     if (EPI == EPI_RESID && norm) {
-                        ssq[lp / 4][i] += o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w;
+                        ssq[lp / 8][i] += o.x * o.x + o.y * o.y + o.z * o.z + o.w * o.w;
                         if (row < row_end)
                             *reinterpret_cast<uint2*>(p.norm_out + (size_t)row * p.N + col) =
                                 make_uint2(pack_bf2(o.x * gf[0], o.y * gf[1]),
@@ -329,10 +328,10 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
             }
         }
         if (norm) {
-            // the four lanes of a row hold each block's columns between them
-            const int parts = p.N / 64;
+            // the four lanes of a row hold each half's columns between them
+            const int parts = p.N / 128;
 #pragma unroll
-            for (int hb = 0; hb < NC / 2; ++hb)
+            for (int hb = 0; hb < NC / 4; ++hb)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float t = ssq[hb][i];
@@ -340,7 +339,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
                     t += __shfl_xor_sync(0xffffffffu, t, 2);
                     const int row = row_base + 8 * i + (lane >> 2);
                     if ((lane & 3) == 0 && row < row_end)
-                        p.ss_out[(size_t)row * parts + (n0 + 32 * cb) / 64 + hb] = t;
+                        p.ss_out[(size_t)row * parts + (n0 + 32 * cb) / 128 + hb] = t;
                 }
         }
     } else if constexpr (EPI == EPI_GLU) {
@@ -772,13 +771,14 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
         int lj = 0;
         uint32_t lphase = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; ok && tile < num_tiles && !*abort_flag; tile += gridDim.x) {
+        for (int tile = blockIdx.x; ok && tile < num_tiles && !__any_sync(0xffffffffu, *abort_flag);
+             tile += gridDim.x) {
             const TileGeo g = tile_geo<EPI, LORA, BN>(tile, num_m, num_n, p, lg);
             int brow = 0;
             if constexpr (LORA)
                 if (lg.seg_b) brow = lg.seg_tenant[g.seg] * p.N;
             for (int kb = 0; kb < num_k; ++kb) {
-                if (!mbar_wait(&empty[stage], phase ^ 1)) {
+                if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
                     ok = false;
                     break;
                 }
@@ -802,7 +802,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
                 if (!ok) break;
                 if (lg.n_parts == 0) continue;  // segmented weights only
                 // this tile's t rows (its part) and its tenant's B rows
-                if (!mbar_wait(&lempty[lj], lphase ^ 1)) {
+                if (!mbar_wait_warp(&lempty[lj], lphase ^ 1)) {
                     ok = false;
                     break;
                 }
@@ -836,18 +836,18 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
         bool ok = true;
         const uint32_t a_lo = sw128_desc_lo(smem_u32(smem));
         const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + a_bytes);
-        for (int tile = blockIdx.x; ok && tile < num_tiles && !*abort_flag;
+        for (int tile = blockIdx.x; ok && tile < num_tiles && !__any_sync(0xffffffffu, *abort_flag);
              tile += gridDim.x, ++local) {
             const int acc = local & 1;
             const uint32_t acc_phase = (local >> 1) & 1;
-            if (!mbar_wait(&tempty[acc], acc_phase ^ 1)) {
+            if (!mbar_wait_warp(&tempty[acc], acc_phase ^ 1)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
             const uint32_t d = tmem_base + acc * BN;
             for (int kb = 0; kb < num_k; ++kb) {
-                if (!mbar_wait(&full[stage], phase)) {
+                if (!mbar_wait_warp(&full[stage], phase)) {
                     ok = false;
                     break;
                 }
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
                 // D += t[rows, part] . B_part[tenant][cols]^T (one K = 16 step);
                 // none with segmented weights only (n_parts == 0)
                 if (ok && lg.n_parts > 0) {
-                    if (!mbar_wait(&lfull[lj], lphase)) {
+                    if (!mbar_wait_warp(&lfull[lj], lphase)) {
                         ok = false;
                     } else {
                         ++l_used;
@@ -1046,12 +1046,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true;
-        for (int tile = first; ok && tile < num_tiles && !*abort_flag; tile += step) {
+        for (int tile = first; ok && tile < num_tiles && !__any_sync(0xffffffffu, *abort_flag);
+             tile += step) {
             int mb, nb;
             tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
             const int arow = mb * BM + (int)rank * 128, brow = nb * BN + (int)rank * 128;
             for (int kb = 0; kb < num_k; ++kb) {
-                if (!mbar_wait(&empty[stage], phase ^ 1)) {
+                if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
                     ok = false;
                     break;
                 }
@@ -1079,16 +1080,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
         bool ok = true;
         const uint32_t a_lo = sw128_desc_lo(smem_u32(smem));
         const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + HALF_BYTES);
-        for (int tile = first; ok && tile < num_tiles && !*abort_flag; tile += step, ++local) {
+        for (int tile = first; ok && tile < num_tiles && !__any_sync(0xffffffffu, *abort_flag);
+             tile += step, ++local) {
             const int acc = local & 1;
-            if (!mbar_wait_cluster(&tempty[acc], ((local >> 1) & 1) ^ 1)) {
+            if (!mbar_wait_cluster_warp(&tempty[acc], ((local >> 1) & 1) ^ 1)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
             const uint32_t d = tmem_base + acc * BN;
             for (int kb = 0; kb < num_k; ++kb) {
-                if (!mbar_wait_cluster(&full[stage], phase)) {
+                if (!mbar_wait_cluster_warp(&full[stage], phase)) {
                     ok = false;
                     break;
                 }
@@ -1240,13 +1242,13 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
 // 16,384): a tile alone on its SM, and two narrow tiles sharing one, which is
 // how a narrow launch of more tiles than SMs runs.  A 256-wide tile is the
 // fastest per column, so narrower ones win only where it leaves SMs idle:
-// 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide tiles, 61 in 80 of 128
-// and 76 in 160 of 64; 300 rows 96, 60 and 55; 4,800 rows 196, 237 and 348.
+// 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide tiles, 59 in 80 of 128
+// and 76 in 160 of 64; 300 rows 94, 57 and 47; 4,800 rows 190, 235 and 351.
 // A pair's tile (plain launches only) takes 0.33 for the same work per SM as
 // a wide one's 0.385, so it wins wherever its tiles divide as well over the
 // SMs: 2,400 rows x N 32,768 177 us against 188, but x N 2,048 33 against 23.
-// RoPE needs a tile within one head; the GLU backward with dm has wide tiles
-// only.
+// RoPE needs a tile within one head, a folded norm's sums of squares one of 128
+// columns; the GLU backward with dm has wide tiles only.
 constexpr int kPairTile = 512;
 
 static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
@@ -1264,10 +1266,10 @@ static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
         }
     }
     if (p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn)) return best;
-    static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.235, 0.39},
-                                                                     {64, 0.215, 0.334}};
+    static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.225, 0.38},
+                                                                     {64, 0.18, 0.33}};
     for (const auto& w : kNarrow) {
-        if (p.epi == EPI_ROPE && w.bn > p.hd) continue;
+        if ((p.epi == EPI_ROPE && w.bn > p.hd) || (p.norm_gamma && w.bn < 128)) continue;
         const long long tiles = (long long)m_tiles * (p.N / w.bn);
         const double t = tiles <= sms ? w.alone : rounds(tiles, 2 * sms) * w.two;
         if (t < least) {

@@ -167,6 +167,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
     return true;
 }
 
+// mbar_wait by a fully active warp: all lanes wait and the result is one vote,
+// so that a loop it steers stays warp-uniform to the compiler (see elect_one).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
+                                               long long limit_cycles = 4000000000LL) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+        if (__any_sync(0xffffffffu, clock64() - t0 > limit_cycles)) return false;
+    }
+    return true;
+}
+
 // --------------------------------------------------------------------------
 // TMA
 // --------------------------------------------------------------------------
@@ -466,24 +478,26 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
                  : "memory");
 }
 
-// As mbar_wait, with acquire at cluster scope (arrivals from the peer CTA).
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity,
-                                                  long long limit_cycles = 4000000000LL) {
-    long long t0 = 0;
-    for (;;) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        const long long t = clock64();
-        if (t0 == 0) t0 = t;
-        if (t - t0 > limit_cycles) return false;
+// As mbar_wait_warp, with acquire at cluster scope (arrivals from the peer CTA).
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity,
+                                                       long long limit_cycles = 4000000000LL) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
+    const long long t0 = clock64();
+    while (!__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) {
+        if (__any_sync(0xffffffffu, clock64() - t0 > limit_cycles)) return false;
     }
+    return true;
 }
 
 // 2D tiled load into this CTA's shared memory that completes on a barrier of

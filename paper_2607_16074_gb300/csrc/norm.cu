@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
 }
 
 // First half of a folded RMSNorm (the residual GEMM epilogue does the same for
-// every later norm): y = bf16(x * gamma) and, per row and 64-column block,
+// every later norm): y = bf16(x * gamma) and, per row and 128-column block,
 // the sum of x^2; the consuming GEMM scales its output rows by
 // rsqrt(sum / d + eps).  One warp per row.
 template <int V>
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256) k_rms_prep(const float* __restrict__ x,
                                                   const uint16_t* __restrict__ gamma, int M,
                                                   uint16_t* __restrict__ y, float* __restrict__ ss) {
     constexpr int D = V * 128;
-    constexpr int P = D / 64;  // a 64-column block is half a warp's float4 i
+    constexpr int P = D / 128;  // 128-column blocks: lane float4 i = b
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= M) return;
@@ -125,11 +125,12 @@ __global__ void __launch_bounds__(256) k_rms_prep(const float* __restrict__ x,
 #pragma unroll
     for (int i = 0; i < V; ++i) v[i] = __ldg(xr + lane + 32 * i);
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-        float t = v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+    for (int b = 0; b < P; ++b) {
+        float t = 0.f;
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if ((lane & 15) == 0) ss[(size_t)row * P + 2 * i + (lane >> 4)] = t;
+        t += v[b].x * v[b].x + v[b].y * v[b].y + v[b].z * v[b].z + v[b].w * v[b].w;
+        t = warp_sum(t);
+        if (lane == 0) ss[(size_t)row * P + b] = t;
     }
     uint2* orow = reinterpret_cast<uint2*>(y + (size_t)row * D);
     const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
