@@ -521,15 +521,18 @@ HeadsWs carve_heads(const jnx_head* heads, const jnx_group* g, void* base) {
     if (hd.any_x) {
         w.sc.kbuf = take(N * hd.ldkv * 4);
         w.sc.vbuf = take(N * hd.ldkv * 4);
-        w.sc.dk = take(N * hd.ldkv * 4);
-        w.sc.dv = take(N * hd.ldkv * 4);
         w.sc.P = take(N * hd.nq * 4);
         w.sc.dS = take(N * hd.nq * 4);
         w.sc.dQs = take(S * hd.ld_h * 4);
-        w.sc.dkv_bf = reinterpret_cast<uint16_t*>(take(N * 2 * hd.ldkv * 2));
-        w.sc.Gs = take(S * 32 * hd.d_in * 4);
-        w.sc.Hs = take(S * 32 * hd.d_in * 4);
+        w.sc.dkv = reinterpret_cast<uint16_t*>(take(N * 2 * hd.ldkv * 2));
+        w.sc.HG = take(S * 64 * hd.d_in * 4);
+        int longest = 1;
+        for (int i = 0; g->h_cu_seqlens && i < g->n_samples; ++i)
+            longest = std::max(longest, g->h_cu_seqlens[i + 1] - g->h_cu_seqlens[i]);
+        w.sc.ldp = 2 * ((longest + 63) / 64 * 64);
+        w.sc.planes = reinterpret_cast<uint16_t*>(take(S * 64 * (size_t)w.sc.ldp * 2));
     }
+    w.sc.status = w.status;
     w.bytes = off;
     return w;
 }
@@ -712,22 +715,34 @@ extern "C" jnx_status jnx_heads_forward(const jnx_head* heads, int32_t n_tenants
         const int n = std::min(kMaxSlots, g->n_slots - g0);
         HeadBatch b = fill_table(tab, heads, nullptr, g, g0, n);
         TraceScope ts(JNX_K_HEADS_FWD, heads_flops(tab, n, false), s);
-        for (int i = 0; i < n && b.any_xattn; ++i) {
-            const HeadSlot& hs = tab.slot[i];
-            if (hs.kind != JNX_HEAD_XATTN || hs.r1 == hs.r0) continue;
-            for (int which = 0; which < 2; ++which) {
-                GemmParams p{};
-                p.M = hs.r1 - hs.r0;
-                p.N = hs.dq;
-                p.K = d;
-                p.epi = EPI_F32;
-                p.out = (which ? w.sc.vbuf : w.sc.kbuf) + (size_t)hs.r0 * w.sc.ldkv;
-                p.ldo = w.sc.ldkv;
-                p.status = w.status;
-                if ((st = gemm_launch(hidden + (size_t)hs.r0 * d, d, which ? hs.wv : hs.wk, d, p,
-                                      s)))
-                    return st;
+        if (b.any_xattn) {
+            // k = X Wk^T and v = X Wv^T of every query-head slot in one launch
+            // (two a slot before: 16 launches of 18 us for eight tenants of 4,400
+            // rows, 63 us now)
+            static thread_local GemmBatch gb;  // staging of the kernel argument
+            gb.n_maps = gb.n = gb.tiles = 0;
+            gb.ldo = w.sc.ldkv;
+            gb.status = w.status;
+            const int mx = batch_map(gb, hidden, g->n_tokens, d, d, false, 128);
+            for (int i = 0; i < n; ++i) {
+                const HeadSlot& hs = tab.slot[i];
+                if (hs.kind != JNX_HEAD_XATTN || hs.r1 == hs.r0) continue;
+                for (int which = 0; which < 2; ++which) {
+                    GemmBatch::Problem q{};
+                    q.out = (which ? w.sc.vbuf : w.sc.kbuf) + (size_t)hs.r0 * w.sc.ldkv;
+                    q.a = mx;
+                    q.b = q.b2 = batch_map(gb, which ? hs.wv : hs.wk, hs.dq, d, d, false, 256);
+                    if (mx < 0 || q.b < 0)
+                        return fail(JNX_ERR_CUDA,
+                                    "heads: tensor map encode failed (alignment or driver)");
+                    q.k1 = q.k = d / 64;
+                    q.m = hs.r1 - hs.r0;
+                    q.arow = hs.r0;
+                    q.nb = hs.dq / 256;
+                    batch_add(gb, q);
+                }
             }
+            if ((st = gemm_batch_launch(gb, EPI_F32, false, false, s))) return st;
         }
         if ((st = heads_forward_launch(tab, b, w.sc, pooled, d, g->cu_seqlens, g->sample_slot,
                                        g->sample_target, targets, preds, loss, s)))
@@ -757,8 +772,7 @@ static jnx_status heads_backward(const jnx_head* heads, int32_t n_tenants, const
         const int n = std::min(kMaxSlots, g->n_slots - g0);
         HeadBatch b = fill_table(tab, heads, grads, g, g0, n, accum);
         TraceScope ts(JNX_K_HEADS_BWD, heads_flops(tab, n, true), s);
-        if ((st = heads_backward_launch(tab, b, w.sc, pooled, d, hidden, g->cu_seqlens,
-                                        g->sample_slot, kv_grads, s)))
+        if ((st = heads_backward_launch(tab, b, w.sc, pooled, d, hidden, g, kv_grads, s)))
             return st;
     }
     return JNX_OK;
@@ -816,9 +830,40 @@ static jnx_status heads_feature_grad(const jnx_head* heads, const jnx_group* g, 
         return st;
     if (!any_x) return JNX_OK;
     const int ld = w.sc.ldkv;
-    if ((st = to_bf16_launch(w.sc.dk, ld, N, ld, w.sc.dkv_bf, 2 * ld, s)) ||
-        (st = to_bf16_launch(w.sc.dv, ld, N, ld, w.sc.dkv_bf + ld, 2 * ld, s)))
-        return st;
+    if (d % 256 == 0) {
+        // [dk | dv] [Wk; Wv] per tenant, the weights as they lie (rows are K):
+        // one tcgen05 launch per 64 tenants (mma.sync tiles of 64 x 128 took 283
+        // us for 35,000 rows x 2,048 columns, this 61)
+        static thread_local GemmBatch gb;  // staging of the kernel argument
+        for (int g0 = 0; g0 < g->n_slots; g0 += kMaxSlots) {
+            gb.n_maps = gb.n = gb.tiles = 0;
+            gb.ldo = d;
+            gb.status = w.status;
+            const int ma = batch_map(gb, w.sc.dkv, N, 2 * ld, 2 * ld, false, 128);
+            for (int i = g0; i < std::min(g0 + kMaxSlots, g->n_slots); ++i) {
+                const jnx_head& h = heads[g->h_slot_tenant[i]];
+                if (h.kind != JNX_HEAD_XATTN) continue;
+                GemmBatch::Problem q{};
+                q.arow = g->h_cu_seqlens[g->h_seg_offsets[i]];
+                q.m = g->h_cu_seqlens[g->h_seg_offsets[i + 1]] - q.arow;
+                if (q.m == 0) continue;
+                q.out = d_hidden + (size_t)q.arow * d;
+                q.a = ma;
+                q.b = batch_map(gb, h.wk, h.q_dim, d, d, true, 0);
+                q.b2 = batch_map(gb, h.wv, h.q_dim, d, d, true, 0);
+                if (ma < 0 || q.b < 0 || q.b2 < 0)
+                    return fail(JNX_ERR_CUDA,
+                                "heads: tensor map encode failed (alignment or driver)");
+                q.k1 = h.q_dim / 64;
+                q.k = 2 * q.k1;
+                q.ax2 = ld;
+                q.nb = d / 256;
+                batch_add(gb, q);
+            }
+            if ((st = gemm_batch_launch(gb, EPI_F32, false, true, s))) return st;
+        }
+        return JNX_OK;
+    }
     // one launch per distinct query width; other slots are skipped
     std::vector<int> widths;
     for (int i = 0; i < g->n_slots; ++i) {
@@ -831,8 +876,8 @@ static jnx_status heads_feature_grad(const jnx_head* heads, const jnx_group* g, 
     for (int dq : widths) {
         sp = SegUpParts{};
         sp.n_parts = 2;
-        sp.t[0] = w.sc.dkv_bf;
-        sp.t[1] = w.sc.dkv_bf + ld;
+        sp.t[0] = w.sc.dkv;
+        sp.t[1] = w.sc.dkv + ld;
         sp.ldt[0] = sp.ldt[1] = 2 * ld;
         sp.k[0] = sp.k[1] = dq;
         for (int i = 0; i < g->n_slots; ++i) {
@@ -925,8 +970,8 @@ extern "C" jnx_status jnx_heads_backward_adamw(const jnx_head* heads, int32_t n_
         for (int g0 = 0; g0 < g->n_slots; g0 += kMaxSlots) {
             const int n = std::min(kMaxSlots, g->n_slots - g0);
             HeadBatch b = fill_table(tab, heads, grads, g, g0, n, accumulate != 0);
-            if ((st = heads_backward_front_launch(tab, b, w.sc, d, hidden, g->cu_seqlens,
-                                                  g->sample_slot, d_hidden != nullptr, s)))
+            if ((st = heads_backward_front_launch(tab, b, w.sc, d, hidden, g, d_hidden != nullptr,
+                                                  s)))
                 return st;
         }
     }

@@ -764,25 +764,4 @@ jnx_status mlp_dfeat_launch(const float* dz, int ldz, const int* cu, const int* 
                             : fail(JNX_ERR_CUDA, "MLP feature gradient: %s", cudaGetErrorString(e));
 }
 
-// fp32 -> bf16 of a [rows, cols] block with row strides (the query heads'
-// dk | dv rows into one bf16 operand).
-__global__ void __launch_bounds__(256) k_to_bf16(const float* __restrict__ src, int lds, int rows,
-                                                 int cols, uint16_t* __restrict__ dst, int ldd) {
-    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (i >= (long long)rows * (cols / 2)) return;
-    const int r = (int)(i / (cols / 2)), c = (int)(i % (cols / 2)) * 2;
-    const float2 v = *reinterpret_cast<const float2*>(src + (size_t)r * lds + c);
-    *reinterpret_cast<uint32_t*>(dst + (size_t)r * ldd + c) = pack_bf2(v.x, v.y);
-}
-
-jnx_status to_bf16_launch(const float* src, int lds, int rows, int cols, uint16_t* dst, int ldd,
-                          cudaStream_t s) {
-    if (cols % 2 || lds % 2 || ldd % 2) return fail(JNX_ERR_UNSUPPORTED, "to bf16: odd widths");
-    const long long n = (long long)rows * (cols / 2);
-    if (n <= 0) return JNX_OK;
-    k_to_bf16<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(src, lds, rows, cols, dst, ldd);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "to bf16: %s", cudaGetErrorString(e));
-}
-
 }  // namespace jnx

@@ -1176,6 +1176,218 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
 }
 
 // ---------------------------------------------------------------------------
+// A batch of GEMMs in one launch (GemmBatch): the wide single-CTA kernel over
+// the tiles of all problems in turn, each with its own tensor maps and output.
+// An operand may be MN-major (its rows are K): 64 x 64 boxes of it, 128-byte
+// swizzled, are the tensor core's transposed operand as they are, which saves
+// a transposed copy in memory.  What it replaces and the times stand at its
+// callers.
+// ---------------------------------------------------------------------------
+template <int EPI, bool AMN, bool BMN>
+__global__ void __launch_bounds__(192, 1) k_gemm_batch(const __grid_constant__ GemmBatch gb) {
+    using namespace gemm;
+    constexpr uint32_t IDESC =
+        idesc_bf16_f32(BM, BN) | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    uint64_t* empty = full + STAGES;
+    uint64_t* tfull = empty + STAGES;
+    uint64_t* tempty = tfull + 2;
+    uint64_t* drain = tempty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* consumed = abort_flag + 1;
+    const int warp = warp_uniform(threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(&tfull[a], 1);
+            mbar_init(&tempty[a], 128);
+        }
+        mbar_init(drain, 1);
+        *abort_flag = 0;
+        *consumed = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, TMEM_COLS);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
+    int issued = 0;
+
+    // the problem of a tile, and the tile's place in it (row blocks fastest)
+    int pi = 0;
+    auto find = [&](int tile, int& mb, int& nb) -> const GemmBatch::Problem& {
+        while (pi + 1 < gb.n && gb.p[pi + 1].tile0 <= tile) ++pi;
+        const GemmBatch::Problem& q = gb.p[pi];
+        const int mt = (q.m + BM - 1) / BM, in = tile - q.tile0;
+        mb = in % mt;
+        nb = in / mt;
+        return q;
+    };
+
+    if (warp == 0) {
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; ok && tile < gb.tiles && !__any_sync(0xffffffffu, *abort_flag);
+             tile += gridDim.x) {
+            int mb, nb;
+            const GemmBatch::Problem& q = find(tile, mb, nb);
+            for (int kb = 0; kb < q.k; ++kb) {
+                if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
+                    ok = false;
+                    break;
+                }
+                const bool second = kb >= q.k1;
+                const int bk = (second ? kb - q.k1 : kb) * BK;
+                const CUtensorMap* ma = &gb.map[q.a];
+                const CUtensorMap* mbp = &gb.map[second ? q.b2 : q.b];
+                if (elect_one()) {
+                    uint8_t* sa = smem + stage * STAGE_BYTES;
+                    mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
+                    if constexpr (AMN) {
+#pragma unroll
+                        for (int i = 0; i < BM / 64; ++i)
+                            tma_load_2d(sa + i * 64 * BK * 2, ma, mb * BM + 64 * i, kb * BK,
+                                        &full[stage]);
+                    } else {
+                        tma_load_2d(sa, ma, second ? q.ax2 + bk : bk, q.arow + mb * BM,
+                                    &full[stage]);
+                    }
+                    if constexpr (BMN) {
+#pragma unroll
+                        for (int i = 0; i < BN / 64; ++i)
+                            tma_load_2d(sa + A_BYTES + i * 64 * BK * 2, mbp, nb * BN + 64 * i, bk,
+                                        &full[stage]);
+                    } else {
+                        tma_load_2d(sa + A_BYTES, mbp, bk, nb * BN, &full[stage]);
+                    }
+                }
+                __syncwarp();
+                ++issued;
+                if (++stage == STAGES) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+            }
+        }
+        if (!ok) {
+            *abort_flag = 1;
+            report(gb.status, JNX_ERR_TIMEOUT);
+        }
+    } else if (warp == 1) {
+        int stage = 0, local = 0, n_used = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        const uint32_t a0 = smem_u32(smem), b0 = a0 + A_BYTES;
+        for (int tile = blockIdx.x; ok && tile < gb.tiles && !__any_sync(0xffffffffu, *abort_flag);
+             tile += gridDim.x, ++local) {
+            int mb, nb;
+            const GemmBatch::Problem& q = find(tile, mb, nb);
+            const int acc = local & 1;
+            if (!mbar_wait_warp(&tempty[acc], ((local >> 1) & 1) ^ 1)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem_base + acc * BN;
+            for (int kb = 0; kb < q.k; ++kb) {
+                if (!mbar_wait_warp(&full[stage], phase)) {
+                    ok = false;
+                    break;
+                }
+                ++n_used;
+                tc_fence_after();
+                const uint32_t off = stage * STAGE_BYTES;
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        // 16 K rows of an MN-major operand are two 8-row atoms
+                        const uint64_t da =
+                            AMN ? sw128_desc_mn(a0 + off + kk * 2048, 64 * BK * 2, 1024)
+                                : sw128_desc(a0 + off + kk * 32);
+                        const uint64_t db =
+                            BMN ? sw128_desc_mn(b0 + off + kk * 2048, 64 * BK * 2, 1024)
+                                : sw128_desc(b0 + off + kk * 32);
+                        tc_mma_f16(d, da, db, IDESC, (kb | kk) != 0);
+                    }
+                    tc_commit(&empty[stage]);
+                }
+                __syncwarp();
+                if (++stage == STAGES) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+            }
+            if (!ok) break;
+            if (elect_one()) tc_commit(&tfull[acc]);
+            __syncwarp();
+        }
+        if (!ok) {
+            *abort_flag = 1;
+            report(gb.status, JNX_ERR_TIMEOUT);
+        }
+        *consumed = n_used;
+        if (elect_one()) tc_commit(drain);
+        __syncwarp();
+        mbar_wait(drain, 0);
+    } else {
+        const int q4 = warp & 3;  // TMEM lane quarter this warp may access
+        uint8_t* stg = reinterpret_cast<uint8_t*>(full) + 256 + (warp - 2) * 2048;
+        int local = 0;
+        for (int tile = blockIdx.x; tile < gb.tiles; tile += gridDim.x, ++local) {
+            int mb, nb;
+            const GemmBatch::Problem& q = find(tile, mb, nb);
+            const int acc = local & 1;
+            if (!mbar_wait(&tfull[acc], (local >> 1) & 1) || *abort_flag) {
+                *abort_flag = 1;
+                report(gb.status, JNX_ERR_TIMEOUT);
+                break;
+            }
+            tc_fence_after();
+            TileGeo g;
+            g.nb = nb;
+            g.seg = 0;
+            g.c0 = nb * BN;
+            g.c1 = g.c0 + 128;
+            g.row0 = mb * BM;
+            g.row_end = min(g.row0 + BM, q.m);
+            GemmParams p{};
+            p.out = p.resid = q.out;
+            p.ldo = p.ldr = gb.ldo;
+            epilogue_tile<EPI, 8, 256>(tmem_base + acc * BN + ((uint32_t)(q4 * 32) << 16), stg,
+                                       lane, g.row0 + q4 * 32, g.row_end, g, p, 0);
+            tc_fence_before();
+            mbar_arrive(&tempty[acc]);
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (*abort_flag && warp == 0 && lane == 0) {
+        // wait (bounded) for TMA copies this CTA issued but nobody consumed
+        for (int i = *consumed; i < issued; ++i)
+            mbar_wait(&full[i % STAGES], (i / STAGES) & 1, 100000000LL);
+    }
+    __syncwarp();
+    if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 
@@ -1451,6 +1663,43 @@ jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ld
         default: return fail(JNX_ERR_INVALID_ARG, "gemm: epilogue %d unsupported here", p.epi);
     }
     if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
+    return JNX_OK;
+}
+
+int batch_map(GemmBatch& gb, const uint16_t* ptr, uint64_t rows, uint64_t cols, uint64_t ld,
+              bool mn, int box) {
+    if (gb.n_maps >= kBatchMaps) return -1;
+    if (!make_tmap_bf16(&gb.map[gb.n_maps], ptr, rows, cols, ld, mn ? gemm::BK : box, 64)) return -1;
+    return gb.n_maps++;
+}
+
+bool batch_add(GemmBatch& gb, GemmBatch::Problem p) {
+    if (gb.n >= kBatchMax) return false;
+    p.tile0 = gb.tiles;
+    gb.tiles += (p.m + gemm::BM - 1) / gemm::BM * p.nb;
+    gb.p[gb.n++] = p;
+    return true;
+}
+
+template <int EPI, bool AMN, bool BMN>
+static cudaError_t launch_batch(const GemmBatch& gb, cudaStream_t s) {
+    static std::atomic<uint64_t> attr{0};
+    cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(k_gemm_batch<EPI, AMN, BMN>),
+                                   gemm::SMEM_BYTES, attr);
+    if (e != cudaSuccess) return e;
+    k_gemm_batch<EPI, AMN, BMN>
+        <<<std::min(gb.tiles, num_sms()), 192, gemm::SMEM_BYTES, s>>>(gb);
+    return cudaGetLastError();
+}
+
+jnx_status gemm_batch_launch(const GemmBatch& gb, int epi, bool a_mn, bool b_mn, cudaStream_t s) {
+    if (gb.tiles == 0) return JNX_OK;
+    cudaError_t e = cudaErrorInvalidValue;
+    if (epi == EPI_F32 && !a_mn && !b_mn) e = launch_batch<EPI_F32, false, false>(gb, s);
+    if (epi == EPI_F32 && !a_mn && b_mn) e = launch_batch<EPI_F32, false, true>(gb, s);
+    if (epi == EPI_F32 && a_mn && b_mn) e = launch_batch<EPI_F32, true, true>(gb, s);
+    if (epi == EPI_RESID && a_mn && b_mn) e = launch_batch<EPI_RESID, true, true>(gb, s);
+    if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm batch launch: %s", cudaGetErrorString(e));
     return JNX_OK;
 }
 

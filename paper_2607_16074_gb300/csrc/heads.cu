@@ -702,6 +702,23 @@ __device__ __forceinline__ void xattn_chunk_xr(float (&acc)[2][4][4], const uint
     }
 }
 
+// The chunk's query-major split tiles of dS (tq) and P (the two planes after
+// them) into the sample's weight-gradient operands (see k_xattn_bwd); pad: zeros
+// for the 32 keys after the chunk, too.
+__device__ __forceinline__ void xattn_store_planes(uint16_t* __restrict__ dst, int ldp,
+                                                   const uint16_t* tq, int j0, bool pad) {
+    static_assert(kXRows == 32 && kMaxQ == 32, "four 16-byte units a row");
+    for (int i = threadIdx.x; i < 4 * kMaxQ * 4; i += 256) {
+        const int u = i & 3, q = (i >> 2) & 31, pl = i >> 7;  // planes: dS hi, dS lo, P hi, P lo
+        const uint4 v =
+            *reinterpret_cast<const uint4*>(tq + (size_t)(pl * kMaxQ + q) * kXPad + 8 * u);
+        uint16_t* o = dst + (size_t)((pl < 2 ? kMaxQ : 0) + q) * ldp + (pl & 1) * (ldp / 2) + j0 +
+                      8 * u;
+        *reinterpret_cast<uint4*>(o) = v;
+        if (pad) *reinterpret_cast<uint4*>(o + kXRows) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
 // A query-head sample is shared by a cluster of kXCtas CTAs: rank k takes an
 // equal share of the sample's 32-key chunks, keys [ja, jz) (empty for the
 // last ranks of a short sample).
@@ -864,7 +881,11 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 3)
 // D_q = sum_j dP P, dS = P (dP - D_q) in place, this sample's dQ
 // contribution scale dS k (summed per tenant later in sample order), and,
 // when kv_grads is set (the feature gradient needs them), the key rows'
-// dv = P^T dO and dk = scale dS^T Q.
+// dk = scale dS^T Q and dv = P^T dO as bf16 rows dk | dv of dkv (row stride 2
+// ldkv).  Also P and dS query-major as the bf16 hi and lo operands of the
+// weight gradients' products: planes[s][P: 0 .. 31, dS: 32 .. 63][hi: key, lo:
+// ldp / 2 + key], zero past the queries and, up to the next multiple of 64, past
+// the keys.
 __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
     k_xattn_bwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
@@ -874,7 +895,8 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
                                                    const float* __restrict__ P,
                                                    float* __restrict__ dS,
                                                    const float* __restrict__ dO, int ld_h,
-                                                   float* __restrict__ dk, float* __restrict__ dv,
+                                                   uint16_t* __restrict__ dkv,
+                                                   uint16_t* __restrict__ planes, int ldp,
                                                    float* __restrict__ dQs, int kv_grads) {
     extern __shared__ __align__(16) uint8_t xsm[];
     __shared__ float red[8 * 32], slot_d[32];
@@ -927,8 +949,12 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
             __syncthreads();
             xattn_split_rows(sR, kXRows, kXCols + 8, kbuf, ldkv, (size_t)r0 + j0, nr, c0, kXCols);
             xattn_split_chunk(sT, kv_grads ? uD : nullptr, dSs, j0, nr, nq);
-            if (kv_grads) xattn_split_chunk(nullptr, uP, Ps, j0, nr, nq);
+            if (c0 == 0 || kv_grads)
+                xattn_split_chunk(sT + 2 * kMaxQ * kXPad, kv_grads ? uP : nullptr, Ps, j0, nr, nq);
             __syncthreads();
+            if (c0 == 0)
+                xattn_store_planes(planes + (size_t)s * 2 * kMaxQ * ldp, ldp, sT, j0,
+                                   j0 + kXRows >= L && ((L + kXRows - 1) / kXRows & 1));
             xattn_chunk_xr(aq, sT, sR);  // dQ += dS k
             if (!kv_grads) continue;
             // dv[j, c] = sum_q P[q, j] dO[q, c], dk[j, c] = scale sum_q dS[q, j] Q[q, c]:
@@ -976,13 +1002,14 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
                 for (int hf = 0; hf < 2; ++hf) {
                     const int j = 16 * m + g + 8 * hf;
                     if (j >= nr) continue;
-                    const size_t row = (size_t)(r0 + j0 + j) * ldkv + c0 + 32 * warp + 2 * t;
+                    uint16_t* row =
+                        dkv + (size_t)(r0 + j0 + j) * 2 * ldkv + c0 + 32 * warp + 2 * t;
 #pragma unroll
                     for (int n = 0; n < 4; ++n) {
-                        *reinterpret_cast<float2*>(dv + row + 8 * n) =
-                            make_float2(av[m][n][2 * hf], av[m][n][2 * hf + 1]);
-                        *reinterpret_cast<float2*>(dk + row + 8 * n) =
-                            make_float2(ak[m][n][2 * hf] * scale, ak[m][n][2 * hf + 1] * scale);
+                        *reinterpret_cast<uint32_t*>(row + 8 * n) =
+                            pack_bf2(ak[m][n][2 * hf] * scale, ak[m][n][2 * hf + 1] * scale);
+                        *reinterpret_cast<uint32_t*>(row + ldkv + 8 * n) =
+                            pack_bf2(av[m][n][2 * hf], av[m][n][2 * hf + 1]);
                     }
                 }
         }
@@ -1014,15 +1041,19 @@ __global__ void __launch_bounds__(256) k_xattn_dq(const __grid_constant__ HeadTa
 // key-major), so
 //   dWk = sum_rows dk^T X = scale Q^T (sum_s G_s),  G_s = dS_s^T X_s  [nq, d]
 //   dWv = sum_rows dv^T X = sum_s dO_s^T H_s,       H_s = P_s^T X_s   [nq, d]
-// which takes 2 nq d flops per row and product instead of 2 dq d.  Both
-// steps run in fp32 on CUDA cores (X is exact in bf16), every sum in a fixed
-// order, so a tenant's gradients do not depend on the batch around it.
+// which takes 2 nq d flops per row and product instead of 2 dq d.  X is exact in
+// bf16; P and dS are fp32 and enter as two bf16 operands each, hi = bf16(P) and
+// lo = bf16(P - hi), so P X = hi X + lo X to about 2^-17 of P.  HG holds, per
+// sample, H_s in rows 0 .. 31 and G_s in rows 32 .. 63.
 //
-// k_xattn_gh: one CTA per (sample, 128 columns e of X), on the bf16 tensor
-// cores (mma.sync m16n8k16, fp32 accumulation).  X is bf16 already; P and dS
-// are fp32 and enter as two bf16 operands each, hi = bf16(P) and lo =
-// bf16(P - hi), so P X = hi X + lo X to about 2^-17 of P, i.e. within the
-// fp32 path's accuracy for these sums.  The sample's rows are staged 32 keys
+// Where d is a multiple of 256 they are one batched tcgen05 GEMM (gh_launch):
+// per sample [P | dS] planes [64, keys] (k_xattn_bwd wrote them) times X, whose
+// rows are K, the hi planes' K-steps before the lo planes':
+// 61 us for 64 samples of 547 rows x 2,048 columns, where k_xattn_gh, whose
+// sixteen column blocks each split P and dS again, took 246.
+//
+// k_xattn_gh, for other widths: one CTA per (sample, 128 columns e of X), on
+// mma.sync (m16n8k16, fp32 accumulation).  The sample's rows are staged 32 keys
 // at a time by cp.async (X rows into padded rows; the P / dS rows, nq
 // floats each, contiguous per sample), then split and transposed into
 // [query][key] operands in shared memory by all threads.  Warp w computes
@@ -1039,8 +1070,7 @@ __global__ void __launch_bounds__(256) k_xattn_gh(const __grid_constant__ HeadTa
                                                   int sample0, const float* __restrict__ P,
                                                   const float* __restrict__ dS,
                                                   const uint16_t* __restrict__ X, int ldx,
-                                                  float* __restrict__ Gs, float* __restrict__ Hs,
-                                                  int ldg) {
+                                                  float* __restrict__ HG, int ldg) {
     static_assert(kMaxQ == 32, "two 16-row query tiles");
     __shared__ __align__(16) uint16_t sx[2][kGhRows][kGhXPad];
     __shared__ __align__(16) float sp[2][kGhRows * kMaxQ], sd[2][kGhRows * kMaxQ];
@@ -1142,107 +1172,117 @@ __global__ void __launch_bounds__(256) k_xattn_gh(const __grid_constant__ HeadTa
             if (q >= nq) continue;
 #pragma unroll
             for (int n = 0; n < 2; ++n) {
-                const size_t o = ((size_t)s * kMaxQ + q) * ldg + e0 + 16 * w + 8 * n + 2 * (lane & 3);
-                *reinterpret_cast<float2*>(Hs + o) =
+                float* o = HG + ((size_t)s * 2 * kMaxQ + q) * ldg + e0 + 16 * w + 8 * n +
+                           2 * (lane & 3);
+                *reinterpret_cast<float2*>(o) =
                     make_float2(acc[0][m][n][2 * half], acc[0][m][n][2 * half + 1]);
-                *reinterpret_cast<float2*>(Gs + o) =
+                *reinterpret_cast<float2*>(o + (size_t)kMaxQ * ldg) =
                     make_float2(acc[1][m][n][2 * half], acc[1][m][n][2 * half + 1]);
             }
         }
 }
 
-// k_xattn_wgrad: one CTA per (slot, 32 value columns c, 64 columns e); warp
-// w takes c = c0 + 4w..4w+3 (and the running sum of G_s over rows
-// q = 4w..4w+3), a lane two consecutive columns e.  The slot's samples in
-// order: dWv += dO_s^T H_s with dO_s [nq, 32] and H_s [nq, 64] staged; at the
-// end dWk = scale Q^T G_t with G_t staged.
+// k_xattn_wgrad: one CTA per (slot, 64 value columns c, 128 columns e), fp32 on
+// CUDA cores; warp w takes c = c0 + 8 w .. + 7 (and the running sum of G_s over
+// rows q = 4 w .. + 3), a lane four consecutive columns e.  The slot's samples in
+// order: dWv += dO_s^T H_s with dO_s [nq, 64] and H_s [nq, 128] staged; at the
+// end dWk = scale Q^T G_t with G_t staged.  Bound by shared-memory reads of the
+// staged operands: a thread's 8 x 4 block takes three 16-byte reads for its 32
+// multiply-adds (4 x 2 took two for 8: 115 us for eight tenants of eight samples,
+// d 2,048; this 90).
+constexpr int kWgC = 64, kWgE = 128;
+
 template <class OT>
 __global__ void __launch_bounds__(256) k_xattn_wgrad(const __grid_constant__ HeadTable tab,
                                                      const __grid_constant__ OT opt, AdamHp hp,
-                                                     const float* __restrict__ Gs,
-                                                     const float* __restrict__ Hs, int ldg,
+                                                     const float* __restrict__ HG, int ldg,
                                                      const float* __restrict__ dO, int ld_h) {
-    __shared__ __align__(16) float sh[kMaxQ][64];
-    __shared__ __align__(16) float so[kMaxQ][32];
-    __shared__ __align__(16) float sg[kMaxQ][64];
+    __shared__ __align__(16) float sh[kMaxQ][kWgE];  // H_s, then G_t
+    __shared__ __align__(16) float so[kMaxQ][kWgC];  // dO_s, then Q
     const HeadSlot& hs = tab.slot[blockIdx.x];
     if (hs.kind != JNX_HEAD_XATTN) return;
-    const int nq = hs.nq, dq = hs.dq, c0 = blockIdx.y * 32, e0 = blockIdx.z * 64;
+    const int nq = hs.nq, dq = hs.dq, c0 = blockIdx.y * kWgC, e0 = blockIdx.z * kWgE;
     if (c0 >= dq || e0 >= hs.d_in) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float av[4][2], gt[4][2];
+    float av[8][4] = {}, gt[4][4] = {};
+    auto product = [&](float (&acc)[8][4]) {
+        for (int q = 0; q < nq; ++q) {
+            const float4 oa = *reinterpret_cast<const float4*>(&so[q][8 * w]);
+            const float4 ob = *reinterpret_cast<const float4*>(&so[q][8 * w + 4]);
+            const float4 hv = *reinterpret_cast<const float4*>(&sh[q][4 * lane]);
+            const float o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) av[i][0] = av[i][1] = gt[i][0] = gt[i][1] = 0.f;
-    for (int s = hs.s0; s < hs.s1; ++s) {
-        __syncthreads();  // the previous sample's staged rows are read
-        for (int i = threadIdx.x; i < nq * 16; i += 256) {  // H_s [nq, 64]: 16 float4 per row
-            const int q = i >> 4, u = i & 15;
-            *reinterpret_cast<float4*>(&sh[q][4 * u]) = *reinterpret_cast<const float4*>(
-                Hs + ((size_t)s * kMaxQ + q) * ldg + e0 + 4 * u);
+            for (int i = 0; i < 8; ++i) {
+                acc[i][0] = fmaf(o[i], hv.x, acc[i][0]);
+                acc[i][1] = fmaf(o[i], hv.y, acc[i][1]);
+                acc[i][2] = fmaf(o[i], hv.z, acc[i][2]);
+                acc[i][3] = fmaf(o[i], hv.w, acc[i][3]);
+            }
         }
-        for (int i = threadIdx.x; i < nq * 8; i += 256) {  // dO_s [nq, 32]: 8 float4 per row
-            const int q = i >> 3, u = i & 7;
+    };
+    for (int s = hs.s0; s < hs.s1; ++s) {
+        const float* H = HG + (size_t)s * 2 * kMaxQ * ldg + e0;
+        __syncthreads();  // the previous sample's staged rows are read
+        for (int i = threadIdx.x; i < nq * (kWgE / 4); i += 256) {
+            const int q = i / (kWgE / 4), u = i % (kWgE / 4);
+            *reinterpret_cast<float4*>(&sh[q][4 * u]) =
+                *reinterpret_cast<const float4*>(H + (size_t)q * ldg + 4 * u);
+        }
+        for (int i = threadIdx.x; i < nq * (kWgC / 4); i += 256) {
+            const int q = i / (kWgC / 4), u = i % (kWgC / 4);
             *reinterpret_cast<float4*>(&so[q][4 * u]) = *reinterpret_cast<const float4*>(
                 dO + (size_t)s * ld_h + (size_t)q * dq + c0 + 4 * u);
         }
         if (4 * w < nq) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float2 gv = *reinterpret_cast<const float2*>(
-                    Gs + ((size_t)s * kMaxQ + 4 * w + i) * ldg + e0 + 2 * lane);
+                const float4 gv = *reinterpret_cast<const float4*>(
+                    H + (size_t)(kMaxQ + 4 * w + i) * ldg + 4 * lane);
                 gt[i][0] += gv.x;
                 gt[i][1] += gv.y;
+                gt[i][2] += gv.z;
+                gt[i][3] += gv.w;
             }
         }
         __syncthreads();
-        for (int q = 0; q < nq; ++q) {
-            const float4 o4 = *reinterpret_cast<const float4*>(&so[q][4 * w]);
-            const float2 hv = *reinterpret_cast<const float2*>(&sh[q][2 * lane]);
-            const float o[4] = {o4.x, o4.y, o4.z, o4.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                av[i][0] = fmaf(o[i], hv.x, av[i][0]);
-                av[i][1] = fmaf(o[i], hv.y, av[i][1]);
-            }
-        }
+        product(av);
     }
     __syncthreads();
     if (4 * w < nq) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float2*>(&sg[4 * w + i][2 * lane]) = make_float2(gt[i][0], gt[i][1]);
+            *reinterpret_cast<float4*>(&sh[4 * w + i][4 * lane]) =
+                make_float4(gt[i][0], gt[i][1], gt[i][2], gt[i][3]);
+    }
+    for (int i = threadIdx.x; i < nq * kWgC; i += 256) {
+        const int q = i / kWgC, c = i % kWgC;
+        so[q][c] = bf2f(hs.q[(size_t)q * dq + c0 + c]);
     }
     __syncthreads();
     const float scale = rsqrtf((float)dq);
-    float ak[4][2] = {};
-    for (int q = 0; q < nq; ++q) {
-        const float2 gv = *reinterpret_cast<const float2*>(&sg[q][2 * lane]);
+    float ak[8][4] = {};
+    product(ak);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float qv = bf2f(hs.q[(size_t)q * dq + c0 + 4 * w + i]);
-            ak[i][0] = fmaf(qv, gv.x, ak[i][0]);
-            ak[i][1] = fmaf(qv, gv.y, ak[i][1]);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const size_t o = (size_t)(c0 + 4 * w + i) * hs.d_in + e0 + 2 * lane;
-        float2 vk = make_float2(ak[i][0] * scale, ak[i][1] * scale);
-        float2 vv = make_float2(av[i][0], av[i][1]);
+    for (int i = 0; i < 8; ++i) {
+        const size_t o = (size_t)(c0 + 8 * w + i) * hs.d_in + e0 + 4 * lane;
+        float4 vk = make_float4(ak[i][0] * scale, ak[i][1] * scale, ak[i][2] * scale,
+                                ak[i][3] * scale);
+        float4 vv = make_float4(av[i][0], av[i][1], av[i][2], av[i][3]);
         if (hs.accum) {
-            const float2 ok = *reinterpret_cast<const float2*>(hs.g_wk + o);
-            const float2 ov = *reinterpret_cast<const float2*>(hs.g_wv + o);
-            vk.x += ok.x;
-            vk.y += ok.y;
-            vv.x += ov.x;
-            vv.y += ov.y;
+            const float4 ok = *reinterpret_cast<const float4*>(hs.g_wk + o);
+            const float4 ov = *reinterpret_cast<const float4*>(hs.g_wv + o);
+            vk = make_float4(vk.x + ok.x, vk.y + ok.y, vk.z + ok.z, vk.w + ok.w);
+            vv = make_float4(vv.x + ov.x, vv.y + ov.y, vv.z + ov.z, vv.w + ov.w);
         }
         if constexpr (kFused<OT>) {
-            opt_step2(opt.slot[blockIdx.x], 5, o, vk, hp);
-            opt_step2(opt.slot[blockIdx.x], 6, o, vv, hp);
+            // Wk's and Wv's optimizer state need only be 8-byte aligned
+            opt_step2(opt.slot[blockIdx.x], 5, o, make_float2(vk.x, vk.y), hp);
+            opt_step2(opt.slot[blockIdx.x], 5, o + 2, make_float2(vk.z, vk.w), hp);
+            opt_step2(opt.slot[blockIdx.x], 6, o, make_float2(vv.x, vv.y), hp);
+            opt_step2(opt.slot[blockIdx.x], 6, o + 2, make_float2(vv.z, vv.w), hp);
         } else {
-            *reinterpret_cast<float2*>(hs.g_wk + o) = vk;
-            *reinterpret_cast<float2*>(hs.g_wv + o) = vv;
+            *reinterpret_cast<float4*>(hs.g_wk + o) = vk;
+            *reinterpret_cast<float4*>(hs.g_wv + o) = vv;
         }
     }
 }
@@ -1253,6 +1293,57 @@ __global__ void __launch_bounds__(256) k_xattn_wgrad(const __grid_constant__ Hea
 static jnx_status cuda_ok(const char* what) {
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
+}
+
+// H_s = P_s^T X_s and G_s = dS_s^T X_s of the batch's query-head samples (see
+// k_xattn_gh).
+static jnx_status gh_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws, int d,
+                            const uint16_t* hidden, const jnx_group* g, cudaStream_t s) {
+    if (d % 256) {
+        k_xattn_gh<<<dim3(b.sample1 - b.sample0, d / 128), 256, 0, s>>>(
+            tab, b.g0, g->cu_seqlens, g->sample_slot, b.sample0, ws.P, ws.dS, hidden, d, ws.HG, d);
+        return JNX_OK;
+    }
+    static thread_local GemmBatch gb;  // staging of the kernel argument (copied at launch)
+    jnx_status st;
+    auto begin = [&]() -> bool {
+        gb.n_maps = gb.n = gb.tiles = 0;
+        gb.ldo = d;
+        gb.status = ws.status;
+        return batch_map(gb, ws.planes, (uint64_t)g->n_samples * 2 * kMaxQ, ws.ldp, ws.ldp, false,
+                         128) == 0;
+    };
+    if (!begin()) return fail(JNX_ERR_CUDA, "heads backward: tensor map");
+    for (int i = 0; i < b.n; ++i) {
+        const HeadSlot& hs = tab.slot[i];
+        if (hs.kind != JNX_HEAD_XATTN) continue;
+        for (int sm = hs.s0; sm < hs.s1; ++sm) {
+            const int r0 = g->h_cu_seqlens[sm], L = g->h_cu_seqlens[sm + 1] - r0;
+            float* out = ws.HG + (size_t)sm * 2 * kMaxQ * d;
+            if (L <= 0) {
+                if (cudaMemsetAsync(out, 0, (size_t)2 * kMaxQ * d * sizeof(float), s))
+                    return fail(JNX_ERR_CUDA, "heads backward: empty sample");
+                continue;
+            }
+            if (gb.n == kBatchMax) {
+                if ((st = gemm_batch_launch(gb, EPI_F32, false, true, s))) return st;
+                if (!begin()) return fail(JNX_ERR_CUDA, "heads backward: tensor map");
+            }
+            GemmBatch::Problem q{};
+            q.out = out;
+            q.a = 0;
+            q.b = q.b2 = batch_map(gb, hidden + (size_t)r0 * d, L, d, d, true, 0);
+            if (q.b < 0) return fail(JNX_ERR_CUDA, "heads backward: tensor map");
+            q.k1 = (L + 63) / 64;
+            q.k = 2 * q.k1;
+            q.ax2 = ws.ldp / 2;
+            q.m = 2 * kMaxQ;
+            q.arow = sm * 2 * kMaxQ;
+            q.nb = d / 256;
+            batch_add(gb, q);
+        }
+    }
+    return gemm_batch_launch(gb, EPI_F32, false, true, s);
 }
 
 jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws,
@@ -1282,9 +1373,9 @@ jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const 
 
 jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws,
                                  const float* pooled, int d, const uint16_t* hidden,
-                                 const int* cu, const int* sample_slot, bool kv_grads,
-                                 cudaStream_t s) {
+                                 const jnx_group* g, bool kv_grads, cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
+    const int *cu = g->cu_seqlens, *sample_slot = g->sample_slot;
     const NoOpt no{};
     const AdamHp nh{};
     k_head_dw_out<NoOpt>
@@ -1300,31 +1391,31 @@ jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
         k_xattn_bwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(
             tab, b.g0, cu, sample_slot, b.sample0, ws.kbuf, ws.vbuf, ws.ldkv, ws.P, ws.dS, ws.dh,
-            ws.ld_h, ws.dk, ws.dv, ws.dQs, kv_grads ? 1 : 0);
+            ws.ld_h, ws.dkv, ws.planes, ws.ldp, ws.dQs, kv_grads ? 1 : 0);
         k_xattn_dq<NoOpt><<<dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s>>>(
             tab, no, nh, ws.dQs, ws.ld_h);
-        k_xattn_gh<<<dim3(b.sample1 - b.sample0, d / 128), 256, 0, s>>>(
-            tab, b.g0, cu, sample_slot, b.sample0, ws.P, ws.dS, hidden, d, ws.Gs, ws.Hs, d);
-        k_xattn_wgrad<NoOpt><<<dim3(b.n, b.max_dq / 32, d / 64), 256, 0, s>>>(
-            tab, no, nh, ws.Gs, ws.Hs, d, ws.dh, ws.ld_h);
+        jnx_status st = gh_launch(tab, b, ws, d, hidden, g, s);
+        if (st) return st;
+        k_xattn_wgrad<NoOpt><<<dim3(b.n, b.max_dq / kWgC, d / kWgE), 256, 0, s>>>(
+            tab, no, nh, ws.HG, d, ws.dh, ws.ld_h);
     }
     return cuda_ok("heads backward");
 }
 
 jnx_status heads_backward_front_launch(const HeadTable& tab, const HeadBatch& b,
                                        const HeadScratch& ws, int d, const uint16_t* hidden,
-                                       const int* cu, const int* sample_slot, bool kv_grads,
-                                       cudaStream_t s) {
+                                       const jnx_group* g, bool kv_grads, cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
+    const int *cu = g->cu_seqlens, *sample_slot = g->sample_slot;
     k_head_back_in<<<dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s>>>(
         tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
         k_xattn_bwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(
             tab, b.g0, cu, sample_slot, b.sample0, ws.kbuf, ws.vbuf, ws.ldkv, ws.P, ws.dS, ws.dh,
-            ws.ld_h, ws.dk, ws.dv, ws.dQs, kv_grads ? 1 : 0);
-        k_xattn_gh<<<dim3(b.sample1 - b.sample0, d / 128), 256, 0, s>>>(
-            tab, b.g0, cu, sample_slot, b.sample0, ws.P, ws.dS, hidden, d, ws.Gs, ws.Hs, d);
+            ws.ld_h, ws.dkv, ws.planes, ws.ldp, ws.dQs, kv_grads ? 1 : 0);
+        jnx_status st = gh_launch(tab, b, ws, d, hidden, g, s);
+        if (st) return st;
     }
     return cuda_ok("heads backward");
 }
@@ -1344,8 +1435,8 @@ jnx_status heads_backward_step_launch(const HeadTable& tab, const HeadOptTable& 
             tab, opt, hp, ws.dh, ws.ld_h, pooled, d);
     if (b.any_xattn) {
         // wgrad reads the learned queries, which dq then updates
-        k_xattn_wgrad<HeadOptTable><<<dim3(b.n, b.max_dq / 32, d / 64), 256, 0, s>>>(
-            tab, opt, hp, ws.Gs, ws.Hs, d, ws.dh, ws.ld_h);
+        k_xattn_wgrad<HeadOptTable><<<dim3(b.n, b.max_dq / kWgC, d / kWgE), 256, 0, s>>>(
+            tab, opt, hp, ws.HG, d, ws.dh, ws.ld_h);
         k_xattn_dq<HeadOptTable><<<dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s>>>(
             tab, opt, hp, ws.dQs, ws.ld_h);
     }

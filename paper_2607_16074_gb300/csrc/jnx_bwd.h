@@ -81,8 +81,6 @@ jnx_status seg_wgrad_launch(const SegRows& sr, const uint16_t* U, int ldu, const
 jnx_status mlp_dfeat_launch(const float* dz, int ldz, const int* cu, const int* sample_slot,
                             int n_samples, const MlpFeatTable& tab, int d, float* dh,
                             cudaStream_t s);
-jnx_status to_bf16_launch(const float* src, int lds, int rows, int cols, uint16_t* dst, int ldd,
-                          cudaStream_t s);
 
 // Attention backward over the packed samples (bidirectional inside each
 // sample), from q, k, v (after RoPE, [N, (H + 2 Hkv) hd]), the saved

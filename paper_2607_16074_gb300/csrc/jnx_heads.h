@@ -65,12 +65,15 @@ struct HeadScratch {
     float *y, *dy;       // [n_samples, ld_y]
     int ld_h, ld_y;
     // query heads
-    float *kbuf, *vbuf, *dk, *dv;  // [n_tokens, ldkv]
+    float *kbuf, *vbuf;            // [n_tokens, ldkv]
     int ldkv;
     float *P, *dS;                 // [nq * n_tokens], key-major per sample
     float* dQs;                    // [n_samples, ld_h]
-    float *Gs, *Hs;                // [n_samples, 32, d]: dS_s^T X_s and P_s^T X_s (32 query rows)
-    uint16_t* dkv_bf;              // feature gradient: bf16 [dk | dv] rows [n_tokens, 2 ldkv]
+    float* HG;                     // [n_samples, 64, d]: P_s^T X_s and dS_s^T X_s (32 rows each)
+    uint16_t* planes;              // their bf16 operands [n_samples, 64, ldp] (see k_xattn_bwd)
+    int ldp;                       // twice the longest sample, in whole 64s
+    uint16_t* dkv;                 // feature gradient: bf16 [dk | dv] rows [n_tokens, 2 ldkv]
+    int* status;                   // device status word
 };
 
 jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws,
@@ -81,8 +84,7 @@ jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const 
 // gradient only).
 jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws,
                                  const float* pooled, int d, const uint16_t* hidden,
-                                 const int* cu, const int* sample_slot, bool kv_grads,
-                                 cudaStream_t s);
+                                 const jnx_group* g, bool kv_grads, cudaStream_t s);
 // The backward with the tenant-private AdamW step fused into it, in two
 // launches so that nothing updates a parameter before every read of it:
 // front: the output layer's input gradient (reads W2 / Wout) and the query
@@ -94,8 +96,7 @@ jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const
 // the queries' own update.
 jnx_status heads_backward_front_launch(const HeadTable& tab, const HeadBatch& b,
                                        const HeadScratch& ws, int d, const uint16_t* hidden,
-                                       const int* cu, const int* sample_slot, bool kv_grads,
-                                       cudaStream_t s);
+                                       const jnx_group* g, bool kv_grads, cudaStream_t s);
 jnx_status heads_backward_step_launch(const HeadTable& tab, const HeadOptTable& opt,
                                       const AdamHp& hp, const HeadBatch& b,
                                       const HeadScratch& ws, const float* pooled, int d,

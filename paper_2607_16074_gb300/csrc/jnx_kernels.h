@@ -127,6 +127,33 @@ struct LoraDown {
 jnx_status lora_down_launch(const jnx_group* g, const uint16_t* x, int ldx, int K, int n_parts,
                             const uint16_t* const* a, uint16_t* t, int ldt, cudaStream_t s);
 
+// Many small GEMMs of one launch: problem i is out_i [m, nb * 256] (fp32, row
+// stride ldo) = A_i . B_i^T over k K-steps of 64.  A_i comes from map[a], rows
+// arow + row (K-major) or columns row (a_mn: A is [K, m] row-major); B_i from
+// map[b] for the first k1 K-steps and from map[b2] (restarting at its first K
+// row) for the rest, whose A columns start at ax2; b_mn: B is [K, N] row-major.
+// A K extent that is no multiple of 64 ends in the maps' zero fill, so a map
+// whose rows are K covers one problem's rows only.
+constexpr int kBatchMaps = 130, kBatchMax = 128;
+struct GemmBatch {
+    CUtensorMap map[kBatchMaps];
+    struct Problem {
+        float* out;
+        int a, b, b2, k1, k, m, arow, ax2, nb, tile0;
+    } p[kBatchMax];
+    int n_maps, n, tiles, ldo;
+    int* status;
+};
+// An operand's map: K-major [rows, K] with `box` rows a stage, or MN-major
+// [K rows, cols].  Returns its index, -1 when the table is full or the layout
+// is not one TMA takes.
+int batch_map(GemmBatch& gb, const uint16_t* ptr, uint64_t rows, uint64_t cols, uint64_t ld,
+              bool mn, int box);
+// Adds a problem; false when the table is full.
+bool batch_add(GemmBatch& gb, GemmBatch::Problem p);
+// epi: EPI_F32 or EPI_RESID (out += product).
+jnx_status gemm_batch_launch(const GemmBatch& gb, int epi, bool a_mn, bool b_mn, cudaStream_t s);
+
 // GEMM C = A . B^T with A [M, K] (row stride lda), B [N, K] (row stride ldb).
 jnx_status gemm_check(int M, int N, int K);
 jnx_status gemm_launch(const uint16_t* A, int lda, const uint16_t* B, int ldb, GemmParams p,
