@@ -152,10 +152,27 @@ __global__ void __launch_bounds__(256) k_flow_embed(
     }
     __syncthreads();
     const uint16_t* W = w_in + (size_t)t * dm * D;
+    // a weight row is 2 D contiguous bytes: 16-byte loads where rows allow them
+    // (2-byte ones kept a row's 32 loads in turn: 37.6 us for 512 rows, 10.6 now)
+    const bool vec = D % 8 == 0 && (reinterpret_cast<uintptr_t>(w_in) & 15) == 0;
     for (int j = threadIdx.x; j < dm; j += blockDim.x) {
         float acc = bf2f(b_in[(size_t)t * dm + j]) + bf2f(pos[((size_t)t * C + c) * dm + j]) +
                     phi[(size_t)s * dm + j];
-        for (int k = 0; k < D; ++k) acc += xs[k] * bf2f(W[(size_t)j * D + k]);
+        const uint16_t* wr = W + (size_t)j * D;
+        if (vec) {
+#pragma unroll 4
+            for (int k = 0; k < D; k += 8) {
+                const uint4 q = __ldg(reinterpret_cast<const uint4*>(wr + k));
+                const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    acc += xs[k + 2 * e] * __uint_as_float(u[e] << 16);
+                    acc += xs[k + 2 * e + 1] * __uint_as_float(u[e] & 0xffff0000u);
+                }
+            }
+        } else {
+            for (int k = 0; k < D; ++k) acc += xs[k] * bf2f(wr[k]);
+        }
         h[(size_t)r * dm + j] = acc;
     }
 }
@@ -695,75 +712,75 @@ __global__ void __launch_bounds__(128) k_flow_attn_bwd_kv(
 }
 
 // ---------------------------------------------------------------------------
-// output: v = nf W_out^T + b_out, and (training) dv = 2 (v - u) / n_t and
-// the row's sum of (v - u)^2.  One warp per action row.
+// output: v = nf W_out^T + b_out, and (training) dv = 2 (v - u) / n_t.  One warp
+// per output element (a warp per row took its outputs in turn, a load and a
+// shuffle tree each: 34 us for 32 rows x 32 outputs of depth 1,024, 5.3 now).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_flow_out(const uint16_t* __restrict__ nf,
                                                   const int* __restrict__ sample_slot,
                                                   const __grid_constant__ FlowSlots fs, FlowDims dd,
                                                   const uint16_t* __restrict__ w_out,
                                                   const uint16_t* __restrict__ b_out,
-                                                  const float* __restrict__ u, int M,
-                                                  float* __restrict__ v, float* __restrict__ dv,
-                                                  float* __restrict__ rowsq) {
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= M) return;
+                                                  const float* __restrict__ u,
+                                                  float* __restrict__ v, float* __restrict__ dv) {
+    const int r = blockIdx.x, lane = threadIdx.x & 31;
     const int dm = dd.dm, D = dd.D, C = dd.C;
+    const int k = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (k >= D) return;
     const int slot = sample_slot[r / C];
     const int t = fs.tenant[slot];
-    const float nt = (float)(fs.s1[slot] - fs.s0[slot]) * C * D;
-    // the row in registers: lane holds columns 8 lane + 256 i, i < dm / 256
-    float xr[4][8];
+    const uint16_t* xr = nf + (size_t)r * dm + 8 * lane;
+    const uint16_t* wr = w_out + ((size_t)t * D + k) * dm + 8 * lane;
+    float acc = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i)  // columns 8 lane + 256 i, i < dm / 256
         if (256 * i < dm) {
-            const uint4 q = *reinterpret_cast<const uint4*>(nf + (size_t)r * dm + 256 * i + 8 * lane);
-            const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
+            const uint4 x = *reinterpret_cast<const uint4*>(xr + 256 * i);
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(wr + 256 * i));
+            const uint32_t x4[4] = {x.x, x.y, x.z, x.w}, w4[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                xr[i][2 * e] = __uint_as_float(w4[e] << 16);
-                xr[i][2 * e + 1] = __uint_as_float(w4[e] & 0xffff0000u);
+                acc = fmaf(__uint_as_float(x4[e] << 16), __uint_as_float(w4[e] << 16), acc);
+                acc = fmaf(__uint_as_float(x4[e] & 0xffff0000u),
+                           __uint_as_float(w4[e] & 0xffff0000u), acc);
             }
         }
-    float sq = 0.f;
-    for (int k = 0; k < D; ++k) {
-        const uint16_t* wr = w_out + ((size_t)t * D + k) * dm + 8 * lane;
-        float acc = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (256 * i < dm) {
-                const uint4 q = *reinterpret_cast<const uint4*>(wr + 256 * i);
-                const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc = fmaf(xr[i][2 * e], __uint_as_float(w4[e] << 16), acc);
-                    acc = fmaf(xr[i][2 * e + 1], __uint_as_float(w4[e] & 0xffff0000u), acc);
-                }
-            }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
         acc += bf2f(b_out[(size_t)t * D + k]);
-        if (lane == 0) {
-            const size_t e = (size_t)r * D + k;
-            v[e] = acc;
-            if (u) {
-                const float diff = acc - u[e];
-                dv[e] = 2.f * diff / nt;
-                sq += diff * diff;
-            }
+        const size_t e = (size_t)r * D + k;
+        v[e] = acc;
+        if (u) {
+            const float nt = (float)(fs.s1[slot] - fs.s0[slot]) * C * D;
+            dv[e] = 2.f * (acc - u[e]) / nt;
         }
     }
-    if (u && lane == 0) rowsq[r] = sq;
 }
 
-// loss[tenant] = sum of the tenant's row sums in row order / n_t.
-__global__ void k_flow_loss(const __grid_constant__ FlowSlots fs, FlowDims dd,
-                            const float* __restrict__ rowsq, float* __restrict__ loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= fs.n) return;
+// loss[tenant] = sum over its elements of (v - u)^2 / n_t: one CTA per slot,
+// thread i its elements i, i + 256, ..., then a fixed tree.
+__global__ void __launch_bounds__(256) k_flow_loss(const __grid_constant__ FlowSlots fs,
+                                                   FlowDims dd, const float* __restrict__ v,
+                                                   const float* __restrict__ u,
+                                                   float* __restrict__ loss) {
+    __shared__ float red[8];
+    const int i = blockIdx.x;
+    const size_t e0 = (size_t)fs.s0[i] * dd.C * dd.D, e1 = (size_t)fs.s1[i] * dd.C * dd.D;
     float acc = 0.f;
-    for (int r = fs.s0[i] * dd.C; r < fs.s1[i] * dd.C; ++r) acc += rowsq[r];
-    loss[fs.tenant[i]] = acc / ((float)(fs.s1[i] - fs.s0[i]) * dd.C * dd.D);
+    for (size_t e = e0 + threadIdx.x; e < e1; e += 256) {
+        const float diff = v[e] - u[e];
+        acc += diff * diff;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        loss[fs.tenant[i]] = t / ((float)(fs.s1[i] - fs.s0[i]) * dd.C * dd.D);
+    }
 }
 
 // Euler step of the sampler: x += dt v.
@@ -787,10 +804,34 @@ __global__ void __launch_bounds__(256) k_flow_out_bwd(const float* __restrict__ 
     __shared__ float g[kMaxD];
     if (threadIdx.x < D) g[threadIdx.x] = dv[(size_t)r * D + threadIdx.x];
     __syncthreads();
-    for (int j = threadIdx.x; j < dm; j += blockDim.x) {
-        float acc = 0.f;
-        for (int k = 0; k < D; ++k) acc += g[k] * bf2f(w_out[((size_t)t * D + k) * dm + j]);
-        dnf[(size_t)r * dm + j] = acc;
+    // four consecutive columns a thread (dm is a multiple of 4, w_out 16-byte
+    // aligned), eight weight rows' loads in flight
+    for (int j = 4 * threadIdx.x; j < dm; j += 4 * blockDim.x) {
+        float acc[4] = {};
+        const uint16_t* wc = w_out + (size_t)t * D * dm + j;
+#pragma unroll 8
+        for (int k = 0; k < D; ++k) {
+            const uint2 q = __ldg(reinterpret_cast<const uint2*>(wc + (size_t)k * dm));
+            acc[0] += g[k] * __uint_as_float(q.x << 16);
+            acc[1] += g[k] * __uint_as_float(q.x & 0xffff0000u);
+            acc[2] += g[k] * __uint_as_float(q.y << 16);
+            acc[3] += g[k] * __uint_as_float(q.y & 0xffff0000u);
+        }
+        *reinterpret_cast<float4*>(dnf + (size_t)r * dm + j) =
+            make_float4(acc[0], acc[1], acc[2], acc[3]);
+    }
+}
+
+// Four consecutive gradient elements written or, with add, added to.
+__device__ __forceinline__ void store4(float* p, const float (&v)[4], int add) {
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (add) o = *reinterpret_cast<const float4*>(p);
+        *reinterpret_cast<float4*>(p) = add ? make_float4(o.x + v[0], o.y + v[1], o.z + v[2], o.w + v[3])
+                                            : make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) p[e] = add ? p[e] + v[e] : v[e];
     }
 }
 
@@ -804,11 +845,18 @@ __global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* __restrict_
     const int i = blockIdx.x, k = blockIdx.y, dm = dd.dm, D = dd.D, C = dd.C;
     const int t = fs.tenant[i];
     const int r0 = fs.s0[i] * C, r1 = fs.s1[i] * C;
-    for (int j = threadIdx.x; j < dm; j += blockDim.x) {
-        float acc = 0.f;
-        for (int r = r0; r < r1; ++r) acc += dv[(size_t)r * D + k] * bf2f(nf[(size_t)r * dm + j]);
-        float* p = gw + ((size_t)t * D + k) * dm + j;
-        *p = add ? *p + acc : acc;
+    for (int j = 4 * threadIdx.x; j < dm; j += 4 * blockDim.x) {
+        float acc[4] = {};
+#pragma unroll 8
+        for (int r = r0; r < r1; ++r) {
+            const float g = dv[(size_t)r * D + k];
+            const uint2 q = __ldg(reinterpret_cast<const uint2*>(nf + (size_t)r * dm + j));
+            acc[0] += g * __uint_as_float(q.x << 16);
+            acc[1] += g * __uint_as_float(q.x & 0xffff0000u);
+            acc[2] += g * __uint_as_float(q.y << 16);
+            acc[3] += g * __uint_as_float(q.y & 0xffff0000u);
+        }
+        store4(gw + ((size_t)t * D + k) * dm + j, acc, add);
     }
     if (threadIdx.x == 0) {
         float acc = 0.f;
@@ -821,8 +869,12 @@ __global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* __restrict_
 // ---------------------------------------------------------------------------
 // backward of the embedding and of the time MLP
 // ---------------------------------------------------------------------------
-// Per slot, thread per width column j: dW_in[t][j, :] = sum_r dh[r, j] x[r, :],
+// Per slot and width column j: dW_in[t][j, :] = sum_r dh[r, j] x[r, :],
 // db_in[t][j] = sum_r dh[r, j], dpos[t][c, j] = sum over samples dh[s C + c, j].
+// One CTA per (slot, 32 columns): lane = column, warp w takes the action
+// dimensions 8 w .. + 7 and the chunk steps c = w (mod 8); rows in order, several
+// loads in flight (a thread per column with every dimension: 90 us for eight
+// tenants of 64 rows, 31 now).
 __global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* __restrict__ dh,
                                                           const float* __restrict__ x,
                                                           const __grid_constant__ FlowSlots fs,
@@ -830,31 +882,29 @@ __global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* __restric
                                                           float* __restrict__ gb,
                                                           float* __restrict__ gpos, int add) {
     const int i = blockIdx.x, dm = dd.dm, D = dd.D, C = dd.C;
-    const int j = blockIdx.y * blockDim.x + threadIdx.x;
-    if (j >= dm) return;
-    const int t = fs.tenant[i];
-    float w[kMaxD];
-#pragma unroll
-    for (int k = 0; k < kMaxD; ++k) w[k] = 0.f;
-    float b = 0.f;
-    for (int s = fs.s0[i]; s < fs.s1[i]; ++s)
-        for (int c = 0; c < C; ++c) {
-            const size_t r = (size_t)s * C + c;
-            const float g = dh[r * dm + j];
+    const int warp = threadIdx.x >> 5, j = blockIdx.y * 32 + (threadIdx.x & 31);
+    const int t = fs.tenant[i], k0 = 8 * warp;
+    const int r0 = fs.s0[i] * C, r1 = fs.s1[i] * C;
+    if (k0 < D || warp == 0) {
+        float w[8] = {}, b = 0.f;
+#pragma unroll 4
+        for (int r = r0; r < r1; ++r) {
+            const float g = dh[(size_t)r * dm + j];
             b += g;
 #pragma unroll
-            for (int k = 0; k < kMaxD; ++k)
-                if (k < D) w[k] += g * x[r * D + k];
+            for (int k = 0; k < 8; ++k)
+                if (k0 + k < D) w[k] += g * x[(size_t)r * D + k0 + k];
         }
+        float* p = gw + ((size_t)t * dm + j) * D + k0;
 #pragma unroll
-    for (int k = 0; k < kMaxD; ++k)
-        if (k < D) {
-            float* p = gw + ((size_t)t * dm + j) * D + k;
-            *p = add ? *p + w[k] : w[k];
+        for (int k = 0; k < 8; ++k)
+            if (k0 + k < D) p[k] = add ? p[k] + w[k] : w[k];
+        if (warp == 0) {
+            float* pb = gb + (size_t)t * dm + j;
+            *pb = add ? *pb + b : b;
         }
-    float* pb = gb + (size_t)t * dm + j;
-    *pb = add ? *pb + b : b;
-    for (int c = 0; c < C; ++c) {
+    }
+    for (int c = warp; c < C; c += 8) {
         float acc = 0.f;
         for (int s = fs.s0[i]; s < fs.s1[i]; ++s) acc += dh[((size_t)s * C + c) * dm + j];
         float* p = gpos + ((size_t)t * C + c) * dm + j;
@@ -918,24 +968,42 @@ __global__ void __launch_bounds__(256) k_flow_time_bwd(const int* __restrict__ s
 // Per slot, row j of an outer-product sum over the tenant's samples:
 //   G[t][j, k] = sum_s A[s, j] f(B[s, k]),  gb[t][j] = sum_s A[s, j]
 // with f = SiLU (T2: A = dphi, B = z1) or the identity (T1: A = dz1, B = s(tau)).
+// One CTA per (slot, kOuterRows rows j): a thread's four columns k of a sample's
+// B row serve all of the rows (one row a CTA evaluated SiLU per row and wrote 4
+// bytes a store: 55 us for eight experts of width 1,024, 14 now).
+constexpr int kOuterRows = 8;
+
 template <bool SILU>
 __global__ void __launch_bounds__(256) k_flow_outer(const float* __restrict__ A,
                                                     const float* __restrict__ Bm,
                                                     const __grid_constant__ FlowSlots fs,
                                                     FlowDims dd, float* __restrict__ gw,
                                                     float* __restrict__ gb, int add) {
-    const int i = blockIdx.x, j = blockIdx.y, dm = dd.dm;
+    const int i = blockIdx.x, j0 = blockIdx.y * kOuterRows, dm = dd.dm;
     const int t = fs.tenant[i];
-    for (int k = threadIdx.x; k < dm; k += blockDim.x) {
-        float acc = 0.f;
+    for (int k = 4 * threadIdx.x; k < dm; k += 4 * 256) {
+        float acc[kOuterRows][4] = {};
         for (int s = fs.s0[i]; s < fs.s1[i]; ++s) {
-            const float b = Bm[(size_t)s * dm + k];
-            acc += A[(size_t)s * dm + j] * (SILU ? silu_f(b) : b);
+            const float4 q = *reinterpret_cast<const float4*>(Bm + (size_t)s * dm + k);
+            float b[4] = {q.x, q.y, q.z, q.w};
+            if (SILU)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) b[e] = silu_f(b[e]);
+            const float4 a0 = *reinterpret_cast<const float4*>(A + (size_t)s * dm + j0);
+            const float4 a1 = *reinterpret_cast<const float4*>(A + (size_t)s * dm + j0 + 4);
+            const float a[kOuterRows] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int r = 0; r < kOuterRows; ++r)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[r][e] += a[r] * b[e];
         }
-        float* p = gw + ((size_t)t * dm + j) * dm + k;
-        *p = add ? *p + acc : acc;
+#pragma unroll
+        for (int r = 0; r < kOuterRows; ++r) {
+            store4(gw + ((size_t)t * dm + j0 + r) * dm + k, acc[r], add);
+        }
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < kOuterRows) {
+        const int j = j0 + threadIdx.x;
         float acc = 0.f;
         for (int s = fs.s0[i]; s < fs.s1[i]; ++s) acc += A[(size_t)s * dm + j];
         float* p = gb + (size_t)t * dm + j;
@@ -954,7 +1022,6 @@ struct FlowWs {
     uint16_t* ones;      // [dm] bf16 1.0 (the non-affine norm's gain)
     float *sfeat, *z1, *phi;  // [S, dm]
     float *x, *u, *v, *dv;    // [M_a, D]
-    float* rowsq;             // [M_a]
     float* h;                 // [M_a, dm] the residual stream
     float* h_out;             // [M_a, dm]
     uint16_t* nf;             // [M_a, dm]
@@ -965,21 +1032,17 @@ struct FlowWs {
     float* lse;               // [nb][M_a, nh]
     uint16_t* m;              // [nb][M_a, F]
     uint16_t* kvc;            // [nb][N, 2 dm]
-    // the context weight gradient on the tensor cores: the hidden rows and
-    // dKV_c transposed, each tenant's rows at a 64-aligned column offset
-    uint16_t *xT, *dkT;       // [d, kpad], [2 dm, kpad]
     // backward scratch
     float *dh, *dn, *dO;      // [M_a, dm]
     uint16_t* dh_bf;          // [M_a, dm]
     uint16_t* gu;             // [M_a, 2 F]
     uint16_t* dqkv;           // [M_a, 3 dm]
     uint16_t* dkvc;           // [N, 2 dm]
-    uint16_t* wt;             // transposed weights of one block [T, max]
     float *dphi, *dz1;        // [S, dm]
     size_t bytes;
 };
 
-FlowWs carve_flow(const FlowDims& d, int S, int N, int n_slots, void* base) {
+FlowWs carve_flow(const FlowDims& d, int S, int N, void* base) {
     uint8_t* p = static_cast<uint8_t*>(base);
     FlowWs w{};
     size_t off = 0;
@@ -1000,7 +1063,6 @@ FlowWs carve_flow(const FlowDims& d, int S, int N, int n_slots, void* base) {
     w.u = f32(Ma * d.D);
     w.v = f32(Ma * d.D);
     w.dv = f32(Ma * d.D);
-    w.rowsq = f32(Ma);
     w.h = f32(Ma * dm);
     w.h_out = f32(Ma * dm);
     w.nf = b16(Ma * dm);
@@ -1020,12 +1082,8 @@ FlowWs carve_flow(const FlowDims& d, int S, int N, int n_slots, void* base) {
     w.gu = b16(Ma * 2 * d.F);
     w.dqkv = b16(Ma * 3 * dm);
     w.dkvc = b16(n * 2 * dm);
-    w.wt = b16((size_t)d.T * std::max(3 * dm * dm, 2 * (size_t)d.F * dm));
     w.dphi = f32(s * dm);
     w.dz1 = f32(s * dm);
-    const size_t kpad = (n + 63) / 64 * 64 + 64 * (size_t)std::max(n_slots, 0);
-    w.xT = b16((size_t)d.d * kpad);
-    w.dkT = b16(2 * dm * kpad);
     w.bytes = off;
     return w;
 }
@@ -1281,12 +1339,48 @@ jnx_status flow_network(const jnx_flow_head* fh, const FlowDims& d, const jnx_gr
         cudaSuccess)
         return last("flow: copy");
     if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, w.nf, s))) return st;
-    k_flow_out<<<(Ma + 7) / 8, 256, 0, s>>>(w.nf, g->sample_slot, fs, d, fh->w_out, fh->b_out,
-                                            train ? w.u : nullptr, Ma, w.v, w.dv, w.rowsq);
+    k_flow_out<<<dim3(Ma, (d.D + 7) / 8), 256, 0, s>>>(w.nf, g->sample_slot, fs, d, fh->w_out,
+                                                       fh->b_out, train ? w.u : nullptr, w.v, w.dv);
     if ((st = last("flow output"))) return st;
     if (train && loss) {
-        k_flow_loss<<<(nsl + 63) / 64, 64, 0, s>>>(fs, d, w.rowsq, loss);
+        k_flow_loss<<<nsl, 256, 0, s>>>(fs, d, w.v, w.u, loss);
         if ((st = last("flow loss"))) return st;
+    }
+    return JNX_OK;
+}
+
+// dW_kvc[t] (+)= dKV_c^T X over each tenant's token rows, one batched launch per
+// 64 tenants (transposed copies of the rows and a launch per tenant took 200 us a
+// block for eight tenants of 1,200 rows, 66 now).
+jnx_status ctx_wgrad(const FlowDims& d, const SegRows& rt, const FlowWs& w,
+                     const uint16_t* hidden, float* grad, int add, cudaStream_t s) {
+    static thread_local GemmBatch gb;  // staging of the kernel argument (copied at launch)
+    const int M2 = 2 * d.dm;
+    for (int i0 = 0; i0 < rt.n; i0 += 64) {
+        gb.n_maps = gb.n = gb.tiles = 0;
+        gb.ldo = d.d;
+        gb.status = w.status;
+        for (int i = i0; i < std::min(i0 + 64, rt.n); ++i) {
+            float* gw = grad + (size_t)rt.tenant[i] * M2 * d.d;
+            const int r0 = rt.r0[i], rows = rt.r1[i] - r0;
+            if (rows <= 0) {  // no context rows: a zero gradient
+                if (!add && cudaMemsetAsync(gw, 0, sizeof(float) * M2 * d.d, s))
+                    return last("flow context weight gradient");
+                continue;
+            }
+            GemmBatch::Problem q{};
+            q.out = gw;
+            q.a = batch_map(gb, w.dkvc + (size_t)r0 * M2, rows, M2, M2, true, 0);
+            q.b = q.b2 = batch_map(gb, hidden + (size_t)r0 * d.d, rows, d.d, d.d, true, 0);
+            if (q.a < 0 || q.b < 0)
+                return fail(JNX_ERR_CUDA, "flow: tensor map encode failed (alignment or driver)");
+            q.k1 = q.k = (rows + 63) / 64;
+            q.m = M2;
+            q.nb = d.d / 256;
+            batch_add(gb, q);
+        }
+        jnx_status st = gemm_batch_launch(gb, add ? EPI_RESID : EPI_F32, true, true, s);
+        if (st) return st;
     }
     return JNX_OK;
 }
@@ -1300,7 +1394,7 @@ extern "C" size_t jnx_flow_workspace_bytes(const jnx_flow_head* fh, const jnx_gr
     if (!fh || !g) return 0;
     FlowDims d{fh->d_model, fh->d_ff, fh->n_blocks, fh->chunk, fh->action_dim, fh->d_in,
                fh->n_tenants, fh->d_model / kHd};
-    return carve_flow(d, g->n_samples, g->n_tokens, g->n_slots, nullptr).bytes;
+    return carve_flow(d, g->n_samples, g->n_tokens, nullptr).bytes;
 }
 
 static jnx_status flow_begin(const jnx_flow_head* fh, const jnx_group* g, const uint16_t* hidden,
@@ -1311,7 +1405,7 @@ static jnx_status flow_begin(const jnx_flow_head* fh, const jnx_group* g, const 
         return fail(JNX_ERR_INVALID_ARG, "flow: null workspace or hidden rows");
     if (reinterpret_cast<uintptr_t>(workspace) & 255)
         return fail(JNX_ERR_INVALID_ARG, "flow: workspace must be 256-byte aligned");
-    w = carve_flow(d, g->n_samples, g->n_tokens, g->n_slots, workspace);
+    w = carve_flow(d, g->n_samples, g->n_tokens, workspace);
     if (ws_bytes < w.bytes)
         return fail(JNX_ERR_WORKSPACE, "flow: workspace %zu < %zu bytes", ws_bytes, w.bytes);
     return JNX_OK;
@@ -1427,20 +1521,10 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
         rt.r1[i] = sg.t1[i];
     }
     // the context weight gradient dW_kvc[t] = dKV_c^T X over tenant t's token
-    // rows runs as one tcgen05 GEMM per tenant (K = its rows, padded to 64)
-    // on transposed copies; widths that are not a multiple of 256 keep the
+    // rows runs as one batched tcgen05 launch, both operands read as they lie
+    // (their rows are K); widths that are not a multiple of 256 keep the
     // mma.sync segmented kernel
     const bool tc_kvc = d.d % 256 == 0;
-    static thread_local SegRows rp;  // token-row segments at padded offsets
-    rp = rt;
-    std::vector<int> kp(nsl);
-    int kpad = 0;
-    for (int i = 0; i < nsl; ++i) {
-        rp.tile_start[i] = kpad;
-        kp[i] = (rt.r1[i] - rt.r0[i] + 63) / 64 * 64;
-        kpad += kp[i];
-    }
-    if (tc_kvc && (st = transpose_seg_launch(hidden, d.d, d.d, rp, kpad, w.xT, s))) return st;
     // output layer
     {
         TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * d.D * 4.0, s);
@@ -1487,7 +1571,6 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
         }
         {
             TraceScope ts(JNX_K_FLOW_GEMM, 2.0 * Ma * F * dm, s);
-            if ((st = transpose_launch(B.w_d, T, dm, F, w.wt, s))) return st;  // [T, F, dm]
             p = GemmParams{};
             p.M = Ma;
             p.N = F;
@@ -1498,8 +1581,8 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
             p.aux = w.gu;
             p.ldaux = 2 * F;
             p.status = w.status;
-            if ((st = gemm_launch_seg(w.dh_bf, dm, w.wt, dm, T, p, nsl, sg.a0.data(),
-                                      sg.a1.data(), sg.ten.data(), s)))
+            if ((st = gemm_launch_seg(w.dh_bf, dm, B.w_d, F, T, p, nsl, sg.a0.data(),
+                                      sg.a1.data(), sg.ten.data(), s, true)))
                 return st;
         }
         {
@@ -1510,7 +1593,6 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
         }
         {
             TraceScope ts(JNX_K_FLOW_GEMM, 2.0 * Ma * dm * 2 * F, s);
-            if ((st = transpose_launch(B.w_gu, T, 2 * F, dm, w.wt, s))) return st;  // [T, dm, 2F]
             p = GemmParams{};
             p.M = Ma;
             p.N = dm;
@@ -1519,8 +1601,8 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
             p.out = w.dn;
             p.ldo = dm;
             p.status = w.status;
-            if ((st = gemm_launch_seg(w.gu, 2 * F, w.wt, 2 * F, T, p, nsl, sg.a0.data(),
-                                      sg.a1.data(), sg.ten.data(), s)))
+            if ((st = gemm_launch_seg(w.gu, 2 * F, B.w_gu, dm, T, p, nsl, sg.a0.data(),
+                                      sg.a1.data(), sg.ten.data(), s, true)))
                 return st;
         }
         {
@@ -1537,7 +1619,6 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
         }
         {
             TraceScope ts(JNX_K_FLOW_GEMM, 2.0 * Ma * dm * dm, s);
-            if ((st = transpose_launch(B.w_o, T, dm, dm, w.wt, s))) return st;
             p = GemmParams{};
             p.M = Ma;
             p.N = dm;
@@ -1546,8 +1627,8 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
             p.out = w.dO;
             p.ldo = dm;
             p.status = w.status;
-            if ((st = gemm_launch_seg(w.dh_bf, dm, w.wt, dm, T, p, nsl, sg.a0.data(),
-                                      sg.a1.data(), sg.ten.data(), s)))
+            if ((st = gemm_launch_seg(w.dh_bf, dm, B.w_o, dm, T, p, nsl, sg.a0.data(),
+                                      sg.a1.data(), sg.ten.data(), s, true)))
                 return st;
         }
         {
@@ -1569,38 +1650,11 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
                                            G.w_kvc, (long long)2 * dm * d.d, add, s)))
                     return st;
             } else {
-                if ((st = transpose_seg_launch(w.dkvc, 2 * dm, 2 * dm, rp, kpad, w.dkT, s)))
-                    return st;
-                for (int i = 0; i < nsl; ++i) {
-                    float* gw = G.w_kvc + (size_t)rt.tenant[i] * 2 * dm * d.d;
-                    if (kp[i] == 0) {  // no context rows: a zero gradient
-                        if (!add && cudaMemsetAsync(gw, 0, sizeof(float) * 2 * dm * d.d, s))
-                            return last("flow context weight gradient");
-                        continue;
-                    }
-                    GemmParams q{};
-                    q.M = 2 * dm;
-                    q.N = d.d;
-                    q.K = kp[i];
-                    q.status = w.status;
-                    if (add) {
-                        q.epi = EPI_RESID;
-                        q.resid = gw;
-                        q.ldr = d.d;
-                    } else {
-                        q.epi = EPI_F32;
-                        q.out = gw;
-                        q.ldo = d.d;
-                    }
-                    if ((st = gemm_launch(w.dkT + rp.tile_start[i], kpad, w.xT + rp.tile_start[i],
-                                          kpad, q, s)))
-                        return st;
-                }
+                if ((st = ctx_wgrad(d, rt, w, hidden, G.w_kvc, add, s))) return st;
             }
         }
         {
             TraceScope ts(JNX_K_FLOW_GEMM, 2.0 * Ma * dm * 3 * dm, s);
-            if ((st = transpose_launch(B.w_qkv, T, 3 * dm, dm, w.wt, s))) return st;  // [T, dm, 3dm]
             p = GemmParams{};
             p.M = Ma;
             p.N = dm;
@@ -1609,8 +1663,8 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
             p.out = w.dn;
             p.ldo = dm;
             p.status = w.status;
-            if ((st = gemm_launch_seg(w.dqkv, 3 * dm, w.wt, 3 * dm, T, p, nsl, sg.a0.data(),
-                                      sg.a1.data(), sg.ten.data(), s)))
+            if ((st = gemm_launch_seg(w.dqkv, 3 * dm, B.w_qkv, dm, T, p, nsl, sg.a0.data(),
+                                      sg.a1.data(), sg.ten.data(), s, true)))
                 return st;
         }
         {
@@ -1621,12 +1675,12 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
     }
     // ---- embedding and time MLP ----
     TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * 8.0 + (double)S * dm * dm * 8.0, s);
-    k_flow_embed_wgrad<<<dim3(nsl, (dm + 255) / 256), 256, 0, s>>>(w.dh, w.x, fs, d, gr->w_in,
+    k_flow_embed_wgrad<<<dim3(nsl, dm / 32), 256, 0, s>>>(w.dh, w.x, fs, d, gr->w_in,
                                                                     gr->b_in, gr->pos, add);
     k_flow_dphi<<<dim3(S, (dm + 255) / 256), 256, 0, s>>>(w.dh, d, w.dphi);
     k_flow_time_bwd<<<dim3(S, dm / 128), 256, (dm + 16 * 128) * sizeof(float), s>>>(
         g->sample_slot, fs, d, fh->t2, w.z1, w.dphi, w.dz1);
-    k_flow_outer<true><<<dim3(nsl, dm), 256, 0, s>>>(w.dphi, w.z1, fs, d, gr->t2, gr->tb2, add);
-    k_flow_outer<false><<<dim3(nsl, dm), 256, 0, s>>>(w.dz1, w.sfeat, fs, d, gr->t1, gr->tb1, add);
+    k_flow_outer<true><<<dim3(nsl, dm / kOuterRows), 256, 0, s>>>(w.dphi, w.z1, fs, d, gr->t2, gr->tb2, add);
+    k_flow_outer<false><<<dim3(nsl, dm / kOuterRows), 256, 0, s>>>(w.dz1, w.sfeat, fs, d, gr->t1, gr->tb1, add);
     return last("flow embedding backward");
 }

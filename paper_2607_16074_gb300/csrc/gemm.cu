@@ -689,7 +689,9 @@ __device__ __forceinline__ void lora_part(const LoraGemm& lg, int c, int& part, 
     c0 = c;
 }
 
-template <int EPI, bool LORA, int EW, int BN>
+// BMN: B is MN-major, [K rows, N] as it lies (segmented launches: a tenant's K
+// rows), for the gradient through a projection.
+template <int EPI, bool LORA, int EW, int BN, bool BMN>
 __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
     k_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
            const __grid_constant__ typename std::conditional<LORA, LoraGemm, NoLora>::type lg,
@@ -698,7 +700,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
     using gemm::BK;
     using gemm::BM;
     constexpr bool WIDE = BN == 256;
-    constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
+    constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN) | (BMN ? 1u << 16 : 0u);
+    static_assert(!BMN || EPI == EPI_F32 || EPI == EPI_GLU_BWD, "contiguous tile columns");
     constexpr int LT_BYTES = gemm::LT_BYTES, LSTAGE = LT_BYTES + BN * 32;
     constexpr int RING = WIDE ? gemm::STAGES : gemm::RING_MAX;  // barriers per direction
     constexpr uint32_t TMEM_COLS = 2 * BN;
@@ -776,7 +779,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
             const TileGeo g = tile_geo<EPI, LORA, BN>(tile, num_m, num_n, p, lg);
             int brow = 0;
             if constexpr (LORA)
-                if (lg.seg_b) brow = lg.seg_tenant[g.seg] * p.N;
+                if (lg.seg_b) brow = lg.seg_tenant[g.seg] * (BMN ? p.K : p.N);
             for (int kb = 0; kb < num_k; ++kb) {
                 if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
                     ok = false;
@@ -786,10 +789,17 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
                     uint8_t* sa = smem + stage * stage_bytes;
                     mbar_arrive_expect_tx(&full[stage], stage_bytes);
                     tma_load_2d(sa, &ta, kb * BK, g.row0, &full[stage]);
-                    tma_load_2d(sa + a_bytes, &tb, kb * BK, brow + g.c0, &full[stage]);
-                    if constexpr (!WIDE)
-                        tma_load_2d(sa + a_bytes + BN / 2 * BK * 2, &tb, kb * BK, brow + g.c1,
-                                    &full[stage]);
+                    if constexpr (BMN) {
+#pragma unroll
+                        for (int i = 0; i < BN / 64; ++i)
+                            tma_load_2d(sa + a_bytes + i * 64 * BK * 2, &tb, g.c0 + 64 * i,
+                                        brow + kb * BK, &full[stage]);
+                    } else {
+                        tma_load_2d(sa + a_bytes, &tb, kb * BK, brow + g.c0, &full[stage]);
+                        if constexpr (!WIDE)
+                            tma_load_2d(sa + a_bytes + BN / 2 * BK * 2, &tb, kb * BK, brow + g.c1,
+                                        &full[stage]);
+                    }
                 }
                 __syncwarp();
                 ++issued;
@@ -856,10 +866,15 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
                 const uint32_t off = (uint32_t)(stage * stage_bytes) >> 4;
                 if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk)
-                        tc_mma_f16(d, desc_of(a_lo + off + 2 * kk, kSw128DescHi),
-                                   desc_of(b_lo + off + 2 * kk, kSw128DescHi), IDESC,
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        uint64_t db = desc_of(b_lo + off + 2 * kk, kSw128DescHi);
+                        if constexpr (BMN)  // 16 K rows are two 8-row atoms
+                            db = sw128_desc_mn(
+                                smem_u32(smem) + stage * stage_bytes + a_bytes + kk * 2048,
+                                64 * BK * 2, 1024);
+                        tc_mma_f16(d, desc_of(a_lo + off + 2 * kk, kSw128DescHi), db, IDESC,
                                    (kb | kk) != 0);
+                    }
                     tc_commit(&empty[stage]);
                 }
                 __syncwarp();
@@ -1451,16 +1466,16 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
 // Width of a launch's output tiles: the one with the least estimated time,
 // (tiles an SM works through) x (its time per 64-deep K step).  The step times
 // are GB300's in microseconds, from launches of 8 to 10,000 tiles (K = 2,048 to
-// 16,384): a tile alone on its SM, and two narrow tiles sharing one, which is
-// how a narrow launch of more tiles than SMs runs.  A 256-wide tile is the
-// fastest per column, so narrower ones win only where it leaves SMs idle:
-// 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide tiles, 59 in 80 of 128
-// and 76 in 160 of 64; 300 rows 94, 57 and 47; 4,800 rows 190, 235 and 351.
-// A pair's tile (plain launches only) takes 0.33 for the same work per SM as
-// a wide one's 0.385, so it wins wherever its tiles divide as well over the
-// SMs: 2,400 rows x N 32,768 177 us against 188, but x N 2,048 33 against 23.
-// RoPE needs a tile within one head, a folded norm's sums of squares one of 128
-// columns; the GLU backward with dm has wide tiles only.
+// 16,384): `alone` where every tile has an SM of its own, `two` for a round of
+// two narrow tiles sharing one, which is how a narrow launch of more tiles than
+// SMs runs.  A 256-wide tile is faster per column, so narrower ones win only
+// where it leaves SMs idle: 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide
+// tiles, 59 in 80 of 128 and 76 in 160 of 64; 300 rows 94, 57 and 47; 4,800 rows
+// 190, 235 and 351.  A pair's tile (plain launches only) takes 0.32 for the same
+// work per SM as a wide one's 0.355 (0.385 alone), so it wins wherever its tiles
+// divide as well over the SMs: 2,400 rows x N 32,768 177 us against 188, but x N
+// 2,048 33 against 23.  RoPE needs a tile within one head, a folded norm's sums of
+// squares one of 128 columns; the GLU backward with dm has wide tiles only.
 constexpr int kPairTile = 512;
 
 static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
@@ -1468,18 +1483,17 @@ static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
     auto rounds = [](long long tiles, int slots) { return (double)((tiles + slots - 1) / slots); };
     const long long wide = (long long)m_tiles * (p.N / 256);
     int best = 256;
-    double least = rounds(wide, sms) * 0.385;
+    double least = wide <= sms ? 0.385 : rounds(wide, sms) * 0.355;
     if (pairs) {
-        const double t =
-            rounds((long long)((m_tiles + 1) / 2) * (p.N / 256), sms / 2) * 0.33;
+        const double t = rounds((long long)((m_tiles + 1) / 2) * (p.N / 256), sms / 2) * 0.32;
         if (t < least) {
             best = kPairTile;
             least = t;
         }
     }
     if (p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn)) return best;
-    static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.225, 0.38},
-                                                                     {64, 0.18, 0.33}};
+    static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.225, 0.40},
+                                                                     {64, 0.18, 0.335}};
     for (const auto& w : kNarrow) {
         if ((p.epi == EPI_ROPE && w.bn > p.hd) || (p.norm_gamma && w.bn < 128)) continue;
         const long long tiles = (long long)m_tiles * (p.N / w.bn);
@@ -1500,7 +1514,7 @@ static void narrow_ring(GemmParams& p, int bn, long long tiles, bool lora) {
     while (p.stages > 2 && gemm::narrow_smem(bn, p.stages, p.a_rows, lora) > budget) --p.stages;
 }
 
-template <int EPI, bool LORA, class LG, int EW, int BN>
+template <int EPI, bool LORA, class LG, int EW, int BN, bool BMN>
 static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
                              GemmParams p, long long tiles, cudaStream_t s) {
     static_assert(EW == 4 || (EW == 8 && !LORA && BN == 256 &&
@@ -1516,9 +1530,9 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const
     const int grid = (int)std::min<long long>(tiles, (long long)num_sms() * per_sm);
     static std::atomic<uint64_t> attr{0};  // per instantiation, one bit per device
     cudaError_t e =
-        set_smem_limit(reinterpret_cast<const void*>(k_gemm<EPI, LORA, EW, BN>), limit, attr);
+        set_smem_limit(reinterpret_cast<const void*>(k_gemm<EPI, LORA, EW, BN, BMN>), limit, attr);
     if (e != cudaSuccess) return e;
-    k_gemm<EPI, LORA, EW, BN><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, lg, p);
+    k_gemm<EPI, LORA, EW, BN, BMN><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, lg, p);
     return cudaGetLastError();
 }
 
@@ -1538,16 +1552,16 @@ static cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, Gem
 }
 
 // The launch of one epilogue at the tile width bn (kPairTile: a CTA pair's).
-template <int EPI, bool LORA, class LG, int EW = 4>
+template <int EPI, bool LORA, class LG, int EW = 4, bool BMN = false>
 static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
                               const GemmParams& p, int bn, long long tiles, cudaStream_t s) {
     if constexpr (!LORA)
         if (bn == kPairTile) return launch_pair<EPI, EW>(ta, tb, p, s);
     if constexpr (EW == 4) {
-        if (bn == 64) return launch_bn<EPI, LORA, LG, EW, 64>(ta, tb, lg, p, tiles, s);
-        if (bn == 128) return launch_bn<EPI, LORA, LG, EW, 128>(ta, tb, lg, p, tiles, s);
+        if (bn == 64) return launch_bn<EPI, LORA, LG, EW, 64, BMN>(ta, tb, lg, p, tiles, s);
+        if (bn == 128) return launch_bn<EPI, LORA, LG, EW, 128, BMN>(ta, tb, lg, p, tiles, s);
     }
-    return launch_bn<EPI, LORA, LG, EW, 256>(ta, tb, lg, p, tiles, s);
+    return launch_bn<EPI, LORA, LG, EW, 256, BMN>(ta, tb, lg, p, tiles, s);
 }
 
 // Box rows of the two operands' tensor maps at tile width bn.
@@ -1618,7 +1632,7 @@ jnx_status gemm_launch(const uint16_t* A, int lda, const uint16_t* B, int ldb, G
 
 jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ldb, int n_tenants,
                            GemmParams p, int n_seg, const int* seg_r0, const int* seg_r1,
-                           const int* seg_tenant, cudaStream_t s) {
+                           const int* seg_tenant, cudaStream_t s, bool b_mn) {
     jnx_status st = gemm_check(p.M, p.N, p.K);
     if (st != JNX_OK) return st;
     if (n_seg < 0 || n_seg > kLoraMaxSlots || n_tenants <= 0)
@@ -1648,18 +1662,28 @@ jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ld
     p.a_rows = a_box(bn, most);
     CUtensorMap ta, tb;
     if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) ||
-        !make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.N, p.K, ldb, b_box(bn), gemm::BK))
+        !(b_mn ? make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.K, p.N, ldb, gemm::BK, 64)
+               : make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.N, p.K, ldb, b_box(bn), gemm::BK)))
         return fail(JNX_ERR_CUDA, "gemm: tensor map encode failed (alignment or driver)");
     const long long total = (long long)tiles * (p.N / bn);
     if (p.group_m <= 0) p.group_m = default_group_m(p.K);
     cudaError_t e;
+    if (b_mn) {
+        if (p.epi == EPI_F32)
+            e = launch_epi<EPI_F32, true, LoraGemm, 4, true>(ta, tb, lg, p, bn, total, s);
+        else if (p.epi == EPI_GLU_BWD)
+            e = launch_epi<EPI_GLU_BWD, true, LoraGemm, 4, true>(ta, tb, lg, p, bn, total, s);
+        else
+            return fail(JNX_ERR_INVALID_ARG, "gemm: epilogue %d unsupported here", p.epi);
+        if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
+        return JNX_OK;
+    }
     switch (p.epi) {
         case EPI_BF16: e = launch_epi<EPI_BF16, true>(ta, tb, lg, p, bn, total, s); break;
         case EPI_F32: e = launch_epi<EPI_F32, true>(ta, tb, lg, p, bn, total, s); break;
         case EPI_RESID: e = launch_epi<EPI_RESID, true>(ta, tb, lg, p, bn, total, s); break;
         case EPI_GLU: e = launch_epi<EPI_GLU, true>(ta, tb, lg, p, bn, total, s); break;
         case EPI_GLU_SAVE: e = launch_epi<EPI_GLU_SAVE, true>(ta, tb, lg, p, bn, total, s); break;
-        case EPI_GLU_BWD: e = launch_epi<EPI_GLU_BWD, true>(ta, tb, lg, p, bn, total, s); break;
         default: return fail(JNX_ERR_INVALID_ARG, "gemm: epilogue %d unsupported here", p.epi);
     }
     if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
