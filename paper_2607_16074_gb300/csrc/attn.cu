@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(HD == 256 ? 384 : 640, 1)
         fence_barrier_init();
         fence_proxy_async();
     }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
     if (warp == 2) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
@@ -655,7 +656,7 @@ static jnx_status launch_attn_ws(const uint16_t* qkv, int ldq, int n_tokens, int
     if (n_work == 0) return JNX_OK;
     const int grid = std::min((n_work + C::NST - 1) / C::NST, num_sms());
     const float scale_log2 = (float)(1.4426950408889634 / sqrt((double)HD));
-    k_attn_ws<HD, BN><<<grid, C::THREADS, C::SMEM, s>>>(tq, tkv, cu, it, H, Hkv, scale_log2, out, ldo,
+    pdl(k_attn_ws<HD, BN>, grid, C::THREADS, C::SMEM, s)(tq, tkv, cu, it, H, Hkv, scale_log2, out, ldo,
                                                  lse, status);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "attention: %s", cudaGetErrorString(e));

@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(192, 1)
         fence_barrier_init();
         fence_proxy_async();
     }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
@@ -578,7 +579,7 @@ static jnx_status launch_bwd(const CUtensorMap (&maps)[4], const int* cu, const 
     const int grid = (int)std::min<long long>(n_work, num_sms());
     const float scale_log2 = (float)(1.4426950408889634 / sqrt((double)HD));
     const float scale = (float)(1.0 / sqrt((double)HD));
-    k_attn_bwd<HD, MODE><<<grid, 192, C::SMEM, s>>>(maps[0], maps[1], maps[2], maps[3], cu, it, H,
+    pdl(k_attn_bwd<HD, MODE>, grid, 192, C::SMEM, s)(maps[0], maps[1], maps[2], maps[3], cu, it, H,
                                                    Hkv, scale_log2, scale, lse, D, pos, rope,
                                                    rope_ld, dqkv, ldq, status);
     cudaError_t e = cudaGetLastError();

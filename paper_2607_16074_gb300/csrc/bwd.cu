@@ -24,6 +24,7 @@
 
 #include "jnx_bwd.h"
 #include "jnx_dev.cuh"
+#include "jnx_kernels.h"
 
 namespace jnx {
 
@@ -35,6 +36,7 @@ namespace jnx {
 // aligned (vec), element by element at the edges and otherwise.
 __global__ void __launch_bounds__(256) k_transpose(const uint16_t* __restrict__ src, int rows,
                                                    int cols, uint16_t* __restrict__ dst, int vec) {
+    pdl_entry();
     __shared__ uint16_t tile[64][64 + 2];
     const size_t plane = (size_t)rows * cols;
     src += (size_t)blockIdx.z * plane;
@@ -83,7 +85,7 @@ jnx_status transpose_launch(const uint16_t* src, int batch, int rows, int cols, 
     if ((rows + 63) / 64 > 65535 || batch > 65535)
         return fail(JNX_ERR_UNSUPPORTED, "transpose: too many rows or planes");
     const int vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
-    k_transpose<<<dim3((cols + 63) / 64, (rows + 63) / 64, batch), 256, 0, s>>>(src, rows, cols,
+    pdl(k_transpose, dim3((cols + 63) / 64, (rows + 63) / 64, batch), 256, 0, s)(src, rows, cols,
                                                                              dst, vec);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "transpose: %s", cudaGetErrorString(e));
@@ -99,6 +101,7 @@ __global__ void __launch_bounds__(256) k_rms_bwd(const float* __restrict__ x,
                                                  const uint16_t* __restrict__ gamma, float eps,
                                                  const float* __restrict__ dn, const float* dres,
                                                  int M, int d, float* dx, uint16_t* dx_bf) {
+    pdl_entry();
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (row >= M) return;
     const float* xr = x + (size_t)row * d;
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(256) k_rms_bwd_row(const float* __restrict__ x
                                                      const uint16_t* __restrict__ gamma, float eps,
                                                      const float* __restrict__ dn, const float* dres,
                                                      int d, float* dx, uint16_t* dx_bf) {
+    pdl_entry();
     __shared__ float red[2][8];
     const size_t row = blockIdx.x;
     const int units = d / 4, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -209,13 +213,13 @@ jnx_status rms_bwd_launch(const float* x, const uint16_t* gamma, float eps, cons
     if (M <= 0) return JNX_OK;
     if (d >= 1024 && d <= 4096) {
         if (d <= 1024)
-            k_rms_bwd_row<1><<<M, 256, 0, s>>>(x, gamma, eps, dn, dres, d, dx, dx_bf);
+            pdl(k_rms_bwd_row<1>, M, 256, 0, s)(x, gamma, eps, dn, dres, d, dx, dx_bf);
         else if (d <= 2048)
-            k_rms_bwd_row<2><<<M, 256, 0, s>>>(x, gamma, eps, dn, dres, d, dx, dx_bf);
+            pdl(k_rms_bwd_row<2>, M, 256, 0, s)(x, gamma, eps, dn, dres, d, dx, dx_bf);
         else
-            k_rms_bwd_row<4><<<M, 256, 0, s>>>(x, gamma, eps, dn, dres, d, dx, dx_bf);
+            pdl(k_rms_bwd_row<4>, M, 256, 0, s)(x, gamma, eps, dn, dres, d, dx, dx_bf);
     } else {
-        k_rms_bwd<<<(M + 7) / 8, 256, 0, s>>>(x, gamma, eps, dn, dres, M, d, dx, dx_bf);
+        pdl(k_rms_bwd, (M + 7) / 8, 256, 0, s)(x, gamma, eps, dn, dres, M, d, dx, dx_bf);
     }
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "rms backward: %s", cudaGetErrorString(e));
@@ -230,6 +234,7 @@ __global__ void __launch_bounds__(256) k_attn_bwd_prep(const float* __restrict__
                                                        const uint16_t* __restrict__ att, int M,
                                                        int H, int hd, uint16_t* __restrict__ dO,
                                                        float* __restrict__ D) {
+    pdl_entry();
     const long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (w >= (long long)M * H) return;
@@ -254,7 +259,7 @@ jnx_status attn_bwd_prep_launch(const float* datt, const uint16_t* att, int M, i
     if (hd % 128 && hd != 64) return fail(JNX_ERR_UNSUPPORTED, "attention prep: head dim");
     if (M <= 0) return JNX_OK;
     const long long warps = (long long)M * H;
-    k_attn_bwd_prep<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(datt, att, M, H, hd, dO, D);
+    pdl(k_attn_bwd_prep, (unsigned)((warps + 7) / 8), 256, 0, s)(datt, att, M, H, hd, dO, D);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK
                             : fail(JNX_ERR_CUDA, "attention prep: %s", cudaGetErrorString(e));
@@ -278,6 +283,7 @@ template <bool ADD>
 __global__ void __launch_bounds__(128) k_seg_up(const __grid_constant__ SegRows sr,
                                                 const __grid_constant__ SegUpParts sp, int ncols,
                                                 float* __restrict__ out, int ldo) {
+    pdl_entry();
     using namespace seg;
     __shared__ __align__(128) uint8_t sT[2][UP_BM * 32];
     __shared__ __align__(128) uint8_t sW[2][UP_BK * 256];
@@ -380,6 +386,7 @@ __global__ void __launch_bounds__(128) k_seg_tn(const __grid_constant__ SegChunk
                                                 const uint16_t* __restrict__ U, int ldu,
                                                 const uint16_t* __restrict__ V, int ldv, int n,
                                                 float* __restrict__ part) {
+    pdl_entry();
     using namespace seg;
     __shared__ __align__(128) uint8_t sU[2][TN_ROWS * 32];
     __shared__ __align__(128) uint8_t sV[2][TN_ROWS * 512];
@@ -453,6 +460,7 @@ __global__ void __launch_bounds__(256) k_seg_reduce(const __grid_constant__ SegC
                                                     const float* __restrict__ part, int n,
                                                     float* __restrict__ grad, long long gstride,
                                                     int add) {
+    pdl_entry();
     const int slot = blockIdx.y;
     const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
     if (e >= 16LL * n) return;
@@ -500,9 +508,9 @@ jnx_status seg_up_launch(const jnx_group* g, const SegUpParts& sp, int ncols, fl
     if (tiles == 0) return JNX_OK;
     const dim3 grid(tiles, ncols / seg::UP_BN);
     if (add)
-        k_seg_up<true><<<grid, 128, 0, s>>>(sr, sp, ncols, out, ldo);
+        pdl(k_seg_up<true>, grid, 128, 0, s)(sr, sp, ncols, out, ldo);
     else
-        k_seg_up<false><<<grid, 128, 0, s>>>(sr, sp, ncols, out, ldo);
+        pdl(k_seg_up<false>, grid, 128, 0, s)(sr, sp, ncols, out, ldo);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK
                             : fail(JNX_ERR_CUDA, "segmented up-projection: %s", cudaGetErrorString(e));
@@ -543,13 +551,13 @@ jnx_status seg_tn_launch(const jnx_group* g, const uint16_t* U, int ldu, const u
     ch.slot_chunk0[g->n_slots] = nc;
     if ((size_t)nc * 16 * n > part_floats)
         return fail(JNX_ERR_WORKSPACE, "adapter gradient: partial buffer too small");
-    if (nc > 0) k_seg_tn<<<dim3(nc, n / seg::TN_BN), 128, 0, s>>>(ch, U, ldu, V, ldv, n, part);
+    if (nc > 0) pdl(k_seg_tn, dim3(nc, n / seg::TN_BN), 128, 0, s)(ch, U, ldu, V, ldv, n, part);
     if (g->n_slots > 0) {
         const dim3 grid((unsigned)((16LL * n + 255) / 256), g->n_slots);
         if (trans)
-            k_seg_reduce<true><<<grid, 256, 0, s>>>(ch, part, n, grad, gstride, add ? 1 : 0);
+            pdl(k_seg_reduce<true>, grid, 256, 0, s)(ch, part, n, grad, gstride, add ? 1 : 0);
         else
-            k_seg_reduce<false><<<grid, 256, 0, s>>>(ch, part, n, grad, gstride, add ? 1 : 0);
+            pdl(k_seg_reduce<false>, grid, 256, 0, s)(ch, part, n, grad, gstride, add ? 1 : 0);
     }
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK
@@ -573,6 +581,7 @@ __global__ void __launch_bounds__(128) k_seg_wgrad(const __grid_constant__ SegRo
                                                    const uint16_t* __restrict__ V, int ldv,
                                                    int m, int n, float* __restrict__ grad,
                                                    long long gstride, int add) {
+    pdl_entry();
     using namespace seg;
     __shared__ __align__(128) uint8_t sU[2][WG_ROWS * 128];
     __shared__ __align__(128) uint8_t sV[2][WG_ROWS * 256];
@@ -667,7 +676,7 @@ jnx_status seg_wgrad_launch(const SegRows& sr, const uint16_t* U, int ldu, const
     if (sr.n <= 0) return JNX_OK;
     if (m / seg::WG_BM > 65535 || sr.n > 65535)
         return fail(JNX_ERR_UNSUPPORTED, "weight gradient: grid too large");
-    k_seg_wgrad<<<dim3(n / seg::WG_BN, m / seg::WG_BM, sr.n), 128, 0, s>>>(sr, U, ldu, V, ldv, m,
+    pdl(k_seg_wgrad, dim3(n / seg::WG_BN, m / seg::WG_BM, sr.n), 128, 0, s)(sr, U, ldu, V, ldv, m,
                                                                           n, grad, gstride,
                                                                           add ? 1 : 0);
     cudaError_t e = cudaGetLastError();
@@ -684,6 +693,7 @@ __global__ void __launch_bounds__(256) k_mlp_dfeat(const float* __restrict__ dz,
                                                    const int* __restrict__ sample_slot,
                                                    const __grid_constant__ MlpFeatTable tab, int d,
                                                    float* __restrict__ dh) {
+    pdl_entry();
     const int s = blockIdx.x;
     const int c = blockIdx.y * 256 + threadIdx.x;
     const int slot = sample_slot[s];
@@ -701,7 +711,7 @@ jnx_status mlp_dfeat_launch(const float* dz, int ldz, const int* cu, const int* 
                             int n_samples, const MlpFeatTable& tab, int d, float* dh,
                             cudaStream_t s) {
     if (n_samples <= 0) return JNX_OK;
-    k_mlp_dfeat<<<dim3(n_samples, (d + 255) / 256), 256, 0, s>>>(dz, ldz, cu, sample_slot, tab, d,
+    pdl(k_mlp_dfeat, dim3(n_samples, (d + 255) / 256), 256, 0, s)(dz, ldz, cu, sample_slot, tab, d,
                                                                 dh);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK

@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(256) k_flow_time1(const float* __restrict__ ta
                                                     const uint16_t* __restrict__ tb1,
                                                     float* __restrict__ sfeat,
                                                     float* __restrict__ z1) {
+    pdl_entry();
     extern __shared__ float sh[];  // s(tau) [dm]
     const int s = blockIdx.x, dm = dd.dm, half = dm / 2;
     const int t = fs.tenant[sample_slot[s]];
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(256) k_flow_time2(const int* __restrict__ samp
                                                     const uint16_t* __restrict__ tb2,
                                                     const float* __restrict__ z1,
                                                     float* __restrict__ phi) {
+    pdl_entry();
     extern __shared__ float sh[];  // SiLU(z1) [dm]
     const int s = blockIdx.x, dm = dd.dm;
     const int t = fs.tenant[sample_slot[s]];
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(256) k_flow_embed(
     const uint16_t* __restrict__ w_in, const uint16_t* __restrict__ b_in,
     const uint16_t* __restrict__ pos, const float* __restrict__ phi, float* __restrict__ x_out,
     float* __restrict__ u_out, float* __restrict__ h) {
+    pdl_entry();
     __shared__ float xs[kMaxD];
     const int r = blockIdx.x, C = dd.C, D = dd.D, dm = dd.dm;
     const int s = r / C, c = r % C;
@@ -287,6 +290,7 @@ __global__ void __launch_bounds__(128) k_flow_attn_fwd(const uint16_t* __restric
                                                        const int* __restrict__ cu, FlowDims dd,
                                                        uint16_t* __restrict__ o,
                                                        float* __restrict__ lse) {
+    pdl_entry();
     constexpr int NK = kKT / KS, NT = NK / 8;
     __shared__ __align__(128) uint8_t sbuf[4 * kTileB];  // (K, V) x 2 buffers
     const int s = blockIdx.x, h = blockIdx.y, C = dd.C, dm = dd.dm;
@@ -484,6 +488,7 @@ __global__ void __launch_bounds__(128) k_flow_attn_bwd_q(
     const uint16_t* __restrict__ qkv, const uint16_t* __restrict__ kvc, const int* __restrict__ cu,
     FlowDims dd, const uint16_t* __restrict__ o, const float* __restrict__ dO,
     const float* __restrict__ lse, uint16_t* __restrict__ dqkv) {
+    pdl_entry();
     constexpr int NK = kKT / KS, NT = NK / 8;
     __shared__ __align__(128) uint8_t sbuf[4 * kTileB];
     __shared__ float sD[kMaxC], sL[kMaxC];
@@ -621,6 +626,7 @@ __global__ void __launch_bounds__(128) k_flow_attn_bwd_kv(
     const uint16_t* __restrict__ qkv, const uint16_t* __restrict__ kvc, const int* __restrict__ cu,
     FlowDims dd, const uint16_t* __restrict__ o, const float* __restrict__ dO,
     const float* __restrict__ lse, uint16_t* __restrict__ dqkv, uint16_t* __restrict__ dkvc) {
+    pdl_entry();
     constexpr int NT = 2 * NQ;  // n8 query tiles
     __shared__ __align__(128) uint8_t sbuf[4 * kTileB];  // q, dO, K, V
     __shared__ float sD[kMaxC], sL[kMaxC];
@@ -723,6 +729,7 @@ __global__ void __launch_bounds__(256) k_flow_out(const uint16_t* __restrict__ n
                                                   const uint16_t* __restrict__ b_out,
                                                   const float* __restrict__ u,
                                                   float* __restrict__ v, float* __restrict__ dv) {
+    pdl_entry();
     const int r = blockIdx.x, lane = threadIdx.x & 31;
     const int dm = dd.dm, D = dd.D, C = dd.C;
     const int k = blockIdx.y * 8 + (threadIdx.x >> 5);
@@ -764,6 +771,7 @@ __global__ void __launch_bounds__(256) k_flow_loss(const __grid_constant__ FlowS
                                                    FlowDims dd, const float* __restrict__ v,
                                                    const float* __restrict__ u,
                                                    float* __restrict__ loss) {
+    pdl_entry();
     __shared__ float red[8];
     const int i = blockIdx.x;
     const size_t e0 = (size_t)fs.s0[i] * dd.C * dd.D, e1 = (size_t)fs.s1[i] * dd.C * dd.D;
@@ -785,6 +793,7 @@ __global__ void __launch_bounds__(256) k_flow_loss(const __grid_constant__ FlowS
 
 // Euler step of the sampler: x += dt v.
 __global__ void k_flow_euler(float* __restrict__ x, const float* __restrict__ v, float dt, int n) {
+    pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) x[i] += dt * v[i];
 }
@@ -799,6 +808,7 @@ __global__ void __launch_bounds__(256) k_flow_out_bwd(const float* __restrict__ 
                                                       FlowDims dd,
                                                       const uint16_t* __restrict__ w_out,
                                                       float* __restrict__ dnf) {
+    pdl_entry();
     const int r = blockIdx.x, dm = dd.dm, D = dd.D;
     const int t = fs.tenant[sample_slot[r / dd.C]];
     __shared__ float g[kMaxD];
@@ -842,6 +852,7 @@ __global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* __restrict_
                                                         const __grid_constant__ FlowSlots fs,
                                                         FlowDims dd, float* __restrict__ gw,
                                                         float* __restrict__ gb, int add) {
+    pdl_entry();
     const int i = blockIdx.x, k = blockIdx.y, dm = dd.dm, D = dd.D, C = dd.C;
     const int t = fs.tenant[i];
     const int r0 = fs.s0[i] * C, r1 = fs.s1[i] * C;
@@ -881,6 +892,7 @@ __global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* __restric
                                                           FlowDims dd, float* __restrict__ gw,
                                                           float* __restrict__ gb,
                                                           float* __restrict__ gpos, int add) {
+    pdl_entry();
     const int i = blockIdx.x, dm = dd.dm, D = dd.D, C = dd.C;
     const int warp = threadIdx.x >> 5, j = blockIdx.y * 32 + (threadIdx.x & 31);
     const int t = fs.tenant[i], k0 = 8 * warp;
@@ -916,6 +928,7 @@ __global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* __restric
 // action row of the sample), c in order.
 __global__ void __launch_bounds__(256) k_flow_dphi(const float* __restrict__ dh, FlowDims dd,
                                                    float* __restrict__ dphi) {
+    pdl_entry();
     const int s = blockIdx.x, dm = dd.dm, C = dd.C;
     const int j = blockIdx.y * blockDim.x + threadIdx.x;
     if (j >= dm) return;
@@ -933,6 +946,7 @@ __global__ void __launch_bounds__(256) k_flow_time_bwd(const int* __restrict__ s
                                                        const float* __restrict__ z1,
                                                        const float* __restrict__ dphi,
                                                        float* __restrict__ dz1) {
+    pdl_entry();
     extern __shared__ float sh[];  // dphi [dm], then partials [16][128]
     const int s = blockIdx.x, dm = dd.dm, k0 = blockIdx.y * 128;
     const int t = fs.tenant[sample_slot[s]];
@@ -979,6 +993,7 @@ __global__ void __launch_bounds__(256) k_flow_outer(const float* __restrict__ A,
                                                     const __grid_constant__ FlowSlots fs,
                                                     FlowDims dd, float* __restrict__ gw,
                                                     float* __restrict__ gb, int add) {
+    pdl_entry();
     const int i = blockIdx.x, j0 = blockIdx.y * kOuterRows, dm = dd.dm;
     const int t = fs.tenant[i];
     for (int k = 4 * threadIdx.x; k < dm; k += 4 * 256) {
@@ -1102,11 +1117,11 @@ jnx_status flow_attn_fwd_launch(const uint16_t* qkv, const uint16_t* kvc, const 
     const int MT = (d.C + 15) / 16;
     const dim3 grid(S, d.nh);
     if (MT == 1)
-        k_flow_attn_fwd<4><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, lse);
+        pdl(k_flow_attn_fwd<4>, grid, 128, 0, s)(qkv, kvc, cu, d, o, lse);
     else if (MT == 2)
-        k_flow_attn_fwd<2><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, lse);
+        pdl(k_flow_attn_fwd<2>, grid, 128, 0, s)(qkv, kvc, cu, d, o, lse);
     else
-        k_flow_attn_fwd<1><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, lse);
+        pdl(k_flow_attn_fwd<1>, grid, 128, 0, s)(qkv, kvc, cu, d, o, lse);
     return last("flow attention");
 }
 
@@ -1114,7 +1129,7 @@ template <int NQ>
 void launch_bwd_kv(dim3 grid, const uint16_t* qkv, const uint16_t* kvc, const int* cu,
                    const FlowDims& d, const uint16_t* o, const float* dO, const float* lse,
                    uint16_t* dqkv, uint16_t* dkvc, cudaStream_t s) {
-    k_flow_attn_bwd_kv<NQ><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, dO, lse, dqkv, dkvc);
+    pdl(k_flow_attn_bwd_kv<NQ>, grid, 128, 0, s)(qkv, kvc, cu, d, o, dO, lse, dqkv, dkvc);
 }
 
 // dq (query side), then dk / dv (key side: one CTA per sample, head and
@@ -1129,11 +1144,11 @@ jnx_status flow_attn_bwd_launch(const uint16_t* qkv, const uint16_t* kvc, const 
     const int* cu = g->cu_seqlens;
     const dim3 grid(S, d.nh);
     if (MT == 1)
-        k_flow_attn_bwd_q<4><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, dO, lse, dqkv);
+        pdl(k_flow_attn_bwd_q<4>, grid, 128, 0, s)(qkv, kvc, cu, d, o, dO, lse, dqkv);
     else if (MT == 2)
-        k_flow_attn_bwd_q<2><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, dO, lse, dqkv);
+        pdl(k_flow_attn_bwd_q<2>, grid, 128, 0, s)(qkv, kvc, cu, d, o, dO, lse, dqkv);
     else
-        k_flow_attn_bwd_q<1><<<grid, 128, 0, s>>>(qkv, kvc, cu, d, o, dO, lse, dqkv);
+        pdl(k_flow_attn_bwd_q<1>, grid, 128, 0, s)(qkv, kvc, cu, d, o, dO, lse, dqkv);
     int tiles = 1;
     for (int i = 0; i < S; ++i)
         tiles = std::max(tiles, (g->h_cu_seqlens[i + 1] - g->h_cu_seqlens[i] + d.C + kKT - 1) / kKT);
@@ -1213,11 +1228,13 @@ Segs make_segs(const jnx_group* g, int C) {
 }
 
 __global__ void k_fill_bf16(uint16_t* p, int n, uint16_t v) {
+    pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) p[i] = v;
 }
 
 __global__ void k_fill_f32(float* p, int n, float v) {
+    pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) p[i] = v;
 }
@@ -1339,11 +1356,11 @@ jnx_status flow_network(const jnx_flow_head* fh, const FlowDims& d, const jnx_gr
         cudaSuccess)
         return last("flow: copy");
     if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, w.nf, s))) return st;
-    k_flow_out<<<dim3(Ma, (d.D + 7) / 8), 256, 0, s>>>(w.nf, g->sample_slot, fs, d, fh->w_out,
+    pdl(k_flow_out, dim3(Ma, (d.D + 7) / 8), 256, 0, s)(w.nf, g->sample_slot, fs, d, fh->w_out,
                                                        fh->b_out, train ? w.u : nullptr, w.v, w.dv);
     if ((st = last("flow output"))) return st;
     if (train && loss) {
-        k_flow_loss<<<nsl, 256, 0, s>>>(fs, d, w.v, w.u, loss);
+        pdl(k_flow_loss, nsl, 256, 0, s)(fs, d, w.v, w.u, loss);
         if ((st = last("flow loss"))) return st;
     }
     return JNX_OK;
@@ -1418,13 +1435,13 @@ static jnx_status flow_embed(const jnx_flow_head* fh, const FlowDims& d, const j
                              cudaStream_t s) {
     const int S = g->n_samples, Ma = S * d.C;
     TraceScope ts(JNX_K_FLOW_MISC, (double)S * d.dm * d.dm * 4.0, s);
-    k_fill_bf16<<<(d.dm + 255) / 256, 256, 0, s>>>(w.ones, d.dm, (uint16_t)0x3F80);
+    pdl(k_fill_bf16, (d.dm + 255) / 256, 256, 0, s)(w.ones, d.dm, (uint16_t)0x3F80);
     const dim3 tg(S, d.dm / kTimeRows);
-    k_flow_time1<<<tg, 256, d.dm * sizeof(float), s>>>(tau, g->sample_slot, fs, d, fh->t1, fh->tb1,
+    pdl(k_flow_time1, tg, 256, d.dm * sizeof(float), s)(tau, g->sample_slot, fs, d, fh->t1, fh->tb1,
                                                        w.sfeat, w.z1);
-    k_flow_time2<<<tg, 256, d.dm * sizeof(float), s>>>(g->sample_slot, fs, d, fh->t2, fh->tb2,
+    pdl(k_flow_time2, tg, 256, d.dm * sizeof(float), s)(g->sample_slot, fs, d, fh->t2, fh->tb2,
                                                        w.z1, w.phi);
-    k_flow_embed<<<Ma, 256, 0, s>>>(actions, noise, tau, xin, g->sample_slot, fs, d, fh->w_in,
+    pdl(k_flow_embed, Ma, 256, 0, s)(actions, noise, tau, xin, g->sample_slot, fs, d, fh->w_in,
                                     fh->b_in, fh->pos, w.phi, w.x, w.u, w.h);
     return last("flow embedding");
 }
@@ -1475,11 +1492,11 @@ extern "C" jnx_status jnx_flow_sample(const jnx_flow_head* fh, const jnx_group* 
         return last("flow: copy");
     // tau of step i for every sample, in the u buffer (no target when sampling)
     for (int i = 0; i < n_steps; ++i) {
-        k_fill_f32<<<(g->n_samples + 255) / 256, 256, 0, s>>>(w.u, g->n_samples,
+        pdl(k_fill_f32, (g->n_samples + 255) / 256, 256, 0, s)(w.u, g->n_samples,
                                                              (float)i / (float)n_steps);
         if ((st = flow_embed(fh, d, g, w, fs, nullptr, nullptr, w.u, actions, s))) return st;
         if ((st = flow_network(fh, d, g, hidden, w, fs, sg, i > 0, false, nullptr, s))) return st;
-        k_flow_euler<<<(n + 255) / 256, 256, 0, s>>>(actions, w.v, 1.f / (float)n_steps, n);
+        pdl(k_flow_euler, (n + 255) / 256, 256, 0, s)(actions, w.v, 1.f / (float)n_steps, n);
         if ((st = last("flow euler"))) return st;
     }
     return JNX_OK;
@@ -1528,9 +1545,9 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
     // output layer
     {
         TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * d.D * 4.0, s);
-        k_flow_out_wgrad<<<dim3(nsl, d.D), 256, 0, s>>>(w.dv, w.nf, fs, d, gr->w_out, gr->b_out,
+        pdl(k_flow_out_wgrad, dim3(nsl, d.D), 256, 0, s)(w.dv, w.nf, fs, d, gr->w_out, gr->b_out,
                                                         add);
-        k_flow_out_bwd<<<Ma, 256, 0, s>>>(w.dv, g->sample_slot, fs, d, fh->w_out, w.dn);
+        pdl(k_flow_out_bwd, Ma, 256, 0, s)(w.dv, g->sample_slot, fs, d, fh->w_out, w.dn);
         if ((st = last("flow output backward"))) return st;
         if ((st = rms_bwd_launch(w.h_out, w.ones, kEps, w.dn, nullptr, Ma, dm, w.dh, w.dh_bf, s)))
             return st;
@@ -1675,12 +1692,12 @@ extern "C" jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group
     }
     // ---- embedding and time MLP ----
     TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * 8.0 + (double)S * dm * dm * 8.0, s);
-    k_flow_embed_wgrad<<<dim3(nsl, dm / 32), 256, 0, s>>>(w.dh, w.x, fs, d, gr->w_in,
+    pdl(k_flow_embed_wgrad, dim3(nsl, dm / 32), 256, 0, s)(w.dh, w.x, fs, d, gr->w_in,
                                                                     gr->b_in, gr->pos, add);
-    k_flow_dphi<<<dim3(S, (dm + 255) / 256), 256, 0, s>>>(w.dh, d, w.dphi);
-    k_flow_time_bwd<<<dim3(S, dm / 128), 256, (dm + 16 * 128) * sizeof(float), s>>>(
+    pdl(k_flow_dphi, dim3(S, (dm + 255) / 256), 256, 0, s)(w.dh, d, w.dphi);
+    pdl(k_flow_time_bwd, dim3(S, dm / 128), 256, (dm + 16 * 128) * sizeof(float), s)(
         g->sample_slot, fs, d, fh->t2, w.z1, w.dphi, w.dz1);
-    k_flow_outer<true><<<dim3(nsl, dm / kOuterRows), 256, 0, s>>>(w.dphi, w.z1, fs, d, gr->t2, gr->tb2, add);
-    k_flow_outer<false><<<dim3(nsl, dm / kOuterRows), 256, 0, s>>>(w.dz1, w.sfeat, fs, d, gr->t1, gr->tb1, add);
+    pdl(k_flow_outer<true>, dim3(nsl, dm / kOuterRows), 256, 0, s)(w.dphi, w.z1, fs, d, gr->t2, gr->tb2, add);
+    pdl(k_flow_outer<false>, dim3(nsl, dm / kOuterRows), 256, 0, s)(w.dz1, w.sfeat, fs, d, gr->t1, gr->tb1, add);
     return last("flow embedding backward");
 }

@@ -745,6 +745,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
         fence_barrier_init();
         fence_proxy_async();
     }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
     if (warp == 1) {
         tmem_alloc(tmem_slot, TMEM_COLS);
         tmem_relinquish();
@@ -1038,6 +1039,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
         fence_barrier_init();
         fence_proxy_async();
     }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
     if (warp == 1) {
         tmem_alloc_pair(tmem_slot, 512);
         tmem_relinquish_pair();
@@ -1232,6 +1234,7 @@ __global__ void __launch_bounds__(192, 1) k_gemm_batch(const __grid_constant__ G
         fence_barrier_init();
         fence_proxy_async();
     }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
     if (warp == 1) {
         tmem_alloc(tmem_slot, TMEM_COLS);
         tmem_relinquish();
@@ -1532,7 +1535,7 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const
     cudaError_t e =
         set_smem_limit(reinterpret_cast<const void*>(k_gemm<EPI, LORA, EW, BN, BMN>), limit, attr);
     if (e != cudaSuccess) return e;
-    k_gemm<EPI, LORA, EW, BN, BMN><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, lg, p);
+    pdl(k_gemm<EPI, LORA, EW, BN, BMN>, grid, 64 + 32 * EW, smem, s)(ta, tb, lg, p);
     return cudaGetLastError();
 }
 
@@ -1547,7 +1550,7 @@ static cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, Gem
     cudaError_t e =
         set_smem_limit(reinterpret_cast<const void*>(k_gemm_pair<EPI, EW>), smem, attr);
     if (e != cudaSuccess) return e;
-    k_gemm_pair<EPI, EW><<<grid, 64 + 32 * EW, smem, s>>>(ta, tb, p);
+    pdl(k_gemm_pair<EPI, EW>, grid, 64 + 32 * EW, smem, s)(ta, tb, p);
     return cudaGetLastError();
 }
 
@@ -1711,8 +1714,7 @@ static cudaError_t launch_batch(const GemmBatch& gb, cudaStream_t s) {
     cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(k_gemm_batch<EPI, AMN, BMN>),
                                    gemm::SMEM_BYTES, attr);
     if (e != cudaSuccess) return e;
-    k_gemm_batch<EPI, AMN, BMN>
-        <<<std::min(gb.tiles, num_sms()), 192, gemm::SMEM_BYTES, s>>>(gb);
+    pdl(k_gemm_batch<EPI, AMN, BMN>, std::min(gb.tiles, num_sms()), 192, gemm::SMEM_BYTES, s)(gb);
     return cudaGetLastError();
 }
 

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(256, 2) k_head_lin(const __grid_constant__ Hea
                                                   float* __restrict__ z_out, float* __restrict__ h_out,
                                                   int ld_out, const int* __restrict__ sample_target,
                                                   float* __restrict__ preds) {
+    pdl_entry();
     extern __shared__ __align__(16) uint8_t lin_smem[];
     const HeadSlot& hs = tab.slot[blockIdx.z];
     if (LAYER == 1 && hs.kind != JNX_HEAD_MLP) return;
@@ -264,6 +265,7 @@ __global__ void __launch_bounds__(kLossThreads) k_l2_loss(const __grid_constant_
                                                  const float* __restrict__ targets,
                                                  const int* __restrict__ sample_target,
                                                  float* __restrict__ dy, float* __restrict__ loss) {
+    pdl_entry();
     const HeadSlot& hs = tab.slot[blockIdx.x];
     const int W = hs.width;
     const int n = (hs.s1 - hs.s0) * W;
@@ -295,6 +297,7 @@ __global__ void __launch_bounds__(256) k_head_dw_out(const __grid_constant__ Hea
                                                      const __grid_constant__ OT opt, AdamHp hp,
                                                      const float* __restrict__ dy, int ld_y,
                                                      const float* __restrict__ h, int ld_h) {
+    pdl_entry();
     __shared__ __align__(16) float sh[32][256];
     __shared__ __align__(16) float sd[32][16];
     const HeadSlot& hs = tab.slot[blockIdx.x];
@@ -382,6 +385,7 @@ __global__ void __launch_bounds__(256, 3) k_head_back_in(const __grid_constant__
                                                       const float* __restrict__ dy, int ld_y,
                                                       const float* __restrict__ z, int ld_h,
                                                       float* __restrict__ dh) {
+    pdl_entry();
     __shared__ __align__(16) float sdy[kBackO][8];
     __shared__ __align__(16) float red[8][8][kBackCols];  // [warp][sample][column]
     const HeadSlot& hs = tab.slot[blockIdx.x];
@@ -471,6 +475,7 @@ __global__ void __launch_bounds__(256) k_mlp_dw1(const __grid_constant__ HeadTab
                                                  const __grid_constant__ OT opt, AdamHp hp,
                                                  const float* __restrict__ dz, int ld,
                                                  const float* __restrict__ p, int ld_p) {
+    pdl_entry();
     const HeadSlot& hs = tab.slot[blockIdx.x];
     if (hs.kind != JNX_HEAD_MLP) return;
     const int j0 = blockIdx.y * kDw1Rows;
@@ -823,6 +828,7 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 3)
                                                    const float* __restrict__ vbuf, int ldkv,
                                                    float* __restrict__ P, float* __restrict__ h,
                                                    int ld_h) {
+    pdl_entry();
     static_assert(kMaxQ == 32 && kXRows == 32, "two 16-row tiles of queries and of keys");
     extern __shared__ __align__(16) uint8_t xsm[];
     __shared__ float red[8 * 32], slot_m[32], slot_s[32];
@@ -898,6 +904,7 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
                                                    uint16_t* __restrict__ dkv,
                                                    uint16_t* __restrict__ planes, int ldp,
                                                    float* __restrict__ dQs, int kv_grads) {
+    pdl_entry();
     extern __shared__ __align__(16) uint8_t xsm[];
     __shared__ float red[8 * 32], slot_d[32];
     cg::cluster_group cluster = cg::this_cluster();
@@ -1023,6 +1030,7 @@ template <class OT>
 __global__ void __launch_bounds__(256) k_xattn_dq(const __grid_constant__ HeadTable tab,
                                                   const __grid_constant__ OT opt, AdamHp hp,
                                                   const float* __restrict__ dQs, int ld_h) {
+    pdl_entry();
     const HeadSlot& hs = tab.slot[blockIdx.x];
     if (hs.kind != JNX_HEAD_XATTN) return;
     const int i = blockIdx.y * 256 + threadIdx.x;
@@ -1071,6 +1079,7 @@ __global__ void __launch_bounds__(256) k_xattn_gh(const __grid_constant__ HeadTa
                                                   const float* __restrict__ dS,
                                                   const uint16_t* __restrict__ X, int ldx,
                                                   float* __restrict__ HG, int ldg) {
+    pdl_entry();
     static_assert(kMaxQ == 32, "two 16-row query tiles");
     __shared__ __align__(16) uint16_t sx[2][kGhRows][kGhXPad];
     __shared__ __align__(16) float sp[2][kGhRows * kMaxQ], sd[2][kGhRows * kMaxQ];
@@ -1197,6 +1206,7 @@ __global__ void __launch_bounds__(256) k_xattn_wgrad(const __grid_constant__ Hea
                                                      const __grid_constant__ OT opt, AdamHp hp,
                                                      const float* __restrict__ HG, int ldg,
                                                      const float* __restrict__ dO, int ld_h) {
+    pdl_entry();
     __shared__ __align__(16) float sh[kMaxQ][kWgE];  // H_s, then G_t
     __shared__ __align__(16) float so[kMaxQ][kWgC];  // dO_s, then Q
     const HeadSlot& hs = tab.slot[blockIdx.x];
@@ -1300,7 +1310,7 @@ static jnx_status cuda_ok(const char* what) {
 static jnx_status gh_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws, int d,
                             const uint16_t* hidden, const jnx_group* g, cudaStream_t s) {
     if (d % 256) {
-        k_xattn_gh<<<dim3(b.sample1 - b.sample0, d / 128), 256, 0, s>>>(
+        pdl(k_xattn_gh, dim3(b.sample1 - b.sample0, d / 128), 256, 0, s)(
             tab, b.g0, g->cu_seqlens, g->sample_slot, b.sample0, ws.P, ws.dS, hidden, d, ws.HG, d);
         return JNX_OK;
     }
@@ -1352,22 +1362,22 @@ jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const 
                                 float* loss, cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
     if (b.any_mlp)
-        k_head_lin<1><<<dim3((b.max_ns + kLinS - 1) / kLinS,
+        pdl(k_head_lin<1>, dim3((b.max_ns + kLinS - 1) / kLinS,
                              (b.max_mlp_hid + kLinCols - 1) / kLinCols, b.n),
-                        256, kLinSmem, s>>>(
+                        256, kLinSmem, s)(
             tab, pooled, d, ws.z, ws.h, ws.ld_h, sample_target, preds);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, false);
-        k_xattn_fwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(tab, b.g0, cu, sample_slot,
+        pdl(k_xattn_fwd, (b.sample1 - b.sample0) * kXCtas, 256, smem, s)(tab, b.g0, cu, sample_slot,
                                                              b.sample0, ws.kbuf, ws.vbuf, ws.ldkv,
                                                              ws.P, ws.h, ws.ld_h);
     }
-    k_head_lin<2><<<dim3((b.max_ns + kLinS - 1) / kLinS,
+    pdl(k_head_lin<2>, dim3((b.max_ns + kLinS - 1) / kLinS,
                          (b.max_width + kLinCols - 1) / kLinCols, b.n),
-                    256, kLinSmem, s>>>(
+                    256, kLinSmem, s)(
         tab, ws.h, ws.ld_h, ws.y, nullptr, ws.ld_y, sample_target, preds);
     if (targets)  // without targets (inference) there is no loss
-        k_l2_loss<<<b.n, kLossThreads, 0, s>>>(tab, ws.y, ws.ld_y, targets, sample_target, ws.dy, loss);
+        pdl(k_l2_loss, b.n, kLossThreads, 0, s)(tab, ws.y, ws.ld_y, targets, sample_target, ws.dy, loss);
     return cuda_ok("heads forward");
 }
 
@@ -1378,25 +1388,24 @@ jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const
     const int *cu = g->cu_seqlens, *sample_slot = g->sample_slot;
     const NoOpt no{};
     const AdamHp nh{};
-    k_head_dw_out<NoOpt>
-        <<<dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s>>>(
+    pdl(k_head_dw_out<NoOpt>, dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s)(
             tab, no, nh, ws.dy, ws.ld_y, ws.h, ws.ld_h);
-    k_head_back_in<<<dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s>>>(
+    pdl(k_head_back_in, dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s)(
         tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_mlp)
-        k_mlp_dw1<NoOpt><<<dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256),
-                           256, 0, s>>>(
+        pdl(k_mlp_dw1<NoOpt>, dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256),
+                           256, 0, s)(
             tab, no, nh, ws.dh, ws.ld_h, pooled, d);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
-        k_xattn_bwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(
+        pdl(k_xattn_bwd, (b.sample1 - b.sample0) * kXCtas, 256, smem, s)(
             tab, b.g0, cu, sample_slot, b.sample0, ws.kbuf, ws.vbuf, ws.ldkv, ws.P, ws.dS, ws.dh,
             ws.ld_h, ws.dkv, ws.planes, ws.ldp, ws.dQs, kv_grads ? 1 : 0);
-        k_xattn_dq<NoOpt><<<dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s>>>(
+        pdl(k_xattn_dq<NoOpt>, dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s)(
             tab, no, nh, ws.dQs, ws.ld_h);
         jnx_status st = gh_launch(tab, b, ws, d, hidden, g, s);
         if (st) return st;
-        k_xattn_wgrad<NoOpt><<<dim3(b.n, b.max_dq / kWgC, d / kWgE), 256, 0, s>>>(
+        pdl(k_xattn_wgrad<NoOpt>, dim3(b.n, b.max_dq / kWgC, d / kWgE), 256, 0, s)(
             tab, no, nh, ws.HG, d, ws.dh, ws.ld_h);
     }
     return cuda_ok("heads backward");
@@ -1407,11 +1416,11 @@ jnx_status heads_backward_front_launch(const HeadTable& tab, const HeadBatch& b,
                                        const jnx_group* g, bool kv_grads, cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
     const int *cu = g->cu_seqlens, *sample_slot = g->sample_slot;
-    k_head_back_in<<<dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s>>>(
+    pdl(k_head_back_in, dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s)(
         tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
-        k_xattn_bwd<<<(b.sample1 - b.sample0) * kXCtas, 256, smem, s>>>(
+        pdl(k_xattn_bwd, (b.sample1 - b.sample0) * kXCtas, 256, smem, s)(
             tab, b.g0, cu, sample_slot, b.sample0, ws.kbuf, ws.vbuf, ws.ldkv, ws.P, ws.dS, ws.dh,
             ws.ld_h, ws.dkv, ws.planes, ws.ldp, ws.dQs, kv_grads ? 1 : 0);
         jnx_status st = gh_launch(tab, b, ws, d, hidden, g, s);
@@ -1425,19 +1434,17 @@ jnx_status heads_backward_step_launch(const HeadTable& tab, const HeadOptTable& 
                                       const HeadScratch& ws, const float* pooled, int d,
                                       cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
-    k_head_dw_out<HeadOptTable>
-        <<<dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s>>>(
+    pdl(k_head_dw_out<HeadOptTable>, dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s)(
             tab, opt, hp, ws.dy, ws.ld_y, ws.h, ws.ld_h);
     if (b.any_mlp)
-        k_mlp_dw1<HeadOptTable>
-            <<<dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256), 256, 0,
-               s>>>(
+        pdl(k_mlp_dw1<HeadOptTable>, dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256), 256, 0,
+               s)(
             tab, opt, hp, ws.dh, ws.ld_h, pooled, d);
     if (b.any_xattn) {
         // wgrad reads the learned queries, which dq then updates
-        k_xattn_wgrad<HeadOptTable><<<dim3(b.n, b.max_dq / kWgC, d / kWgE), 256, 0, s>>>(
+        pdl(k_xattn_wgrad<HeadOptTable>, dim3(b.n, b.max_dq / kWgC, d / kWgE), 256, 0, s)(
             tab, opt, hp, ws.HG, d, ws.dh, ws.ld_h);
-        k_xattn_dq<HeadOptTable><<<dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s>>>(
+        pdl(k_xattn_dq<HeadOptTable>, dim3(b.n, (b.max_nq * b.max_dq + 255) / 256), 256, 0, s)(
             tab, opt, hp, ws.dQs, ws.ld_h);
     }
     return cuda_ok("heads backward step");

@@ -109,6 +109,17 @@ __device__ __forceinline__ float adamw_elem(float g, float& m, float& v, float p
     return __fsub_rn(p, __fmul_rn(lr, upd));
 }
 
+// Programmatic dependent launch: a kernel launched by pdl() (jnx_kernels.h) may
+// be on the SMs before the one ahead of it on its stream has ended.  Every such
+// kernel calls this before it touches global memory or TMEM: it waits until the
+// grid ahead is complete and its writes are visible, then lets the grid behind
+// be set up.  Since every kernel in a chain waits, the grid ahead being complete
+// means that all before it are, too.
+__device__ __forceinline__ void pdl_entry() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Record the first device-side error in the status word (never traps).
 __device__ __forceinline__ void report(int* status, int code) {
     if (status) atomicCAS(status, 0, code);

@@ -14,6 +14,36 @@ namespace jnx {
 enum { EPI_BF16 = 0, EPI_F32 = 1, EPI_RESID = 2, EPI_GLU = 3, EPI_ROPE = 4, EPI_GLU_BWD = 5,
        EPI_GLU_SAVE = 6, EPI_GLU_DM = 7 };
 
+// kernel<<<grid, block, smem, s>>>(args...) as a programmatic dependent launch:
+// pdl(kernel, grid, block, smem, s)(args...).  The kernel's CTAs are set up while
+// the one ahead on the stream drains and wait in pdl_entry() (jnx_dev.cuh), which
+// every kernel launched this way calls first.  It takes the launch latency out of
+// chains of short kernels: 17 launches of a small training step 95 -> 60 us, 300 of
+// a sampling call 3.48 -> 2.66 ms, 113 of an 18-block inference 3.21 -> 3.02 ms.
+template <class... P>
+struct PdlLaunch {
+    void (*kernel)(P...);
+    cudaLaunchConfig_t cfg;
+    template <class... A>
+    cudaError_t operator()(A&&... a) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(a)...);
+    }
+};
+template <class... P>
+PdlLaunch<P...> pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
+    PdlLaunch<P...> l{kernel, {}};
+    l.cfg.gridDim = grid;
+    l.cfg.blockDim = block;
+    l.cfg.dynamicSmemBytes = smem;
+    l.cfg.stream = s;
+    return l;
+}
+
 struct GemmParams {
     int M, N, K;
     int epi;

@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(128) k_lora_down(const uint16_t* __restrict__ 
                                                    const __grid_constant__ LoraSlots ls,
                                                    const __grid_constant__ LoraDown ld,
                                                    uint16_t* __restrict__ t, int ldt) {
+    pdl_entry();
     using lora::BK;
     using lora::BM;
     constexpr int R = kLoraRank;
@@ -131,9 +132,9 @@ jnx_status lora_down_launch(const jnx_group* g, const uint16_t* x, int ldx, int 
         }
         if (tiles == 0) continue;
         if (n_parts == 3)
-            k_lora_down<3><<<tiles, 128, 0, s>>>(x, ldx, K, ls, ld, t, ldt);
+            pdl(k_lora_down<3>, tiles, 128, 0, s)(x, ldx, K, ls, ld, t, ldt);
         else
-            k_lora_down<1><<<tiles, 128, 0, s>>>(x, ldx, K, ls, ld, t, ldt);
+            pdl(k_lora_down<1>, tiles, 128, 0, s)(x, ldx, K, ls, ld, t, ldt);
     }
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "lora down: %s", cudaGetErrorString(e));

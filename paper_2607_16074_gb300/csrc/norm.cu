@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ gather
                                               const int32_t* __restrict__ text_ids, int64_t n_text,
                                               const uint16_t* __restrict__ table, int vocab, int d,
                                               float* __restrict__ x, int* status) {
+    pdl_entry();
     const int tok = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (tok >= n_tokens) return;
@@ -60,7 +61,7 @@ jnx_status pack_launch(const jnx_group* g, const uint16_t* vision, int64_t n_vis
                        int d, float* x, int* status, cudaStream_t s) {
     if (d % 8) return fail(JNX_ERR_UNSUPPORTED, "pack: d %% 8 != 0");
     if (g->n_tokens == 0) return JNX_OK;
-    k_pack<<<(g->n_tokens + 7) / 8, 256, 0, s>>>(g->gather_src, g->n_tokens, vision, n_vision,
+    pdl(k_pack, (g->n_tokens + 7) / 8, 256, 0, s)(g->gather_src, g->n_tokens, vision, n_vision,
                                                  text_ids, n_text, table, vocab, d, x, status);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "pack: %s", cudaGetErrorString(e));
@@ -81,6 +82,7 @@ template <int V>
 __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
                                                  const uint16_t* __restrict__ gamma, float eps,
                                                  int M, uint16_t* __restrict__ out) {
+    pdl_entry();
     constexpr int D = V * 128;
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -115,6 +117,7 @@ template <int V>
 __global__ void __launch_bounds__(256) k_rms_prep(const float* __restrict__ x,
                                                   const uint16_t* __restrict__ gamma, int M,
                                                   uint16_t* __restrict__ y, float* __restrict__ ss) {
+    pdl_entry();
     constexpr int D = V * 128;
     constexpr int P = D / 128;  // 128-column blocks: lane float4 i = b
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -149,11 +152,11 @@ jnx_status rms_prep_launch(const float* x, const uint16_t* gamma, int M, int d, 
     if (M == 0) return JNX_OK;
     const int grid = (M + 7) / 8;
     switch (d) {
-        case 256: k_rms_prep<2><<<grid, 256, 0, s>>>(x, gamma, M, y, ss); break;
-        case 512: k_rms_prep<4><<<grid, 256, 0, s>>>(x, gamma, M, y, ss); break;
-        case 1024: k_rms_prep<8><<<grid, 256, 0, s>>>(x, gamma, M, y, ss); break;
-        case 2048: k_rms_prep<16><<<grid, 256, 0, s>>>(x, gamma, M, y, ss); break;
-        case 4096: k_rms_prep<32><<<grid, 256, 0, s>>>(x, gamma, M, y, ss); break;
+        case 256: pdl(k_rms_prep<2>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
+        case 512: pdl(k_rms_prep<4>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
+        case 1024: pdl(k_rms_prep<8>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
+        case 2048: pdl(k_rms_prep<16>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
+        case 4096: pdl(k_rms_prep<32>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
         default: return fail(JNX_ERR_UNSUPPORTED, "rms prep: d=%d not in {256..4096}", d);
     }
     cudaError_t e = cudaGetLastError();
@@ -165,11 +168,11 @@ jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int 
     if (M == 0) return JNX_OK;
     const int grid = (M + 7) / 8;
     switch (d) {
-        case 256: k_rmsnorm<2><<<grid, 256, 0, s>>>(x, gamma, eps, M, out); break;
-        case 512: k_rmsnorm<4><<<grid, 256, 0, s>>>(x, gamma, eps, M, out); break;
-        case 1024: k_rmsnorm<8><<<grid, 256, 0, s>>>(x, gamma, eps, M, out); break;
-        case 2048: k_rmsnorm<16><<<grid, 256, 0, s>>>(x, gamma, eps, M, out); break;
-        case 4096: k_rmsnorm<32><<<grid, 256, 0, s>>>(x, gamma, eps, M, out); break;
+        case 256: pdl(k_rmsnorm<2>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
+        case 512: pdl(k_rmsnorm<4>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
+        case 1024: pdl(k_rmsnorm<8>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
+        case 2048: pdl(k_rmsnorm<16>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
+        case 4096: pdl(k_rmsnorm<32>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
         default: return fail(JNX_ERR_UNSUPPORTED, "rmsnorm: d=%d not in {256..4096}", d);
     }
     cudaError_t e = cudaGetLastError();
@@ -202,6 +205,7 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
     k_final_pool(const float* __restrict__ x, const uint16_t* __restrict__ gamma, float eps,
                  const int* __restrict__ cu, int parts, float* __restrict__ pooled,
                  uint16_t* __restrict__ hidden) {
+    pdl_entry();
     constexpr int D = C * 256;
     constexpr int R = PRE && C == 16 ? 2 : 4;  // rows of a round
     __shared__ float red[2][R][8];
@@ -298,9 +302,9 @@ jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, c
     const bool pre = grid < 4 * num_sms();
     auto launch = [&](auto deep, auto flat) {
         if (pre)
-            deep<<<grid, 256, 0, s>>>(x, gamma, eps, cu, parts, pooled, hidden);
+            pdl(deep, grid, 256, 0, s)(x, gamma, eps, cu, parts, pooled, hidden);
         else
-            flat<<<grid, 256, 0, s>>>(x, gamma, eps, cu, parts, pooled, hidden);
+            pdl(flat, grid, 256, 0, s)(x, gamma, eps, cu, parts, pooled, hidden);
     };
     switch (d) {
         case 256: launch(k_final_pool<1, true>, k_final_pool<1, false>); break;
@@ -335,6 +339,7 @@ struct RopeFreqs {
 
 __global__ void __launch_bounds__(256) k_rope_table(float2* tab, int max_pos,
                                                     const __grid_constant__ RopeFreqs fr) {
+    pdl_entry();
     __shared__ double2 fine[kRopeFine], coarse[kRopeCoarse];
     const int i = blockIdx.x, p0 = blockIdx.y * kRopeSpan;
     const int t = threadIdx.x;
@@ -361,7 +366,7 @@ jnx_status rope_table_launch(float2* tab, int max_pos, int hd, float theta, cuda
     if (half > 128) return fail(JNX_ERR_UNSUPPORTED, "rope table: head dim %d", hd);
     RopeFreqs fr;
     for (int i = 0; i < half; ++i) fr.inv[i] = pow((double)theta, -2.0 * i / (2.0 * half));
-    k_rope_table<<<dim3(half, (max_pos + kRopeSpan - 1) / kRopeSpan), 256, 0, s>>>(tab, max_pos,
+    pdl(k_rope_table, dim3(half, (max_pos + kRopeSpan - 1) / kRopeSpan), 256, 0, s)(tab, max_pos,
                                                                                   fr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "rope table: %s", cudaGetErrorString(e));

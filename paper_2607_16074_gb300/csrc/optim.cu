@@ -15,6 +15,7 @@
 
 #include "../../include/jnx.h"
 #include "jnx_dev.cuh"
+#include "jnx_kernels.h"
 #include "jnx_trace.h"
 
 namespace jnx {
@@ -40,6 +41,7 @@ struct AdamTable {
 // it, then a scalar tail.
 __global__ void __launch_bounds__(256) k_adamw(const __grid_constant__ AdamTable tab, float lr,
                                                float b1, float b2, float eps, float wd) {
+    pdl_entry();
     const AdamSeg& s = tab.seg[blockIdx.y];
     const long long stride = (long long)gridDim.x * 256;
     const long long t0 = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -96,7 +98,7 @@ static jnx_status launch_segments(const std::vector<AdamSeg>& segs, const jnx_ad
         }
         if (mx == 0) continue;
         const int bx = (int)std::min<long long>((mx / 4 + 255) / 256 + 1, 1024);
-        k_adamw<<<dim3(bx, ns), 256, 0, s>>>(tab, hp->lr, hp->beta1, hp->beta2, hp->eps,
+        pdl(k_adamw, dim3(bx, ns), 256, 0, s)(tab, hp->lr, hp->beta1, hp->beta2, hp->eps,
                                              hp->weight_decay);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "adamw: %s", cudaGetErrorString(e));
