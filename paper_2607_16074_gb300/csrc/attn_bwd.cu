@@ -71,6 +71,14 @@ struct AttnBwdCfg {
     static constexpr int IB = BN * HD * 2;  // one inner operand tile
     static constexpr int NB1 = HD == 256 ? 2 : 3;
     static constexpr int NB2 = (HD == 256 && NEED_DP) ? 1 : 2;
+    // The accumulating product of tile j holds B1's tile until it is done, so with
+    // two B1 slots the scores of tile j + 2 would wait for their whole load right
+    // after it, and the product of tile j + 1 behind them.  There tiles go in
+    // pairs instead: both accumulating products, then both tiles' scores, whose
+    // loads have been under way since.  (MMA warp of head dim 256: 1,080 clocks a
+    // tile waiting for B1 in the dQ pass and 1,940 in the dK pass of 4,350 and
+    // 4,100; 24,000 tokens, dQ 283 -> 250 us and dK 380 -> 319.)
+    static constexpr bool PAIRED = NB1 == 2 && NEED_DP;
     static constexpr int OFF_A2 = OB;
     static constexpr int OFF_B1 = NEED_DP ? 2 * OB : OB;
     static constexpr int OFF_B2 = OFF_B1 + NB1 * IB;
@@ -342,7 +350,8 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                 ++no;
                 tc_fence_after();
                 ok = issue_scores() && (n < 2 || issue_scores());
-                if (ok && n <= 2) commit(o_empty);
+                int ns = min(n, 2);  // score tiles issued
+                if (ok && ns == n) commit(o_empty);
                 for (int kt = 0; kt < n && ok; ++kt) {
                     const uint32_t pb = gp & 1;
                     if (!(ok = mbar_wait_warp(&p_full[pb], (gp >> 1) & 1))) break;
@@ -379,9 +388,10 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                     // the score products of tile kt + 2 reuse buffer pb: the
                     // tensor core runs this thread's MMAs in issue order, so
                     // the products above have read it before they land
-                    if (kt + 2 < n) {
+                    const int upto = !C::PAIRED ? kt + 3 : kt & 1 ? kt + 3 : 0;
+                    for (; ok && ns < min(upto, n); ++ns) {
                         ok = issue_scores();
-                        if (ok && kt + 3 == n) commit(o_empty);
+                        if (ok && ns + 1 == n) commit(o_empty);
                     }
                 }
                 if (!ok) break;
