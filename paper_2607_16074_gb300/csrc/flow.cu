@@ -50,9 +50,13 @@ __device__ __forceinline__ float silu_grad_f(float z) {
 
 // ---------------------------------------------------------------------------
 // time embedding: s(tau), z1 = T1 s + tb1, phi = T2 SiLU(z1) + tb2.  Each
-// layer is one launch over (sample, block of 32 output rows): one warp per
+// layer is one launch over (row, block of 32 output rows): one warp per
 // row, lanes along the dot product with 16-byte weight loads (dm is a
-// multiple of 256), the row sum in a fixed butterfly order.
+// multiple of 256), the row sum in a fixed butterfly order.  A row is a sample
+// with its own tau, or, when sampling (tau null), an Euler step and slot: row r
+// is slot r % n at time (step0 + r / n) / n_steps, since all of a tenant's samples
+// are at the same time then.  One pair of launches serves every step (a fill and
+// two launches of a row per sample in each step before: 20 of 265 us).
 // ---------------------------------------------------------------------------
 constexpr int kTimeRows = 32;
 
@@ -81,19 +85,20 @@ __global__ void __launch_bounds__(256) k_flow_time1(const float* __restrict__ ta
                                                     FlowDims dd, const uint16_t* __restrict__ t1,
                                                     const uint16_t* __restrict__ tb1,
                                                     float* __restrict__ sfeat,
-                                                    float* __restrict__ z1) {
+                                                    float* __restrict__ z1, int step0,
+                                                    int n_steps) {
     pdl_entry();
     extern __shared__ float sh[];  // s(tau) [dm]
     const int s = blockIdx.x, dm = dd.dm, half = dm / 2;
-    const int t = fs.tenant[sample_slot[s]];
-    const float tv = tau[s];
+    const int t = fs.tenant[tau ? sample_slot[s] : s % fs.n];
+    const float tv = tau ? tau[s] : (float)(step0 + s / fs.n) / (float)n_steps;
     for (int i = threadIdx.x; i < dm; i += blockDim.x) {
         const int k = i < half ? i : i - half;
         const float w = powf(10000.f, -(float)k / (float)half);
         const float a = 1000.f * tv * w;
         const float v = i < half ? sinf(a) : cosf(a);
         sh[i] = v;
-        if (blockIdx.y == 0) sfeat[(size_t)s * dm + i] = v;
+        if (sfeat && blockIdx.y == 0) sfeat[(size_t)s * dm + i] = v;
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -109,11 +114,11 @@ __global__ void __launch_bounds__(256) k_flow_time2(const int* __restrict__ samp
                                                     FlowDims dd, const uint16_t* __restrict__ t2,
                                                     const uint16_t* __restrict__ tb2,
                                                     const float* __restrict__ z1,
-                                                    float* __restrict__ phi) {
+                                                    float* __restrict__ phi, int by_slot) {
     pdl_entry();
     extern __shared__ float sh[];  // SiLU(z1) [dm]
     const int s = blockIdx.x, dm = dd.dm;
-    const int t = fs.tenant[sample_slot[s]];
+    const int t = fs.tenant[by_slot ? s % fs.n : sample_slot[s]];
     for (int i = threadIdx.x; i < dm; i += blockDim.x) sh[i] = silu_f(z1[(size_t)s * dm + i]);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -133,13 +138,14 @@ __global__ void __launch_bounds__(256) k_flow_embed(
     const float* __restrict__ tau, const float* __restrict__ xin,
     const int* __restrict__ sample_slot, const __grid_constant__ FlowSlots fs, FlowDims dd,
     const uint16_t* __restrict__ w_in, const uint16_t* __restrict__ b_in,
-    const uint16_t* __restrict__ pos, const float* __restrict__ phi, float* __restrict__ x_out,
-    float* __restrict__ u_out, float* __restrict__ h) {
+    const uint16_t* __restrict__ pos, const float* __restrict__ phi, int phi_by_slot,
+    float* __restrict__ x_out, float* __restrict__ u_out, float* __restrict__ h) {
     pdl_entry();
     __shared__ float xs[kMaxD];
     const int r = blockIdx.x, C = dd.C, D = dd.D, dm = dd.dm;
     const int s = r / C, c = r % C;
-    const int t = fs.tenant[sample_slot[s]];
+    const int slot = sample_slot[s], t = fs.tenant[slot];
+    const float* ph = phi + (size_t)(phi_by_slot ? slot : s) * dm;
     if (threadIdx.x < D) {
         const size_t e = (size_t)r * D + threadIdx.x;
         float x;
@@ -160,7 +166,7 @@ __global__ void __launch_bounds__(256) k_flow_embed(
     const bool vec = D % 8 == 0 && (reinterpret_cast<uintptr_t>(w_in) & 15) == 0;
     for (int j = threadIdx.x; j < dm; j += blockDim.x) {
         float acc = bf2f(b_in[(size_t)t * dm + j]) + bf2f(pos[((size_t)t * C + c) * dm + j]) +
-                    phi[(size_t)s * dm + j];
+                    ph[j];
         const uint16_t* wr = W + (size_t)j * D;
         if (vec) {
 #pragma unroll 4
@@ -1233,12 +1239,6 @@ __global__ void k_fill_bf16(uint16_t* p, int n, uint16_t v) {
     if (i < n) p[i] = v;
 }
 
-__global__ void k_fill_f32(float* p, int n, float v) {
-    pdl_entry();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
-}
-
 // The network from h (embedded) through the blocks to v (and, with u, dv
 // and the loss); saves every block's activations.  With reuse_ctx, the
 // context K/V of every block are already in the workspace.
@@ -1258,12 +1258,10 @@ jnx_status flow_network(const jnx_flow_head* fh, const FlowDims& d, const jnx_gr
         float* lse = w.lse + (size_t)b * Ma * d.nh;
         uint16_t* m = w.m + (size_t)b * Ma * d.F;
         uint16_t* kvc = w.kvc + (size_t)b * N * 2 * dm;
-        if (cudaMemcpyAsync(h_in, w.h, (size_t)Ma * dm * 4, cudaMemcpyDeviceToDevice, s) !=
-            cudaSuccess)
-            return last("flow: copy");
         {
             TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * 6.0, s);
-            if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, n1, s))) return st;
+            if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, n1, s, train ? h_in : nullptr)))
+                return st;
         }
         GemmParams p{};
         p.M = Ma;
@@ -1314,12 +1312,10 @@ jnx_status flow_network(const jnx_flow_head* fh, const FlowDims& d, const jnx_gr
                                       sg.ten.data(), s)))
                 return st;
         }
-        if (cudaMemcpyAsync(h_mid, w.h, (size_t)Ma * dm * 4, cudaMemcpyDeviceToDevice, s) !=
-            cudaSuccess)
-            return last("flow: copy");
         {
             TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * 6.0, s);
-            if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, n2, s))) return st;
+            if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, n2, s, train ? h_mid : nullptr)))
+                return st;
         }
         p = GemmParams{};
         p.M = Ma;
@@ -1352,10 +1348,8 @@ jnx_status flow_network(const jnx_flow_head* fh, const FlowDims& d, const jnx_gr
         }
     }
     TraceScope ts(JNX_K_FLOW_MISC, (double)Ma * dm * 8.0, s);
-    if (cudaMemcpyAsync(w.h_out, w.h, (size_t)Ma * dm * 4, cudaMemcpyDeviceToDevice, s) !=
-        cudaSuccess)
-        return last("flow: copy");
-    if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, w.nf, s))) return st;
+    if ((st = rmsnorm_launch(w.h, w.ones, kEps, Ma, dm, w.nf, s, train ? w.h_out : nullptr)))
+        return st;
     pdl(k_flow_out, dim3(Ma, (d.D + 7) / 8), 256, 0, s)(w.nf, g->sample_slot, fs, d, fh->w_out,
                                                        fh->b_out, train ? w.u : nullptr, w.v, w.dv);
     if ((st = last("flow output"))) return st;
@@ -1428,22 +1422,23 @@ static jnx_status flow_begin(const jnx_flow_head* fh, const jnx_group* g, const 
     return JNX_OK;
 }
 
-// time embedding + token embedding into w.h
-static jnx_status flow_embed(const jnx_flow_head* fh, const FlowDims& d, const jnx_group* g,
-                             const FlowWs& w, const FlowSlots& fs, const float* actions,
-                             const float* noise, const float* tau, const float* xin,
-                             cudaStream_t s) {
-    const int S = g->n_samples, Ma = S * d.C;
-    TraceScope ts(JNX_K_FLOW_MISC, (double)S * d.dm * d.dm * 4.0, s);
+// The time embedding of every sample (tau), or of Euler steps [step0, step0 +
+// rows / slots) of n_steps for every slot (tau null), into z1 and phi.
+static jnx_status flow_time(const jnx_flow_head* fh, const FlowDims& d, const jnx_group* g,
+                            const FlowSlots& fs, const float* tau, int rows, int step0,
+                            int n_steps, float* sfeat, float* z1, float* phi, cudaStream_t s) {
+    const dim3 tg(rows, d.dm / kTimeRows);
+    pdl(k_flow_time1, tg, 256, d.dm * sizeof(float), s)(tau, g->sample_slot, fs, d, fh->t1,
+                                                        fh->tb1, sfeat, z1, step0, n_steps);
+    pdl(k_flow_time2, tg, 256, d.dm * sizeof(float), s)(g->sample_slot, fs, d, fh->t2, fh->tb2, z1,
+                                                        phi, tau ? 0 : 1);
+    return last("flow time embedding");
+}
+
+// the norm's unit gain
+static jnx_status flow_ones(const FlowDims& d, const FlowWs& w, cudaStream_t s) {
     pdl(k_fill_bf16, (d.dm + 255) / 256, 256, 0, s)(w.ones, d.dm, (uint16_t)0x3F80);
-    const dim3 tg(S, d.dm / kTimeRows);
-    pdl(k_flow_time1, tg, 256, d.dm * sizeof(float), s)(tau, g->sample_slot, fs, d, fh->t1, fh->tb1,
-                                                       w.sfeat, w.z1);
-    pdl(k_flow_time2, tg, 256, d.dm * sizeof(float), s)(g->sample_slot, fs, d, fh->t2, fh->tb2,
-                                                       w.z1, w.phi);
-    pdl(k_flow_embed, Ma, 256, 0, s)(actions, noise, tau, xin, g->sample_slot, fs, d, fh->w_in,
-                                    fh->b_in, fh->pos, w.phi, w.x, w.u, w.h);
-    return last("flow embedding");
+    return last("flow gain");
 }
 
 extern "C" jnx_status jnx_flow_forward(const jnx_flow_head* fh, const jnx_group* g,
@@ -1463,7 +1458,16 @@ extern "C" jnx_status jnx_flow_forward(const jnx_flow_head* fh, const jnx_group*
     static thread_local FlowSlots fs;
     fill_slots(g, fs);
     const Segs sg = make_segs(g, d.C);
-    if ((st = flow_embed(fh, d, g, w, fs, actions, noise, tau, nullptr, s))) return st;
+    {
+        TraceScope ts(JNX_K_FLOW_MISC, (double)g->n_samples * d.dm * d.dm * 4.0, s);
+        if ((st = flow_ones(d, w, s)) ||
+            (st = flow_time(fh, d, g, fs, tau, g->n_samples, 0, 1, w.sfeat, w.z1, w.phi, s)))
+            return st;
+        pdl(k_flow_embed, g->n_samples * d.C, 256, 0, s)(actions, noise, tau, (const float*)nullptr,
+                                                         g->sample_slot, fs, d, fh->w_in, fh->b_in,
+                                                         fh->pos, w.phi, 0, w.x, w.u, w.h);
+        if ((st = last("flow embedding"))) return st;
+    }
     if ((st = flow_network(fh, d, g, hidden, w, fs, sg, false, true, loss, s))) return st;
     if (cudaMemcpyAsync(velocity, w.v, (size_t)g->n_samples * d.C * d.D * 4,
                         cudaMemcpyDeviceToDevice, s) != cudaSuccess)
@@ -1490,11 +1494,28 @@ extern "C" jnx_status jnx_flow_sample(const jnx_flow_head* fh, const jnx_group* 
     const int n = g->n_samples * d.C * d.D;
     if (cudaMemcpyAsync(actions, noise, (size_t)n * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return last("flow: copy");
-    // tau of step i for every sample, in the u buffer (no target when sampling)
+    if ((st = flow_ones(d, w, s))) return st;
+    // time embeddings of as many steps as the buffers hold at once (the blocks'
+    // saved inputs are not kept when sampling, so theirs are free)
+    float* tz = d.nb > 0 ? w.h_in : w.z1;
+    float* tp = d.nb > 0 ? w.h_mid : w.phi;
+    const size_t cap = d.nb > 0 ? (size_t)d.nb * g->n_samples * d.C : (size_t)g->n_samples;
+    const int chunk = (int)std::max<size_t>(1, cap / g->n_slots);
     for (int i = 0; i < n_steps; ++i) {
-        pdl(k_fill_f32, (g->n_samples + 255) / 256, 256, 0, s)(w.u, g->n_samples,
-                                                             (float)i / (float)n_steps);
-        if ((st = flow_embed(fh, d, g, w, fs, nullptr, nullptr, w.u, actions, s))) return st;
+        if (i % chunk == 0) {
+            const int rows = std::min(chunk, n_steps - i) * g->n_slots;
+            TraceScope ts(JNX_K_FLOW_MISC, (double)rows * d.dm * d.dm * 4.0, s);
+            if ((st = flow_time(fh, d, g, fs, nullptr, rows, i, n_steps, nullptr, tz, tp, s)))
+                return st;
+        }
+        {
+            TraceScope ts(JNX_K_FLOW_MISC, (double)n * 4.0, s);
+            pdl(k_flow_embed, g->n_samples * d.C, 256, 0, s)(
+                (const float*)nullptr, (const float*)nullptr, (const float*)nullptr, actions,
+                g->sample_slot, fs, d, fh->w_in, fh->b_in, fh->pos,
+                tp + (size_t)(i % chunk) * g->n_slots * d.dm, 1, w.x, w.u, w.h);
+            if ((st = last("flow embedding"))) return st;
+        }
         if ((st = flow_network(fh, d, g, hidden, w, fs, sg, i > 0, false, nullptr, s))) return st;
         pdl(k_flow_euler, (n + 255) / 256, 256, 0, s)(actions, w.v, 1.f / (float)n_steps, n);
         if ((st = last("flow euler"))) return st;

@@ -205,9 +205,10 @@ jnx_status pack_launch(const jnx_group* g, const uint16_t* vision, int64_t n_vis
                        const int32_t* text_ids, int64_t n_text, const uint16_t* table, int vocab,
                        int d, float* x, int* status, cudaStream_t s);
 
-// RMSNorm: out[M, d] bf16 = x / sqrt(mean(x^2) + eps) * gamma.
+// RMSNorm: out[M, d] bf16 = x / sqrt(mean(x^2) + eps) * gamma; copy (optional)
+// receives x.
 jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int M, int d,
-                          uint16_t* out, cudaStream_t s);
+                          uint16_t* out, cudaStream_t s, float* copy = nullptr);
 
 // Final RMSNorm fused with the per-sample mean pool.
 jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, const int* cu,

@@ -68,7 +68,8 @@ jnx_status pack_launch(const jnx_group* g, const uint16_t* vision, int64_t n_vis
 }
 
 // ---------------------------------------------------------------------------
-// RMSNorm: one warp per row, the row held in registers (V float4 per lane),
+// RMSNorm: one warp per row, the row held in registers (V float4 per lane) and,
+// with `copy`, written out as it came,
 // fp32 sum of squares reduced lane-wise then by a fixed shuffle tree, so a
 // row's result does not depend on where it sits in the batch.
 // ---------------------------------------------------------------------------
@@ -81,7 +82,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 template <int V>
 __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
                                                  const uint16_t* __restrict__ gamma, float eps,
-                                                 int M, uint16_t* __restrict__ out) {
+                                                 int M, uint16_t* __restrict__ out,
+                                                 float* __restrict__ copy) {
     pdl_entry();
     constexpr int D = V * 128;
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -97,6 +99,11 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
     }
     ss = warp_sum(ss);
     const float r = rsqrtf(ss / (float)D + eps);
+    if (copy) {
+        float4* crow = reinterpret_cast<float4*>(copy + (size_t)row * D);
+#pragma unroll
+        for (int i = 0; i < V; ++i) crow[lane + 32 * i] = v[i];
+    }
     uint2* orow = reinterpret_cast<uint2*>(out + (size_t)row * D);
     const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
 #pragma unroll
@@ -164,15 +171,15 @@ jnx_status rms_prep_launch(const float* x, const uint16_t* gamma, int M, int d, 
 }
 
 jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int M, int d,
-                          uint16_t* out, cudaStream_t s) {
+                          uint16_t* out, cudaStream_t s, float* copy) {
     if (M == 0) return JNX_OK;
     const int grid = (M + 7) / 8;
     switch (d) {
-        case 256: pdl(k_rmsnorm<2>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
-        case 512: pdl(k_rmsnorm<4>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
-        case 1024: pdl(k_rmsnorm<8>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
-        case 2048: pdl(k_rmsnorm<16>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
-        case 4096: pdl(k_rmsnorm<32>, grid, 256, 0, s)(x, gamma, eps, M, out); break;
+        case 256: pdl(k_rmsnorm<2>, grid, 256, 0, s)(x, gamma, eps, M, out, copy); break;
+        case 512: pdl(k_rmsnorm<4>, grid, 256, 0, s)(x, gamma, eps, M, out, copy); break;
+        case 1024: pdl(k_rmsnorm<8>, grid, 256, 0, s)(x, gamma, eps, M, out, copy); break;
+        case 2048: pdl(k_rmsnorm<16>, grid, 256, 0, s)(x, gamma, eps, M, out, copy); break;
+        case 4096: pdl(k_rmsnorm<32>, grid, 256, 0, s)(x, gamma, eps, M, out, copy); break;
         default: return fail(JNX_ERR_UNSUPPORTED, "rmsnorm: d=%d not in {256..4096}", d);
     }
     cudaError_t e = cudaGetLastError();
