@@ -1343,7 +1343,7 @@ jnx_status flow_network(const jnx_flow_head* fh, const FlowDims& d, const jnx_gr
         {
             TraceScope ts(JNX_K_FLOW_GEMM, 2.0 * Ma * dm * d.F, s);
             if ((st = gemm_launch_seg(m, d.F, B.w_d, d.F, d.T, p, nsl, sg.a0.data(), sg.a1.data(),
-                                      sg.ten.data(), s)))
+                                      sg.ten.data(), s, false, !train)))
                 return st;
         }
     }

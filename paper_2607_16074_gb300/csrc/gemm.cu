@@ -1193,6 +1193,192 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
 }
 
 // ---------------------------------------------------------------------------
+// Segmented residual GEMM with K split over a cluster: x += A . B_t^T in tiles
+// of 128 x 64, one per cluster of kSplit CTAs, each over its share of the K
+// steps; the partial tiles meet in distributed shared memory and are added in
+// rank order, then to x.  For the experts' long contractions over a tenant's few
+// rows: a chain of 64 K steps of 0.18 us is all a narrow tile does (K = 4,096, 16
+// rows: 17 us, 10.0 split).  Taken by the sampler for K >= 2,048, whatever the
+// rows, so that a tenant's bits do not depend on its group; a training step's
+// rows fill the SMs without it (5,300 us against 5,322 for eight tenants of 64).
+// ---------------------------------------------------------------------------
+constexpr int kSplit = 4;
+constexpr int kSplitPad = 68;  // row stride of a partial tile (floats)
+constexpr int split_smem(int stages, int a_rows) {
+    return gemm::narrow_smem(64, stages, a_rows, false) - gemm::STG_BYTES +
+           gemm::BM * kSplitPad * 4;
+}
+
+__global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(192)
+    k_gemm_split(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+                 const __grid_constant__ LoraGemm lg, GemmParams p) {
+    using gemm::A_BYTES;
+    using gemm::BK;
+    using gemm::BM;
+    constexpr int BN = 64, RING = gemm::RING_MAX;
+    constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
+    const int stages = p.stages, a_bytes = p.a_rows * BK * 2, stage_bytes = a_bytes + BN * BK * 2;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + stages * stage_bytes + A_BYTES - a_bytes);
+    uint64_t* empty = full + RING;
+    uint64_t* tfull = empty + RING;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* consumed = abort_flag + 1;
+    float* part = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full) + gemm::NARROW_BAR);
+    const int warp = warp_uniform(threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    const int rank = (int)cluster_rank();
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < RING; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(tfull, 1);
+        *abort_flag = 0;
+        *consumed = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+    }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, BN);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
+
+    const TileGeo g = tile_geo<EPI_RESID, true, BN>(blockIdx.x / kSplit, lg.seg_tile0[lg.n_seg],
+                                                    p.N / BN, p, lg);
+    const int num_k = p.K / BK;
+    const int k0 = rank * num_k / kSplit, k1 = (rank + 1) * num_k / kSplit;
+    int issued = 0;
+    if (warp == 0) {
+        const int brow = lg.seg_tenant[g.seg] * p.N + g.c0;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int kb = k0; kb < k1; ++kb) {
+            if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
+                ok = false;
+                break;
+            }
+            if (elect_one()) {
+                uint8_t* sa = smem + stage * stage_bytes;
+                mbar_arrive_expect_tx(&full[stage], stage_bytes);
+                tma_load_2d(sa, &ta, kb * BK, g.row0, &full[stage]);
+                tma_load_2d(sa + a_bytes, &tb, kb * BK, brow, &full[stage]);
+            }
+            __syncwarp();
+            ++issued;
+            if (++stage == stages) {
+                stage = 0;
+                phase ^= 1;
+            }
+        }
+        if (!ok) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        }
+    } else if (warp == 1) {
+        int stage = 0, n_used = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        const uint32_t a_lo = sw128_desc_lo(smem_u32(smem));
+        const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + a_bytes);
+        for (int kb = k0; kb < k1; ++kb) {
+            if (!mbar_wait_warp(&full[stage], phase)) {
+                ok = false;
+                break;
+            }
+            ++n_used;
+            tc_fence_after();
+            const uint32_t off = (uint32_t)(stage * stage_bytes) >> 4;
+            if (elect_one()) {
+#pragma unroll
+                for (int kk = 0; kk < BK / 16; ++kk)
+                    tc_mma_f16(tmem_base, desc_of(a_lo + off + 2 * kk, kSw128DescHi),
+                               desc_of(b_lo + off + 2 * kk, kSw128DescHi), IDESC,
+                               kb > k0 || kk > 0);
+                tc_commit(&empty[stage]);
+            }
+            __syncwarp();
+            if (++stage == stages) {
+                stage = 0;
+                phase ^= 1;
+            }
+        }
+        if (!ok) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        }
+        *consumed = n_used;
+        if (elect_one()) tc_commit(tfull);  // all MMAs of this CTA
+        __syncwarp();
+        mbar_wait_warp(tfull, 0);
+    } else {
+        const int q = warp & 3;  // TMEM lane quarter this warp may access
+        if (!mbar_wait_warp(tfull, 0)) {
+            *abort_flag = 1;
+            report(p.status, JNX_ERR_TIMEOUT);
+        } else if (g.row0 + q * 32 < g.row_end) {
+            tc_fence_after();
+            float* row = part + (q * 32 + lane) * kSplitPad;
+#pragma unroll
+            for (int c = 0; c < BN / 32; ++c) {
+                uint32_t r[32];
+                tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + c * 32, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    *reinterpret_cast<uint4*>(row + c * 32 + 4 * u) =
+                        make_uint4(r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
+            }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc(tmem_base, BN);
+    __syncwarp();
+    cluster_sync_all();
+    if (warp >= 2 && !*abort_flag) {
+        // this rank's quarter of the columns: four threads a row, 32 rows a pass
+        const int i = threadIdx.x - 64, c = rank * (BN / kSplit) + 4 * (i & 3);
+        for (int r = i >> 2; g.row0 + r < g.row_end; r += 32) {
+            float4* xp = reinterpret_cast<float4*>(p.resid + (size_t)(g.row0 + r) * p.ldr + g.c0 + c);
+            const float4 x = *xp;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < kSplit; ++k) {
+                float4 t;
+                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w)
+                             : "r"(map_rank(part + r * kSplitPad + c, k))
+                             : "memory");
+                v.x += t.x;
+                v.y += t.y;
+                v.z += t.z;
+                v.w += t.w;
+            }
+            *xp = make_float4(x.x + v.x, x.y + v.y, x.z + v.z, x.w + v.w);
+        }
+    }
+    if (*abort_flag && warp == 0 && lane == 0)
+        // wait (bounded) for TMA copies this CTA issued but nobody consumed
+        for (int i = *consumed; i < issued; ++i)
+            mbar_wait(&full[i % stages], (i / stages) & 1, 100000000LL);
+    __syncwarp();
+    cluster_sync_all();  // no CTA's partial tile goes away while another reads it
+}
+
+// ---------------------------------------------------------------------------
 // A batch of GEMMs in one launch (GemmBatch): the wide single-CTA kernel over
 // the tiles of all problems in turn, each with its own tensor maps and output.
 // An operand may be MN-major (its rows are K): 64 x 64 boxes of it, 128-byte
@@ -1635,7 +1821,7 @@ jnx_status gemm_launch(const uint16_t* A, int lda, const uint16_t* B, int ldb, G
 
 jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ldb, int n_tenants,
                            GemmParams p, int n_seg, const int* seg_r0, const int* seg_r1,
-                           const int* seg_tenant, cudaStream_t s, bool b_mn) {
+                           const int* seg_tenant, cudaStream_t s, bool b_mn, bool split_k) {
     jnx_status st = gemm_check(p.M, p.N, p.K);
     if (st != JNX_OK) return st;
     if (n_seg < 0 || n_seg > kLoraMaxSlots || n_tenants <= 0)
@@ -1661,16 +1847,32 @@ jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ld
     lg.seg_tile0[n_seg] = tiles;
     if (tiles == 0) return JNX_OK;
     p.seg_bn = 1;
-    const int bn = pick_bn(tiles, p, false);
+    const bool split = split_k && p.epi == EPI_RESID && !b_mn && !p.norm_gamma && p.K >= 2048;
+    const int bn = split ? 64 : pick_bn(tiles, p, false);
     p.a_rows = a_box(bn, most);
     CUtensorMap ta, tb;
     if (!make_tmap_bf16(&ta, A, p.M, p.K, lda, p.a_rows, gemm::BK) ||
         !(b_mn ? make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.K, p.N, ldb, gemm::BK, 64)
-               : make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.N, p.K, ldb, b_box(bn), gemm::BK)))
+               : make_tmap_bf16(&tb, B, (uint64_t)n_tenants * p.N, p.K, ldb,
+                                split ? 64 : b_box(bn), gemm::BK)))
         return fail(JNX_ERR_CUDA, "gemm: tensor map encode failed (alignment or driver)");
     const long long total = (long long)tiles * (p.N / bn);
     if (p.group_m <= 0) p.group_m = default_group_m(p.K);
     cudaError_t e;
+    if (split) {
+        const long long ctas = total * kSplit;
+        if (ctas > 0x7FFFFFFFLL) return fail(JNX_ERR_UNSUPPORTED, "gemm: too many tiles");
+        const int budget = (ctas > num_sms() ? 112 : 224) * 1024;
+        p.stages = std::min(gemm::RING_MAX, std::max(2, p.K / gemm::BK / kSplit));
+        while (p.stages > 2 && split_smem(p.stages, p.a_rows) > budget) --p.stages;
+        static std::atomic<uint64_t> attr{0};
+        e = set_smem_limit(reinterpret_cast<const void*>(k_gemm_split), 224 * 1024, attr);
+        if (e == cudaSuccess)
+            e = pdl(k_gemm_split, (unsigned)ctas, 192, split_smem(p.stages, p.a_rows), s)(ta, tb,
+                                                                                        lg, p);
+        if (e != cudaSuccess) return fail(JNX_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
+        return JNX_OK;
+    }
     if (b_mn) {
         if (p.epi == EPI_F32)
             e = launch_epi<EPI_F32, true, LoraGemm, 4, true>(ta, tb, lg, p, bn, total, s);

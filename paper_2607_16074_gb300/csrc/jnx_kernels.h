@@ -143,10 +143,12 @@ jnx_status gemm_launch_lora(const uint16_t* A, int lda, const uint16_t* B, int l
 // [N, K] slice of tenant seg_tenant[i] in B = [n_tenants * N, K] (row stride
 // ldb).  Output tiles never straddle two segments.  b_mn (EPI_F32, EPI_GLU_BWD):
 // C = A . B_t with B_t the [K, N] rows of the tenant in B = [n_tenants * K, N],
-// read as they lie.
+// read as they lie.  split_k (EPI_RESID): K >= 2,048 is split over a cluster
+// (k_gemm_split).
 jnx_status gemm_launch_seg(const uint16_t* A, int lda, const uint16_t* B, int ldb, int n_tenants,
                            GemmParams p, int n_seg, const int* seg_r0, const int* seg_r1,
-                           const int* seg_tenant, cudaStream_t s, bool b_mn = false);
+                           const int* seg_tenant, cudaStream_t s, bool b_mn = false,
+                           bool split_k = false);
 struct LoraSlots {
     int g0, n, sample0, pad_;
     int tenant[kLoraMaxSlots];
