@@ -226,11 +226,22 @@ static jnx_status backbone_forward(const jnx_backbone* bb, const jnx_group* g,
     const int qkvw = (H + 2 * Hkv) * hd;
 
     const double Nd = (double)N * d;
+    // Fold an RMSNorm into the residual GEMM before it (for the first block, the
+    // packer) only where that GEMM's K loop is long enough to hide the extra
+    // epilogue work (writing y and the sums of squares).  Measured on GB300: at K =
+    // 4096 (7B-class O projection) the fold saves ~0.12 ms per launch against
+    // k_rmsnorm, at K = 2048 (2B-class O projection) it costs ~0.2 ms more.
+    const bool fold_ffn = H * hd >= 4096;  // pre-FFN norm, after the O projection
+    const bool fold_attn = F >= 4096;      // pre-attention norm, after the down projection
     {
-        TraceScope ts(JNX_K_PACK, Nd * 6.0, s);
-        if ((st = pack_launch(g, vision, n_vision_rows, text_ids, n_text, bb->text_table,
-                              bb->vocab, d, w.x, w.status, s)))
-            return st;
+        const bool prep = fold_attn && bb->n_layers > 0;
+        TraceScope ts(JNX_K_PACK, Nd * (prep ? 8.0 : 6.0), s);
+        st = prep ? pack_prep_launch(g, vision, n_vision_rows, text_ids, n_text, bb->text_table,
+                                     bb->vocab, d, w.x, w.status, bb->layers[0].attn_norm, w.nrm,
+                                     w.ss, s)
+                  : pack_launch(g, vision, n_vision_rows, text_ids, n_text, bb->text_table,
+                                bb->vocab, d, w.x, w.status, s);
+        if (st) return st;
     }
     {
         TraceScope ts(JNX_K_ROPE_TABLE, (double)g->max_seqlen * hd * 4.0, s);
@@ -272,13 +283,6 @@ static jnx_status backbone_forward(const jnx_backbone* bb, const jnx_group* g,
         attn_flops += 4.0 * L * L * H * hd;
     }
 
-    // Fold an RMSNorm into the residual GEMM before it only where that GEMM's
-    // K loop is long enough to hide the extra epilogue work (writing y and
-    // the sums of squares).  Measured on GB300: at K = 4096 (7B-class O
-    // projection) the fold saves ~0.12 ms per launch against k_rmsnorm, at
-    // K = 2048 (2B-class O projection) it costs ~0.2 ms more.
-    const bool fold_ffn = H * hd >= 4096;  // pre-FFN norm, after the O projection
-    const bool fold_attn = F >= 4096;      // pre-attention norm, after the down projection
     auto save = [&](int l) -> jnx_status {
         if (!saved) return JNX_OK;
         return cudaMemcpyAsync(saved + (size_t)l * N * d, w.x, (size_t)N * d * sizeof(float),
@@ -290,13 +294,10 @@ static jnx_status backbone_forward(const jnx_backbone* bb, const jnx_group* g,
         const jnx_layer& L = bb->layers[l];
         if ((st = save(l))) return st;
         // attention sub-block.  A folded RMSNorm: the residual GEMM before it
-        // (or, for the first block, rms_prep) writes y = bf16(x * gamma) and
+        // (or, for the first block, the packer) writes y = bf16(x * gamma) and
         // the row's sums of x^2; the GEMM after it reads y and scales each
         // output row by rsqrt(mean(x^2) + eps).  Unfolded: k_rmsnorm.
-        if (l == 0 && fold_attn) {
-            TraceScope ts(JNX_K_RMSNORM, Nd * 6.0, s);
-            if ((st = rms_prep_launch(w.x, L.attn_norm, N, d, w.nrm, w.ss, s))) return st;
-        } else if (!fold_attn) {
+        if (!fold_attn) {
             TraceScope ts(JNX_K_RMSNORM, Nd * 6.0, s);
             if ((st = rmsnorm_launch(w.x, L.attn_norm, bb->eps, N, d, w.nrm, s))) return st;
         }

@@ -216,10 +216,12 @@ jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int 
 jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, const int* cu,
                              int S, int d, float* pooled, uint16_t* hidden, cudaStream_t s);
 
-// Folded RMSNorm, first half: y = bf16(x * gamma) [M, d] and per row and
-// 128-column block the sum of x^2 (ss [M, d / 128]).
-jnx_status rms_prep_launch(const float* x, const uint16_t* gamma, int M, int d, uint16_t* y,
-                           float* ss, cudaStream_t s);
+// The packer with the first block's folded RMSNorm's first half: also y = bf16(x *
+// gamma) [N, d] and, per row and 128-column block, the sum of x^2 (ss [N, d / 128]).
+jnx_status pack_prep_launch(const jnx_group* g, const uint16_t* vision, int64_t n_vision,
+                            const int32_t* text_ids, int64_t n_text, const uint16_t* table,
+                            int vocab, int d, float* x, int* status, const uint16_t* gamma,
+                            uint16_t* y, float* ss, cudaStream_t s);
 
 // (cos, sin) table for positions [0, max_pos) of head dim hd.
 jnx_status rope_table_launch(float2* tab, int max_pos, int hd, float theta, cudaStream_t s);

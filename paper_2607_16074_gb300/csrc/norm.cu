@@ -19,6 +19,18 @@ namespace jnx {
 // the fp32 residual stream.  The canonical packed batch is where the samples
 // of all tenants are concatenated (§4.3); gather_src comes from the plan.
 // ---------------------------------------------------------------------------
+// The bf16 source row of a gather index, null outside its buffer.
+__device__ __forceinline__ const uint16_t* pack_source(int src, const uint16_t* vision,
+                                                       int64_t n_vision, const int32_t* text_ids,
+                                                       int64_t n_text, const uint16_t* table,
+                                                       int vocab, int d) {
+    if (src >= 0) return src < n_vision ? vision + (size_t)src * d : nullptr;
+    const int64_t p = -(int64_t)src - 1;
+    if (p >= n_text) return nullptr;
+    const int id = text_ids[p];
+    return id >= 0 && id < vocab ? table + (size_t)id * d : nullptr;
+}
+
 __global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ gather, int n_tokens,
                                               const uint16_t* __restrict__ vision, int64_t n_vision,
                                               const int32_t* __restrict__ text_ids, int64_t n_text,
@@ -28,17 +40,8 @@ __global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ gather
     const int tok = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (tok >= n_tokens) return;
-    const int src = gather[tok];
-    const uint16_t* row = nullptr;
-    if (src >= 0) {
-        if (src < n_vision) row = vision + (size_t)src * d;
-    } else {
-        const int64_t p = -(int64_t)src - 1;
-        if (p < n_text) {
-            const int id = text_ids[p];
-            if (id >= 0 && id < vocab) row = table + (size_t)id * d;
-        }
-    }
+    const uint16_t* row =
+        pack_source(gather[tok], vision, n_vision, text_ids, n_text, table, vocab, d);
     if (row == nullptr && lane == 0) report(status, JNX_ERR_DEVICE_BOUNDS);
     float4* out = reinterpret_cast<float4*>(x + (size_t)tok * d);
     const int nchunk = d / 8;
@@ -116,58 +119,73 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
     }
 }
 
-// First half of a folded RMSNorm (the residual GEMM epilogue does the same for
-// every later norm): y = bf16(x * gamma) and, per row and 128-column block,
-// the sum of x^2; the consuming GEMM scales its output rows by
-// rsqrt(sum / d + eps).  One warp per row.
+// The packer with the first block's folded RMSNorm's first half (the residual
+// GEMM epilogue does the same for every later norm): beside x, y = bf16(x * gamma)
+// and, per row and 128-column block, the sum of x^2; the consuming GEMM scales its
+// output rows by rsqrt(sum / d + eps).  One warp per row.  Bound by HBM: 2 bytes
+// in, 6 out per element in one pass, where a packer and a kernel that read the
+// fp32 rows back moved 12 (65,725 rows x 4,096: 340 + 400 us, now 329).
 template <int V>
-__global__ void __launch_bounds__(256) k_rms_prep(const float* __restrict__ x,
-                                                  const uint16_t* __restrict__ gamma, int M,
-                                                  uint16_t* __restrict__ y, float* __restrict__ ss) {
+__global__ void __launch_bounds__(256)
+    k_pack_prep(const int32_t* __restrict__ gather, int n_tokens,
+                const uint16_t* __restrict__ vision, int64_t n_vision,
+                const int32_t* __restrict__ text_ids, int64_t n_text,
+                const uint16_t* __restrict__ table, int vocab, float* __restrict__ x, int* status,
+                const uint16_t* __restrict__ gamma, uint16_t* __restrict__ y,
+                float* __restrict__ ss) {
     pdl_entry();
-    constexpr int D = V * 128;
-    constexpr int P = D / 128;  // 128-column blocks: lane float4 i = b
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    constexpr int D = V * 128;  // lane float4 i = 128-column block i
+    const int tok = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (row >= M) return;
-    const float4* xr = reinterpret_cast<const float4*>(x + (size_t)row * D);
-    float4 v[V];
+    if (tok >= n_tokens) return;
+    const uint16_t* row =
+        pack_source(gather[tok], vision, n_vision, text_ids, n_text, table, vocab, D);
+    if (row == nullptr && lane == 0) report(status, JNX_ERR_DEVICE_BOUNDS);
+    uint2 w[V];
 #pragma unroll
-    for (int i = 0; i < V; ++i) v[i] = __ldg(xr + lane + 32 * i);
-#pragma unroll
-    for (int b = 0; b < P; ++b) {
-        float t = 0.f;
-#pragma unroll
-        t += v[b].x * v[b].x + v[b].y * v[b].y + v[b].z * v[b].z + v[b].w * v[b].w;
-        t = warp_sum(t);
-        if (lane == 0) ss[(size_t)row * P + b] = t;
-    }
-    uint2* orow = reinterpret_cast<uint2*>(y + (size_t)row * D);
+    for (int i = 0; i < V; ++i)
+        w[i] = row ? __ldg(reinterpret_cast<const uint2*>(row) + lane + 32 * i) : make_uint2(0u, 0u);
+    float4* xr = reinterpret_cast<float4*>(x + (size_t)tok * D);
+    uint2* yr = reinterpret_cast<uint2*>(y + (size_t)tok * D);
     const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
 #pragma unroll
     for (int i = 0; i < V; ++i) {
+        const float4 v = make_float4(__uint_as_float(w[i].x << 16),
+                                     __uint_as_float(w[i].x & 0xFFFF0000u),
+                                     __uint_as_float(w[i].y << 16),
+                                     __uint_as_float(w[i].y & 0xFFFF0000u));
+        xr[lane + 32 * i] = v;
+        float t = 0.f;
+        t += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        t = warp_sum(t);
+        if (lane == 0) ss[(size_t)tok * V + i] = t;
         const uint2 gg = __ldg(g2 + lane + 32 * i);
-        uint2 o;
-        o.x = pack_bf2(v[i].x * bf2f(gg.x & 0xFFFF), v[i].y * bf2f(gg.x >> 16));
-        o.y = pack_bf2(v[i].z * bf2f(gg.y & 0xFFFF), v[i].w * bf2f(gg.y >> 16));
-        orow[lane + 32 * i] = o;
+        yr[lane + 32 * i] =
+            make_uint2(pack_bf2(v.x * bf2f(gg.x & 0xFFFF), v.y * bf2f(gg.x >> 16)),
+                       pack_bf2(v.z * bf2f(gg.y & 0xFFFF), v.w * bf2f(gg.y >> 16)));
     }
 }
 
-jnx_status rms_prep_launch(const float* x, const uint16_t* gamma, int M, int d, uint16_t* y,
-                           float* ss, cudaStream_t s) {
-    if (M == 0) return JNX_OK;
-    const int grid = (M + 7) / 8;
+jnx_status pack_prep_launch(const jnx_group* g, const uint16_t* vision, int64_t n_vision,
+                            const int32_t* text_ids, int64_t n_text, const uint16_t* table,
+                            int vocab, int d, float* x, int* status, const uint16_t* gamma,
+                            uint16_t* y, float* ss, cudaStream_t s) {
+    if (g->n_tokens == 0) return JNX_OK;
+    auto launch = [&](auto k) {
+        pdl(k, (g->n_tokens + 7) / 8, 256, 0, s)(g->gather_src, g->n_tokens, vision, n_vision,
+                                                 text_ids, n_text, table, vocab, x, status, gamma,
+                                                 y, ss);
+    };
     switch (d) {
-        case 256: pdl(k_rms_prep<2>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
-        case 512: pdl(k_rms_prep<4>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
-        case 1024: pdl(k_rms_prep<8>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
-        case 2048: pdl(k_rms_prep<16>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
-        case 4096: pdl(k_rms_prep<32>, grid, 256, 0, s)(x, gamma, M, y, ss); break;
-        default: return fail(JNX_ERR_UNSUPPORTED, "rms prep: d=%d not in {256..4096}", d);
+        case 256: launch(k_pack_prep<2>); break;
+        case 512: launch(k_pack_prep<4>); break;
+        case 1024: launch(k_pack_prep<8>); break;
+        case 2048: launch(k_pack_prep<16>); break;
+        case 4096: launch(k_pack_prep<32>); break;
+        default: return fail(JNX_ERR_UNSUPPORTED, "pack: d=%d not in {256..4096}", d);
     }
     cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "rms prep: %s", cudaGetErrorString(e));
+    return e == cudaSuccess ? JNX_OK : fail(JNX_ERR_CUDA, "pack: %s", cudaGetErrorString(e));
 }
 
 jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int M, int d,
