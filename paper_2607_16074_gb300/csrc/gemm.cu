@@ -645,12 +645,9 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
     }
 }
 
-template <int EPI, bool LORA, int BN, class LG>
-__device__ __forceinline__ TileGeo tile_geo(int tile, int num_m, int num_n, const GemmParams& p,
-                                            const LG& lg) {
-    int mb, nb;
-    tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
-    TileGeo g;
+// The two column groups of tile column nb.
+template <int EPI, int BN>
+__device__ __forceinline__ void tile_columns(int nb, const GemmParams& p, TileGeo& g) {
     g.nb = nb;
     constexpr int HB = BN / 2;
     if (BN < 256 && EPI == EPI_ROPE) {  // BN <= hd: a slice of one head and its rotation partner
@@ -665,6 +662,15 @@ __device__ __forceinline__ TileGeo tile_geo(int tile, int num_m, int num_n, cons
         g.c0 = nb * BN;
         g.c1 = g.c0 + HB;
     }
+}
+
+template <int EPI, bool LORA, int BN, class LG>
+__device__ __forceinline__ TileGeo tile_geo(int tile, int num_m, int num_n, const GemmParams& p,
+                                            const LG& lg) {
+    int mb, nb;
+    tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
+    TileGeo g;
+    tile_columns<EPI, BN>(nb, p, g);
     if constexpr (LORA) {
         int sg = 0;
         while (sg + 1 < lg.n_seg && lg.seg_tile0[sg + 1] <= mb) ++sg;
@@ -676,6 +682,20 @@ __device__ __forceinline__ TileGeo tile_geo(int tile, int num_m, int num_n, cons
         g.row0 = mb * gemm::BM;
         g.row_end = min(g.row0 + gemm::BM, p.M);
     }
+    return g;
+}
+
+// One CTA's rows of a pair's 256-row tile, and the tile's columns.
+template <int EPI, int BN>
+__device__ __forceinline__ TileGeo pair_geo(int tile, int num_m, int num_n, const GemmParams& p,
+                                            uint32_t rank) {
+    int mb, nb;
+    tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
+    TileGeo g;
+    tile_columns<EPI, BN>(nb, p, g);
+    g.seg = 0;
+    g.row0 = mb * 256 + (int)rank * 128;
+    g.row_end = min(g.row0 + 128, p.M);
     return g;
 }
 
@@ -974,8 +994,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
 }
 
 // ---------------------------------------------------------------------------
-// The same GEMM on CTA pairs: tiles of 256 x 256 shared by the two SMs of a
-// cluster.  Each CTA stages its 128 A rows and its 128 of the tile's 256 B rows;
+// The same GEMM on CTA pairs: tiles of 256 x BN shared by the two SMs of a
+// cluster.  Each CTA stages its 128 A rows and its half of the tile's B rows;
 // the leader's MMA warp issues M = 256 instructions over both CTAs' operands,
 // and each CTA's epilogue warps take its own 128 accumulator rows.
 //
@@ -986,6 +1006,9 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
 // instead of four, and the MMAs bound it.  Single-CTA tiles against
 // pairs: 8,192 x 4,096 x K 4,096 with the residual 187 -> 162 us (1,696 TFLOP/s),
 // GeGLU gate/up of 4,800 rows x N 32,768 x K 2,048 364 -> 323 us (1,994).
+// Tiles of 256 x 128 (24 KB a step and CTA, eight stages) are for the few rows that
+// a chain of K steps bounds: 607 x 2,048 x K 16,384 with the residual 56.4 us in lone
+// 128 x 128 tiles, 47.2 here.
 //
 // Barriers: `full` (leader only) counts both CTAs' bytes; `empty` and `tfull`
 // are signalled in both CTAs by the leader's commits; `tempty` (leader only)
@@ -993,21 +1016,26 @@ __global__ void __launch_bounds__(64 + 32 * EW, BN == 256 ? 1 : 2)
 // so no barrier, operand or accumulator goes away under its peer.
 // ---------------------------------------------------------------------------
 namespace pair {
-constexpr int BM = 256, BN = 256, BK = 64, STAGES = 6;
-constexpr int HALF_BYTES = 128 * BK * 2;         // one operand of one CTA's stage
-constexpr int STAGE_BYTES = 2 * HALF_BYTES;
-constexpr int smem_bytes(int ew) {
-    return STAGES * STAGE_BYTES + 1024 + 256 + (ew == 8 ? 8 * gemm::STG_SLOT_EW8 : gemm::STG_BYTES);
+constexpr int BM = 256, BK = 64;
+constexpr int A_BYTES = 128 * BK * 2;  // one CTA's rows of a stage
+constexpr int stages(int bn) { return bn == 256 ? 6 : 8; }
+constexpr int stage_bytes(int bn) { return A_BYTES + bn / 2 * BK * 2; }
+constexpr int smem_bytes(int bn, int ew) {
+    return stages(bn) * stage_bytes(bn) + 1024 + 256 +
+           (ew == 8 ? 8 * gemm::STG_SLOT_EW8 : gemm::STG_BYTES);
 }
-static_assert(smem_bytes(8) <= 227 * 1024, "shared memory per CTA");
-constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
+static_assert(smem_bytes(256, 8) <= 227 * 1024 && smem_bytes(128, 4) <= 227 * 1024,
+              "shared memory per CTA");
 }  // namespace pair
 
-template <int EPI, int EW>
+template <int EPI, int EW, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
     k_gemm_pair(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                 GemmParams p) {
-    using namespace pair;
+    using pair::A_BYTES;
+    using pair::BK;
+    constexpr int STAGES = pair::stages(BN), STAGE_BYTES = pair::stage_bytes(BN);
+    constexpr uint32_t IDESC = idesc_bf16_f32(pair::BM, BN);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1041,7 +1069,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
     }
     pdl_entry();  // TMEM is taken once the grid ahead has given its own back
     if (warp == 1) {
-        tmem_alloc_pair(tmem_slot, 512);
+        tmem_alloc_pair(tmem_slot, 2 * BN);
         tmem_relinquish_pair();
     }
     if (warp == 0 && lane == 0) {
@@ -1053,7 +1081,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
     tc_fence_after();
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
-    const int num_m = (p.M + BM - 1) / BM;
+    const int num_m = (p.M + pair::BM - 1) / pair::BM;
     const int num_n = p.N / BN;
     const int num_k = p.K / BK;
     const int num_tiles = num_m * num_n;
@@ -1065,9 +1093,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
         bool ok = true;
         for (int tile = first; ok && tile < num_tiles && !__any_sync(0xffffffffu, *abort_flag);
              tile += step) {
-            int mb, nb;
-            tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
-            const int arow = mb * BM + (int)rank * 128, brow = nb * BN + (int)rank * 128;
+            const TileGeo g = pair_geo<EPI, BN>(tile, num_m, num_n, p, rank);
+            const int brow = rank ? g.c1 : g.c0;
             for (int kb = 0; kb < num_k; ++kb) {
                 if (!mbar_wait_warp(&empty[stage], phase ^ 1)) {
                     ok = false;
@@ -1077,8 +1104,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
                     uint8_t* sa = smem + stage * STAGE_BYTES;
                     const uint32_t bar = map_rank(&full[stage], 0);
                     if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE_BYTES);
-                    tma_load_2d_pair(sa, &ta, kb * BK, arow, bar);
-                    tma_load_2d_pair(sa + HALF_BYTES, &tb, kb * BK, brow, bar);
+                    tma_load_2d_pair(sa, &ta, kb * BK, g.row0, bar);
+                    tma_load_2d_pair(sa + A_BYTES, &tb, kb * BK, brow, bar);
                 }
                 __syncwarp();
                 if (++stage == STAGES) {
@@ -1096,7 +1123,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
         uint32_t phase = 0;
         bool ok = true;
         const uint32_t a_lo = sw128_desc_lo(smem_u32(smem));
-        const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + HALF_BYTES);
+        const uint32_t b_lo = sw128_desc_lo(smem_u32(smem) + A_BYTES);
         for (int tile = first; ok && tile < num_tiles && !__any_sync(0xffffffffu, *abort_flag);
              tile += step, ++local) {
             const int acc = local & 1;
@@ -1149,15 +1176,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
         int local = 0;
         for (int tile = first; tile < num_tiles; tile += step, ++local) {
             const int acc = local & 1;
-            int mb, nb;
-            tile_coords(tile, num_m, num_n, p.group_m, mb, nb);
-            TileGeo g;
-            g.nb = nb;
-            g.seg = 0;
-            g.c0 = nb * BN;
-            g.c1 = g.c0 + 128;
-            g.row0 = mb * BM + (int)rank * 128;
-            g.row_end = min(g.row0 + 128, p.M);
+            const TileGeo g = pair_geo<EPI, BN>(tile, num_m, num_n, p, rank);
             const int row_base = g.row0 + q * 32;
             if constexpr (EPI == EPI_GLU_DM) {
                 // this thread's dm for the tile into L2 while its K loop runs
@@ -1171,7 +1190,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
                 break;
             }
             tc_fence_after();
-            epilogue_tile<EPI, EW == 8 ? 4 : 8, 256>(
+            epilogue_tile<EPI, EW == 8 ? BN / 64 : BN / 32, BN>(
                 tmem_base + acc * BN + ((uint32_t)(q * 32) << 16), stg, lane, row_base, g.row_end,
                 g, p, cb);
             tc_fence_before();
@@ -1189,7 +1208,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
     __syncthreads();
     cluster_sync_all();
     tc_fence_after();
-    if (warp == 1) tmem_dealloc_pair(tmem_base, 512);
+    if (warp == 1) tmem_dealloc_pair(tmem_base, 2 * BN);
 }
 
 // ---------------------------------------------------------------------------
@@ -1652,43 +1671,42 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
     return e;
 }
 
-// Width of a launch's output tiles: the one with the least estimated time,
-// (tiles an SM works through) x (its time per 64-deep K step).  The step times
-// are GB300's in microseconds, from launches of 8 to 10,000 tiles (K = 2,048 to
-// 16,384): `alone` where every tile has an SM of its own, `two` for a round of
-// two narrow tiles sharing one, which is how a narrow launch of more tiles than
-// SMs runs.  A 256-wide tile is faster per column, so narrower ones win only
-// where it leaves SMs idle: 607 rows x N 2,048 x K 16,384 takes 96 us in 40 wide
-// tiles, 59 in 80 of 128 and 76 in 160 of 64; 300 rows 94, 57 and 47; 4,800 rows
-// 190, 235 and 351.  A pair's tile (plain launches only) takes 0.32 for the same
-// work per SM as a wide one's 0.355 (0.385 alone), so it wins wherever its tiles
-// divide as well over the SMs: 2,400 rows x N 32,768 177 us against 188, but x N
-// 2,048 33 against 23.  RoPE needs a tile within one head, a folded norm's sums of
-// squares one of 128 columns; the GLU backward with dm has wide tiles only.
-constexpr int kPairTile = 512;
+// A launch's output tiles: the form with the least estimated time, `fixed` (the
+// launch, the first loads, the last tile's epilogue) + (rounds of tiles an SM works
+// through) x (K / 64 steps) x the step.  GB300's times in microseconds, fitted over
+// 42 launches of 8 to 10,000 tiles (K = 1,024 to 16,384; the picks lose 1 % to the
+// best form): `alone` where every tile has its own SM (or pair), `busy` otherwise,
+// which for a narrow tile is a round of two CTAs an SM.  Wide tiles are faster per
+// column, so narrower ones win only where wide ones leave SMs idle, and pairs wherever
+// they divide as well over the SMs.  N 2,048 x K 16,384, in the order of the table:
+// 300 rows 92, 79, 46, 55 and 45 us; 607 rows 93, 80, 47, 56 and 73; 2,400 rows 97,
+// 169, 142, 112 and 167; and 1,000 rows x N 32,768 x K 2,048 86, 75, 86, 93 and 131.
+// RoPE needs a tile within one head, a folded norm's sums of squares one of 128
+// columns; the GLU backward with dm has wide tiles only, other operands no pairs.
+constexpr int kPairTile = 512, kPairNarrow = 384;  // a pair's tiles of 256 and of 128 columns
 
 static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
+    static const struct { int form, bn, rows, per_sm; double fixed, alone, busy; } kForms[] = {
+        {256, 256, 1, 1, 6.1, 0.34, 0.345},
+        {kPairTile, 256, 2, 1, 9.4, 0.273, 0.295},
+        {kPairNarrow, 128, 2, 1, 6.9, 0.157, 0.17},
+        {128, 128, 1, 2, 5.3, 0.197, 0.395},
+        {64, 64, 1, 2, 4.8, 0.156, 0.32}};
     const int sms = num_sms();
-    auto rounds = [](long long tiles, int slots) { return (double)((tiles + slots - 1) / slots); };
-    const long long wide = (long long)m_tiles * (p.N / 256);
+    const bool wide_only = p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn);
     int best = 256;
-    double least = wide <= sms ? 0.385 : rounds(wide, sms) * 0.355;
-    if (pairs) {
-        const double t = rounds((long long)((m_tiles + 1) / 2) * (p.N / 256), sms / 2) * 0.32;
+    double least = 1e30;
+    for (const auto& f : kForms) {
+        if (f.rows == 2 && !pairs) continue;
+        if (f.bn < 256 && (wide_only || (p.epi == EPI_ROPE && f.bn > p.hd) ||
+                           (p.norm_gamma && f.bn < 128)))
+            continue;
+        const long long tiles = (long long)((m_tiles + f.rows - 1) / f.rows) * (p.N / f.bn);
+        const int slots = sms / f.rows * f.per_sm;
+        const double step = tiles <= sms / f.rows ? f.alone : (tiles + slots - 1) / slots * f.busy;
+        const double t = f.fixed + step * (p.K / gemm::BK);
         if (t < least) {
-            best = kPairTile;
-            least = t;
-        }
-    }
-    if (p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn)) return best;
-    static const struct { int bn; double alone, two; } kNarrow[] = {{128, 0.225, 0.40},
-                                                                     {64, 0.18, 0.335}};
-    for (const auto& w : kNarrow) {
-        if ((p.epi == EPI_ROPE && w.bn > p.hd) || (p.norm_gamma && w.bn < 128)) continue;
-        const long long tiles = (long long)m_tiles * (p.N / w.bn);
-        const double t = tiles <= sms ? w.alone : rounds(tiles, 2 * sms) * w.two;
-        if (t < least) {
-            best = w.bn;
+            best = f.form;
             least = t;
         }
     }
@@ -1725,18 +1743,18 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const
     return cudaGetLastError();
 }
 
-template <int EPI, int EW>
+template <int EPI, int EW, int BN>
 static cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, GemmParams p,
                                cudaStream_t s) {
-    constexpr int smem = pair::smem_bytes(EW);
+    constexpr int smem = pair::smem_bytes(BN, EW);
     p.group_m = std::max(1, p.group_m / 2);  // row blocks of 256
-    const long long tiles = (long long)((p.M + pair::BM - 1) / pair::BM) * (p.N / pair::BN);
+    const long long tiles = (long long)((p.M + pair::BM - 1) / pair::BM) * (p.N / BN);
     const int grid = 2 * (int)std::min<long long>(tiles, num_sms() / 2);
     static std::atomic<uint64_t> attr{0};
     cudaError_t e =
-        set_smem_limit(reinterpret_cast<const void*>(k_gemm_pair<EPI, EW>), smem, attr);
+        set_smem_limit(reinterpret_cast<const void*>(k_gemm_pair<EPI, EW, BN>), smem, attr);
     if (e != cudaSuccess) return e;
-    pdl(k_gemm_pair<EPI, EW>, grid, 64 + 32 * EW, smem, s)(ta, tb, p);
+    pdl(k_gemm_pair<EPI, EW, BN>, grid, 64 + 32 * EW, smem, s)(ta, tb, p);
     return cudaGetLastError();
 }
 
@@ -1745,8 +1763,10 @@ template <int EPI, bool LORA, class LG, int EW = 4, bool BMN = false>
 static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
                               const GemmParams& p, int bn, long long tiles, cudaStream_t s) {
     if constexpr (!LORA)
-        if (bn == kPairTile) return launch_pair<EPI, EW>(ta, tb, p, s);
+        if (bn == kPairTile) return launch_pair<EPI, EW, 256>(ta, tb, p, s);
     if constexpr (EW == 4) {
+        if constexpr (!LORA)
+            if (bn == kPairNarrow) return launch_pair<EPI, EW, 128>(ta, tb, p, s);
         if (bn == 64) return launch_bn<EPI, LORA, LG, EW, 64, BMN>(ta, tb, lg, p, tiles, s);
         if (bn == 128) return launch_bn<EPI, LORA, LG, EW, 128, BMN>(ta, tb, lg, p, tiles, s);
     }
@@ -1754,7 +1774,10 @@ static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, cons
 }
 
 // Box rows of the two operands' tensor maps at tile width bn.
-static int b_box(int bn) { return bn == kPairTile ? 128 : bn == 256 ? 256 : bn / 2; }
+static int b_box(int bn) {
+    if (bn == kPairTile || bn == kPairNarrow) return bn == kPairTile ? 128 : 64;
+    return bn == 256 ? 256 : bn / 2;
+}
 
 // Rows of A a narrow stage holds: the tallest tile's rows, in powers of two.
 static int a_box(int bn, int most_rows) {

@@ -1,6 +1,7 @@
 """The GEMM's tile widths against each other and the oracle: a launch picks its
 tiles by its size, and a row's result must have the same bits in all of them
-(M = 1 .. 607 rows take the narrow ones here, the larger the wide ones)."""
+(at K = 320 the fewer rows take the narrow ones, the more the wide ones; at K = 4,160
+607 rows take a CTA pair's narrow ones and the full rows its wide ones)."""
 import pytest
 import torch
 
@@ -12,7 +13,8 @@ from tests.helpers import check_bf16_out, rel_err
 pytestmark = pytest.mark.gpu
 
 ROWS = 5000
-N, K = 2048, 320  # five K steps: shorter than, and not a multiple of, the rings
+N = 2048
+KS = 320, 4160  # five K steps, shorter than the rings, and 65: no multiple of them
 
 
 def _run(A, W, rows, epi, x0, pos, hd, act):
@@ -22,7 +24,7 @@ def _run(A, W, rows, epi, x0, pos, hd, act):
            }.get(epi, lambda: torch.zeros((rows, N), dtype=torch.bfloat16, device="cuda"))()
     ws = torch.zeros(J.lib().jnx_op_gemm_workspace_bytes(900, hd or 64), dtype=torch.uint8,
                      device="cuda")
-    rope = epi == J.JNX_EPI_ROPE
+    rope, K = epi == J.JNX_EPI_ROPE, A.shape[1]
     J.check(J.lib().jnx_op_gemm(A.data_ptr(), W.data_ptr(), rows, N, K, epi, out.data_ptr(),
                                 out.shape[1], pos.data_ptr(), 900 if rope else 0,
                                 N // 2 if rope else 0, hd, 10000.0, act, ws.data_ptr(), ws.numel(),
@@ -31,11 +33,12 @@ def _run(A, W, rows, epi, x0, pos, hd, act):
     return out
 
 
+@pytest.mark.parametrize("K", KS)
 @pytest.mark.parametrize("epi,hd,act", [
     (J.JNX_EPI_F32, 0, 0), (J.JNX_EPI_BF16, 0, 0), (J.JNX_EPI_RESID, 0, 0), (J.JNX_EPI_GLU, 0, 0),
     (J.JNX_EPI_GLU, 0, 1), (J.JNX_EPI_GLU_SAVE, 0, 0), (J.JNX_EPI_ROPE, 64, 0),
     (J.JNX_EPI_ROPE, 128, 0), (J.JNX_EPI_ROPE, 256, 0)])
-def test_rows_have_the_same_bits_in_every_tile_width(epi, hd, act):
+def test_rows_have_the_same_bits_in_every_tile_width(epi, hd, act, K):
     A, W = randn_bf16((ROWS, K), 1), randn_bf16((N, K), 2, 0.05)
     x0 = torch.randn((ROWS, N), generator=torch.Generator().manual_seed(3)).cuda()
     pos = (torch.arange(ROWS, dtype=torch.int32) * 7 % 900).cuda()
