@@ -202,6 +202,15 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)map) : "memory");
 }
 
+// A box of a tensor map into L2: a hint that reads no data, so it may run before
+// pdl_entry() whatever the grid ahead still writes.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int32_t x, int32_t y) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                     (uint64_t)map),
+                 "r"(x), "r"(y)
+                 : "memory");
+}
+
 // L2 eviction policy for data that is touched once (a streamed output, the
 // residual read-modify-write): its lines go first, so they do not push out
 // operand tiles that other CTAs are still reusing.
