@@ -290,6 +290,12 @@ __device__ __forceinline__ void mma4(float (&c)[4], const uint32_t (&a)[4], uint
 // tile w / KS (16 rows) and the w % KS-th of the 64 / KS-key slices of every
 // staged tile, with its own running maximum and sum; the KS slices are
 // merged at the end in slice order.
+// A sampling call's CTAs are few (32 for two samples) and each is a chain of five
+// tiles, so the loads' latency bounds it: a ring of four tiles, three in flight
+// beside the query rows, and one barrier a tile
+// (two tiles, the queries first: 1,932 us a call of 40 such launches, 1,892 now).
+constexpr int kFwdRing = 4;
+constexpr int kFwdSmem = kFwdRing * 2 * kTileB + kMaxC * kRowB;
 template <int KS>
 __global__ void __launch_bounds__(128) k_flow_attn_fwd(const uint16_t* __restrict__ qkv,
                                                        const uint16_t* __restrict__ kvc,
@@ -298,40 +304,37 @@ __global__ void __launch_bounds__(128) k_flow_attn_fwd(const uint16_t* __restric
                                                        float* __restrict__ lse) {
     pdl_entry();
     constexpr int NK = kKT / KS, NT = NK / 8;
-    __shared__ __align__(128) uint8_t sbuf[4 * kTileB];  // (K, V) x 2 buffers
+    extern __shared__ __align__(128) uint8_t sbuf[];  // the ring's (K, V), the query rows
     const int s = blockIdx.x, h = blockIdx.y, C = dd.C, dm = dd.dm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
     const int MT = (C + 15) >> 4, mt = warp / KS, ks = warp % KS;
     const bool active = mt < MT;
     const int ctx0 = cu[s], L = cu[s + 1] - ctx0, act0 = s * C, nkeys = L + C;
     const uint32_t sb = smem_u32(sbuf);
-    load_rows(sb, qkv + (size_t)act0 * 3 * dm + h * kHd, 3 * dm, C, MT * 16);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
+    const uint32_t sq = sb + kFwdRing * 2 * kTileB;
+    const int ntiles = (nkeys + kKT - 1) / kKT;
+    auto load_tile = [&](int t) {  // one group a call, empty past the last tile
+        const uint32_t nk = sb + t % kFwdRing * 2 * kTileB;
+        if (t < ntiles) load_kv_tile(nk, nk + kTileB, t * kKT, nkeys, L, kvc, ctx0, qkv, act0, dm, h);
+        cp_async_commit();
+    };
+    load_rows(sq, qkv + (size_t)act0 * 3 * dm + h * kHd, 3 * dm, C, MT * 16);
+    for (int t = 0; t < kFwdRing - 1; ++t) load_tile(t);
     uint32_t qa[4][4];
-    if (active)
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) ld_a(sb, mt * 16, kk, lane, qa[kk]);
-    __syncthreads();
     float oacc[8][4];
 #pragma unroll
     for (int i = 0; i < 8; ++i) oacc[i][0] = oacc[i][1] = oacc[i][2] = oacc[i][3] = 0.f;
     float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.f, 0.f};
     const float sc2 = kLog2e / sqrtf((float)kHd);
-    const int ntiles = (nkeys + kKT - 1) / kKT;
-    load_kv_tile(sb, sb + kTileB, 0, nkeys, L, kvc, ctx0, qkv, act0, dm, h);
-    cp_async_commit();
     for (int t = 0; t < ntiles; ++t) {
-        const uint32_t kb = sb + (t & 1) * 2 * kTileB, vb = kb + kTileB;
-        if (t + 1 < ntiles) {
-            const uint32_t nk = sb + ((t + 1) & 1) * 2 * kTileB;
-            load_kv_tile(nk, nk + kTileB, (t + 1) * kKT, nkeys, L, kvc, ctx0, qkv, act0, dm, h);
-        }
-        cp_async_commit();
-        cp_async_wait<1>();
-        __syncthreads();
+        const uint32_t kb = sb + t % kFwdRing * 2 * kTileB, vb = kb + kTileB;
+        cp_async_wait<kFwdRing - 2>();
+        __syncthreads();  // tile t is there, and every warp is done with tile t - 1
+        load_tile(t + kFwdRing - 1);
         if (active) {
+            if (t == 0)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) ld_a(sq, mt * 16, kk, lane, qa[kk]);
             float sacc[NT][4];
 #pragma unroll
             for (int i = 0; i < NT; ++i) sacc[i][0] = sacc[i][1] = sacc[i][2] = sacc[i][3] = 0.f;
@@ -392,8 +395,8 @@ __global__ void __launch_bounds__(128) k_flow_attn_fwd(const uint16_t* __restric
                 }
             }
         }
-        __syncthreads();
     }
+    __syncthreads();  // the ring is free for the merge
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         lrow[i] += __shfl_xor_sync(0xffffffffu, lrow[i], 1);
@@ -1121,14 +1124,15 @@ jnx_status flow_attn_fwd_launch(const uint16_t* qkv, const uint16_t* kvc, const 
                                 cudaStream_t s) {
     if (S == 0) return JNX_OK;
     const int MT = (d.C + 15) / 16;
-    const dim3 grid(S, d.nh);
-    if (MT == 1)
-        pdl(k_flow_attn_fwd<4>, grid, 128, 0, s)(qkv, kvc, cu, d, o, lse);
-    else if (MT == 2)
-        pdl(k_flow_attn_fwd<2>, grid, 128, 0, s)(qkv, kvc, cu, d, o, lse);
-    else
-        pdl(k_flow_attn_fwd<1>, grid, 128, 0, s)(qkv, kvc, cu, d, o, lse);
-    return last("flow attention");
+    auto go = [&](auto kernel, std::atomic<uint64_t>& attr) {
+        if (set_smem_limit(reinterpret_cast<const void*>(kernel), kFwdSmem, attr) == cudaSuccess)
+            pdl(kernel, dim3(S, d.nh), 128, kFwdSmem, s)(qkv, kvc, cu, d, o, lse);
+        return last("flow attention");
+    };
+    static std::atomic<uint64_t> a4{0}, a2{0}, a1{0};  // per kernel, one bit per device
+    return MT == 1   ? go(k_flow_attn_fwd<4>, a4)
+           : MT == 2 ? go(k_flow_attn_fwd<2>, a2)
+                     : go(k_flow_attn_fwd<1>, a1);
 }
 
 template <int NQ>
