@@ -8,7 +8,7 @@
 // P is recomputed from the forward's saved log2-sum-exp of each row, so no
 // row max or normalisation is needed here.
 //
-// One kernel template k_attn_bwd<HD, MODE> runs one pass:
+// One kernel k_attn_bwd<HD> runs the passes of its head dim (bwd_pass<HD, MODE>):
 //   DQ   outer tile = 128 queries of head h, inner loop over the sample's
 //        64-key tiles:       S = Q K^T, dP = dO V^T, dS, dQ += dS K
 //   DKV  outer tile = 128 keys of K/V head g, inner loop over (query head
@@ -16,14 +16,20 @@
 //        dS^T, dK += dS^T Q, dV += P^T dO       (head dims 64 / 128)
 //   DK   as DKV without dV; DV as DKV without dP and dK (head dim 256,
 //        whose two 256-column accumulators do not fit TMEM together)
+// A CTA claims items from one queue of all passes, those of the keys before those of
+// the queries, so the long ones start first and the short ones fill the end.  A launch
+// a pass, its items dealt out in turn, left SMs idle at the end of each, and every
+// warp looked each item up for itself (24,000 tokens with the forward: 995 -> 826 us
+// at head dim 256, 1,344 -> 1,332 at 128, 571 -> 563 at 64).
 // Each pass accumulates in TMEM and writes its rows once, so no atomics and
 // a fixed summation order: a sample's gradients do not depend on where it
 // sits in the packed batch.
 //
 // Warp roles (320 threads, one CTA per SM, persistent over work items):
-//   warp 0     TMA producer: the item's outer operands (A1, and A2 when the
-//              pass has a dP product) into one buffer, inner operands B1 /
-//              B2 through rings that run on from item to item
+//   warp 0     claims the items and hands them to the other warps; TMA producer:
+//              the item's outer operands (A1, and A2 when the pass has a dP
+//              product) into one buffer, inner operands B1 / B2 through rings that
+//              run on from item to item
 //   warp 1     MMA issuer: the two score-shaped products of inner tile j
 //              into score buffer j % 2 (S at column 64 b, dP at 128 + 64 b),
 //              issued two tiles ahead of the accumulating products, which
@@ -57,7 +63,7 @@ namespace abwd {
 constexpr int BM = 128;  // outer rows per item
 constexpr int BN = 64;   // inner rows per tile
 enum { DQ = 0, DKV = 1, DK = 2, DV = 3 };
-constexpr int kBars = 23;
+constexpr int kBars = 27;  // of one pass; each pass of a launch has its own
 constexpr int EW = 8;    // elementwise warps: two per TMEM lane quarter, one column half each
 }  // namespace abwd
 
@@ -82,70 +88,76 @@ struct AttnBwdCfg {
     static constexpr int OFF_A2 = OB;
     static constexpr int OFF_B1 = NEED_DP ? 2 * OB : OB;
     static constexpr int OFF_B2 = OFF_B1 + NB1 * IB;
-    static constexpr int OFF_BAR = OFF_B2 + NB2 * IB;
-    static constexpr int SMEM = OFF_BAR + abwd::kBars * 8 + 16 + 1024;
+    static constexpr int END = OFF_B2 + NB2 * IB;
     static constexpr uint32_t S_COL = 0;        // score buffer b at b * BN
     static constexpr uint32_t DP_COL = 2 * BN;  // dP buffer b at 2 BN + b * BN
     static constexpr uint32_t ACC_COL = 256;
-    static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
     static_assert(ACC_COL + NACC * HD <= 512, "TMEM columns");
     static_assert(MODE != abwd::DKV || HD <= 128, "dK and dV together need head dim <= 128");
+};
+
+// The passes of a head dim, in the queue's order, and a launch's shared memory.
+template <int HD>
+struct AttnBwdPasses {
+    static constexpr int N = HD == 256 ? 3 : 2;
+    static constexpr int KEY = HD == 256 ? abwd::DK : abwd::DKV;  // the first
+    static constexpr int K_END = AttnBwdCfg<HD, KEY>::END, Q_END = AttnBwdCfg<HD, abwd::DQ>::END;
+    static constexpr int OFF_BAR = K_END > Q_END ? K_END : Q_END;  // DV stages less than DK
+    static constexpr int SMEM = OFF_BAR + N * abwd::kBars * 8 + 48 + 1024;
+    static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
 };
 
 struct BwdItems {
     const int2* list;  // (sample, 128-row tile), most expensive first
     int n;
+    int* claimed;      // items taken beyond the grid's first, 0 at launch
 };
 
+// A launch's arguments beyond the tensor maps.
+struct BwdArgs {
+    const int* cu;
+    BwdItems items;
+    int H, Hkv;
+    float scale_log2, scale;
+    const float *lse, *Dsum;
+    const int* pos;
+    const float2* rope;
+    int rope_ld;
+    uint16_t* dqkv;
+    int ldq;
+    int* status;
+};
+
+// Item w of a pass: list entry w / HP, head (query head for DQ, K/V head otherwise)
+// w % HP.  L < 0: past the pass's last.
 struct BwdWork {
     int tile, hp, start, L;
-    bool valid;
 };
 
-// Item w: list entry w / HP, head (query head for DQ, K/V head otherwise) w % HP.
-__device__ __forceinline__ BwdWork bwd_fetch(const BwdItems& it, const int* __restrict__ cu, int HP,
-                                             int w, int n_work) {
-    BwdWork a{0, 0, 0, 0, false};
-    if (w >= n_work) return a;
-    a.hp = w % HP;
-    const int2 e = it.list[w / HP];
-    a.tile = e.y;
-    a.start = cu[e.x];
-    a.L = cu[e.x + 1] - a.start;
-    a.valid = a.tile * abwd::BM < a.L;
-    return a;
-}
-
-// The item as warp-uniform values.
-__device__ __forceinline__ BwdWork bwd_uniform(BwdWork a) {
-    a.tile = warp_uniform(a.tile);
-    a.hp = warp_uniform(a.hp);
-    a.start = warp_uniform(a.start);
-    a.L = warp_uniform(a.L);
-    a.valid = warp_uniform(a.valid);
-    return a;
-}
-
+// The items of one pass, [q0, q0 + items) of the queue.  Warp 0 passes its claim and
+// gets back the first one past the pass.
 template <int HD, int MODE>
-__global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
-    k_attn_bwd(const __grid_constant__ CUtensorMap t_qkv_o, const __grid_constant__ CUtensorMap t_qkv_i,
-               const __grid_constant__ CUtensorMap t_do_o, const __grid_constant__ CUtensorMap t_do_i,
-               const int* __restrict__ cu, BwdItems items, int H, int Hkv, float scale_log2,
-               float scale, const float* __restrict__ lse, const float* __restrict__ Dsum,
-               const int* __restrict__ pos, const float2* __restrict__ rope, int rope_ld,
-               uint16_t* __restrict__ dqkv, int ldq, int* status) {
+__device__ __forceinline__ int bwd_pass(const CUtensorMap& t_qkv_o, const CUtensorMap& t_qkv_i,
+                                        const CUtensorMap& t_do_o, const CUtensorMap& t_do_i,
+                                        const BwdArgs& p, uint8_t* sm, uint64_t* bars,
+                                        volatile int* fail_flag, uint32_t tbase, int q0,
+                                        int claim) {
     using C = AttnBwdCfg<HD, MODE>;
     constexpr int BM = C::BM, BN = C::BN;
     constexpr int NCH = HD / 64;  // 64-column (128-byte) chunks of an operand row
     constexpr bool IS_DQ = MODE == abwd::DQ;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* sm = reinterpret_cast<uint8_t*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int H = p.H, Hkv = p.Hkv, rope_ld = p.rope_ld, ldq = p.ldq;
+    const int* __restrict__ cu = p.cu;
+    const float* __restrict__ lse = p.lse;
+    const float* __restrict__ Dsum = p.Dsum;
+    const int* __restrict__ pos = p.pos;
+    const float2* __restrict__ rope = p.rope;
+    uint16_t* __restrict__ dqkv = p.dqkv;
+    const float scale_log2 = p.scale_log2, scale = p.scale;
     uint8_t* sA1 = sm;
     uint8_t* sA2 = sm + C::OFF_A2;
     auto sB1 = [&](int b) { return sm + C::OFF_B1 + b * C::IB; };
     auto sB2 = [&](int b) { return sm + C::OFF_B2 + b * C::IB; };
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + C::OFF_BAR);
     uint64_t* o_full = bars + 0;
     uint64_t* o_empty = bars + 1;
     uint64_t* b1_full = bars + 2;   // [3]
@@ -158,29 +170,25 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
     uint64_t* acc_free = bars + 17;
     uint64_t* drain = bars + 18;
     uint64_t* xbar = bars + 19;  // [4] the two warps of a lane quarter have read a score tile
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + abwd::kBars);
-    volatile int* fail_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+    uint64_t* w_full = bars + 23;   // [2] an item is in its slot; at 25 [2]: its readers have it
+    uint64_t* w_empty = bars + 25;
+    volatile int* slot = fail_flag + 1;  // [2] items
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int group = H / Hkv;
     const int HP = IS_DQ ? H : Hkv;
-    const int n_work = items.n * HP;
-    if (tid == 0) {
-        for (int i = 0; i < abwd::kBars; ++i)
-            mbar_init(&bars[i], (i == 14 || i == 15 || i == 17) ? abwd::EW : i >= 19 ? 2 : 1);
-        *fail_flag = 0;
-        fence_barrier_init();
-        fence_proxy_async();
-    }
-    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
-    if (warp == 1) {
-        tmem_alloc(tmem_slot, 512);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tbase = warp_uniform(*tmem_slot);
+    const int n_work = p.items.n * HP;
+    // the next item as warp 0 hands it to the others
+    int seen = 0;
+    auto next_item = [&](bool& ok) -> BwdWork {
+        const int b = seen & 1;
+        if (!(ok = mbar_wait_warp(&w_full[b], (seen >> 1) & 1))) return BwdWork{0, 0, 0, -1};
+        const BwdWork a{warp_uniform(slot[4 * b]), warp_uniform(slot[4 * b + 1]),
+                        warp_uniform(slot[4 * b + 2]), warp_uniform(slot[4 * b + 3])};
+        if (elect_one()) mbar_arrive(&w_empty[b]);
+        __syncwarp();
+        ++seen;
+        return a;
+    };
     // inner tiles of an item
     auto n_inner = [&](int L) { return IS_DQ ? (L + BN - 1) / BN : group * ((L + BN - 1) / BN); };
 
@@ -195,6 +203,21 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                 tma_prefetch_desc(&t_do_i);
             }
             bool ok = true;
+            int told = 0;            // items handed out
+            auto tell = [&](const BwdWork& a) {
+                const int b = told & 1;
+                if (!mbar_wait_warp(&w_empty[b], ((told >> 1) & 1) ^ 1)) return false;
+                if (elect_one()) {
+                    slot[4 * b] = a.tile;
+                    slot[4 * b + 1] = a.hp;
+                    slot[4 * b + 2] = a.start;
+                    slot[4 * b + 3] = a.L;
+                    mbar_arrive(&w_full[b]);
+                }
+                __syncwarp();
+                ++told;
+                return true;
+            };
             int no = 0;              // outer tiles loaded
             uint32_t g1 = 0, g2 = 0;  // inner tiles loaded into each ring
             auto load_inner = [&](const CUtensorMap* map, uint8_t* dst, int col, int row,
@@ -207,35 +230,59 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                 }
                 __syncwarp();
             };
-            for (int w = blockIdx.x; w < n_work && ok && !__any_sync(0xffffffffu, *fail_flag); w += gridDim.x) {
-                const BwdWork a = bwd_uniform(bwd_fetch(items, cu, HP, w, n_work));
-                if (!a.valid) continue;
+            // The next item is claimed at an item's start, its list entry fetched with the
+            // second tile's loads and its rows with the third's, each a step later than
+            // what it needs was asked for: none of the three is waited for.
+            int2 entry = make_int2(0, 0);
+            int r0 = 0, r1 = 0;
+            auto fetch_entry = [&]() {
+                claim = __shfl_sync(0xffffffffu, claim, 0);
+                if (claim - q0 < n_work) entry = p.items.list[(claim - q0) / HP];
+            };
+            auto fetch_rows = [&]() {
+                if (claim - q0 < n_work) {
+                    r0 = cu[entry.x];
+                    r1 = cu[entry.x + 1];
+                }
+            };
+            fetch_entry();
+            fetch_rows();
+            while (claim - q0 < n_work) {
+                if (__any_sync(0xffffffffu, *fail_flag)) {
+                    ok = false;
+                    break;
+                }
+                const BwdWork a{warp_uniform(entry.y), warp_uniform((claim - q0) % HP),
+                                warp_uniform(r0), warp_uniform(r1 - r0)};
+                if (lane == 0) claim = (int)gridDim.x + atomicAdd(p.items.claimed, 1);
+                __syncwarp();
+                if (a.tile * BM >= a.L) {  // no rows
+                    fetch_entry();
+                    fetch_rows();
+                    continue;
+                }
+                if (!(ok = tell(a))) break;
                 const int row0 = a.start + a.tile * BM;
                 if (no > 0 && !(ok = mbar_wait_warp(o_empty, (no - 1) & 1))) break;
                 if (elect_one()) {
-                mbar_arrive_expect_tx(o_full, C::NEED_DP ? 2 * C::OB : C::OB);
-                if (IS_DQ) {
+                    mbar_arrive_expect_tx(o_full, C::NEED_DP ? 2 * C::OB : C::OB);
+                    const int k1 = (IS_DQ ? a.hp : H + a.hp) * HD;
+                    const int k2 = (IS_DQ ? a.hp : H + Hkv + a.hp) * HD;
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) {
-                        tma_load_2d(sA1 + c * BM * 128, &t_qkv_o, a.hp * HD + c * 64, row0, o_full);
-                        tma_load_2d(sA2 + c * BM * 128, &t_do_o, a.hp * HD + c * 64, row0, o_full);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < NCH; ++c) {
-                        tma_load_2d(sA1 + c * BM * 128, &t_qkv_o, (H + a.hp) * HD + c * 64, row0,
-                                    o_full);
+                        tma_load_2d(sA1 + c * BM * 128, &t_qkv_o, k1 + c * 64, row0, o_full);
                         if (C::NEED_DP)
-                            tma_load_2d(sA2 + c * BM * 128, &t_qkv_o, (H + Hkv + a.hp) * HD + c * 64,
+                            tma_load_2d(sA2 + c * BM * 128, IS_DQ ? &t_do_o : &t_qkv_o, k2 + c * 64,
                                         row0, o_full);
                     }
-                }
                 }
                 __syncwarp();
                 ++no;
                 const int n = n_inner(a.L);
                 const int nq = (a.L + BN - 1) / BN;
                 for (int j = 0; j < n && ok; ++j) {
+                    if (j == 1) fetch_entry();
+                    if (j == 2) fetch_rows();
                     int row, c1, c2;
                     const CUtensorMap* m2;
                     if (IS_DQ) {
@@ -260,7 +307,11 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                     load_inner(m2, sB2(s2), c2, row, &b2_full[s2]);
                     ++g2;
                 }
+                if (!ok) break;
+                if (n < 2) fetch_entry();
+                if (n < 3) fetch_rows();
             }
+            ok = ok && tell(BwdWork{0, 0, 0, -1});
             if (!ok) *fail_flag = 1;
             // teardown: every copy issued has landed before the CTA exits
             if (no > 0) mbar_wait_warp(o_full, (no - 1) & 1, 100000000LL);
@@ -342,9 +393,9 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                 if (elect_one()) tc_commit(bar);
                 __syncwarp();
             };
-            for (int w = blockIdx.x; w < n_work && ok && !__any_sync(0xffffffffu, *fail_flag); w += gridDim.x) {
-                const BwdWork a = bwd_uniform(bwd_fetch(items, cu, HP, w, n_work));
-                if (!a.valid) continue;
+            while (ok) {
+                const BwdWork a = next_item(ok);
+                if (a.L < 0 || __any_sync(0xffffffffu, *fail_flag)) break;
                 const int n = n_inner(a.L);
                 if (!(ok = mbar_wait_warp(o_full, no & 1))) break;
                 ++no;
@@ -412,10 +463,9 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
         uint32_t gs = 0;
         int items_done = 0;
         bool ok = true;
-        for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
-            if (__any_sync(0xffffffffu, *fail_flag != 0)) break;
-            const BwdWork a = bwd_fetch(items, cu, HP, w, n_work);
-            if (!a.valid) continue;
+        while (ok) {
+            const BwdWork a = next_item(ok);
+            if (a.L < 0 || __any_sync(0xffffffffu, *fail_flag != 0)) break;
             const int L = a.L, n = n_inner(L);
             const int nq = (L + BN - 1) / BN;
             const int r = a.tile * BM + quarter * 32 + lane;  // this thread's outer row
@@ -511,7 +561,7 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
                     // and read as position 0 (no rotation)
                     int pr = rv ? pos[grow] : 0;
                     if (pr < 0 || pr >= rope_ld) {
-                        if (rv) report(status, JNX_ERR_DEVICE_BOUNDS);
+                        if (rv) report(p.status, JNX_ERR_DEVICE_BOUNDS);
                         pr = 0;
                     }
 #pragma unroll 1
@@ -577,33 +627,96 @@ __global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
         }
         if (!ok) *fail_flag = 1;
     }
+    return claim;
+}
+
+template <int HD>
+__global__ void __launch_bounds__(64 + 32 * abwd::EW, 1)
+    k_attn_bwd(const __grid_constant__ CUtensorMap t_qkv_o, const __grid_constant__ CUtensorMap t_qkv_i,
+               const __grid_constant__ CUtensorMap t_do_o, const __grid_constant__ CUtensorMap t_do_i,
+               const __grid_constant__ BwdArgs p) {
+    using P = AttnBwdPasses<HD>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* sm = reinterpret_cast<uint8_t*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + P::OFF_BAR);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + P::N * abwd::kBars);
+    volatile int* fail_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);  // then the slots
+
+    const int warp = warp_uniform(threadIdx.x >> 5);
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < P::N * abwd::kBars; ++k) {
+            const int i = k % abwd::kBars;
+            mbar_init(&bars[k], i == 14 || i == 15 || i == 17 ? abwd::EW
+                                : i >= 25                     ? abwd::EW + 1
+                                : i >= 19 && i < 23           ? 2
+                                                              : 1);
+        }
+        *fail_flag = 0;
+        fence_barrier_init();
+        fence_proxy_async();
+    }
+    pdl_entry();  // TMEM is taken once the grid ahead has given its own back
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (*fail_flag && tid == 0) report(status, JNX_ERR_TIMEOUT);
+    const uint32_t tbase = warp_uniform(*tmem_slot);
+
+    // A pass leaves no copy, MMA or TMEM read of its own behind, so the next may
+    // reuse the buffers; its barriers are its own.
+    const int nk = p.items.n * p.Hkv;
+    bool failed;
+    auto end_pass = [&]() {
+        __syncwarp();
+        tc_fence_before();
+        failed = __syncthreads_or(*fail_flag);
+        tc_fence_after();
+    };
+    int claim = blockIdx.x, q0 = 0;
+    claim = bwd_pass<HD, P::KEY>(t_qkv_o, t_qkv_i, t_do_o, t_do_i, p, sm, bars, fail_flag, tbase,
+                                 q0, claim);
+    q0 += nk;
+    bars += abwd::kBars;
+    end_pass();
+    if constexpr (HD == 256) {
+        if (!failed) {
+            claim = bwd_pass<HD, abwd::DV>(t_qkv_o, t_qkv_i, t_do_o, t_do_i, p, sm, bars, fail_flag,
+                                           tbase, q0, claim);
+            q0 += nk;
+            bars += abwd::kBars;
+            end_pass();
+        }
+    }
+    if (!failed) {
+        bwd_pass<HD, abwd::DQ>(t_qkv_o, t_qkv_i, t_do_o, t_do_i, p, sm, bars, fail_flag, tbase, q0,
+                               claim);
+        end_pass();
+    }
+    if (failed && threadIdx.x == 0) report(p.status, JNX_ERR_TIMEOUT);
     if (warp == 1) tmem_dealloc(tbase, 512);
 }
 
-template <int HD, int MODE>
-static jnx_status launch_bwd(const CUtensorMap (&maps)[4], const int* cu, const BwdItems& it, int H,
-                             int Hkv, const float* lse, const float* D, const int* pos,
-                             const float2* rope, int rope_ld, uint16_t* dqkv, int ldq, int* status,
-                             cudaStream_t s) {
-    using C = AttnBwdCfg<HD, MODE>;
+template <int HD>
+static jnx_status launch_bwd(const CUtensorMap (&maps)[4], BwdArgs p, cudaStream_t s) {
+    constexpr int smem = AttnBwdPasses<HD>::SMEM;
     static std::atomic<uint64_t> attr{0};
-    if (set_smem_limit(reinterpret_cast<const void*>(k_attn_bwd<HD, MODE>), C::SMEM, attr) !=
-        cudaSuccess)
+    if (set_smem_limit(reinterpret_cast<const void*>(k_attn_bwd<HD>), smem, attr) != cudaSuccess)
         return fail(JNX_ERR_CUDA, "attention backward: smem attribute");
-    const int HP = MODE == abwd::DQ ? H : Hkv;
-    const long long n_work = (long long)it.n * HP;
-    if (n_work > 0x7FFFFFFFLL) return fail(JNX_ERR_UNSUPPORTED, "attention backward: too many items");
-    if (n_work == 0) return JNX_OK;
+    const int key_passes = AttnBwdPasses<HD>::N - 1;
+    const long long n_work = (long long)p.items.n * (key_passes * p.Hkv + p.H);
+    // (claims run past the last item by one for each CTA)
+    if (n_work > 0x7FFFFFFFLL - 2 * num_sms())
+        return fail(JNX_ERR_UNSUPPORTED, "attention backward: too many items");
     const int grid = (int)std::min<long long>(n_work, num_sms());
-    const float scale_log2 = (float)(1.4426950408889634 / sqrt((double)HD));
-    const float scale = (float)(1.0 / sqrt((double)HD));
-    pdl(k_attn_bwd<HD, MODE>, grid, 64 + 32 * abwd::EW, C::SMEM, s)(maps[0], maps[1], maps[2], maps[3], cu, it, H,
-                                                   Hkv, scale_log2, scale, lse, D, pos, rope,
-                                                   rope_ld, dqkv, ldq, status);
+    p.scale_log2 = (float)(1.4426950408889634 / sqrt((double)HD));
+    p.scale = (float)(1.0 / sqrt((double)HD));
+    if (cudaMemsetAsync(p.items.claimed, 0, sizeof(int), s) != cudaSuccess)
+        return fail(JNX_ERR_CUDA, "attention backward: %s", cudaGetErrorString(cudaGetLastError()));
+    pdl(k_attn_bwd<HD>, grid, 64 + 32 * abwd::EW, smem, s)(maps[0], maps[1], maps[2], maps[3], p);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? JNX_OK
                             : fail(JNX_ERR_CUDA, "attention backward: %s", cudaGetErrorString(e));
@@ -612,10 +725,10 @@ static jnx_status launch_bwd(const CUtensorMap (&maps)[4], const int* cu, const 
 jnx_status attention_bwd_launch(const uint16_t* qkv, int ldq, const uint16_t* dO, const float* lse,
                                 const float* D, int n_tokens, int H, int Hkv, int hd,
                                 const int* cu, const int* pos, const float2* rope, int rope_ld,
-                                const int2* items, int n_items, uint16_t* dqkv, int* status,
-                                cudaStream_t s) {
+                                const int2* items, int n_items, int* claimed, uint16_t* dqkv,
+                                int* status, cudaStream_t s) {
     if (n_tokens == 0 || n_items == 0) return JNX_OK;
-    if (!items) return fail(JNX_ERR_INVALID_ARG, "attention backward: null work items");
+    if (!items || !claimed) return fail(JNX_ERR_INVALID_ARG, "attention backward: null work items");
     if (Hkv <= 0 || H % Hkv) return fail(JNX_ERR_UNSUPPORTED, "attention backward: H %% Hkv != 0");
     if (ldq != (H + 2 * Hkv) * hd)
         return fail(JNX_ERR_INVALID_ARG, "attention backward: q|k|v row stride");
@@ -625,29 +738,12 @@ jnx_status attention_bwd_launch(const uint16_t* qkv, int ldq, const uint16_t* dO
         !make_tmap_bf16(&maps[2], dO, n_tokens, (uint64_t)H * hd, (uint64_t)H * hd, abwd::BM, 64) ||
         !make_tmap_bf16(&maps[3], dO, n_tokens, (uint64_t)H * hd, (uint64_t)H * hd, abwd::BN, 64))
         return fail(JNX_ERR_CUDA, "attention backward: tensor map encode failed");
-    BwdItems it{items, n_items};
-    jnx_status st;
+    const BwdArgs p{cu, {items, n_items, claimed}, H, Hkv, 0.f, 0.f, lse, D, pos, rope, rope_ld,
+                    dqkv, ldq, status};
     switch (hd) {
-        case 64:
-            if ((st = launch_bwd<64, abwd::DQ>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld, dqkv,
-                                               ldq, status, s)))
-                return st;
-            return launch_bwd<64, abwd::DKV>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld, dqkv,
-                                             ldq, status, s);
-        case 128:
-            if ((st = launch_bwd<128, abwd::DQ>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld,
-                                                dqkv, ldq, status, s)))
-                return st;
-            return launch_bwd<128, abwd::DKV>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld, dqkv,
-                                              ldq, status, s);
-        case 256:
-            if ((st = launch_bwd<256, abwd::DQ>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld,
-                                                dqkv, ldq, status, s)) ||
-                (st = launch_bwd<256, abwd::DK>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld,
-                                                dqkv, ldq, status, s)))
-                return st;
-            return launch_bwd<256, abwd::DV>(maps, cu, it, H, Hkv, lse, D, pos, rope, rope_ld, dqkv,
-                                             ldq, status, s);
+        case 64: return launch_bwd<64>(maps, p, s);
+        case 128: return launch_bwd<128>(maps, p, s);
+        case 256: return launch_bwd<256>(maps, p, s);
         default:
             return fail(JNX_ERR_UNSUPPORTED, "attention backward: head_dim %d", hd);
     }

@@ -87,11 +87,11 @@ jnx_status mlp_dfeat_launch(const float* dz, int ldz, const int* cu, const int* 
 // log2-sum-exp lse [N, H] of the forward, dO [N, H hd] bf16 and
 // D = rowsum(dO * O) [N, H].  Writes dq, dk, dv with the inverse RoPE
 // applied to dq and dk (the gradients of the pre-RoPE projections) into
-// dqkv [N, (H + 2 Hkv) hd] bf16.
+// dqkv [N, (H + 2 Hkv) hd] bf16.  claimed: one int of scratch.
 jnx_status attention_bwd_launch(const uint16_t* qkv, int ldq, const uint16_t* dO, const float* lse,
                                 const float* D, int n_tokens, int H, int Hkv, int hd,
                                 const int* cu, const int* pos, const float2* rope, int rope_ld,
-                                const int2* items, int n_items, uint16_t* dqkv, int* status,
-                                cudaStream_t s);
+                                const int2* items, int n_items, int* claimed, uint16_t* dqkv,
+                                int* status, cudaStream_t s);
 
 }  // namespace jnx

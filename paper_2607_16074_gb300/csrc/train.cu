@@ -46,6 +46,7 @@ struct BwdWs {
     uint16_t *t_qkv, *t_o, *dt_qkv, *dt_o, *bt[4];
     float2* rope;
     int2* items;
+    int* claimed;  // the attention backward's work counter
     size_t part_floats;
     size_t bytes;
 };
@@ -130,6 +131,7 @@ BwdWs carve_bwd(const jnx_backbone* bb, int64_t N, void* base) {
     for (int i = 0; i < 4; ++i) w.bt[i] = b16(T * kLoraRank * cols[i]);
     w.rope = reinterpret_cast<float2*>(take((size_t)kMaxRopePos * (hd / 2) * 8));
     w.items = reinterpret_cast<int2*>(take((n + n / 128 + 1) * sizeof(int2)));
+    w.claimed = reinterpret_cast<int*>(w.items + n + n / 128);  // past the last item there can be
     w.bytes = off;
     return w;
 }
@@ -377,7 +379,7 @@ extern "C" jnx_status jnx_backbone_backward_lora(const jnx_backbone* bb, const j
             TraceScope ts(JNX_K_ATTN_BWD, 2.5 * attn_flops, s);
             if ((st = attention_bwd_launch(w.qkv, qkvw, w.dO, w.lse, w.Dsum, N, H, Hkv, hd,
                                            g->cu_seqlens, g->pos_ids, w.rope, g->max_seqlen,
-                                           items, n_items, w.dqkv, w.status, s)))
+                                           items, n_items, w.claimed, w.dqkv, w.status, s)))
                 return st;
         }
 
@@ -511,7 +513,8 @@ extern "C" jnx_status jnx_op_attention_backward(const uint16_t* qkv, const uint1
     TraceScope ts(JNX_K_ATTN_BWD, 0.0, s);
     return attention_bwd_launch(qkv, ldq, dO, lse, D, n_tokens, n_heads, n_kv_heads, head_dim,
                                 cu_seqlens, pos, rope, max_seqlen, items_d, (int)items.size(),
-                                dqkv, status, s);
+                                reinterpret_cast<int*>(items_d + n_tokens + n_tokens / 128), dqkv,
+                                status, s);
 }
 
 extern "C" jnx_status jnx_op_rms_backward(const float* x, const uint16_t* gamma, float eps,
