@@ -8,7 +8,8 @@
 // the backbone's token rows for the context.  Every per-tenant projection
 // is one segmented tcgen05 GEMM over the group (gemm_launch_seg: a tenant's
 // rows times its slice of the stacked weights); weight gradients are
-// k_seg_wgrad (mma.sync, a tenant's rows in a fixed order); the attention
+// k_seg_wgrad for the action rows (mma.sync, a tenant's rows in a fixed order)
+// and a batched GEMM for the context rows; the attention
 // (C <= 64 queries per sample against its L context rows and C action rows)
 // runs on bf16 mma.sync tiles with fp32 softmax; the small per-row and
 // per-sample pieces run on CUDA cores in fp32.

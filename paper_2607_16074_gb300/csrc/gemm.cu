@@ -2,16 +2,25 @@
 //
 //   C[M, N] = A[M, K] . B[N, K]^T      (A = activations, B = weights [out, in])
 //
-// One persistent CTA per SM walks output tiles of 128 x 256.  Warp roles:
-//   warp 0     TMA producer: 128x64 A and 256x64 B boxes (128-byte swizzle)
-//              into a 4-stage shared-memory ring, completion on mbarriers;
-//   warp 1     MMA issuer: one thread issues tcgen05.mma (M=128, N=256,
-//              K=16) into a TMEM accumulator, double-buffered (2 x 256
-//              columns) so the epilogue of tile i overlaps the mainloop of
-//              tile i+1; tcgen05.commit frees smem stages / signals the
-//              epilogue;
+// Five kernels share the epilogues and the order of every K reduction:
+//   k_gemm        persistent CTAs over output tiles of 128 x 256, 128 or 64
+//                 (narrower for the fewer rows), with the per-tenant forms (LoRA
+//                 up-projections, segmented weights)
+//   k_gemm_pair   plain launches on CTA pairs (cta_group::2), tiles of 256 x 256
+//                 or 128
+//   k_gemm_batch  a table of products in one launch, either operand as it lies
+//   k_gemm_split  K over a cluster of four CTAs (the samplers' long contractions;
+//                 the one with partial sums, added in rank order)
+// pick_bn has the rule among the first two.  Warp roles:
+//   warp 0     TMA producer: A and B boxes of 64 K columns (128-byte swizzle)
+//              into a shared-memory ring (4 stages of 128 x 256), completion on
+//              mbarriers; all lanes wait, an elected one issues;
+//   warp 1     MMA issuer: tcgen05.mma (K=16) into a TMEM accumulator,
+//              double-buffered so the epilogue of tile i overlaps the
+//              mainloop of tile i+1; tcgen05.commit frees smem stages /
+//              signals the epilogue;
 //   warps 2-5  epilogue: tcgen05.ld of their 32-lane TMEM quarter (one row
-//              per thread), fused op, global store.
+//              per thread), fused op, global store (2-9 where it is the bound).
 // Fused epilogues used by the backbone block:
 //   EPI_BF16   C -> bf16
 //   EPI_F32    C -> fp32

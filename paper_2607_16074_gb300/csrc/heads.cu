@@ -19,8 +19,8 @@
 //   (the weight gradients formed through the queries per sample:
 //    dWk = Q^T (sum_s dS_s^T X_s) / sqrt(dq), dWv = sum_s dO_s^T (P_s^T X_s))
 // Loss (both): l_t = sum (y - t)^2 / (n_t * width), dy = 2 (y - t) / (n_t width).
-// All sums run in a fixed order inside one thread, one CTA or one
-// tensor-core instruction sequence (no atomics), so a tenant's results are
+// All sums run in a fixed order inside one thread, one CTA, one cluster (in
+// rank order) or one tensor-core instruction sequence (no atomics), so a tenant's results are
 // identical whether it runs grouped or alone.
 #include <cooperative_groups.h>
 
@@ -1377,7 +1377,8 @@ jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const 
                     256, kLinSmem, s)(
         tab, ws.h, ws.ld_h, ws.y, nullptr, ws.ld_y, sample_target, preds);
     if (targets)  // without targets (inference) there is no loss
-        pdl(k_l2_loss, b.n, kLossThreads, 0, s)(tab, ws.y, ws.ld_y, targets, sample_target, ws.dy, loss);
+        pdl(k_l2_loss, b.n, kLossThreads, 0, s)(tab, ws.y, ws.ld_y, targets, sample_target, ws.dy,
+                                                loss);
     return cuda_ok("heads forward");
 }
 
@@ -1388,13 +1389,13 @@ jnx_status heads_backward_launch(const HeadTable& tab, const HeadBatch& b, const
     const int *cu = g->cu_seqlens, *sample_slot = g->sample_slot;
     const NoOpt no{};
     const AdamHp nh{};
-    pdl(k_head_dw_out<NoOpt>, dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s)(
-            tab, no, nh, ws.dy, ws.ld_y, ws.h, ws.ld_h);
-    pdl(k_head_back_in, dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s)(
-        tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
+    pdl(k_head_dw_out<NoOpt>, dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0,
+        s)(tab, no, nh, ws.dy, ws.ld_y, ws.h, ws.ld_h);
+    pdl(k_head_back_in, dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256,
+        0, s)(tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_mlp)
-        pdl(k_mlp_dw1<NoOpt>, dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256),
-                           256, 0, s)(
+        pdl(k_mlp_dw1<NoOpt>,
+            dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256), 256, 0, s)(
             tab, no, nh, ws.dh, ws.ld_h, pooled, d);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
@@ -1416,8 +1417,8 @@ jnx_status heads_backward_front_launch(const HeadTable& tab, const HeadBatch& b,
                                        const jnx_group* g, bool kv_grads, cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
     const int *cu = g->cu_seqlens, *sample_slot = g->sample_slot;
-    pdl(k_head_back_in, dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256, 0, s)(
-        tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
+    pdl(k_head_back_in, dim3(b.n, (b.max_hid + kBackCols - 1) / kBackCols, (b.max_ns + 7) / 8), 256,
+        0, s)(tab, ws.dy, ws.ld_y, ws.z, ws.ld_h, ws.dh);
     if (b.any_xattn) {
         const size_t smem = xattn_smem_bytes(b.max_dq, true);
         pdl(k_xattn_bwd, (b.sample1 - b.sample0) * kXCtas, 256, smem, s)(
@@ -1434,11 +1435,11 @@ jnx_status heads_backward_step_launch(const HeadTable& tab, const HeadOptTable& 
                                       const HeadScratch& ws, const float* pooled, int d,
                                       cudaStream_t s) {
     if (b.n == 0) return JNX_OK;
-    pdl(k_head_dw_out<HeadOptTable>, dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0, s)(
-            tab, opt, hp, ws.dy, ws.ld_y, ws.h, ws.ld_h);
+    pdl(k_head_dw_out<HeadOptTable>, dim3(b.n, (b.max_width + 15) / 16, (b.max_hid + 255) / 256), 256, 0,
+        s)(tab, opt, hp, ws.dy, ws.ld_y, ws.h, ws.ld_h);
     if (b.any_mlp)
-        pdl(k_mlp_dw1<HeadOptTable>, dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256), 256, 0,
-               s)(
+        pdl(k_mlp_dw1<HeadOptTable>,
+            dim3(b.n, (b.max_mlp_hid + kDw1Rows - 1) / kDw1Rows, (d / 4 + 255) / 256), 256, 0, s)(
             tab, opt, hp, ws.dh, ws.ld_h, pooled, d);
     if (b.any_xattn) {
         // wgrad reads the learned queries, which dq then updates
