@@ -238,8 +238,10 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
     cg::cluster_group cluster = cg::this_cluster();
     const int s = blockIdx.x / parts, part = blockIdx.x % parts;
     const int r0 = cu[s], r1 = cu[s + 1];
-    // rows of this CTA: an equal share, in whole rounds
-    const int share = ((r1 - r0 + parts - 1) / parts + R - 1) / R * R;
+    // rows of this CTA: an equal share in whole fours, the same cut in both
+    // variants and for every round length, so that the sums associate alike
+    static_assert(4 % R == 0, "a share is whole rounds");
+    const int share = ((r1 - r0 + parts - 1) / parts + 3) / 4 * 4;
     const int t0 = min(r0 + part * share, r1), t1 = min(t0 + share, r1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float acc[C], gm[C];
