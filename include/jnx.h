@@ -450,7 +450,9 @@ jnx_status jnx_backbone_forward_train(const jnx_backbone* bb, const jnx_group* g
  * of each row's tenant loss with respect to that row's final normed
  * hidden: (dz W1) / L_s on every row of an MLP-head sample (the feature is
  * the mean of the rows), dk W_k + dv W_v on a query-head row.  Every row of
- * the group is written. */
+ * the group is written.  With query heads in the group d_hidden must be
+ * 8-byte aligned (JNX_ERR_INVALID_ARG before any launch otherwise); 16-byte
+ * alignment and d a multiple of 256 let the product run on tcgen05. */
 jnx_status jnx_heads_backward_input(const jnx_head* heads, int32_t n_tenants,
                                     const jnx_group* g, const float* pooled,
                                     const uint16_t* hidden, const float* targets,

@@ -605,6 +605,16 @@ jnx_status check_heads(const jnx_head* heads, int32_t n_tenants, const jnx_group
     return JNX_OK;
 }
 
+// The query heads' rows of d_hidden are written with 8-byte accesses at least.
+jnx_status check_d_hidden(const jnx_head* heads, const jnx_group* g, const float* d_hidden) {
+    for (int i = 0; i < g->n_slots; ++i)
+        if (heads[g->h_slot_tenant[i]].kind == JNX_HEAD_XATTN &&
+            (reinterpret_cast<uintptr_t>(d_hidden) & 7))
+            return fail(JNX_ERR_INVALID_ARG,
+                        "heads backward: the feature gradient must be 8-byte aligned");
+    return JNX_OK;
+}
+
 // Fill the per-slot table for group slots [g0, g0 + n) and describe the batch.
 HeadBatch fill_table(HeadTable& tab, const jnx_head* heads, const jnx_head_grads* grads,
                      const jnx_group* g, int g0, int n, bool accum = false) {
@@ -755,11 +765,13 @@ extern "C" jnx_status jnx_heads_forward(const jnx_head* heads, int32_t n_tenants
 static jnx_status heads_backward(const jnx_head* heads, int32_t n_tenants, const jnx_group* g,
                                  const float* pooled, const uint16_t* hidden,
                                  const jnx_head_grads* grads, void* workspace, size_t ws_bytes,
-                                 void* stream, bool accum, bool kv_grads = false) {
+                                 void* stream, bool accum, const float* d_hidden = nullptr) {
     jnx_status st;
     if (!grads && g && g->n_slots > 0)
         return fail(JNX_ERR_INVALID_ARG, "heads backward: null grads");
-    if ((st = check_heads(heads, n_tenants, g, true, grads, pooled, hidden))) return st;
+    if ((st = check_heads(heads, n_tenants, g, true, grads, pooled, hidden)) ||
+        (st = check_d_hidden(heads, g, d_hidden)))
+        return st;
     if (g->n_slots == 0) return JNX_OK;
     if (!workspace) return fail(JNX_ERR_INVALID_ARG, "heads backward: null workspace");
     HeadsWs w = carve_heads(heads, g, workspace);
@@ -773,7 +785,8 @@ static jnx_status heads_backward(const jnx_head* heads, int32_t n_tenants, const
         const int n = std::min(kMaxSlots, g->n_slots - g0);
         HeadBatch b = fill_table(tab, heads, grads, g, g0, n, accum);
         TraceScope ts(JNX_K_HEADS_BWD, heads_flops(tab, n, true), s);
-        if ((st = heads_backward_launch(tab, b, w.sc, pooled, d, hidden, g, kv_grads, s)))
+        if ((st = heads_backward_launch(tab, b, w.sc, pooled, d, hidden, g, d_hidden != nullptr,
+                                        s)))
             return st;
     }
     return JNX_OK;
@@ -831,10 +844,12 @@ static jnx_status heads_feature_grad(const jnx_head* heads, const jnx_group* g, 
         return st;
     if (!any_x) return JNX_OK;
     const int ld = w.sc.ldkv;
-    if (d % 256 == 0) {
+    if (d % 256 == 0 && (reinterpret_cast<uintptr_t>(d_hidden) & 15) == 0) {
         // [dk | dv] [Wk; Wv] per tenant, the weights as they lie (rows are K):
         // one tcgen05 launch per 64 tenants (mma.sync tiles of 64 x 128 took 283
-        // us for 35,000 rows x 2,048 columns, this 61)
+        // us for 35,000 rows x 2,048 columns, this 61).  Its epilogue stores 16
+        // bytes of a 256-column tile's rows; other widths, and buffers aligned to
+        // 8 bytes only, take those tiles below.
         static thread_local GemmBatch gb;  // staging of the kernel argument
         for (int g0 = 0; g0 < g->n_slots; g0 += kMaxSlots) {
             gb.n_maps = gb.n = gb.tiles = 0;
@@ -903,7 +918,7 @@ extern "C" jnx_status jnx_heads_backward_input(const jnx_head* heads, int32_t n_
     if (!d_hidden && g && g->n_tokens > 0)
         return fail(JNX_ERR_INVALID_ARG, "heads backward: null feature-gradient buffer");
     jnx_status st = heads_backward(heads, n_tenants, g, pooled, hidden, grads, workspace,
-                                   ws_bytes, stream, false, true);
+                                   ws_bytes, stream, false, d_hidden);
     if (st || g->n_slots == 0) return st;
     return heads_feature_grad(heads, g, d_hidden, workspace, static_cast<cudaStream_t>(stream));
 }
@@ -927,7 +942,9 @@ extern "C" jnx_status jnx_heads_backward_adamw(const jnx_head* heads, int32_t n_
     if (accumulate && !grads && g && g->n_slots > 0)
         return fail(JNX_ERR_INVALID_ARG, "heads backward adamw: accumulating needs grads");
     jnx_status st;
-    if ((st = check_heads(heads, n_tenants, g, accumulate != 0, grads, pooled, hidden))) return st;
+    if ((st = check_heads(heads, n_tenants, g, accumulate != 0, grads, pooled, hidden)) ||
+        (st = check_d_hidden(heads, g, d_hidden)))
+        return st;
     if (g->n_slots == 0) return JNX_OK;
     if (!workspace) return fail(JNX_ERR_INVALID_ARG, "heads backward adamw: null workspace");
     // every group tenant's optimizer state, checked before anything is written

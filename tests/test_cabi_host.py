@@ -177,10 +177,22 @@ def test_training_entry_points_reject_bad_arguments_without_a_gpu():
                                       None) == inv
     assert L.jnx_adamw_tensors(None, 1, None, None) == inv
     assert L.jnx_transpose(None, 1, -1, 4, None, None) == inv
-    # a well-formed group: the expert's checks decide, still before any launch
+    # a well-formed group: the heads' and the expert's checks decide, still before any launch
     g, keep = _host_group()
-    fh, blocks = _host_flow_head(384)  # width not in {256, 512, 1024}
     fake = 1 << 20
+    heads = (J.jnx_head * 1)(J.jnx_head(J.JNX_HEAD_XATTN, 512, 0, 4, 256, 7, *([None] * 4),
+                                        *([fake] * 5)))
+    grads = (J.jnx_head_grads * 1)(J.jnx_head_grads(*([None] * 4), *([fake] * 5)))
+    opt = (J.jnx_head_opt * 1)()
+    hp = J.jnx_adamw(1e-3, 0.9, 0.999, 1e-8, 0.0)
+    odd = fake + 4  # the gradient at a query head's rows, off an 8-byte boundary
+    rc = L.jnx_heads_backward_input(heads, 1, C.byref(g), None, fake, fake, grads, odd, fake,
+                                    1 << 40, None)
+    assert rc == inv and "8-byte" in J.jnx_last_error()
+    rc = L.jnx_heads_backward_adamw(heads, 1, C.byref(g), None, fake, fake, None, 0, opt,
+                                    C.byref(hp), odd, fake, 1 << 40, None)
+    assert rc == inv and "8-byte" in J.jnx_last_error()
+    fh, blocks = _host_flow_head(384)  # width not in {256, 512, 1024}
     rc = L.jnx_flow_forward(C.byref(fh), C.byref(g), fake, fake, fake, fake, fake, fake, fake,
                             1 << 30, None)
     assert rc == uns and "d_model" in J.jnx_last_error()
