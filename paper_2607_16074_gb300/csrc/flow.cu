@@ -54,10 +54,12 @@ __device__ __forceinline__ float silu_grad_f(float z) {
 // layer is one launch over (row, block of 32 output rows): one warp per
 // row, lanes along the dot product with 16-byte weight loads (dm is a
 // multiple of 256), the row sum in a fixed butterfly order.  A row is a sample
-// with its own tau, or, when sampling (tau null), an Euler step and slot: row r
-// is slot r % n at time (step0 + r / n) / n_steps, since all of a tenant's samples
-// are at the same time then.  One pair of launches serves every step (a fill and
-// two launches of a row per sample in each step before: 20 of 265 us).
+// with its own tau, or, when sampling (tau null), an Euler step and slot, since
+// all of a tenant's samples are at the same time then: row r is slot r % per at
+// time (step0 + r / per) / n_steps.  One pair of launches serves every step (a
+// fill and two launches of a row per sample in each step before: 20 of 265 us).
+// A group with more slots than samples (some hold none) has a row per sample
+// instead (by_slot 0, per = samples): a step's rows never outnumber the samples.
 // ---------------------------------------------------------------------------
 constexpr int kTimeRows = 32;
 
@@ -86,13 +88,13 @@ __global__ void __launch_bounds__(256) k_flow_time1(const float* __restrict__ ta
                                                     FlowDims dd, const uint16_t* __restrict__ t1,
                                                     const uint16_t* __restrict__ tb1,
                                                     float* __restrict__ sfeat,
-                                                    float* __restrict__ z1, int step0,
-                                                    int n_steps) {
+                                                    float* __restrict__ z1, int per,
+                                                    int by_slot, int step0, int n_steps) {
     pdl_entry();
     extern __shared__ float sh[];  // s(tau) [dm]
     const int s = blockIdx.x, dm = dd.dm, half = dm / 2;
-    const int t = fs.tenant[tau ? sample_slot[s] : s % fs.n];
-    const float tv = tau ? tau[s] : (float)(step0 + s / fs.n) / (float)n_steps;
+    const int t = fs.tenant[by_slot ? s % per : sample_slot[s % per]];
+    const float tv = tau ? tau[s] : (float)(step0 + s / per) / (float)n_steps;
     for (int i = threadIdx.x; i < dm; i += blockDim.x) {
         const int k = i < half ? i : i - half;
         const float w = powf(10000.f, -(float)k / (float)half);
@@ -115,11 +117,12 @@ __global__ void __launch_bounds__(256) k_flow_time2(const int* __restrict__ samp
                                                     FlowDims dd, const uint16_t* __restrict__ t2,
                                                     const uint16_t* __restrict__ tb2,
                                                     const float* __restrict__ z1,
-                                                    float* __restrict__ phi, int by_slot) {
+                                                    float* __restrict__ phi, int per,
+                                                    int by_slot) {
     pdl_entry();
     extern __shared__ float sh[];  // SiLU(z1) [dm]
     const int s = blockIdx.x, dm = dd.dm;
-    const int t = fs.tenant[by_slot ? s % fs.n : sample_slot[s]];
+    const int t = fs.tenant[by_slot ? s % per : sample_slot[s % per]];
     for (int i = threadIdx.x; i < dm; i += blockDim.x) sh[i] = silu_f(z1[(size_t)s * dm + i]);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1428,15 +1431,17 @@ static jnx_status flow_begin(const jnx_flow_head* fh, const jnx_group* g, const 
 }
 
 // The time embedding of every sample (tau), or of Euler steps [step0, step0 +
-// rows / slots) of n_steps for every slot (tau null), into z1 and phi.
+// rows / per) of n_steps (tau null; rows as at k_flow_time1), into z1 and phi.
 static jnx_status flow_time(const jnx_flow_head* fh, const FlowDims& d, const jnx_group* g,
-                            const FlowSlots& fs, const float* tau, int rows, int step0,
-                            int n_steps, float* sfeat, float* z1, float* phi, cudaStream_t s) {
+                            const FlowSlots& fs, const float* tau, int rows, int per, int by_slot,
+                            int step0, int n_steps, float* sfeat, float* z1, float* phi,
+                            cudaStream_t s) {
     const dim3 tg(rows, d.dm / kTimeRows);
     pdl(k_flow_time1, tg, 256, d.dm * sizeof(float), s)(tau, g->sample_slot, fs, d, fh->t1,
-                                                        fh->tb1, sfeat, z1, step0, n_steps);
+                                                        fh->tb1, sfeat, z1, per, by_slot, step0,
+                                                        n_steps);
     pdl(k_flow_time2, tg, 256, d.dm * sizeof(float), s)(g->sample_slot, fs, d, fh->t2, fh->tb2, z1,
-                                                        phi, tau ? 0 : 1);
+                                                        phi, per, by_slot);
     return last("flow time embedding");
 }
 
@@ -1466,7 +1471,8 @@ extern "C" jnx_status jnx_flow_forward(const jnx_flow_head* fh, const jnx_group*
     {
         TraceScope ts(JNX_K_FLOW_MISC, (double)g->n_samples * d.dm * d.dm * 4.0, s);
         if ((st = flow_ones(d, w, s)) ||
-            (st = flow_time(fh, d, g, fs, tau, g->n_samples, 0, 1, w.sfeat, w.z1, w.phi, s)))
+            (st = flow_time(fh, d, g, fs, tau, g->n_samples, g->n_samples, 0, 0, 1, w.sfeat, w.z1,
+                            w.phi, s)))
             return st;
         pdl(k_flow_embed, g->n_samples * d.C, 256, 0, s)(actions, noise, tau, (const float*)nullptr,
                                                          g->sample_slot, fs, d, fh->w_in, fh->b_in,
@@ -1505,12 +1511,15 @@ extern "C" jnx_status jnx_flow_sample(const jnx_flow_head* fh, const jnx_group* 
     float* tz = d.nb > 0 ? w.h_in : w.z1;
     float* tp = d.nb > 0 ? w.h_mid : w.phi;
     const size_t cap = d.nb > 0 ? (size_t)d.nb * g->n_samples * d.C : (size_t)g->n_samples;
-    const int chunk = (int)std::max<size_t>(1, cap / g->n_slots);
+    const int by_slot = g->n_slots > 0 && g->n_slots <= g->n_samples;
+    const int per = by_slot ? g->n_slots : g->n_samples;  // rows of a step, at most cap
+    const int chunk = (int)std::min<size_t>(cap / per, n_steps);
     for (int i = 0; i < n_steps; ++i) {
         if (i % chunk == 0) {
-            const int rows = std::min(chunk, n_steps - i) * g->n_slots;
+            const int rows = std::min(chunk, n_steps - i) * per;
             TraceScope ts(JNX_K_FLOW_MISC, (double)rows * d.dm * d.dm * 4.0, s);
-            if ((st = flow_time(fh, d, g, fs, nullptr, rows, i, n_steps, nullptr, tz, tp, s)))
+            if ((st = flow_time(fh, d, g, fs, nullptr, rows, per, by_slot, i, n_steps, nullptr, tz,
+                                tp, s)))
                 return st;
         }
         {
@@ -1518,7 +1527,7 @@ extern "C" jnx_status jnx_flow_sample(const jnx_flow_head* fh, const jnx_group* 
             pdl(k_flow_embed, g->n_samples * d.C, 256, 0, s)(
                 (const float*)nullptr, (const float*)nullptr, (const float*)nullptr, actions,
                 g->sample_slot, fs, d, fh->w_in, fh->b_in, fh->pos,
-                tp + (size_t)(i % chunk) * g->n_slots * d.dm, 1, w.x, w.u, w.h);
+                tp + (size_t)(i % chunk) * per * d.dm, by_slot, w.x, w.u, w.h);
             if ((st = last("flow embedding"))) return st;
         }
         if ((st = flow_network(fh, d, g, hidden, w, fs, sg, i > 0, false, nullptr, s))) return st;

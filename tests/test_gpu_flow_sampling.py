@@ -1,7 +1,11 @@
 """The flow experts' sampler where its own paths can go wrong: contractions long
 enough to be split over a cluster (F >= 2,048) with one row, one tile and two
-tiles of rows a tenant, and more Euler steps than the time embeddings' buffers
-hold at once (few rows, and no blocks at all)."""
+tiles of rows a tenant, more Euler steps than the time embeddings' buffers
+hold at once (few rows, and no blocks at all), and groups with more slots than
+those buffers have rows."""
+import copy
+
+import numpy as np
 import pytest
 import torch
 
@@ -43,3 +47,23 @@ def test_sampling_vs_oracle_and_alone(F, C, nb, steps):
         alone = _sample(s, s.plan([t]), hidden[cu[s0]:cu[s1]].contiguous(),
                         noise[s0:s1].contiguous(), steps)
         assert torch.equal(alone, out[s0:s1]), t
+
+
+@pytest.mark.parametrize("nb,empty", [(0, 4), (1, 4), (2, 12)])
+def test_slots_without_samples_change_nothing(nb, empty):
+    """One sample, then a group that names it in its last of several slots, the others
+    empty: with a chunk of one row the buffers of a step's time embeddings hold max(1, nb)
+    rows, fewer than there are slots."""
+    s = FlowSetup(F=256, C=1, nb=nb, std=0.05)
+    plan = s.plan([1])
+    many = copy.copy(plan)
+    many.n_slots = empty + 1
+    many.seg_offsets = np.array([0] * (empty + 1) + [1], dtype=np.int32)
+    many.slot_tenant = np.array([0, 2] * (empty // 2) + [1], dtype=np.int32)
+    many.sample_slot = np.array([empty], dtype=np.int32)
+    gen = torch.Generator().manual_seed(2)
+    hidden = torch.randn(plan.n_tokens, 256, generator=gen).to(torch.bfloat16).cuda()
+    noise = torch.randn(1, 1, s.D, generator=gen).cuda()
+    want = _sample(s, plan, hidden, noise, 5)
+    assert torch.isfinite(want).all()
+    assert torch.equal(_sample(s, many, hidden, noise, 5), want)
