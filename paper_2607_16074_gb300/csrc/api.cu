@@ -527,11 +527,8 @@ HeadsWs carve_heads(const jnx_head* heads, const jnx_group* g, void* base) {
         w.sc.dQs = take(S * hd.ld_h * 4);
         w.sc.dkv = reinterpret_cast<uint16_t*>(take(N * 2 * hd.ldkv * 2));
         w.sc.HG = take(S * 64 * hd.d_in * 4);
-        int longest = 1;
-        for (int i = 0; g->h_cu_seqlens && i < g->n_samples; ++i)
-            longest = std::max(longest, g->h_cu_seqlens[i + 1] - g->h_cu_seqlens[i]);
-        w.sc.ldp = 2 * ((longest + 63) / 64 * 64);
-        w.sc.planes = reinterpret_cast<uint16_t*>(take(S * 64 * (size_t)w.sc.ldp * 2));
+        w.sc.ldp = plane_col((int)N, (int)S);
+        w.sc.planes = reinterpret_cast<uint16_t*>(take((size_t)64 * w.sc.ldp * 2));
     }
     w.sc.status = w.status;
     w.bytes = off;

@@ -1531,7 +1531,7 @@ __global__ void __launch_bounds__(192, 1) k_gemm_batch(const __grid_constant__ G
                             tma_load_2d(sa + i * 64 * BK * 2, ma, mb * BM + 64 * i, kb * BK,
                                         &full[stage]);
                     } else {
-                        tma_load_2d(sa, ma, second ? q.ax2 + bk : bk, q.arow + mb * BM,
+                        tma_load_2d(sa, ma, (second ? q.ax2 : q.ax) + bk, q.arow + mb * BM,
                                     &full[stage]);
                     }
                     if constexpr (BMN) {

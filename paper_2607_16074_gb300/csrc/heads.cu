@@ -708,17 +708,16 @@ __device__ __forceinline__ void xattn_chunk_xr(float (&acc)[2][4][4], const uint
 }
 
 // The chunk's query-major split tiles of dS (tq) and P (the two planes after
-// them) into the sample's weight-gradient operands (see k_xattn_bwd); pad: zeros
-// for the 32 keys after the chunk, too.
-__device__ __forceinline__ void xattn_store_planes(uint16_t* __restrict__ dst, int ldp,
+// them) into the sample's weight-gradient operands (see k_xattn_bwd), whose lo
+// half starts at column lo; pad: zeros for the 32 keys after the chunk, too.
+__device__ __forceinline__ void xattn_store_planes(uint16_t* __restrict__ dst, int ldp, int lo,
                                                    const uint16_t* tq, int j0, bool pad) {
     static_assert(kXRows == 32 && kMaxQ == 32, "four 16-byte units a row");
     for (int i = threadIdx.x; i < 4 * kMaxQ * 4; i += 256) {
         const int u = i & 3, q = (i >> 2) & 31, pl = i >> 7;  // planes: dS hi, dS lo, P hi, P lo
         const uint4 v =
             *reinterpret_cast<const uint4*>(tq + (size_t)(pl * kMaxQ + q) * kXPad + 8 * u);
-        uint16_t* o = dst + (size_t)((pl < 2 ? kMaxQ : 0) + q) * ldp + (pl & 1) * (ldp / 2) + j0 +
-                      8 * u;
+        uint16_t* o = dst + (size_t)((pl < 2 ? kMaxQ : 0) + q) * ldp + (pl & 1) * lo + j0 + 8 * u;
         *reinterpret_cast<uint4*>(o) = v;
         if (pad) *reinterpret_cast<uint4*>(o + kXRows) = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -889,9 +888,9 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 3)
 // when kv_grads is set (the feature gradient needs them), the key rows'
 // dk = scale dS^T Q and dv = P^T dO as bf16 rows dk | dv of dkv (row stride 2
 // ldkv).  Also P and dS query-major as the bf16 hi and lo operands of the
-// weight gradients' products: planes[s][P: 0 .. 31, dS: 32 .. 63][hi: key, lo:
-// ldp / 2 + key], zero past the queries and, up to the next multiple of 64, past
-// the keys.
+// weight gradients' products: planes[P: 0 .. 31, dS: 32 .. 63][plane_col + (hi:
+// key, lo: the keys in whole 64s + key)], zero past the queries and, up to the
+// next multiple of 64, past the keys.
 __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
     k_xattn_bwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
@@ -960,7 +959,7 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
                 xattn_split_chunk(sT + 2 * kMaxQ * kXPad, kv_grads ? uP : nullptr, Ps, j0, nr, nq);
             __syncthreads();
             if (c0 == 0)
-                xattn_store_planes(planes + (size_t)s * 2 * kMaxQ * ldp, ldp, sT, j0,
+                xattn_store_planes(planes + plane_col(r0, s), ldp, (L + 63) / 64 * 64, sT, j0,
                                    j0 + kXRows >= L && ((L + kXRows - 1) / kXRows & 1));
             xattn_chunk_xr(aq, sT, sR);  // dQ += dS k
             if (!kv_grads) continue;
@@ -1320,8 +1319,7 @@ static jnx_status gh_launch(const HeadTable& tab, const HeadBatch& b, const Head
         gb.n_maps = gb.n = gb.tiles = 0;
         gb.ldo = d;
         gb.status = ws.status;
-        return batch_map(gb, ws.planes, (uint64_t)g->n_samples * 2 * kMaxQ, ws.ldp, ws.ldp, false,
-                         128) == 0;
+        return batch_map(gb, ws.planes, 2 * kMaxQ, ws.ldp, ws.ldp, false, 128) == 0;
     };
     if (!begin()) return fail(JNX_ERR_CUDA, "heads backward: tensor map");
     for (int i = 0; i < b.n; ++i) {
@@ -1346,9 +1344,9 @@ static jnx_status gh_launch(const HeadTable& tab, const HeadBatch& b, const Head
             if (q.b < 0) return fail(JNX_ERR_CUDA, "heads backward: tensor map");
             q.k1 = (L + 63) / 64;
             q.k = 2 * q.k1;
-            q.ax2 = ws.ldp / 2;
+            q.ax = plane_col(r0, sm);
+            q.ax2 = q.ax + 64 * q.k1;
             q.m = 2 * kMaxQ;
-            q.arow = sm * 2 * kMaxQ;
             q.nb = d / 256;
             batch_add(gb, q);
         }

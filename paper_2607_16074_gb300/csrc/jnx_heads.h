@@ -70,11 +70,18 @@ struct HeadScratch {
     float *P, *dS;                 // [nq * n_tokens], key-major per sample
     float* dQs;                    // [n_samples, ld_h]
     float* HG;                     // [n_samples, 64, d]: P_s^T X_s and dS_s^T X_s (32 rows each)
-    uint16_t* planes;              // their bf16 operands [n_samples, 64, ldp] (see k_xattn_bwd)
-    int ldp;                       // twice the longest sample, in whole 64s
+    uint16_t* planes;              // their bf16 operands [64, ldp] (see plane_col)
+    int ldp;                       // plane columns of all samples
     uint16_t* dkv;                 // feature gradient: bf16 [dk | dv] rows [n_tokens, 2 ldkv]
     int* status;                   // device status word
 };
+
+// Sample s, from token r0 on, has its columns of the planes from plane_col(r0, s)
+// on: two halves (hi, lo) of its keys in whole 64s.  They never reach the next
+// sample's, and all of them together are as many as the tokens ask for, whatever
+// the lengths (a rectangle of samples x longest sample took 545 MB for 512 samples
+// of 12,288 tokens with one of 4,112 among them, this 12 MB).
+__host__ __device__ constexpr int plane_col(int r0, int s) { return 128 * (r0 / 64 + s); }
 
 jnx_status heads_forward_launch(const HeadTable& tab, const HeadBatch& b, const HeadScratch& ws,
                                 const float* pooled, int d, const int* cu, const int* sample_slot,

@@ -206,6 +206,24 @@ def test_training_entry_points_reject_bad_arguments_without_a_gpu():
     assert rc == inv and "aligned" in J.jnx_last_error()
 
 
+def test_query_heads_workspace_grows_with_the_tokens_not_the_longest_sample():
+    L = J.lib()
+    fake = 1 << 20
+    heads = (J.jnx_head * 1)(J.jnx_head(J.JNX_HEAD_XATTN, 2048, 0, 32, 256, 7, *([None] * 4),
+                                        *([fake] * 5)))
+
+    def need(lengths):
+        cu = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+        seg, ten = np.array([0, len(lengths)], np.int32), np.zeros(1, np.int32)
+        g = J.jnx_group(len(lengths), int(cu[-1]), 1, max(lengths), *([fake] * 6),
+                        *(a.ctypes.data_as(J.P32) for a in (cu, seg, ten)))
+        return L.jnx_heads_workspace_bytes(heads, 1, C.byref(g))
+
+    even, ragged = [24] * 512, [16] * 511 + [16 + 8 * 512]
+    assert sum(even) == sum(ragged)
+    assert need(ragged) == need(even) > 0
+
+
 def test_scheduler_bit_exact_vs_oracle_random_queues():
     # jnx_sched_poll (C++) against the scheduler oracle: same queue indices
     # to take and the same wake time, on both collection modes
