@@ -1519,7 +1519,8 @@ __global__ void __launch_bounds__(192, 1) k_gemm_batch(const __grid_constant__ G
                     break;
                 }
                 const bool second = kb >= q.k1;
-                const int bk = (second ? kb - q.k1 : kb) * BK;
+                const int ka = second ? kb - q.k1 : kb;
+                const int bk = (ka >> q.b_twice) * BK;
                 const CUtensorMap* ma = &gb.map[q.a];
                 const CUtensorMap* mbp = &gb.map[second ? q.b2 : q.b];
                 if (elect_one()) {
@@ -1531,7 +1532,7 @@ __global__ void __launch_bounds__(192, 1) k_gemm_batch(const __grid_constant__ G
                             tma_load_2d(sa + i * 64 * BK * 2, ma, mb * BM + 64 * i, kb * BK,
                                         &full[stage]);
                     } else {
-                        tma_load_2d(sa, ma, (second ? q.ax2 : q.ax) + bk, q.arow + mb * BM,
+                        tma_load_2d(sa, ma, (second ? q.ax2 : q.ax) + ka * BK, q.arow + mb * BM,
                                     &full[stage]);
                     }
                     if constexpr (BMN) {

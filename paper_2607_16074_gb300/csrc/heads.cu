@@ -708,16 +708,17 @@ __device__ __forceinline__ void xattn_chunk_xr(float (&acc)[2][4][4], const uint
 }
 
 // The chunk's query-major split tiles of dS (tq) and P (the two planes after
-// them) into the sample's weight-gradient operands (see k_xattn_bwd), whose lo
-// half starts at column lo; pad: zeros for the 32 keys after the chunk, too.
-__device__ __forceinline__ void xattn_store_planes(uint16_t* __restrict__ dst, int ldp, int lo,
+// them) into the sample's weight-gradient operands (see k_xattn_bwd); pad: zeros
+// for the 32 keys after the chunk, too.
+__device__ __forceinline__ void xattn_store_planes(uint16_t* __restrict__ dst, int ldp,
                                                    const uint16_t* tq, int j0, bool pad) {
     static_assert(kXRows == 32 && kMaxQ == 32, "four 16-byte units a row");
     for (int i = threadIdx.x; i < 4 * kMaxQ * 4; i += 256) {
         const int u = i & 3, q = (i >> 2) & 31, pl = i >> 7;  // planes: dS hi, dS lo, P hi, P lo
         const uint4 v =
             *reinterpret_cast<const uint4*>(tq + (size_t)(pl * kMaxQ + q) * kXPad + 8 * u);
-        uint16_t* o = dst + (size_t)((pl < 2 ? kMaxQ : 0) + q) * ldp + (pl & 1) * lo + j0 + 8 * u;
+        uint16_t* o = dst + (size_t)((pl < 2 ? kMaxQ : 0) + q) * ldp + 128 * (j0 / 64) +
+                      64 * (pl & 1) + j0 % 64 + 8 * u;
         *reinterpret_cast<uint4*>(o) = v;
         if (pad) *reinterpret_cast<uint4*>(o + kXRows) = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -888,9 +889,9 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 3)
 // when kv_grads is set (the feature gradient needs them), the key rows'
 // dk = scale dS^T Q and dv = P^T dO as bf16 rows dk | dv of dkv (row stride 2
 // ldkv).  Also P and dS query-major as the bf16 hi and lo operands of the
-// weight gradients' products: planes[P: 0 .. 31, dS: 32 .. 63][plane_col + (hi:
-// key, lo: the keys in whole 64s + key)], zero past the queries and, up to the
-// next multiple of 64, past the keys.
+// weight gradients' products: planes[P: 0 .. 31, dS: 32 .. 63][plane_col + 128
+// (key / 64) + key % 64, lo 64 columns after hi], zero past the queries and, up to
+// the next multiple of 64, past the keys.
 __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
     k_xattn_bwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
@@ -959,7 +960,7 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
                 xattn_split_chunk(sT + 2 * kMaxQ * kXPad, kv_grads ? uP : nullptr, Ps, j0, nr, nq);
             __syncthreads();
             if (c0 == 0)
-                xattn_store_planes(planes + plane_col(r0, s), ldp, (L + 63) / 64 * 64, sT, j0,
+                xattn_store_planes(planes + plane_col(r0, s), ldp, sT, j0,
                                    j0 + kXRows >= L && ((L + kXRows - 1) / kXRows & 1));
             xattn_chunk_xr(aq, sT, sR);  // dQ += dS k
             if (!kv_grads) continue;
@@ -1055,9 +1056,11 @@ __global__ void __launch_bounds__(256) k_xattn_dq(const __grid_constant__ HeadTa
 //
 // Where d is a multiple of 256 they are one batched tcgen05 GEMM (gh_launch):
 // per sample [P | dS] planes [64, keys] (k_xattn_bwd wrote them) times X, whose
-// rows are K, the hi planes' K-steps before the lo planes':
-// 61 us for 64 samples of 547 rows x 2,048 columns, where k_xattn_gh, whose
-// sixteen column blocks each split P and dS again, took 246.
+// rows are K, the hi and the lo K-step of 64 keys in turn: 61 us for 64 samples of
+// 547 rows x 2,048 columns, where k_xattn_gh, whose sixteen column blocks each split
+// P and dS again, took 246.  With all hi steps before all lo ones the small terms met
+// a full sum: W_k's and W_v's gradients there 6.4e-6 and 2.9e-6 off from 64 bits in
+// the 2-norm, 6.1e-6 and 2.7e-6 in turn (k_xattn_gh 6.2e-6 and 2.9e-6), the time alike.
 //
 // k_xattn_gh, for other widths: one CTA per (sample, 128 columns e of X), on
 // mma.sync (m16n8k16, fp32 accumulation).  The sample's rows are staged 32 keys
@@ -1342,10 +1345,9 @@ static jnx_status gh_launch(const HeadTable& tab, const HeadBatch& b, const Head
             q.a = 0;
             q.b = q.b2 = batch_map(gb, hidden + (size_t)r0 * d, L, d, d, true, 0);
             if (q.b < 0) return fail(JNX_ERR_CUDA, "heads backward: tensor map");
-            q.k1 = (L + 63) / 64;
-            q.k = 2 * q.k1;
+            q.k1 = q.k = 2 * ((L + 63) / 64);
+            q.b_twice = 1;
             q.ax = plane_col(r0, sm);
-            q.ax2 = q.ax + 64 * q.k1;
             q.m = 2 * kMaxQ;
             q.nb = d / 256;
             batch_add(gb, q);

@@ -77,7 +77,7 @@ struct HeadScratch {
 };
 
 // Sample s, from token r0 on, has its columns of the planes from plane_col(r0, s)
-// on: two halves (hi, lo) of its keys in whole 64s.  They never reach the next
+// on: 64 of hi and 64 of lo for every 64 of its keys.  They never reach the next
 // sample's, and all of them together are as many as the tokens ask for, whatever
 // the lengths (a rectangle of samples x longest sample took 545 MB for 512 samples
 // of 12,288 tokens with one of 4,112 among them, this 12 MB).

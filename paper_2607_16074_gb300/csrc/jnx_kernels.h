@@ -166,7 +166,7 @@ jnx_status lora_down_launch(const jnx_group* g, const uint16_t* x, int ldx, int 
 // arow + row and columns from ax on (K-major) or columns row (a_mn: A is [K, m]
 // row-major); B_i from map[b] for the first k1 K-steps and from map[b2]
 // (restarting at its first K row) for the rest, whose A columns start at ax2;
-// b_mn: B is [K, N] row-major.
+// b_mn: B is [K, N] row-major; b_twice: B takes each of its K-steps for two of A's.
 // A K extent that is no multiple of 64 ends in the maps' zero fill, so a map
 // whose rows are K covers one problem's rows only.
 constexpr int kBatchMaps = 130, kBatchMax = 128;
@@ -174,7 +174,7 @@ struct GemmBatch {
     CUtensorMap map[kBatchMaps];
     struct Problem {
         float* out;
-        int a, b, b2, k1, k, m, arow, ax, ax2, nb, tile0;
+        int a, b, b2, b_twice, k1, k, m, arow, ax, ax2, nb, tile0;
     } p[kBatchMax];
     int n_maps, n, tiles, ldo;
     int* status;

@@ -102,3 +102,22 @@ def test_step_and_feature_gradient_vs_oracle(d, off):
     X, pooled, targets = _features(plan, d, w)
     preds, loss, dh = _step(heads, plan, g, X, pooled, targets, off)
     _check(w, hw, heads, plan, X, targets, preds, loss, dh)
+
+
+def test_weight_gradients_add_the_small_terms_while_the_sum_is_small():
+    """P and dS enter the weight gradients as two bf16 operands, hi and lo; one long
+    sample of positive rows, where the hi products of W_v's gradient add to one growing
+    sum and the lo ones lose the more bits the later they come.  The bounds lie between
+    the two orders' errors on these inputs: W_k 1.28e-5 and W_v 1.46e-5 with every lo
+    product after the last hi one, 1.02e-5 and 1.26e-5 with 64 keys of each in turn."""
+    d = 512
+    w, hw, heads, plan = _setup(d, [[3000]], kinds=(synth.HEAD_XATTN,))
+    g = R.DeviceGroup(plan)
+    X, _, targets = _features(plan, d, w)
+    X = X.abs()
+    _step(heads, plan, g, X, None, targets)
+    p = M.widen_tree(synth.to_numpy_tree(hw[0]))
+    _, _, gr = M.tenant_step(1, p, [f64(X)], f64(targets)[None])
+    e = {k: np.linalg.norm(f64(heads.grads[0][k]) - gr[k]) / np.linalg.norm(gr[k])
+         for k in ("wk", "wv")}
+    assert e["wk"] < 1.15e-5 and e["wv"] < 1.36e-5, e
