@@ -148,10 +148,10 @@ __device__ __forceinline__ int bwd_pass(const CUtensorMap& t_qkv_o, const CUtens
     constexpr bool IS_DQ = MODE == abwd::DQ;
     const int H = p.H, Hkv = p.Hkv, rope_ld = p.rope_ld, ldq = p.ldq;
     const int* __restrict__ cu = p.cu;
-    const float* __restrict__ lse = p.lse;
-    const float* __restrict__ Dsum = p.Dsum;
+    const float* lse = p.lse;
+    const float* Dsum = p.Dsum;
     const int* __restrict__ pos = p.pos;
-    const float2* __restrict__ rope = p.rope;
+    const float2* rope = p.rope;
     uint16_t* __restrict__ dqkv = p.dqkv;
     const float scale_log2 = p.scale_log2, scale = p.scale;
     uint8_t* sA1 = sm;
@@ -570,7 +570,7 @@ __device__ __forceinline__ int bwd_pass(const CUtensorMap& t_qkv_o, const CUtens
                         if (rv) {
                             const float2* src = rope + (size_t)(c * 32) * rope_ld + pr;
 #pragma unroll
-                            for (int e = 0; e < 32; ++e) cs[e] = __ldg(src + (size_t)e * rope_ld);
+                            for (int e = 0; e < 32; ++e) cs[e] = src[(size_t)e * rope_ld];
                         }
                         uint32_t lo[32], hi[32];
                         tmem_ld32(ta + c * 32, lo);

@@ -34,7 +34,7 @@ namespace jnx {
 // 64 x 64 tiles through shared memory, 16-byte loads along the source rows
 // and 16-byte stores along the destination rows when the buffers are 16-byte
 // aligned (vec), element by element at the edges and otherwise.
-__global__ void __launch_bounds__(256) k_transpose(const uint16_t* __restrict__ src, int rows,
+__global__ void __launch_bounds__(256) k_transpose(const uint16_t* src, int rows,
                                                    int cols, uint16_t* __restrict__ dst, int vec) {
     pdl_entry();
     __shared__ uint16_t tile[64][64 + 2];
@@ -97,9 +97,9 @@ jnx_status transpose_launch(const uint16_t* src, int batch, int rows, int cols, 
 // One warp per row; dres (may be null, may alias dx) is the gradient that
 // reaches x along the residual path.  Also writes bf16(dx) when dx_bf is set.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_rms_bwd(const float* __restrict__ x,
-                                                 const uint16_t* __restrict__ gamma, float eps,
-                                                 const float* __restrict__ dn, const float* dres,
+__global__ void __launch_bounds__(256) k_rms_bwd(const float* x,
+                                                 const uint16_t* gamma, float eps,
+                                                 const float* dn, const float* dres,
                                                  int M, int d, float* dx, uint16_t* dx_bf) {
     pdl_entry();
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -144,9 +144,9 @@ __global__ void __launch_bounds__(256) k_rms_bwd(const float* __restrict__ x,
 // registers, so every input byte is read once; the row sums are combined
 // over the warps in a fixed order.
 template <int NU>
-__global__ void __launch_bounds__(256) k_rms_bwd_row(const float* __restrict__ x,
-                                                     const uint16_t* __restrict__ gamma, float eps,
-                                                     const float* __restrict__ dn, const float* dres,
+__global__ void __launch_bounds__(256) k_rms_bwd_row(const float* x,
+                                                     const uint16_t* gamma, float eps,
+                                                     const float* dn, const float* dres,
                                                      int d, float* dx, uint16_t* dx_bf) {
     pdl_entry();
     __shared__ float red[2][8];
@@ -230,8 +230,8 @@ jnx_status rms_bwd_launch(const float* x, const uint16_t* gamma, float eps, cons
 // columns of dO * O (both as the bf16 values the backward kernels read).
 // One warp per (row, head).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_attn_bwd_prep(const float* __restrict__ datt,
-                                                       const uint16_t* __restrict__ att, int M,
+__global__ void __launch_bounds__(256) k_attn_bwd_prep(const float* datt,
+                                                       const uint16_t* att, int M,
                                                        int H, int hd, uint16_t* __restrict__ dO,
                                                        float* __restrict__ D) {
     pdl_entry();
@@ -241,13 +241,25 @@ __global__ void __launch_bounds__(256) k_attn_bwd_prep(const float* __restrict__
     const int row = (int)(w / H), h = (int)(w % H);
     const size_t base = (size_t)row * H * hd + (size_t)h * hd;
     float acc = 0.f;
-    for (int c = lane * 4; c < hd; c += 128) {
-        const float4 g = *reinterpret_cast<const float4*>(datt + base + c);
-        const uint2 o = *reinterpret_cast<const uint2*>(att + base + c);
-        const uint32_t p0 = pack_bf2(g.x, g.y), p1 = pack_bf2(g.z, g.w);
-        *reinterpret_cast<uint2*>(dO + base + c) = make_uint2(p0, p1);
-        acc += bf2f(p0 & 0xFFFF) * bf2f(o.x & 0xFFFF) + bf2f(p0 >> 16) * bf2f(o.x >> 16) +
-               bf2f(p1 & 0xFFFF) * bf2f(o.y & 0xFFFF) + bf2f(p1 >> 16) * bf2f(o.y >> 16);
+    for (int c0 = lane * 4; c0 < hd; c0 += 256) {  // two columns' loads ahead of the stores
+        float4 g[2];
+        uint2 o[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c = c0 + 128 * k;
+            if (c >= hd) break;
+            g[k] = *reinterpret_cast<const float4*>(datt + base + c);
+            o[k] = *reinterpret_cast<const uint2*>(att + base + c);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c = c0 + 128 * k;
+            if (c >= hd) break;
+            const uint32_t p0 = pack_bf2(g[k].x, g[k].y), p1 = pack_bf2(g[k].z, g[k].w);
+            *reinterpret_cast<uint2*>(dO + base + c) = make_uint2(p0, p1);
+            acc += bf2f(p0 & 0xFFFF) * bf2f(o[k].x & 0xFFFF) + bf2f(p0 >> 16) * bf2f(o[k].x >> 16) +
+                   bf2f(p1 & 0xFFFF) * bf2f(o[k].y & 0xFFFF) + bf2f(p1 >> 16) * bf2f(o[k].y >> 16);
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -383,8 +395,8 @@ __global__ void __launch_bounds__(128) k_seg_up(const __grid_constant__ SegRows 
 // CTA's 256 columns.  4 warps x 64 columns; rows in steps of 32 (two k16
 // steps), double-buffered.
 __global__ void __launch_bounds__(128) k_seg_tn(const __grid_constant__ SegChunks ch,
-                                                const uint16_t* __restrict__ U, int ldu,
-                                                const uint16_t* __restrict__ V, int ldv, int n,
+                                                const uint16_t* U, int ldu,
+                                                const uint16_t* V, int ldv, int n,
                                                 float* __restrict__ part) {
     pdl_entry();
     using namespace seg;
@@ -457,7 +469,7 @@ __global__ void __launch_bounds__(128) k_seg_tn(const __grid_constant__ SegChunk
 // added) to the tenant's gradient slice: [16, n] (TRANS = false) or [n, 16].
 template <bool TRANS>
 __global__ void __launch_bounds__(256) k_seg_reduce(const __grid_constant__ SegChunks ch,
-                                                    const float* __restrict__ part, int n,
+                                                    const float* part, int n,
                                                     float* __restrict__ grad, long long gstride,
                                                     int add) {
     pdl_entry();
@@ -577,8 +589,8 @@ constexpr int WG_BM = 64, WG_BN = 128, WG_ROWS = 32;
 }
 
 __global__ void __launch_bounds__(128) k_seg_wgrad(const __grid_constant__ SegRows sr,
-                                                   const uint16_t* __restrict__ U, int ldu,
-                                                   const uint16_t* __restrict__ V, int ldv,
+                                                   const uint16_t* U, int ldu,
+                                                   const uint16_t* V, int ldv,
                                                    int m, int n, float* __restrict__ grad,
                                                    long long gstride, int add) {
     pdl_entry();
@@ -688,7 +700,7 @@ jnx_status seg_wgrad_launch(const SegRows& sr, const uint16_t* U, int ldu, const
 // MLP heads: d hidden[row] = (dz[s] W1) / L_s for every row of sample s.
 // One CTA per (sample, 256-column block); dz [n_samples, ldz] fp32.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_mlp_dfeat(const float* __restrict__ dz, int ldz,
+__global__ void __launch_bounds__(256) k_mlp_dfeat(const float* dz, int ldz,
                                                    const int* __restrict__ cu,
                                                    const int* __restrict__ sample_slot,
                                                    const __grid_constant__ MlpFeatTable tab, int d,

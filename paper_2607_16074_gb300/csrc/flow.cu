@@ -65,8 +65,8 @@ constexpr int kTimeRows = 32;
 
 // dot product of the bf16 row w [dm] with the fp32 vector v [dm] in shared
 // memory, summed over the warp (every lane returns the sum)
-__device__ __forceinline__ float warp_row_dot(const uint16_t* __restrict__ w,
-                                              const float* __restrict__ v, int dm, int lane) {
+__device__ __forceinline__ float warp_row_dot(const uint16_t* w,
+                                              const float* v, int dm, int lane) {
     float acc = 0.f;
     for (int k = 8 * lane; k < dm; k += 256) {
         const uint4 q = *reinterpret_cast<const uint4*>(w + k);
@@ -82,11 +82,11 @@ __device__ __forceinline__ float warp_row_dot(const uint16_t* __restrict__ w,
     return acc;
 }
 
-__global__ void __launch_bounds__(256) k_flow_time1(const float* __restrict__ tau,
+__global__ void __launch_bounds__(256) k_flow_time1(const float* tau,
                                                     const int* __restrict__ sample_slot,
                                                     const __grid_constant__ FlowSlots fs,
-                                                    FlowDims dd, const uint16_t* __restrict__ t1,
-                                                    const uint16_t* __restrict__ tb1,
+                                                    FlowDims dd, const uint16_t* t1,
+                                                    const uint16_t* tb1,
                                                     float* __restrict__ sfeat,
                                                     float* __restrict__ z1, int per,
                                                     int by_slot, int step0, int n_steps) {
@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(256) k_flow_time1(const float* __restrict__ ta
 
 __global__ void __launch_bounds__(256) k_flow_time2(const int* __restrict__ sample_slot,
                                                     const __grid_constant__ FlowSlots fs,
-                                                    FlowDims dd, const uint16_t* __restrict__ t2,
-                                                    const uint16_t* __restrict__ tb2,
-                                                    const float* __restrict__ z1,
+                                                    FlowDims dd, const uint16_t* t2,
+                                                    const uint16_t* tb2,
+                                                    const float* z1,
                                                     float* __restrict__ phi, int per,
                                                     int by_slot) {
     pdl_entry();
@@ -138,11 +138,11 @@ __global__ void __launch_bounds__(256) k_flow_time2(const int* __restrict__ samp
 // h = x W_in^T + b_in + pos_c + phi_s.  One CTA per action row.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_flow_embed(
-    const float* __restrict__ actions, const float* __restrict__ noise,
-    const float* __restrict__ tau, const float* __restrict__ xin,
+    const float* actions, const float* noise,
+    const float* tau, const float* xin,
     const int* __restrict__ sample_slot, const __grid_constant__ FlowSlots fs, FlowDims dd,
-    const uint16_t* __restrict__ w_in, const uint16_t* __restrict__ b_in,
-    const uint16_t* __restrict__ pos, const float* __restrict__ phi, int phi_by_slot,
+    const uint16_t* w_in, const uint16_t* b_in,
+    const uint16_t* pos, const float* phi, int phi_by_slot,
     float* __restrict__ x_out, float* __restrict__ u_out, float* __restrict__ h) {
     pdl_entry();
     __shared__ float xs[kMaxD];
@@ -150,6 +150,15 @@ __global__ void __launch_bounds__(256) k_flow_embed(
     const int s = r / C, c = r % C;
     const int slot = sample_slot[s], t = fs.tenant[slot];
     const float* ph = phi + (size_t)(phi_by_slot ? slot : s) * dm;
+    // the sums' first terms, loaded before the barrier (dm is at most 1,024)
+    float first[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j = threadIdx.x + 256 * i;
+        if (j < dm)
+            first[i] = bf2f(b_in[(size_t)t * dm + j]) + bf2f(pos[((size_t)t * C + c) * dm + j]) +
+                       ph[j];
+    }
     if (threadIdx.x < D) {
         const size_t e = (size_t)r * D + threadIdx.x;
         float x;
@@ -168,14 +177,16 @@ __global__ void __launch_bounds__(256) k_flow_embed(
     // a weight row is 2 D contiguous bytes: 16-byte loads where rows allow them
     // (2-byte ones kept a row's 32 loads in turn: 37.6 us for 512 rows, 10.6 now)
     const bool vec = D % 8 == 0 && (reinterpret_cast<uintptr_t>(w_in) & 15) == 0;
-    for (int j = threadIdx.x; j < dm; j += blockDim.x) {
-        float acc = bf2f(b_in[(size_t)t * dm + j]) + bf2f(pos[((size_t)t * C + c) * dm + j]) +
-                    ph[j];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j = threadIdx.x + 256 * i;
+        if (j >= dm) break;
+        float acc = first[i];
         const uint16_t* wr = W + (size_t)j * D;
         if (vec) {
 #pragma unroll 4
             for (int k = 0; k < D; k += 8) {
-                const uint4 q = __ldg(reinterpret_cast<const uint4*>(wr + k));
+                const uint4 q = *reinterpret_cast<const uint4*>(wr + k);
                 const uint32_t u[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -301,8 +312,8 @@ __device__ __forceinline__ void mma4(float (&c)[4], const uint32_t (&a)[4], uint
 constexpr int kFwdRing = 4;
 constexpr int kFwdSmem = kFwdRing * 2 * kTileB + kMaxC * kRowB;
 template <int KS>
-__global__ void __launch_bounds__(128) k_flow_attn_fwd(const uint16_t* __restrict__ qkv,
-                                                       const uint16_t* __restrict__ kvc,
+__global__ void __launch_bounds__(128) k_flow_attn_fwd(const uint16_t* qkv,
+                                                       const uint16_t* kvc,
                                                        const int* __restrict__ cu, FlowDims dd,
                                                        uint16_t* __restrict__ o,
                                                        float* __restrict__ lse) {
@@ -498,9 +509,9 @@ __device__ __forceinline__ void bwd_query_side(uint32_t sq, uint8_t* sg_gen, flo
 // (query tile, key slice); the KS partial dq are summed in slice order.
 template <int KS>
 __global__ void __launch_bounds__(128) k_flow_attn_bwd_q(
-    const uint16_t* __restrict__ qkv, const uint16_t* __restrict__ kvc, const int* __restrict__ cu,
-    FlowDims dd, const uint16_t* __restrict__ o, const float* __restrict__ dO,
-    const float* __restrict__ lse, uint16_t* __restrict__ dqkv) {
+    const uint16_t* qkv, const uint16_t* kvc, const int* __restrict__ cu,
+    FlowDims dd, const uint16_t* o, const float* dO,
+    const float* lse, uint16_t* __restrict__ dqkv) {
     pdl_entry();
     constexpr int NK = kKT / KS, NT = NK / 8;
     __shared__ __align__(128) uint8_t sbuf[4 * kTileB];
@@ -636,9 +647,9 @@ __global__ void __launch_bounds__(128) k_flow_attn_bwd_q(
 // gradients are complete in one pass (no accumulation across CTAs).
 template <int NQ>
 __global__ void __launch_bounds__(128) k_flow_attn_bwd_kv(
-    const uint16_t* __restrict__ qkv, const uint16_t* __restrict__ kvc, const int* __restrict__ cu,
-    FlowDims dd, const uint16_t* __restrict__ o, const float* __restrict__ dO,
-    const float* __restrict__ lse, uint16_t* __restrict__ dqkv, uint16_t* __restrict__ dkvc) {
+    const uint16_t* qkv, const uint16_t* kvc, const int* __restrict__ cu,
+    FlowDims dd, const uint16_t* o, const float* dO,
+    const float* lse, uint16_t* __restrict__ dqkv, uint16_t* __restrict__ dkvc) {
     pdl_entry();
     constexpr int NT = 2 * NQ;  // n8 query tiles
     __shared__ __align__(128) uint8_t sbuf[4 * kTileB];  // q, dO, K, V
@@ -735,12 +746,12 @@ __global__ void __launch_bounds__(128) k_flow_attn_bwd_kv(
 // per output element (a warp per row took its outputs in turn, a load and a
 // shuffle tree each: 34 us for 32 rows x 32 outputs of depth 1,024, 5.3 now).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_flow_out(const uint16_t* __restrict__ nf,
+__global__ void __launch_bounds__(256) k_flow_out(const uint16_t* nf,
                                                   const int* __restrict__ sample_slot,
                                                   const __grid_constant__ FlowSlots fs, FlowDims dd,
-                                                  const uint16_t* __restrict__ w_out,
-                                                  const uint16_t* __restrict__ b_out,
-                                                  const float* __restrict__ u,
+                                                  const uint16_t* w_out,
+                                                  const uint16_t* b_out,
+                                                  const float* u,
                                                   float* __restrict__ v, float* __restrict__ dv) {
     pdl_entry();
     const int r = blockIdx.x, lane = threadIdx.x & 31;
@@ -756,7 +767,7 @@ __global__ void __launch_bounds__(256) k_flow_out(const uint16_t* __restrict__ n
     for (int i = 0; i < 4; ++i)  // columns 8 lane + 256 i, i < dm / 256
         if (256 * i < dm) {
             const uint4 x = *reinterpret_cast<const uint4*>(xr + 256 * i);
-            const uint4 q = __ldg(reinterpret_cast<const uint4*>(wr + 256 * i));
+            const uint4 q = *reinterpret_cast<const uint4*>(wr + 256 * i);
             const uint32_t x4[4] = {x.x, x.y, x.z, x.w}, w4[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -781,8 +792,8 @@ __global__ void __launch_bounds__(256) k_flow_out(const uint16_t* __restrict__ n
 // loss[tenant] = sum over its elements of (v - u)^2 / n_t: one CTA per slot,
 // thread i its elements i, i + 256, ..., then a fixed tree.
 __global__ void __launch_bounds__(256) k_flow_loss(const __grid_constant__ FlowSlots fs,
-                                                   FlowDims dd, const float* __restrict__ v,
-                                                   const float* __restrict__ u,
+                                                   FlowDims dd, const float* v,
+                                                   const float* u,
                                                    float* __restrict__ loss) {
     pdl_entry();
     __shared__ float red[8];
@@ -805,7 +816,7 @@ __global__ void __launch_bounds__(256) k_flow_loss(const __grid_constant__ FlowS
 }
 
 // Euler step of the sampler: x += dt v.
-__global__ void k_flow_euler(float* __restrict__ x, const float* __restrict__ v, float dt, int n) {
+__global__ void k_flow_euler(float* x, const float* v, float dt, int n) {
     pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) x[i] += dt * v[i];
@@ -815,34 +826,48 @@ __global__ void k_flow_euler(float* __restrict__ x, const float* __restrict__ v,
 // backward of the output layer
 // ---------------------------------------------------------------------------
 // dnf[r] = dv[r] W_out (per action row).
-__global__ void __launch_bounds__(256) k_flow_out_bwd(const float* __restrict__ dv,
+__global__ void __launch_bounds__(256) k_flow_out_bwd(const float* dv,
                                                       const int* __restrict__ sample_slot,
                                                       const __grid_constant__ FlowSlots fs,
                                                       FlowDims dd,
-                                                      const uint16_t* __restrict__ w_out,
+                                                      const uint16_t* w_out,
                                                       float* __restrict__ dnf) {
     pdl_entry();
     const int r = blockIdx.x, dm = dd.dm, D = dd.D;
     const int t = fs.tenant[sample_slot[r / dd.C]];
     __shared__ float g[kMaxD];
+    // four consecutive columns a thread (dm is a multiple of 4, at most 1,024; w_out
+    // 16-byte aligned), eight weight rows in flight, the first before the barrier
+    constexpr int U = 8;
+    const int j = 4 * threadIdx.x;
+    const uint16_t* wc = w_out + (size_t)t * D * dm + j;
+    uint2 q[U];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            q[u] = make_uint2(0u, 0u);
+            if (j < dm && k0 + u < D)
+                q[u] = *reinterpret_cast<const uint2*>(wc + (size_t)(k0 + u) * dm);
+        }
+    };
+    load(0);
     if (threadIdx.x < D) g[threadIdx.x] = dv[(size_t)r * D + threadIdx.x];
     __syncthreads();
-    // four consecutive columns a thread (dm is a multiple of 4, w_out 16-byte
-    // aligned), eight weight rows' loads in flight
-    for (int j = 4 * threadIdx.x; j < dm; j += 4 * blockDim.x) {
-        float acc[4] = {};
-        const uint16_t* wc = w_out + (size_t)t * D * dm + j;
-#pragma unroll 8
-        for (int k = 0; k < D; ++k) {
-            const uint2 q = __ldg(reinterpret_cast<const uint2*>(wc + (size_t)k * dm));
-            acc[0] += g[k] * __uint_as_float(q.x << 16);
-            acc[1] += g[k] * __uint_as_float(q.x & 0xffff0000u);
-            acc[2] += g[k] * __uint_as_float(q.y << 16);
-            acc[3] += g[k] * __uint_as_float(q.y & 0xffff0000u);
+    if (j >= dm) return;
+    float acc[4] = {};
+    for (int k0 = 0; k0 < D; k0 += U) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float gk = k0 + u < D ? g[k0 + u] : 0.f;
+            acc[0] += gk * __uint_as_float(q[u].x << 16);
+            acc[1] += gk * __uint_as_float(q[u].x & 0xffff0000u);
+            acc[2] += gk * __uint_as_float(q[u].y << 16);
+            acc[3] += gk * __uint_as_float(q[u].y & 0xffff0000u);
         }
-        *reinterpret_cast<float4*>(dnf + (size_t)r * dm + j) =
-            make_float4(acc[0], acc[1], acc[2], acc[3]);
+        load(k0 + U);
     }
+    *reinterpret_cast<float4*>(dnf + (size_t)r * dm + j) =
+        make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
 
 // Four consecutive gradient elements written or, with add, added to.
@@ -860,8 +885,8 @@ __device__ __forceinline__ void store4(float* p, const float (&v)[4], int add) {
 
 // dW_out[t][k, j] = sum over the tenant's rows of dv[r, k] nf[r, j];
 // db_out[t][k] = sum dv[r, k].  One CTA per (slot, k); threads along j.
-__global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* __restrict__ dv,
-                                                        const uint16_t* __restrict__ nf,
+__global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* dv,
+                                                        const uint16_t* nf,
                                                         const __grid_constant__ FlowSlots fs,
                                                         FlowDims dd, float* __restrict__ gw,
                                                         float* __restrict__ gb, int add) {
@@ -874,7 +899,7 @@ __global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* __restrict_
 #pragma unroll 8
         for (int r = r0; r < r1; ++r) {
             const float g = dv[(size_t)r * D + k];
-            const uint2 q = __ldg(reinterpret_cast<const uint2*>(nf + (size_t)r * dm + j));
+            const uint2 q = *reinterpret_cast<const uint2*>(nf + (size_t)r * dm + j);
             acc[0] += g * __uint_as_float(q.x << 16);
             acc[1] += g * __uint_as_float(q.x & 0xffff0000u);
             acc[2] += g * __uint_as_float(q.y << 16);
@@ -899,8 +924,8 @@ __global__ void __launch_bounds__(256) k_flow_out_wgrad(const float* __restrict_
 // dimensions 8 w .. + 7 and the chunk steps c = w (mod 8); rows in order, several
 // loads in flight (a thread per column with every dimension: 90 us for eight
 // tenants of 64 rows, 31 now).
-__global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* __restrict__ dh,
-                                                          const float* __restrict__ x,
+__global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* dh,
+                                                          const float* x,
                                                           const __grid_constant__ FlowSlots fs,
                                                           FlowDims dd, float* __restrict__ gw,
                                                           float* __restrict__ gb,
@@ -939,7 +964,7 @@ __global__ void __launch_bounds__(256) k_flow_embed_wgrad(const float* __restric
 
 // dphi[s, j] = sum_c dh[s C + c, j] (the time embedding is added to every
 // action row of the sample), c in order.
-__global__ void __launch_bounds__(256) k_flow_dphi(const float* __restrict__ dh, FlowDims dd,
+__global__ void __launch_bounds__(256) k_flow_dphi(const float* dh, FlowDims dd,
                                                    float* __restrict__ dphi) {
     pdl_entry();
     const int s = blockIdx.x, dm = dd.dm, C = dd.C;
@@ -955,9 +980,9 @@ __global__ void __launch_bounds__(256) k_flow_dphi(const float* __restrict__ dh,
 // per row), rows j = jg, jg + 16, ...; the 16 row groups are summed in order.
 __global__ void __launch_bounds__(256) k_flow_time_bwd(const int* __restrict__ sample_slot,
                                                        const __grid_constant__ FlowSlots fs,
-                                                       FlowDims dd, const uint16_t* __restrict__ t2,
-                                                       const float* __restrict__ z1,
-                                                       const float* __restrict__ dphi,
+                                                       FlowDims dd, const uint16_t* t2,
+                                                       const float* z1,
+                                                       const float* dphi,
                                                        float* __restrict__ dz1) {
     pdl_entry();
     extern __shared__ float sh[];  // dphi [dm], then partials [16][128]
@@ -1001,8 +1026,8 @@ __global__ void __launch_bounds__(256) k_flow_time_bwd(const int* __restrict__ s
 constexpr int kOuterRows = 8;
 
 template <bool SILU>
-__global__ void __launch_bounds__(256) k_flow_outer(const float* __restrict__ A,
-                                                    const float* __restrict__ Bm,
+__global__ void __launch_bounds__(256) k_flow_outer(const float* A,
+                                                    const float* Bm,
                                                     const __grid_constant__ FlowSlots fs,
                                                     FlowDims dd, float* __restrict__ gw,
                                                     float* __restrict__ gb, int add) {

@@ -625,7 +625,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tbase, uint8_t* stg, int 
             if (rot) {
                 const float2* src = p.rope + (size_t)(hchunk * 32) * p.rope_ld + pos;
 #pragma unroll
-                for (int e = 0; e < 32; ++e) cs[e] = __ldg(src + (size_t)e * p.rope_ld);
+                for (int e = 0; e < 32; ++e) cs[e] = src[(size_t)e * p.rope_ld];
             }
             uint32_t lo[32], hi[32];
             tmem_ld32(tbase + c * 32, lo);

@@ -142,7 +142,7 @@ static_assert(8 * kLinS * kLinRedPad * 4 <= kLinSmem, "partial sums reuse the ri
 
 template <int LAYER>
 __global__ void __launch_bounds__(256, 2) k_head_lin(const __grid_constant__ HeadTable tab,
-                                                  const float* __restrict__ in, int ld_in,
+                                                  const float* in, int ld_in,
                                                   float* __restrict__ z_out, float* __restrict__ h_out,
                                                   int ld_out, const int* __restrict__ sample_target,
                                                   float* __restrict__ preds) {
@@ -261,8 +261,8 @@ __global__ void __launch_bounds__(256, 2) k_head_lin(const __grid_constant__ Hea
 constexpr int kLossThreads = 1024;
 
 __global__ void __launch_bounds__(kLossThreads) k_l2_loss(const __grid_constant__ HeadTable tab,
-                                                 const float* __restrict__ y, int ld_y,
-                                                 const float* __restrict__ targets,
+                                                 const float* y, int ld_y,
+                                                 const float* targets,
                                                  const int* __restrict__ sample_target,
                                                  float* __restrict__ dy, float* __restrict__ loss) {
     pdl_entry();
@@ -295,8 +295,8 @@ __global__ void __launch_bounds__(kLossThreads) k_l2_loss(const __grid_constant_
 template <class OT>
 __global__ void __launch_bounds__(256) k_head_dw_out(const __grid_constant__ HeadTable tab,
                                                      const __grid_constant__ OT opt, AdamHp hp,
-                                                     const float* __restrict__ dy, int ld_y,
-                                                     const float* __restrict__ h, int ld_h) {
+                                                     const float* dy, int ld_y,
+                                                     const float* h, int ld_h) {
     pdl_entry();
     __shared__ __align__(16) float sh[32][256];
     __shared__ __align__(16) float sd[32][16];
@@ -382,8 +382,8 @@ __global__ void __launch_bounds__(256) k_head_dw_out(const __grid_constant__ Hea
 constexpr int kBackCols = 128, kBackO = 64;
 
 __global__ void __launch_bounds__(256, 3) k_head_back_in(const __grid_constant__ HeadTable tab,
-                                                      const float* __restrict__ dy, int ld_y,
-                                                      const float* __restrict__ z, int ld_h,
+                                                      const float* dy, int ld_y,
+                                                      const float* z, int ld_h,
                                                       float* __restrict__ dh) {
     pdl_entry();
     __shared__ __align__(16) float sdy[kBackO][8];
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(256, 3) k_head_back_in(const __grid_constant__
             const int o = o0 + warp + 8 * i;
             wv[i] = make_uint2(0u, 0u);
             if (colok && o < hs.width)
-                wv[i] = __ldg(reinterpret_cast<const uint2*>(hs.w2 + (size_t)o * hs.hid + j0));
+                wv[i] = *reinterpret_cast<const uint2*>(hs.w2 + (size_t)o * hs.hid + j0);
         }
     };
     load(0);
@@ -473,8 +473,8 @@ constexpr int kDw1Rows = 8;
 template <class OT>
 __global__ void __launch_bounds__(256) k_mlp_dw1(const __grid_constant__ HeadTable tab,
                                                  const __grid_constant__ OT opt, AdamHp hp,
-                                                 const float* __restrict__ dz, int ld,
-                                                 const float* __restrict__ p, int ld_p) {
+                                                 const float* dz, int ld,
+                                                 const float* p, int ld_p) {
     pdl_entry();
     const HeadSlot& hs = tab.slot[blockIdx.x];
     if (hs.kind != JNX_HEAD_MLP) return;
@@ -565,7 +565,7 @@ __device__ __forceinline__ void split4(const float4 v, uint2& hi, uint2& lo) {
 // stride ldt); rows nr .. rows - 1 are zero.  16-byte loads: R, ld and c0
 // 16-byte aligned.
 __device__ __forceinline__ void xattn_split_rows(uint16_t* dst, int rows, int ldt,
-                                                 const float* __restrict__ R, int ld, size_t row0,
+                                                 const float* R, int ld, size_t row0,
                                                  int nr, int c0, int nc) {
     // a thread's eight loads are all in flight before the first is used (rows
     // * units is a multiple of 8 x 256: 32 rows, nc a multiple of 256)
@@ -576,7 +576,7 @@ __device__ __forceinline__ void xattn_split_rows(uint16_t* dst, int rows, int ld
         for (int k = 0; k < 8; ++k) {
             const int i = i0 + 256 * k, r = i / units, u = i % units;
             v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r < nr) v[k] = __ldg(reinterpret_cast<const float4*>(R + (row0 + r) * ld + c0 + 4 * u));
+            if (r < nr) v[k] = *reinterpret_cast<const float4*>(R + (row0 + r) * ld + c0 + 4 * u);
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -593,7 +593,7 @@ __device__ __forceinline__ void xattn_split_rows(uint16_t* dst, int rows, int ld
 // planes of a query-major tile tq[plane][q][j] and, if tk, a key-major tile
 // tk[plane][j][q]; entries past nr or nq are zero.
 __device__ __forceinline__ void xattn_split_chunk(uint16_t* tq, uint16_t* tk,
-                                                  const float* __restrict__ X, int j0, int nr,
+                                                  const float* X, int j0, int nr,
                                                   int nq) {
     float v[kMaxQ * kXRows / 256];
 #pragma unroll
@@ -618,7 +618,7 @@ __device__ __forceinline__ void xattn_split_chunk(uint16_t* tq, uint16_t* tk,
 }
 
 // The learned queries (bf16 [nq][dq], 16-byte aligned) into sQ.
-__device__ __forceinline__ void xattn_stage_q(uint16_t* sQ, int ldr, const uint16_t* __restrict__ q,
+__device__ __forceinline__ void xattn_stage_q(uint16_t* sQ, int ldr, const uint16_t* q,
                                               int nq, int dq) {
     const int units = dq / 8;
 #pragma unroll 4
@@ -635,7 +635,7 @@ __device__ __forceinline__ void xattn_stage_q(uint16_t* sQ, int ldr, const uint1
 // Per 32-key chunk (rows split into sR), warp w takes query tile w % 2 and
 // keys 8 (w / 2) .. + 7, over all dq.  Ends with a barrier.
 __device__ void xattn_scores(const uint16_t* ahi, const uint16_t* alo, int ldr, uint16_t* sR,
-                             const float* __restrict__ R, int ldkv, int r0, int ja, int jz,
+                             const float* R, int ldkv, int r0, int ja, int jz,
                              int nq, int dq, float scale, float* __restrict__ out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = warp & 1, nt = warp >> 1, g = lane >> 2, t = lane & 3;
@@ -824,8 +824,8 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 3)
     k_xattn_fwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
                                                    const int* __restrict__ sample_slot,
-                                                   int sample0, const float* __restrict__ kbuf,
-                                                   const float* __restrict__ vbuf, int ldkv,
+                                                   int sample0, const float* kbuf,
+                                                   const float* vbuf, int ldkv,
                                                    float* __restrict__ P, float* __restrict__ h,
                                                    int ld_h) {
     pdl_entry();
@@ -896,11 +896,11 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
     k_xattn_bwd(const __grid_constant__ HeadTable tab, int g0,
                                                    const int* __restrict__ cu,
                                                    const int* __restrict__ sample_slot,
-                                                   int sample0, const float* __restrict__ kbuf,
-                                                   const float* __restrict__ vbuf, int ldkv,
-                                                   const float* __restrict__ P,
+                                                   int sample0, const float* kbuf,
+                                                   const float* vbuf, int ldkv,
+                                                   const float* P,
                                                    float* __restrict__ dS,
-                                                   const float* __restrict__ dO, int ld_h,
+                                                   const float* dO, int ld_h,
                                                    uint16_t* __restrict__ dkv,
                                                    uint16_t* __restrict__ planes, int ldp,
                                                    float* __restrict__ dQs, int kv_grads) {
@@ -1029,7 +1029,7 @@ __global__ void __cluster_dims__(kXCtas, 1, 1) __launch_bounds__(256, 2)
 template <class OT>
 __global__ void __launch_bounds__(256) k_xattn_dq(const __grid_constant__ HeadTable tab,
                                                   const __grid_constant__ OT opt, AdamHp hp,
-                                                  const float* __restrict__ dQs, int ld_h) {
+                                                  const float* dQs, int ld_h) {
     pdl_entry();
     const HeadSlot& hs = tab.slot[blockIdx.x];
     if (hs.kind != JNX_HEAD_XATTN) return;
@@ -1077,9 +1077,9 @@ constexpr int kGhAPad = 40;       // [query][key] operand row stride (bf16)
 __global__ void __launch_bounds__(256) k_xattn_gh(const __grid_constant__ HeadTable tab, int g0,
                                                   const int* __restrict__ cu,
                                                   const int* __restrict__ sample_slot,
-                                                  int sample0, const float* __restrict__ P,
-                                                  const float* __restrict__ dS,
-                                                  const uint16_t* __restrict__ X, int ldx,
+                                                  int sample0, const float* P,
+                                                  const float* dS,
+                                                  const uint16_t* X, int ldx,
                                                   float* __restrict__ HG, int ldg) {
     pdl_entry();
     static_assert(kMaxQ == 32, "two 16-row query tiles");
@@ -1206,8 +1206,8 @@ constexpr int kWgC = 64, kWgE = 128;
 template <class OT>
 __global__ void __launch_bounds__(256) k_xattn_wgrad(const __grid_constant__ HeadTable tab,
                                                      const __grid_constant__ OT opt, AdamHp hp,
-                                                     const float* __restrict__ HG, int ldg,
-                                                     const float* __restrict__ dO, int ld_h) {
+                                                     const float* HG, int ldg,
+                                                     const float* dO, int ld_h) {
     pdl_entry();
     __shared__ __align__(16) float sh[kMaxQ][kWgE];  // H_s, then G_t
     __shared__ __align__(16) float so[kMaxQ][kWgC];  // dO_s, then Q

@@ -115,6 +115,12 @@ __device__ __forceinline__ float adamw_elem(float g, float& m, float& v, float p
 // grid ahead is complete and its writes are visible, then lets the grid behind
 // be set up.  Since every kernel in a chain waits, the grid ahead being complete
 // means that all before it are, too.
+//
+// What a kernel ahead may have written is read by plain loads: no __ldg and no
+// const __restrict__ parameter.  Those allow non-coherent loads, whose data must
+// not change while the kernel lives, and this kernel lives before the one ahead
+// has ended; nor would the compiler have to keep them behind the wait.  Tables of
+// the plan (int), which the host uploads, and outputs may be __restrict__.
 __device__ __forceinline__ void pdl_entry() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -32,7 +32,7 @@ __device__ __forceinline__ uint32_t lsw(int r, int ch) {
 // tiles are about one per SM), so the ring is as deep as 48 KB hold: two slots
 // took 15.2 us (one part) and 24.4 (three) for 9,700 rows of K = 2,048, now 12.1 and 20.6.
 template <int NP>
-__global__ void __launch_bounds__(128) k_lora_down(const uint16_t* __restrict__ x, int ldx, int K,
+__global__ void __launch_bounds__(128) k_lora_down(const uint16_t* x, int ldx, int K,
                                                    const __grid_constant__ LoraSlots ls,
                                                    const __grid_constant__ LoraDown ld,
                                                    uint16_t* __restrict__ t, int ldt) {

@@ -32,9 +32,9 @@ __device__ __forceinline__ const uint16_t* pack_source(int src, const uint16_t* 
 }
 
 __global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ gather, int n_tokens,
-                                              const uint16_t* __restrict__ vision, int64_t n_vision,
+                                              const uint16_t* vision, int64_t n_vision,
                                               const int32_t* __restrict__ text_ids, int64_t n_text,
-                                              const uint16_t* __restrict__ table, int vocab, int d,
+                                              const uint16_t* table, int vocab, int d,
                                               float* __restrict__ x, int* status) {
     pdl_entry();
     const int tok = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -45,17 +45,25 @@ __global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ gather
     if (row == nullptr && lane == 0) report(status, JNX_ERR_DEVICE_BOUNDS);
     float4* out = reinterpret_cast<float4*>(x + (size_t)tok * d);
     const int nchunk = d / 8;
-    for (int c = lane; c < nchunk; c += 32) {
-        float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-        if (row) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + c);
-            lo = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u),
-                             __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
-            hi = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u),
-                             __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xFFFF0000u));
+    for (int c0 = lane; c0 < nchunk; c0 += 128) {  // four loads ahead of their stores
+        uint4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + 32 * k;
+            v[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (row && c < nchunk) v[k] = reinterpret_cast<const uint4*>(row)[c];
         }
-        out[2 * c] = lo;
-        out[2 * c + 1] = hi;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + 32 * k;
+            if (c >= nchunk) break;
+            out[2 * c] =
+                make_float4(__uint_as_float(v[k].x << 16), __uint_as_float(v[k].x & 0xFFFF0000u),
+                            __uint_as_float(v[k].y << 16), __uint_as_float(v[k].y & 0xFFFF0000u));
+            out[2 * c + 1] =
+                make_float4(__uint_as_float(v[k].z << 16), __uint_as_float(v[k].z & 0xFFFF0000u),
+                            __uint_as_float(v[k].w << 16), __uint_as_float(v[k].w & 0xFFFF0000u));
+        }
     }
 }
 
@@ -83,8 +91,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 template <int V>
-__global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
-                                                 const uint16_t* __restrict__ gamma, float eps,
+__global__ void __launch_bounds__(256) k_rmsnorm(const float* x,
+                                                 const uint16_t* gamma, float eps,
                                                  int M, uint16_t* __restrict__ out,
                                                  float* __restrict__ copy) {
     pdl_entry();
@@ -93,13 +101,17 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
     const int lane = threadIdx.x & 31;
     if (row >= M) return;
     const float4* xr = reinterpret_cast<const float4*>(x + (size_t)row * D);
+    const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
     float4 v[V];
+    uint2 gg[V];  // in flight with the row: behind the first store it waited once more
+#pragma unroll
+    for (int i = 0; i < V; ++i) v[i] = xr[lane + 32 * i];
+#pragma unroll
+    for (int i = 0; i < V; ++i) gg[i] = g2[lane + 32 * i];
     float ss = 0.f;
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-        v[i] = __ldg(xr + lane + 32 * i);
+    for (int i = 0; i < V; ++i)
         ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
-    }
     ss = warp_sum(ss);
     const float r = rsqrtf(ss / (float)D + eps);
     if (copy) {
@@ -108,13 +120,11 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
         for (int i = 0; i < V; ++i) crow[lane + 32 * i] = v[i];
     }
     uint2* orow = reinterpret_cast<uint2*>(out + (size_t)row * D);
-    const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
 #pragma unroll
     for (int i = 0; i < V; ++i) {
-        const uint2 gg = __ldg(g2 + lane + 32 * i);
         uint2 o;
-        o.x = pack_bf2(v[i].x * r * bf2f(gg.x & 0xFFFF), v[i].y * r * bf2f(gg.x >> 16));
-        o.y = pack_bf2(v[i].z * r * bf2f(gg.y & 0xFFFF), v[i].w * r * bf2f(gg.y >> 16));
+        o.x = pack_bf2(v[i].x * r * bf2f(gg[i].x & 0xFFFF), v[i].y * r * bf2f(gg[i].x >> 16));
+        o.y = pack_bf2(v[i].z * r * bf2f(gg[i].y & 0xFFFF), v[i].w * r * bf2f(gg[i].y >> 16));
         orow[lane + 32 * i] = o;
     }
 }
@@ -128,10 +138,10 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const float* __restrict__ x,
 template <int V>
 __global__ void __launch_bounds__(256)
     k_pack_prep(const int32_t* __restrict__ gather, int n_tokens,
-                const uint16_t* __restrict__ vision, int64_t n_vision,
+                const uint16_t* vision, int64_t n_vision,
                 const int32_t* __restrict__ text_ids, int64_t n_text,
-                const uint16_t* __restrict__ table, int vocab, float* __restrict__ x, int* status,
-                const uint16_t* __restrict__ gamma, uint16_t* __restrict__ y,
+                const uint16_t* table, int vocab, float* __restrict__ x, int* status,
+                const uint16_t* gamma, uint16_t* __restrict__ y,
                 float* __restrict__ ss) {
     pdl_entry();
     constexpr int D = V * 128;  // lane float4 i = 128-column block i
@@ -141,28 +151,43 @@ __global__ void __launch_bounds__(256)
     const uint16_t* row =
         pack_source(gather[tok], vision, n_vision, text_ids, n_text, table, vocab, D);
     if (row == nullptr && lane == 0) report(status, JNX_ERR_DEVICE_BOUNDS);
-    uint2 w[V];
-#pragma unroll
-    for (int i = 0; i < V; ++i)
-        w[i] = row ? __ldg(reinterpret_cast<const uint2*>(row) + lane + 32 * i) : make_uint2(0u, 0u);
+    const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
     float4* xr = reinterpret_cast<float4*>(x + (size_t)tok * D);
     uint2* yr = reinterpret_cast<uint2*>(y + (size_t)tok * D);
-    const uint2* g2 = reinterpret_cast<const uint2*>(gamma);
+    // G blocks at a time, the next G loaded ahead of the stores of these: a load
+    // behind a store waits for its own data only then
+    constexpr int G = V < 8 ? V : 8;
+    uint2 w[2][G], gg[2][G];
+    auto load = [&](int i0, uint2 (&wl)[G], uint2 (&gl)[G]) {
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const float4 v = make_float4(__uint_as_float(w[i].x << 16),
-                                     __uint_as_float(w[i].x & 0xFFFF0000u),
-                                     __uint_as_float(w[i].y << 16),
-                                     __uint_as_float(w[i].y & 0xFFFF0000u));
-        xr[lane + 32 * i] = v;
-        float t = 0.f;
-        t += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-        t = warp_sum(t);
-        if (lane == 0) ss[(size_t)tok * V + i] = t;
-        const uint2 gg = __ldg(g2 + lane + 32 * i);
-        yr[lane + 32 * i] =
-            make_uint2(pack_bf2(v.x * bf2f(gg.x & 0xFFFF), v.y * bf2f(gg.x >> 16)),
-                       pack_bf2(v.z * bf2f(gg.y & 0xFFFF), v.w * bf2f(gg.y >> 16)));
+        for (int k = 0; k < G; ++k) {
+            wl[k] = row ? reinterpret_cast<const uint2*>(row)[lane + 32 * (i0 + k)]
+                        : make_uint2(0u, 0u);
+            gl[k] = g2[lane + 32 * (i0 + k)];
+        }
+    };
+    load(0, w[0], gg[0]);
+#pragma unroll
+    for (int i0 = 0; i0 < V; i0 += G) {
+        const int b = i0 / G & 1;
+        if (i0 + G < V) load(i0 + G, w[b ^ 1], gg[b ^ 1]);
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            const int i = i0 + k;
+            const uint2 wk = w[b][k], gk = gg[b][k];
+            const float4 v = make_float4(__uint_as_float(wk.x << 16),
+                                         __uint_as_float(wk.x & 0xFFFF0000u),
+                                         __uint_as_float(wk.y << 16),
+                                         __uint_as_float(wk.y & 0xFFFF0000u));
+            xr[lane + 32 * i] = v;
+            float t = 0.f;
+            t += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+            t = warp_sum(t);
+            if (lane == 0) ss[(size_t)tok * V + i] = t;
+            yr[lane + 32 * i] =
+                make_uint2(pack_bf2(v.x * bf2f(gk.x & 0xFFFF), v.y * bf2f(gk.x >> 16)),
+                           pack_bf2(v.z * bf2f(gk.y & 0xFFFF), v.w * bf2f(gk.y >> 16)));
+        }
     }
 }
 
@@ -227,7 +252,7 @@ constexpr int kPoolCtas = 8;
 // of more CTAs.
 template <int C, bool PRE>  // C: columns per thread = d / 256
 __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
-    k_final_pool(const float* __restrict__ x, const uint16_t* __restrict__ gamma, float eps,
+    k_final_pool(const float* x, const uint16_t* gamma, float eps,
                  const int* __restrict__ cu, int parts, float* __restrict__ pooled,
                  uint16_t* __restrict__ hidden) {
     pdl_entry();
@@ -248,7 +273,7 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         acc[c] = 0.f;
-        gm[c] = bf2f(gamma[tid + 256 * c]);
+        gm[c] = hidden ? bf2f(gamma[tid + 256 * c]) : 0.f;
     }
     float nx[R][C];
     auto load = [&](int t) {
@@ -256,7 +281,7 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
         for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int c = 0; c < C; ++c)
-                nx[r][c] = t + r < t1 ? __ldg(x + (size_t)(t + r) * D + tid + 256 * c) : 0.f;
+                nx[r][c] = t + r < t1 ? x[(size_t)(t + r) * D + tid + 256 * c] : 0.f;
     };
     if (PRE) load(t0);
     int buf = 0;
@@ -303,15 +328,22 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
     if (!pooled) return;
 #pragma unroll
     for (int c = 0; c < C; ++c) sums[tid + 256 * c] = acc[c];
-    cluster.sync();
     constexpr int kCols = D / kPoolCtas;  // this CTA finishes columns [part kCols, + kCols)
+    constexpr int kMine = (kCols + 255) / 256;  // of them this thread's, 256 apart
+    float gl[kMine];  // their gains, loaded before the wait for the other CTAs
+#pragma unroll
+    for (int i = 0; i < kMine; ++i)
+        gl[i] = bf2f(gamma[part * kCols + min(tid + 256 * i, kCols - 1)]);
+    cluster.sync();
     const float inv = 1.0f / (float)(r1 - r0);
-    for (int i = tid; i < kCols; i += 256) {
-        const int c = part * kCols + i;
+#pragma unroll
+    for (int i = 0; i < kMine; ++i) {
+        const int c = part * kCols + tid + 256 * i;
+        if (tid + 256 * i >= kCols) break;
         float tot = 0.f;
 #pragma unroll
         for (int k = 0; k < kPoolCtas; ++k) tot += *cluster.map_shared_rank(&sums[c], k);
-        pooled[(size_t)s * D + c] = tot * inv * bf2f(gamma[c]);
+        pooled[(size_t)s * D + c] = tot * inv * gl[i];
     }
     cluster.sync();  // no CTA's shared memory goes away while another reads it
 }
