@@ -241,23 +241,24 @@ jnx_status rmsnorm_launch(const float* x, const uint16_t* gamma, float eps, int 
 // Bound by HBM (4 bytes in, 2 out per element).  With one CTA per sample a
 // group of few samples left most SMs idle and walked each sample's rows one
 // after another.  Before and after: 7 samples of 300 rows x 4096 pooled 123
-// -> 26 us, 38 of 530 x 2048 hidden 333 -> 49 us (5.1 TB/s), 156 of 283 x
+// -> 21 us, 38 of 530 x 2048 hidden 333 -> 49 us (5.1 TB/s), 156 of 283 x
 // 1024 both 92 -> 57 us; 222 of 296 x 4096 pooled, which filled the SMs
-// already, 202 -> 214 us.
+// already, 183 both ways (5.9 TB/s).
 // ---------------------------------------------------------------------------
 constexpr int kPoolCtas = 8;
 
 // PRE: the next round's rows are loaded while this one is summed, for groups
-// whose CTAs do not fill the SMs; otherwise the registers go to longer rounds
-// of more CTAs.
+// whose CTAs do not fill the SMs; otherwise the registers go to more CTAs.  At d
+// = 4096 a round is two rows, so that three CTAs fit an SM (four rows, two CTAs:
+// 222 samples 189 us, 608 489 against 467).
 template <int C, bool PRE>  // C: columns per thread = d / 256
-__global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
+__global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256, C == 16 && !PRE ? 3 : 0)
     k_final_pool(const float* x, const uint16_t* gamma, float eps,
                  const int* __restrict__ cu, int parts, float* __restrict__ pooled,
                  uint16_t* __restrict__ hidden) {
     pdl_entry();
     constexpr int D = C * 256;
-    constexpr int R = PRE && C == 16 ? 2 : 4;  // rows of a round
+    constexpr int R = C == 16 ? 2 : 4;  // rows of a round
     __shared__ float red[2][R][8];
     __shared__ float sums[D];
     cg::cluster_group cluster = cg::this_cluster();
@@ -318,9 +319,11 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(256)
             if (t + r < t1) {
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
-                    const float y = v[r][c] * rs;
-                    acc[c] += y;
-                    if (hidden) hidden[(size_t)(t + r) * D + tid + 256 * c] = f2bf(y * gm[c]);
+                    // a stated multiply-add: left to the compiler it would be one in
+                    // some variants and two roundings in others
+                    acc[c] = fmaf(v[r][c], rs, acc[c]);
+                    if (hidden)
+                        hidden[(size_t)(t + r) * D + tid + 256 * c] = f2bf(v[r][c] * rs * gm[c]);
                 }
             }
         }
@@ -356,8 +359,8 @@ jnx_status final_pool_launch(const float* x, const uint16_t* gamma, float eps, c
     if (S > INT_MAX / parts) return fail(JNX_ERR_UNSUPPORTED, "final_pool: too many samples");
     const int grid = S * parts;
     // under four CTAs an SM the deep variant's loads hide the latency (7 x 4096:
-    // 26 us against 40), above it the flat one's longer rounds are faster (222 x
-    // 4096: 214 us against 221)
+    // 21 us against 26), above it the flat one is faster (222 x 4096: 183 us
+    // against 195; 222 of 530 x 2048: 153 against 173)
     const bool pre = grid < 4 * num_sms();
     auto launch = [&](auto deep, auto flat) {
         if (pre)
