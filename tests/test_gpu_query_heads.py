@@ -94,13 +94,17 @@ def _features(plan, d, w):
     return X, pooled, targets
 
 
-@pytest.mark.parametrize("off", [0, 2])
-@pytest.mark.parametrize("d", [512])
-def test_step_and_feature_gradient_vs_oracle(d, off):
-    w, hw, heads, plan = _setup(d, LENGTHS)
+# widths of whole 256-column tiles and not, buffers on a 16-byte boundary and not, and an
+# MLP head between two query heads
+@pytest.mark.parametrize("mlp", [False, True])
+@pytest.mark.parametrize("d,off", [(512, 0), (512, 2), (384, 0), (640, 0), (640, 2)])
+def test_step_and_feature_gradient_vs_oracle(d, off, mlp):
+    kinds = [synth.HEAD_XATTN, synth.HEAD_MLP if mlp else synth.HEAD_XATTN, synth.HEAD_XATTN]
+    w, hw, heads, plan = _setup(d, LENGTHS, kinds)
     g = R.DeviceGroup(plan)
     X, pooled, targets = _features(plan, d, w)
     preds, loss, dh = _step(heads, plan, g, X, pooled, targets, off)
+    assert torch.isfinite(dh).all()
     _check(w, hw, heads, plan, X, targets, preds, loss, dh)
 
 
