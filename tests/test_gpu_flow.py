@@ -224,6 +224,37 @@ def test_flow_grouped_equals_isolated_and_other_slots_untouched():
             assert torch.all(v[0] == 7.0) and torch.all(v[1] == 7.0), (b, k)
 
 
+def test_flow_tenant_has_the_same_bits_alone_and_among_64():
+    """A tenant's segmented products take narrow tiles alone and 256-wide ones in a
+    group of 64 (width 512, F 1,024): velocities, loss and every gradient bit for bit,
+    for tenants of one, two and nine (two tiles of rows) action chunks."""
+    counts = [1, 2, 9] + [2] * 61
+    per = [[synth.Sample(0, 3 + 7 * (i + j) % 61) for j in range(n)] for i, n in enumerate(counts)]
+    bb = synth.Backbone(n_layers=0, d=256, n_heads=4, n_kv_heads=4, head_dim=64, d_ff=1024,
+                        vision_tokens=32, vocab=100)
+    tenants = [synth.Tenant(synth.HEAD_MLP, chunk=16, action_dim=7, d_hidden=64, max_images=2)
+               for _ in per]
+    w = synth.custom_workload(bb, tenants, per, req_batch=4, seed=3)
+    s = FlowSetup(dm=512, F=1024, nb=1, C=16, D=7, d=256, std=0.03, workload=w)
+    plan = s.plan()
+    hidden = (torch.randn(plan.n_tokens, 256, generator=torch.Generator().manual_seed(5))
+              .to(torch.bfloat16).cuda())
+    inp = _inputs(plan, s.C, s.D)
+    _, vel, loss, _ = s.run(plan, hidden, inp)
+    grads = lambda: list(s.heads.grads.items()) + list(s.heads.block_grads[0].items())
+    full = {k: v.clone() for k, v in grads()}
+    for t in (0, 1, 2, 63):
+        gi = plan.slot_tenant.tolist().index(t)
+        s0, s1 = plan.seg_offsets[gi], plan.seg_offsets[gi + 1]
+        r0, r1 = plan.cu_seqlens[s0], plan.cu_seqlens[s1]
+        _, vel1, loss1, _ = s.run(s.plan([t]), hidden[r0:r1].contiguous(),
+                                  {k: v[s0:s1].contiguous() for k, v in inp.items()})
+        assert torch.equal(vel1, vel[s0:s1]), t
+        assert float(loss1[t]) == float(loss[t]), t
+        for k, v in grads():
+            assert torch.equal(v[t], full[k][t]), (t, k)
+
+
 def test_flow_gradient_accumulation():
     s = FlowSetup(nb=1)
     plan = s.plan()

@@ -5,10 +5,12 @@ tiles by its size, and a row's result must have the same bits in all of them
 import pytest
 import torch
 
+import synth
 from oracle import model as M
 from paper_2607_16074_gb300 import jnx as J
+from paper_2607_16074_gb300 import runtime as R
 from tests.gpu_helpers import f64, randn_bf16, stream
-from tests.helpers import check_bf16_out, rel_err
+from tests.helpers import check_bf16_out, oracle_requests, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -58,3 +60,73 @@ def test_rows_have_the_same_bits_in_every_tile_width(epi, hd, act, K):
         # the output format's own rounding, and beyond it (as the GLU epilogue's
         # other test) fp32 accumulation and the fast sigmoid's few units
         check_bf16_out(f64(full), want, 1e-3, f"glu {act}")
+
+
+@pytest.mark.parametrize("K", [1536, 4160])  # 1,536: lone tiles to 2,120 rows, pairs at 5,000
+def test_glu_backward_rows_have_the_same_bits_in_every_tile_form(K):
+    """The two GLU backward epilogues (256-wide tiles of one CTA or of a pair) at F =
+    2,048: dm into stored multipliers, and dm then the recomputed gate/up product."""
+    F, rows_all = 2048, 5000
+    A, W = randn_bf16((rows_all, K), 1), randn_bf16((F, K), 2, 0.05)
+    Wgu, m0 = randn_bf16((2 * F, K), 3, 0.05), randn_bf16((rows_all, 2 * F), 4)
+    L = J.lib()
+
+    def run(rows):
+        bwd = m0[:rows].clone()
+        J.check(L.jnx_op_gemm_glu_backward(A.data_ptr(), W.data_ptr(), rows, F, K, bwd.data_ptr(),
+                                           0, stream()))
+        dm = torch.full_like(bwd, float("nan"))
+        J.check(L.jnx_op_ffn_glu_backward(A.data_ptr(), W.data_ptr(), A.data_ptr(), Wgu.data_ptr(),
+                                          rows, F, K, 0, dm.data_ptr(), stream()))
+        torch.cuda.synchronize()
+        return bwd, dm
+
+    full = run(rows_all)
+    assert all(torch.isfinite(t.float()).all() for t in full)
+    for rows in (1, 17, 129, 607, 1200, 2120, 4000):
+        for got, want in zip(run(rows), full):
+            assert torch.equal(got, want[:rows]), rows
+
+
+@pytest.mark.parametrize("heads,kv,hd,lora", [(64, 8, 64, 0), (32, 4, 128, 0), (16, 2, 256, 0),
+                                              (16, 2, 256, 16), (32, 4, 128, 16)])
+def test_a_samples_rows_have_the_same_bits_alone_and_in_a_large_group(heads, kv, hd, lora):
+    """Two blocks whose norms are folded into the residual products (4,096-deep: their
+    epilogue also writes the norm's rows and sums of squares, which the RoPE and GLU
+    epilogues read), with and without adapters: tenants of few rows alone, in narrow
+    tiles, against a group of 6,000 rows, in wide ones and pairs."""
+    bb = synth.Backbone(n_layers=2, d=512, n_heads=heads, n_kv_heads=kv, head_dim=hd, d_ff=4096,
+                        vision_tokens=4, vocab=300, lora_rank=lora)
+    lengths = [[9], [100, 1], [170, 120], [596], [600] * 8]
+    tenants = [synth.Tenant(synth.HEAD_MLP, chunk=2, action_dim=3, d_hidden=64, max_images=1)
+               for _ in lengths]
+    w = synth.custom_workload(bb, tenants, [[synth.Sample(1, n) for n in t] for t in lengths],
+                              req_batch=2, seed=5)
+    weights = synth.make_backbone_weights(w)
+    weights = dict(layers=[{k: v.cuda() for k, v in lw.items()} for lw in weights["layers"]],
+                   final_norm=weights["final_norm"].cuda(),
+                   text_table=weights["text_table"].cuda())
+    inp = synth.make_inputs(w)
+    vision, text = inp["vision"].cuda(), inp["text_ids"].cuda()
+    dev = R.DeviceBackbone(bb, weights, len(tenants))
+
+    def run(wsub):
+        plan = J.jnx_group_plan(wsub.schemas(), oracle_requests(wsub), len(tenants), 1 << 30,
+                                1 << 30)
+        g = R.DeviceGroup(plan)
+        ws = torch.zeros(dev.workspace_bytes(plan.n_tokens), dtype=torch.uint8, device="cuda")
+        pooled = torch.full((plan.n_samples, bb.d), float("nan"), device="cuda")
+        hidden = torch.full((plan.n_tokens, bb.d), float("nan"), dtype=torch.bfloat16,
+                            device="cuda")
+        dev.forward(g, vision, text, pooled, hidden, ws)
+        R.check_status(ws)
+        torch.cuda.synchronize()
+        return plan, pooled, hidden
+
+    plan, pooled, hidden = run(w)
+    assert torch.isfinite(pooled).all() and torch.isfinite(hidden.float()).all()
+    seg, cu = plan.seg_offsets, plan.cu_seqlens
+    for slot, t in enumerate(plan.slot_tenant.tolist()):
+        _, p1, h1 = run(w.subset([t]))
+        assert torch.equal(p1, pooled[seg[slot]:seg[slot + 1]]), t
+        assert torch.equal(h1, hidden[cu[seg[slot]]:cu[seg[slot + 1]]]), t
