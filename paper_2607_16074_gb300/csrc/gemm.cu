@@ -1716,6 +1716,15 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
     return e;
 }
 
+// Whether tiles of bn columns hold what the launch's epilogue combines: RoPE needs a
+// tile within one head, a folded norm's sums of squares one of 128 columns; the GLU
+// backward with dm has wide tiles only.
+static bool tile_holds(int bn, const GemmParams& p) {
+    if (bn >= 256) return true;
+    const bool wide_only = p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn);
+    return !(wide_only || (p.epi == EPI_ROPE && bn > p.hd) || (p.norm_gamma && bn < 128));
+}
+
 // A launch's output tiles: the form with the least estimated time, `fixed` (the
 // launch, the first loads, the last tile's epilogue) + (rounds of tiles an SM works
 // through) x (K / 64 steps) x the step.  GB300's times in microseconds, fitted over
@@ -1726,8 +1735,7 @@ cudaError_t set_smem_limit(const void* fn, int bytes, std::atomic<uint64_t>& don
 // they divide as well over the SMs.  N 2,048 x K 16,384, in the order of the table:
 // 300 rows 92, 79, 46, 55 and 45 us; 607 rows 93, 80, 47, 56 and 73; 2,400 rows 97,
 // 169, 142, 112 and 167; and 1,000 rows x N 32,768 x K 2,048 86, 75, 86, 93 and 131.
-// RoPE needs a tile within one head, a folded norm's sums of squares one of 128
-// columns; the GLU backward with dm has wide tiles only, other operands no pairs.
+// Adapters, segments and MN-major operands have no pairs.
 constexpr int kPairTile = 512, kPairNarrow = 384;  // a pair's tiles of 256 and of 128 columns
 
 static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
@@ -1738,14 +1746,11 @@ static int pick_bn(int m_tiles, const GemmParams& p, bool pairs) {
         {128, 128, 1, 2, 5.3, 0.197, 0.395},
         {64, 64, 1, 2, 4.8, 0.156, 0.32}};
     const int sms = num_sms();
-    const bool wide_only = p.epi == EPI_GLU_DM || (p.epi == EPI_GLU_BWD && !p.seg_bn);
     int best = 256;
     double least = 1e30;
     for (const auto& f : kForms) {
         if (f.rows == 2 && !pairs) continue;
-        if (f.bn < 256 && (wide_only || (p.epi == EPI_ROPE && f.bn > p.hd) ||
-                           (p.norm_gamma && f.bn < 128)))
-            continue;
+        if (!tile_holds(f.bn, p)) continue;
         const long long tiles = (long long)((m_tiles + f.rows - 1) / f.rows) * (p.N / f.bn);
         const int slots = sms / f.rows * f.per_sm;
         const double step = tiles <= sms / f.rows ? f.alone : (tiles + slots - 1) / slots * f.busy;
@@ -1807,6 +1812,8 @@ static cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, Gem
 template <int EPI, bool LORA, class LG, int EW = 4, bool BMN = false>
 static cudaError_t launch_epi(const CUtensorMap& ta, const CUtensorMap& tb, const LG& lg,
                               const GemmParams& p, int bn, long long tiles, cudaStream_t s) {
+    // whoever picked bn: a RoPE tile wider than a head would divide by zero heads
+    if (!tile_holds(bn == kPairNarrow ? 128 : bn, p)) return cudaErrorInvalidValue;
     if constexpr (!LORA)
         if (bn == kPairTile) return launch_pair<EPI, EW, 256>(ta, tb, p, s);
     if constexpr (EW == 4) {
