@@ -589,7 +589,8 @@ def run_ours(args, rank, world, local_rank):
     gu_flops, gu_ms = float(work[gu].sum()), float(ms[gu].sum())
     gu_tf = gu_flops / (gu_ms / 1e3) / 1e12 if gu_ms > 0 else 0.0
     tr = recorded_traffic(w.name, (plan.n_tokens, w.backbone.d, w.backbone.d_ff))
-    roofline = dict(kernel="k_gemm<EPI_GLU> (tcgen05): gate/up projection + SwiGLU/GeGLU",
+    roofline = dict(kernel="k_gemm_pair<EPI_GLU> (tcgen05 on CTA pairs; k_gemm for few rows): "
+                           "gate/up projection + SwiGLU/GeGLU",
                     bound="tensor", achieved=round(gu_tf, 1), peak=peaks["bf16_sustained"],
                     unit="TFLOP/s", frac=round(gu_tf / peaks["bf16_sustained"], 4),
                     frac_of_burst=round(gu_tf / peaks["bf16"], 4),

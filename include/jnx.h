@@ -588,7 +588,9 @@ jnx_status jnx_flow_backward(const jnx_flow_head* fh, const jnx_group* g, const 
 /* Inference: from x = noise at tau = 0, n_steps Euler steps of
  * x += v(x, tau) / n_steps up to tau = 1 (the context's K/V projections are
  * computed once and reused by every step).  actions [n_samples, C, D] fp32
- * (out), packed sample order. */
+ * (out), packed sample order.  A tenant's actions have the same bits alone and
+ * in any group; a velocity here may differ from jnx_flow_forward's in its last
+ * bits (contractions of 2,048 and more are summed in another order). */
 jnx_status jnx_flow_sample(const jnx_flow_head* fh, const jnx_group* g, const uint16_t* hidden,
                            const float* noise, int32_t n_steps, float* actions, void* workspace,
                            size_t ws_bytes, void* stream);

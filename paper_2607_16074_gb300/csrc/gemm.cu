@@ -2,15 +2,16 @@
 //
 //   C[M, N] = A[M, K] . B[N, K]^T      (A = activations, B = weights [out, in])
 //
-// Five kernels share the epilogues and the order of every K reduction:
+// Four kernels, of which the first three share the epilogues and the order of every
+// K reduction:
 //   k_gemm        persistent CTAs over output tiles of 128 x 256, 128 or 64
 //                 (narrower for the fewer rows), with the per-tenant forms (LoRA
 //                 up-projections, segmented weights)
 //   k_gemm_pair   plain launches on CTA pairs (cta_group::2), tiles of 256 x 256
 //                 or 128
 //   k_gemm_batch  a table of products in one launch, either operand as it lies
-//   k_gemm_split  K over a cluster of four CTAs (the samplers' long contractions;
-//                 the one with partial sums, added in rank order)
+//   k_gemm_split  K over a cluster of four CTAs (the samplers' long contractions):
+//                 partial sums, added in rank order and stored by itself
 // pick_bn has the rule among the first two.  Warp roles:
 //   warp 0     TMA producer: A and B boxes of 64 K columns (128-byte swizzle)
 //              into a shared-memory ring (4 stages of 128 x 256), completion on
@@ -35,7 +36,8 @@
 // product times a dm already stored in the up columns).
 // Every output element's K reduction runs in the same order whatever M is
 // or where the row sits, so packed (grouped) and per-tenant runs agree
-// bit for bit.
+// bit for bit.  The split's order is another one, taken whatever the rows: an
+// expert's last bits may differ between sampling and training, not by its group.
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
