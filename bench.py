@@ -52,14 +52,13 @@ def workload_desc(w):
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one gate/up
 # GEMM launch: captured by ncu on a small launch of the same kernel whose
 # row blocks fill whole tile groups, as the full launch's do (10,240 rows),
-# and scaled by rows to the full launch (the traffic per row is the same:
-# A once, the weight once per tile group, u once; the summary and command
-# are in profiles/).  Valid only for the GEMM source it was taken on and the
+# and scaled by rows to the full launch (the mean of two launches; the summary
+# and command are in profiles/).  Valid only for the GEMM source it was taken on and the
 # launch shape it is scaled to (packed rows, width, FFN width).
 RECORDED_TRAFFIC = {
     # workload: (sha256 of csrc/gemm.cu, (rows, d, F), bytes per launch, profile)
-    "llama7b": ("8ae0084ca22eba83c00bdc18a9ece2d9956dbc2873b4f8142777cc187087ec5e",
-                (65817, 4096, 11008), (465.714176e6 + 215.440640e6) * 65817 / 10240,
+    "llama7b": ("a9f925d8610dff63ff8f8342cc072081e78f2404c5e741fd90736a0e73e06c53",
+                (65817, 4096, 11008), (640.758656e6 + 216.307072e6) * 65817 / 10240,
                 "profiles/gemm_gate_up_glu_10240_dram.md (10,240 rows, scaled by rows)"),
 }
 
